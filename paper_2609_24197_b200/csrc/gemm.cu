@@ -11,12 +11,6 @@
 //
 // Epilogues: fp32 / bf16 store, fp32 accumulate-into (residual), fp32 K-slice partial, and the
 // LM-head form that reduces each activation row's (max, index) over the CTA's 128 vocabulary rows.
-//
-// A CTA can also own TWO weight tiles (WT = 2, two accumulators in TMEM) so that one activation fill per k-step feeds
-// two MMAs: 1.5 bytes of shared-memory fill per weight byte instead of 2 at 128 activation rows.  Measured on the
-// state projection at 128 rows it changes nothing (5.55 TB/s either way: the profiler shows L2-to-SM traffic down
-// from 2.0x to 1.5x the weight bytes, DRAM at 73 % and the tensor pipe at 43 % - neither the fill nor a pipe is the
-// limit there), so it stays off unless HSPEC_GEMM_WT=2 asks for it.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -46,20 +40,16 @@ struct __align__(8) GemmSmemTail {
 
 __global__ void __launch_bounds__(192, 2)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs g) {
-#ifdef HSPEC_GEMM_CLOCK
-  const long long clk_start = clock64();     // measurement build: one CTA prints where its clocks went
-#endif
   extern __shared__ uint8_t smem_raw[];
   // 128-byte swizzle needs 1024-byte aligned tiles
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t b_stage_bytes = g.BN * TILE_K * 2;
-  const uint32_t a_stage_bytes = uint32_t(g.WT) * A_STAGE_BYTES;
-  const uint32_t stage_bytes = a_stage_bytes + b_stage_bytes;
+  const uint32_t stage_bytes = A_STAGE_BYTES + b_stage_bytes;
   GemmSmemTail* tail = reinterpret_cast<GemmSmemTail*>(smem + size_t(g.stages) * stage_bytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile_m = blockIdx.x;            // activation-row tile (fastest: CTAs sharing a weight tile run together)
-  const int tile_n = blockIdx.y;            // weight-row tile (WT consecutive 128-row tiles)
+  const int tile_n = blockIdx.y;            // 128-row weight tile
   const int split = blockIdx.z;
   const int kt_begin = split * g.k_tiles_per_split;
   const int kt_end = min(g.k_tiles_total, kt_begin + g.k_tiles_per_split);
@@ -87,9 +77,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const uint32_t tmem_acc = tail->tmem_base;
   pdl_wait();                                   // set-up done: now the previous kernel's results may be read
   pdl_trigger();
-#ifdef HSPEC_GEMM_CLOCK
-  const long long clk_setup = clock64();
-#endif
 
   if (warp == 0) {
     if (lane == 0) {
@@ -107,9 +94,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const uint32_t full = smem_u32(&tail->full[s]);
         mbar_expect_tx(full, stage_bytes);
         uint8_t* sa = smem + size_t(s) * stage_bytes;
-        for (int w = 0; w < g.WT; ++w)       // (a tile wholly past the last weight row is zero-filled by the copy)
-          tma_load_2d(smem_u32(sa + w * A_STAGE_BYTES), &tmA, (kt_begin + i) * TILE_K, (tile_n * g.WT + w) * TILE_W, full, pol_w);
-        tma_load_2d(smem_u32(sa + a_stage_bytes), &tmB, (kt_begin + i) * TILE_K, tile_m * g.BN, full, pol_x);
+        tma_load_2d(smem_u32(sa), &tmA, (kt_begin + i) * TILE_K, tile_n * TILE_W, full, pol_w);
+        tma_load_2d(smem_u32(sa + A_STAGE_BYTES), &tmB, (kt_begin + i) * TILE_K, tile_m * g.BN, full, pol_x);
       }
     }
   } else if (warp == 1) {
@@ -127,14 +113,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
         tc_fence_after();
         const uint32_t sa = smem_u32(smem + size_t(s) * stage_bytes);
-        const uint64_t db = umma_desc_kmajor_sw128(sa + a_stage_bytes);
-        for (int w = 0; w < g.WT; ++w) {
-          const uint64_t da = umma_desc_kmajor_sw128(sa + w * A_STAGE_BYTES);
+        const uint64_t da = umma_desc_kmajor_sw128(sa), db = umma_desc_kmajor_sw128(sa + A_STAGE_BYTES);
 #pragma unroll
-          for (int kk = 0; kk < TILE_K / UMMA_K; ++kk) {
-            // advancing K inside the swizzle row: +32 bytes = +2 in the descriptor's 16-byte units
-            umma_bf16(tmem_acc + uint32_t(w * g.BN), da + uint64_t(kk * 2), db + uint64_t(kk * 2), idesc, (i > 0 || kk > 0) ? 1u : 0u);
-          }
+        for (int kk = 0; kk < TILE_K / UMMA_K; ++kk) {
+          // advancing K inside the swizzle row: +32 bytes = +2 in the descriptor's 16-byte units
+          umma_bf16(tmem_acc, da + uint64_t(kk * 2), db + uint64_t(kk * 2), idesc, (i > 0 || kk > 0) ? 1u : 0u);
         }
         umma_commit(smem_u32(&tail->empty[s]));   // stage reusable once these MMAs have read it
       }
@@ -180,9 +163,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       for (int u = 0; u < 4; ++u) load_aq(aq[u], u * 16);
     }
     bool ok = mbar_wait(smem_u32(&tail->tmem_full), 0);
-#ifdef HSPEC_GEMM_CLOCK
-    const long long clk_acc = clock64();
-#endif
     if (!ok) atomicExch(g.status, STATUS_TIMEOUT_EPILOGUE);
     tc_fence_after();
     if (*reinterpret_cast<volatile uint32_t*>(&tail->abort_flag)) ok = false;
@@ -218,12 +198,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
     }
-    for (int w = 0; w < g.WT && g.mode != EPI_ARGMAX_T; ++w) {   // (WT = 2 is never combined with the arg-max epilogues)
-    const int tile_w = tile_n * g.WT + w;           // 128-row weight tile of this pass
-    const int n = tile_w * TILE_W + q * 32 + lane;  // output feature (weight row) of this thread
+    const int n = tile_n * TILE_W + q * 32 + lane;  // output feature (weight row) of this thread
     const bool n_ok = n < g.N_out;
     // Addend of the arg-max epilogue (the causal-correction head): the loads of the next 16 columns are issued before
-    // this batch is reduced.  Measured on that head's CTAs (-DHSPEC_GEMM_CLOCK; K = 256, 128 requests): the epilogue
+    // this batch is reduced.  Measured on that head's CTAs (K = 256, 128 requests): the epilogue
     // takes 23 000 of a CTA's 29 000 clocks - 10 000 with neither addend nor reduction, +6 000 for the reduction network,
     // +7 500 for the addend - and a queue of 64 loads per thread instead of 16 changes nothing: with two CTAs of four
     // epilogue warps per SM it is the warps' instruction latency, not memory, that sets the pace.
@@ -232,19 +210,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int m = m0 + c_first + j;
-#ifdef HSPEC_GEMM_NOADDEND                   // measurement build
-        add_next[j] = float(m);
-#else
         add_next[j] = (n_ok && c_first < g.BN && m < g.M) ? __ldcs(g.addend + size_t(m) * g.ld_add + n) : 0.f;
-#endif
       }
     };
     const bool with_addend = g.mode == EPI_ARGMAX && g.addend != nullptr;
     if (with_addend && ok) load_addend(0);
 
-    for (int c0 = 0; c0 < g.BN && ok; c0 += 16) {
+    for (int c0 = 0; c0 < g.BN && ok && g.mode != EPI_ARGMAX_T; c0 += 16) {
       uint32_t r[16];
-      tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(w * g.BN + c0), r);
+      tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(c0), r);
       tmem_ld_wait();
       if (g.mode == EPI_STORE_F32 || g.mode == EPI_PARTIAL_F32) {
         float* out = reinterpret_cast<float*>(g.out) + (g.mode == EPI_PARTIAL_F32 ? size_t(split) * g.M * g.ldo : 0);
@@ -275,7 +249,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __float2bfloat16_rn(__uint_as_float(r[j]));
         }
       } else if (g.mode == EPI_SWIGLU_F16 || g.mode == EPI_SWIGLU_BF16) {
-        const int f = tile_w * 64 + q * 16 + (lane & 15);
+        const int f = tile_n * 64 + q * 16 + (lane & 15);
         swiglu_store16(r, g.out, g.mode == EPI_SWIGLU_BF16, g.ldo, m0 + c0, g.M, f, 2 * f < g.N_out, lane, g.status);
       } else if (g.mode == EPI_STORE_F16) {
         __half* out = reinterpret_cast<__half*>(g.out);
@@ -299,12 +273,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = v[j];
         }
         int row = 0;
-#ifndef HSPEC_GEMM_NOARGMAX                   // measurement build
         warp_argmax16(v, vi, lane, row);
-#endif
         if ((lane & 1) == 0) { tail->red_val[q][c0 + row] = v[0]; tail->red_idx[q][c0 + row] = vi[0]; }
       }
-    }
     }
     if (g.mode == EPI_ARGMAX_T) {
       // per (column tile, request): [tile_m][N_out]
@@ -333,11 +304,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         g.part_idx[size_t(tile_n) * g.M + m] = idx;
       }
     }
-#ifdef HSPEC_GEMM_CLOCK
-    if (blockIdx.y == gridDim.y / 2 && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 64)
-      printf("gemm cta %d: set-up %lld clocks, until the accumulator is complete %lld, epilogue %lld\n", int(blockIdx.y),
-             clk_setup - clk_start, clk_acc - clk_setup, clock64() - clk_acc);
-#endif
     tc_fence_before();
   }
   __syncthreads();
@@ -524,14 +490,11 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   if (splits > g.k_tiles_total) splits = g.k_tiles_total;
   g.k_tiles_per_split = (g.k_tiles_total + splits - 1) / splits;
   splits = (g.k_tiles_total + g.k_tiles_per_split - 1) / g.k_tiles_per_split;   // no empty slice
-  // Two weight tiles per CTA: only on request (HSPEC_GEMM_WT=2, measurements), see the note at the top of the file.
-  static const int wt_env = [] { const char* e = getenv("HSPEC_GEMM_WT"); return e ? atoi(e) : 0; }();
   const int n_tiles_w = (c.n_out + TILE_W - 1) / TILE_W;
-  g.WT = (wt_env == 2 && g.BN <= 128 && c.mode != EPI_ARGMAX && c.addend == nullptr) ? 2 : 1;
   uint32_t cols = 32;
-  while (cols < uint32_t(g.WT * g.BN)) cols <<= 1;
+  while (cols < uint32_t(g.BN)) cols <<= 1;
   g.tmem_cols = cols;
-  const size_t stage_bytes = size_t(g.WT) * A_STAGE_BYTES + size_t(g.BN) * TILE_K * 2;
+  const size_t stage_bytes = A_STAGE_BYTES + size_t(g.BN) * TILE_K * 2;
   const size_t fixed = sizeof(GemmSmemTail) + 1024;
   // Weight streaming (narrow activation tile): size the ring so that TWO CTAs fit on an SM; one CTA's prologue and
   // epilogue then overlap the other's stream.  Wide tiles take the whole SM.
@@ -558,7 +521,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   }
   CUtensorMap tmB;
   if (!make_tmap_16bit_2d(&tmB, c.x, c.M, c.K, c.ldx, g.BN, c.f16, err)) return cudaErrorInvalidValue;
-  dim3 grid((c.M + g.BN - 1) / g.BN, (n_tiles_w + g.WT - 1) / g.WT, splits);
+  dim3 grid((c.M + g.BN - 1) / g.BN, n_tiles_w, splits);
   const size_t smem = size_t(stages) * stage_bytes + fixed;
   trk_begin(trk, c.label ? c.label : "gemm", 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));

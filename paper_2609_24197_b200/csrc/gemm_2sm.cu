@@ -17,9 +17,7 @@
 // operations, so it is paid once per eight MMAs instead of once per four.  (Three k-steps per stage leave room for two
 // stages only: 1 291 against 1 331 TFLOP/s on M = 2048, n_out = 25600, K = 5120.)
 //
-// Measurement builds (HSPEC_NVCC_FLAGS): -DHSPEC_GEMM2_NOLOAD (no operand is fetched), -DHSPEC_GEMM2_NOMMA (no MMA is
-// issued, stages are released unread), -DHSPEC_GEMM2_NOEPI (accumulators are not read out), -DHSPEC_GEMM2_NOSTORE (read out, not stored), -DHSPEC_GEMM2_NOARGMAX (LM-head epilogue without its reduction network), -DHSPEC_GEMM2_CLOCK (CTA 0 prints its SM clock count and the wall time); HSPEC_GEMM2_KSUB=1 in the
-// environment goes back to one k-step per stage.  On M = 2048, n_out = 25600, K = 5120, SM clocks per 256 x 256 x 16
+// On M = 2048, n_out = 25600, K = 5120, SM clocks per 256 x 256 x 16
 // instruction (the arithmetic needs 128): MMA issue alone, no barrier at all 128; one k-step per stage 167 alone and
 // 182 with loads and read-out; two k-steps per stage 146 and 160.
 #include "common.cuh"
@@ -173,10 +171,6 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   volatile uint32_t* abort_flag = &tail->abort_flag;
   pdl_wait();                                   // set-up done: now the previous kernel's results may be read
   pdl_trigger();
-#ifdef HSPEC_GEMM2_CLOCK
-  const long long clk0 = clock64();
-  const uint64_t ns0 = global_timer_ns();
-#endif
 
   if (warp == 0) {
     if (lane == 0) {
@@ -203,19 +197,12 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           }
           const int n_sub = min(g.ksub, kt_end - kt);
           const uint32_t full = smem_u32(&tail->full[s]);
-#ifdef HSPEC_GEMM2_NOLOAD
-          // measurement build: no operand is fetched, the MMAs run on whatever the stage holds (results are garbage);
-          // shows the rate of the MMA issue + epilogue alone
-          if (rank == 0) mbar_arrive(full);
-          (void)pol_w; (void)pol_x; (void)tn; (void)tm; (void)n_sub;
-#else
           if (rank == 0) mbar_expect_tx(full, 2 * uint32_t(n_sub) * sub_bytes);   // both CTAs' bytes land on the leader's barrier
           for (int sub = 0; sub < n_sub; ++sub) {
             uint8_t* sa = smem + size_t(s) * stage_bytes + size_t(sub) * sub_bytes;
             tma_load_2d_pair(smem_u32(sa), &tmA, (kt + sub) * TILE_K, tn * 256 + int(rank) * 128, full, pol_w);
             tma_load_2d_pair(smem_u32(sa + A_BYTES), &tmB, (kt + sub) * TILE_K, tm * g.BNT + int(rank) * (g.BNT / 2), full, pol_x);
           }
-#endif
         }
       }
     }
@@ -242,13 +229,9 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           for (int sub = 0; sub < n_sub; ++sub) {
             const uint32_t sa = smem_u32(smem + size_t(s) * stage_bytes + size_t(sub) * sub_bytes);
             const uint64_t da = umma_desc_kmajor_sw128(sa), db = umma_desc_kmajor_sw128(sa + A_BYTES);
-#ifndef HSPEC_GEMM2_NOMMA                   // measurement build: stages are released unread (shows the load path's own rate)
 #pragma unroll
             for (int kk = 0; kk < TILE_K / 16; ++kk)
               umma_2sm(tmem_acc, da + uint64_t(kk * 2), db + uint64_t(kk * 2), idesc, (kt > kt_begin || sub > 0 || kk > 0) ? 1u : 0u);
-#else
-            (void)da; (void)db; (void)idesc;
-#endif
           }
           umma_commit_pair(smem_u32(&tail->empty[s]));
         }
@@ -280,20 +263,11 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const bool n_ok = n < g.N_out;
       const int m0 = tm * g.BNT;
       const uint32_t tmem_acc = tmem_base + acc * uint32_t(g.BNT) + (uint32_t(q * 32) << 16);
-#ifdef HSPEC_GEMM2_NOEPI
-      const int c_first = g.BNT;                            // measurement build: the accumulator is handed back unread
-#else
-      const int c_first = 0;
-#endif
-      for (int c0 = c_first; c0 < g.BNT; c0 += 16) {
+      for (int c0 = 0; c0 < g.BNT; c0 += 16) {
         if (m0 + c0 >= g.M && mode != EPI_ARGMAX) break;    // rows past M: nothing to store (warp-uniform)
         uint32_t r[16];
         tmem_ld16(tmem_acc + uint32_t(c0), r);
         tmem_ld_wait();
-#ifdef HSPEC_GEMM2_NOSTORE                   // measurement build: the accumulator is read but nothing is written
-        if (r[0] == 0x7fc12345u && g.M < 0) g.status[0] = r[1];
-        continue;
-#endif
         if (mode == EPI_PARTIAL_F32) {
           // slice of a tail tile: [tail tile][slice][activation row of the tile][256 weight rows of the pair]
           float* out = g.part + (size_t(tile - g.n_full_tiles) * g.tail_splits + sp) * size_t(g.BNT) * 256 +
@@ -351,9 +325,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           // (The network costs the LM head 4 % - 2.34 -> 2.24 ms per step without it - mostly as clock under the power cap.
           // One redux.sync maximum + ballot per column instead of the shuffle rounds: 2.56 ms.)
           int row = 0;
-#ifndef HSPEC_GEMM2_NOARGMAX                 // measurement build: no reduction network (ids are wrong)
           warp_argmax16(v, vi, lane, row);
-#endif
           if ((lane & 1) == 0) { tail->red_val[q][c0 + row] = v[0]; tail->red_idx[q][c0 + row] = vi[0]; }
         }
       }
@@ -381,13 +353,6 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
     }
   }
-#ifdef HSPEC_GEMM2_CLOCK
-  if (blockIdx.x == 0 && threadIdx.x == 64) {
-    const long long dc = clock64() - clk0;
-    const uint64_t dn = global_timer_ns() - ns0;
-    printf("gemm_2sm cta 0: %lld SM clocks in %llu ns = %.0f MHz\n", dc, (unsigned long long)dn, double(dc) * 1e3 / double(dn));
-  }
-#endif
   tc_fence_before();
   cluster_sync_all();           // neither CTA may leave while its pair still reads its shared memory or TMEM
   if (warp == 1) {

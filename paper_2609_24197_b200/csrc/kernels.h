@@ -108,7 +108,6 @@ inline bool epi_is_swiglu(int mode) { return mode == EPI_SWIGLU_F16 || mode == E
 struct GemmArgs {       // kernel argument block
   int M, N_out, K;
   int BN;               // activation rows per CTA = UMMA N (multiple of 16, <= 256)
-  int WT;               // 128-row weight tiles per CTA (1 or 2): with 2, one activation tile fill feeds two MMAs
   int k_tiles_total, k_tiles_per_split;
   int stages;
   uint32_t tmem_cols;
