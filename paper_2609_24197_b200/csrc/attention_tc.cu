@@ -426,7 +426,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
                     is_v ? NSV : NSK);
   } else if (warp == 9) {
     // ================================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       // fp32 accumulate, bf16 x bf16, M = 128, N = 128; scores: A = Q, B = K tile, both K-major in shared memory;
       // P V: A = P from tensor memory, B = V tile (MN-major)
       const uint32_t id_qk = idesc_bf16_128x128(false), id_pv = idesc_bf16_128x128(true);

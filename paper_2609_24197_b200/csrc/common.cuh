@@ -199,6 +199,14 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
 }
 
 // ------------------------------------------------------------------ tcgen05 / TMEM
+// True in exactly one lane of a converged warp.  A role that one thread plays is entered through this and not through
+// lane == 0: with it the compiler knows that a single thread is active around the MMA instructions.
+// 2-SM GEMM, M = 2048, K = 5120: n_out = 51200 818 -> 770 us, n_out = 21664 356 -> 335 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols)
                : "memory");

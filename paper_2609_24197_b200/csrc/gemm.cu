@@ -79,7 +79,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   pdl_trigger();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // weights are streamed once per step, unless the caller runs the same matrix again right away
       const uint64_t pol_w = g.keep_w ? policy_evict_last() : policy_evict_first();
       const uint64_t pol_x = policy_evict_last();    // activations are re-read by every weight tile
@@ -99,7 +99,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = umma_idesc_m128(g.BN, g.f16 != 0);
       bool ok = true;
       for (int i = 0; i < n_kt && ok; ++i) {

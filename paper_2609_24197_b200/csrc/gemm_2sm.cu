@@ -173,7 +173,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   pdl_trigger();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // Weights at normal L2 priority, activations evict-last.  Evict-first weights ran a few percent faster in
       // short isolated runs, but ncu showed 2.4x the algorithmic DRAM reads (the clusters that share a weight tile
       // drift apart and fetch it again), and in a long power-capped step the extra DRAM traffic costs clock:
@@ -207,7 +207,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       const uint32_t idesc = idesc_m256(uint32_t(g.BNT), g.f16 != 0);
       uint32_t it = 0, tile_count = 0;
       bool ok = true;
