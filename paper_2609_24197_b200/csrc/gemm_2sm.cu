@@ -9,7 +9,8 @@
 //
 //   warp 0   TMA producer (both CTAs; both signal the LEADER CTA's "full" barrier)
 //   warp 1   TMEM allocation (both CTAs), MMA issue + commits (leader CTA only, one thread)
-//   warps 2..5  epilogue (both CTAs, their own 128 accumulator lanes)
+//   warps 2..9  epilogue (both CTAs, their own 128 accumulator lanes): two warps per TMEM lane quarter take alternate groups
+//               of 16 accumulator columns
 // No TMA load is multicast; the only cluster-wide signal is tcgen05.commit to both CTAs' barriers.
 //
 // A pipeline stage holds TWO 64-column k-steps (64 KB per CTA at 256-wide tiles, three stages): every barrier round of
@@ -32,6 +33,10 @@ namespace hspec {
 namespace {
 
 constexpr int TILE_K = 64;
+// Eight epilogue warps: with four, reading a 256-column tile out (a TMEM load, then 16 stores, per 16 columns and warp, one
+// after the other) was slow enough to show at the end of every launch.  Burst us, four -> eight warps:
+// M = 512, n_out = 28672, K = 4096 (SwiGLU) 114 -> 107; M = 2048, n_out = 51200, K = 5120 770 -> 760.
+constexpr int EPI_WARPS = 8, EPI_THREADS = 32 * EPI_WARPS, GEMM2_THREADS = 64 + EPI_THREADS;
 constexpr uint32_t A_BYTES = 128 * TILE_K * 2;     // 16 KiB: this CTA's 128 weight rows
 
 struct Gemm2Args {
@@ -116,12 +121,15 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
                ::"r"(bar), "h"(mask)
                : "memory");
 }
+__device__ __forceinline__ void red_add_f32(float* p, float v) {
+  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
 __device__ __forceinline__ uint32_t idesc_m256(uint32_t n, bool f16) {
   const uint32_t fmt = f16 ? 0u : 1u;
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((n >> 3) << 17) | ((256u >> 4) << 24);
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
 gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Gemm2Args g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -155,7 +163,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&tail->tmem_full[a]), 1);
-      mbar_init(smem_u32(&tail->tmem_empty[a]), 256);        // 128 epilogue threads of each CTA (leader's copy is used)
+      mbar_init(smem_u32(&tail->tmem_empty[a]), 2 * EPI_WARPS);   // one arrival per epilogue warp of each CTA (leader's copy is used)
     }
     tail->abort_flag = 0;
     fence_mbar_init();
@@ -263,7 +271,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const bool n_ok = n < g.N_out;
       const int m0 = tm * g.BNT;
       const uint32_t tmem_acc = tmem_base + acc * uint32_t(g.BNT) + (uint32_t(q * 32) << 16);
-      for (int c0 = 0; c0 < g.BNT; c0 += 16) {
+      for (int c0 = ((warp - 2) >> 2) * 16; c0 < g.BNT; c0 += EPI_WARPS * 4) {
         if (m0 + c0 >= g.M && mode != EPI_ARGMAX) break;    // rows past M: nothing to store (warp-uniform)
         uint32_t r[16];
         tmem_ld16(tmem_acc + uint32_t(c0), r);
@@ -282,18 +290,15 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __uint_as_float(r[j]);
           }
         } else if (mode == EPI_ACCUM_F32) {
-          // read-modify-write of the residual stream: issue the 16 loads together, then add and store
+          // Residual stream: y += acc as a reduction in the L2 (one rounding of old + acc, as in registers; every element is
+          // met once per launch, so the result does not depend on any order).  No thread waits for the old value.
+          // Burst us, loads and adds -> reductions: M = 8192, n_out = K = 4096 242 -> 227; M = 512 28.7 -> 25.2 (280 and 33.7
+          // before both this and the eight warps).
           float* out = reinterpret_cast<float*>(g.out);
-          float old[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int m = m0 + c0 + j;
-            old[j] = (n_ok && m < g.M) ? __ldcg(out + size_t(m) * g.ldo + n) : 0.f;
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = old[j] + __uint_as_float(r[j]);
+            if (n_ok && m < g.M) red_add_f32(out + size_t(m) * g.ldo + n, __uint_as_float(r[j]));
           }
         } else if (mode == EPI_SWIGLU_F16 || mode == EPI_SWIGLU_BF16) {
           const int f = tile_n128 * 64 + q * 16 + (lane & 15);
@@ -331,11 +336,12 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
       // accumulator drained: hand it back to the MMA issuer in the leader CTA
       tc_fence_before();
-      mbar_arrive_cluster(acc ? empty_leader1 : empty_leader0);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(acc ? empty_leader1 : empty_leader0);
       if (mode == EPI_ARGMAX) {
-        asm volatile("bar.sync 1, 128;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
         const int t = threadIdx.x - 64;
-        for (int c = t; c < g.BNT; c += 128) {
+        for (int c = t; c < g.BNT; c += EPI_THREADS) {
           const int m = m0 + c;
           if (m >= g.M || tile_n128 * 128 >= g.N_out) continue;   // the pair's second half may lie wholly past V
           float v = tail->red_val[0][c];
@@ -349,7 +355,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           g.part_val[size_t(tile_n128) * g.M + m] = v;
           g.part_idx[size_t(tile_n128) * g.M + m] = idx;
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");        // red_* is reused by the next tile
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");        // red_* is reused by the next tile
       }
     }
   }
@@ -512,7 +518,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   if (c.label) { const char* colon = strchr(c.label, ':'); label += colon ? colon + 1 : c.label; }
   trk_begin(trk, label.c_str(), 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));
-  cudaError_t e = launch_pdl(gemm_2sm_kernel, dim3(2 * clusters), dim3(192), smem, stream, *c.tmW, tmB, g);
+  cudaError_t e = launch_pdl(gemm_2sm_kernel, dim3(2 * clusters), dim3(GEMM2_THREADS), smem, stream, *c.tmW, tmB, g);
   trk_end(trk);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess && splits > 1) {
