@@ -41,7 +41,8 @@ constexpr uint32_t A_BYTES = 128 * TILE_K * 2;     // 16 KiB: this CTA's 128 wei
 
 struct Gemm2Args {
   int M, N_out, K;
-  int BNT;                 // activation rows per cluster tile (128 or 256); each CTA stages BNT/2
+  int BNT;                 // activation rows per cluster tile (a multiple of 32, at most 256); each CTA stages BNT/2
+  uint32_t acc_cols;       // TMEM columns per accumulator: BNT rounded up to a power of two
   int k_tiles, stages;
   int ksub;                // 64-column k-steps per pipeline stage (1 or 2): one barrier round per stage
   int n_tiles_w, n_tiles_m;
@@ -152,7 +153,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     kt_begin = (v % g.tail_splits) * g.k_tiles_per_split;
     kt_end = min(g.k_tiles, kt_begin + g.k_tiles_per_split);
   };
-  const uint32_t tmem_cols = 2u * uint32_t(g.BNT);           // two accumulators (256 or 512 columns)
+  const uint32_t tmem_cols = 2u * g.acc_cols;                // two accumulators
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
@@ -225,7 +226,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const uint32_t acc = tile_count & 1, use = tile_count >> 1;
         if (use > 0 && !mbar_wait(smem_u32(&tail->tmem_empty[acc]), (use - 1) & 1)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tmem_acc = tmem_base + acc * uint32_t(g.BNT);
+        const uint32_t tmem_acc = tmem_base + acc * g.acc_cols;
         for (int kt = kt_begin; kt < kt_end; kt += g.ksub, ++it) {
           const int s = it % g.stages;
           const uint32_t lap = it / g.stages;
@@ -270,7 +271,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const int n = tile_n128 * 128 + q * 32 + lane;
       const bool n_ok = n < g.N_out;
       const int m0 = tm * g.BNT;
-      const uint32_t tmem_acc = tmem_base + acc * uint32_t(g.BNT) + (uint32_t(q * 32) << 16);
+      const uint32_t tmem_acc = tmem_base + acc * g.acc_cols + (uint32_t(q * 32) << 16);
       for (int c0 = ((warp - 2) >> 2) * 16; c0 < g.BNT; c0 += EPI_WARPS * 4) {
         if (m0 + c0 >= g.M && mode != EPI_ARGMAX) break;    // rows past M: nothing to store (warp-uniform)
         uint32_t r[16];
@@ -434,18 +435,22 @@ bool gemm2_preferred(int M, int n_out) {
 // by a simple model: full waves of the 74 SM pairs x k-steps x cost of a k-step, plus the tail wave (k-steps / slices),
 // a fixed cost per wave (pipeline fill, the last epilogue) and, with slices, the pass that sums the partial tiles.
 // One cost unit ~ 2.2 ns (a k-step of a 256-wide pair tile = 256 units ~ 0.56 us).
+// The rows are spread evenly over the tiles, so that the last one is not mostly padding: 549 rows are three tiles of 192
+// and not of 256 (n_out = 28672, K = 4096: 134 -> 122 us; n_out = 4096, K = 14336: 70 -> 66 us).
 void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out) {
   const int tw = (n_out + 255) / 256;
   const int k_tiles = (K + TILE_K - 1) / TILE_K;
   const bool may_split = mode != EPI_ARGMAX;            // every other epilogue can be applied after the slices are summed
   double best_cost = 1e30;
   int best_bnt = 256, best_s = 1;
-  for (int bnt : {256, 128}) {
-    const int tiles = tw * ((M + bnt - 1) / bnt);
+  for (int widest = 256; widest >= 128; widest -= 32) {
+    const int nm = (M + widest - 1) / widest;
+    const int bnt = ((M + nm - 1) / nm + 31) / 32 * 32;
+    const int tiles = tw * nm;
     const int full_waves = tiles / 74, tail = tiles % 74;
-    // a 128-wide tile needs 96 B/clk of shared-memory fill per SM at full MMA rate, a 256-wide one 64 B/clk:
-    // measured, the narrow tile runs ~1.5x slower per flop
-    const double kstep = bnt * (bnt == 128 ? 1.5 : 1.0);
+    // a k-step fills 16 KB of weights and BNT x 64 bytes of activations per SM: below 256 rows it is this fill that sets the
+    // pace (measured, a 128-wide tile runs 1.5x slower per flop than a 256-wide one)
+    const double kstep = 128.0 + 0.5 * bnt;
     for (int s = 1; s <= 8; ++s) {
       if (s > 1 && (!may_split || tail == 0 || tail * s > 74 || k_tiles / s < 8)) continue;
       const int kps = (k_tiles + s - 1) / s;
@@ -458,8 +463,6 @@ void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out
       if (cost < best_cost) { best_cost = cost; best_bnt = bnt; best_s = s; }
     }
   }
-  static const int bnt_env = [] { const char* e = getenv("HSPEC_GEMM2_BNT"); return e ? atoi(e) : 0; }();   // measurements only
-  if (bnt_env == 128 || bnt_env == 256) { best_bnt = bnt_env; best_s = 1; }
   *bnt_out = best_bnt;
   *splits_out = best_s;
 }
@@ -481,6 +484,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   g.M = c.M; g.N_out = c.n_out; g.K = c.K;
   int splits = 1;
   gemm2_pick(c.M, c.n_out, c.K, c.mode, &g.BNT, &splits);
+  g.acc_cols = g.BNT > 128 ? 256 : (g.BNT > 64 ? 128 : 64);
   g.k_tiles = (c.K + TILE_K - 1) / TILE_K;
   g.n_tiles_w = (c.n_out + 255) / 256;
   g.n_tiles_m = (c.M + g.BNT - 1) / g.BNT;
