@@ -138,66 +138,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (m < g.M) asm volatile("prefetch.global.L2 [%0];" ::"l"(g.addend + size_t(m) * g.ld_add + n_w));
         }
     }
-    // EPI_ARGMAX_T: lane = request, its addends for the tile's columns are BN contiguous floats.  They do not depend on
-    // the accumulator: the first 64 are requested before the wait for it, and every group of 16 is re-filled as soon as
-    // it is used (64 loads per thread in flight; one dependent round trip per group made a CTA's epilogue 30 us).
-    float aq[4][16];
-    const int n_t = tile_n * TILE_W + q * 32 + lane;
-    const bool t_on = g.mode == EPI_ARGMAX_T && g.addend != nullptr && n_t < g.N_out;
-    auto load_aq = [&](float (&dst)[16], int c_first) {
-      const int mf = tile_m * g.BN + c_first;
-      const float* arow = g.addend + size_t(n_t) * g.ld_add + mf;
-      if (t_on && c_first < g.BN && mf + 16 <= g.M && (reinterpret_cast<uintptr_t>(arow) & 15) == 0) {
-#pragma unroll
-        for (int j4 = 0; j4 < 4; ++j4) {
-          const float4 t = __ldg(reinterpret_cast<const float4*>(arow) + j4);
-          dst[4 * j4] = t.x; dst[4 * j4 + 1] = t.y; dst[4 * j4 + 2] = t.z; dst[4 * j4 + 3] = t.w;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) dst[j] = (t_on && c_first < g.BN && mf + j < g.M) ? __ldg(arow + j) : 0.f;
-      }
-    };
-    if (g.mode == EPI_ARGMAX_T) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) load_aq(aq[u], u * 16);
-    }
     bool ok = mbar_wait(smem_u32(&tail->tmem_full), 0);
     if (!ok) atomicExch(g.status, STATUS_TIMEOUT_EPILOGUE);
     tc_fence_after();
     if (*reinterpret_cast<volatile uint32_t*>(&tail->abort_flag)) ok = false;
     const int m0 = tile_m * g.BN;
-    // EPI_ARGMAX_T: this lane's running (max, lowest column) over the tile's columns
-    float t_best = -INFINITY;
-    int t_idx = 0x7fffffff;
-    if (g.mode == EPI_ARGMAX_T) {
-      // value = acc + addend[request][vocabulary row]; the arg-max over the tile's vocabulary rows runs inside the
-      // thread (ascending columns, strict comparison: the lowest index wins ties), no shuffles
-      const bool n_ok_t = n_t < g.N_out;
-      for (int c00 = 0; c00 < g.BN && ok; c00 += 64) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c0 = c00 + u * 16;
-          if (c0 >= g.BN) break;                    // warp-uniform
-          uint32_t r[16];
-          tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(c0), r);
-          tmem_ld_wait();
-          float add[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) add[j] = aq[u][j];
-          load_aq(aq[u], c0 + 64);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            const float val = __uint_as_float(r[j]) + add[j];
-            if (n_ok_t && m < g.M) {
-              if (g.logits != nullptr) g.logits[size_t(n_t) * g.ldo + m] = val;
-              if (val > t_best) { t_best = val; t_idx = m; }
-            }
-          }
-        }
-      }
-    }
     const int n = tile_n * TILE_W + q * 32 + lane;  // output feature (weight row) of this thread
     const bool n_ok = n < g.N_out;
     // Addend of the arg-max epilogue (the causal-correction head): the loads of the next 16 columns are issued before
@@ -216,7 +161,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool with_addend = g.mode == EPI_ARGMAX && g.addend != nullptr;
     if (with_addend && ok) load_addend(0);
 
-    for (int c0 = 0; c0 < g.BN && ok && g.mode != EPI_ARGMAX_T; c0 += 16) {
+    for (int c0 = 0; c0 < g.BN && ok; c0 += 16) {
       uint32_t r[16];
       tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(c0), r);
       tmem_ld_wait();
@@ -275,14 +220,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int row = 0;
         warp_argmax16(v, vi, lane, row);
         if ((lane & 1) == 0) { tail->red_val[q][c0 + row] = v[0]; tail->red_idx[q][c0 + row] = vi[0]; }
-      }
-    }
-    if (g.mode == EPI_ARGMAX_T) {
-      // per (column tile, request): [tile_m][N_out]
-      const int n = tile_n * TILE_W + q * 32 + lane;
-      if (n < g.N_out) {
-        g.part_val[size_t(tile_m) * g.N_out + n] = ok ? t_best : -INFINITY;
-        g.part_idx[size_t(tile_m) * g.N_out + n] = ok ? t_idx : 0x7fffffff;
       }
     }
     if (g.mode == EPI_ARGMAX) {
@@ -484,7 +421,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   const int smem_optin = g_smem_optin[current_device()];
   GemmArgs g{};
   g.M = c.M; g.N_out = c.n_out; g.K = c.K;
-  g.BN = c.bn > 0 ? c.bn : gemm_pick_bn(c.M);
+  g.BN = gemm_pick_bn(c.M);
   g.k_tiles_total = (c.K + TILE_K - 1) / TILE_K;
   int splits = c.splits < 1 ? 1 : c.splits;
   if (splits > g.k_tiles_total) splits = g.k_tiles_total;

@@ -160,22 +160,15 @@ cudaError_t token_probs_launch(const float* logits, long long ld, const int* ids
   return cudaGetLastError();
 }
 
-// From 65 to 128 requests the head's GEMM runs with the operands' roles exchanged: the requests' factor rows x [B, r]
-// sit on the MMA's M side (one 128-row tile), the vocabulary matrix W_out on the N side in tiles of 128 rows, so that an
-// accumulator lane is a request and its arg-max over the tile's vocabulary rows runs inside one thread, its addends
-// 512 contiguous bytes fetched four groups ahead.  (With the vocabulary on the lanes every group of 16 columns goes
-// through a 32-shuffle reduction network and 16 separate addend loads: 23 000 of a CTA's 29 000 clocks at 128
-// requests.  Measured per step of 16 positions at 128 requests, V = 152 064, r = 256: 1.68 ms -> 1.42 ms; with 32
-// requests only a quarter of the lanes would work and the vocabulary-on-lanes form is as fast, 0.34 against 0.36 ms
-// for 8 positions.)
-constexpr int MARKOV_T_MIN_B = 65, MARKOV_T_MAX_B = 128, MARKOV_T_TILE = 128;
-
 size_t markov_workspace_bytes(int B, int Vd, int r) {
   const size_t vt = (size_t(Vd) + 127) / 128;
-  return round_up(size_t(B) * r * 2, 256) + 2 * round_up(vt * B * 4, 256) + 256;
+  return round_up(size_t(B) * r * 2, 256) + 2 * round_up(vt * B * 4, 256) + round_up(markov_chain_bytes(B), 256) + 256;
 }
 
+// Up to 128 requests all positions run in one launch (markov_chain.cu: 176 us against 452 for 8 positions at 32 requests and
+// V = 151 936, 375 against 861 for 16 positions at 96 requests and V = 32 000); above that one GEMM and one reduction per position.
 cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk, std::string* err) {
+  if (markov_chain_supported(c.B, c.Vd, c.r)) return markov_chain_launch(c, stream, trk);
   const size_t vt = (size_t(c.Vd) + 127) / 128;
   uint8_t* ws = reinterpret_cast<uint8_t*>(c.ws);
   uint16_t* x = reinterpret_cast<uint16_t*>(ws);
@@ -186,17 +179,9 @@ cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk
   trk_end(trk);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const bool transposed = c.B >= MARKOV_T_MIN_B && c.B <= MARKOV_T_MAX_B && c.W_out != nullptr;
-  CUtensorMap tm_x;
-  if (transposed && !make_tmap_16bit_2d(&tm_x, x, c.B, c.r, c.r, 128, c.f16, err)) return cudaErrorInvalidValue;
-  const size_t n_part = transposed ? (size_t(c.Vd) + MARKOV_T_TILE - 1) / MARKOV_T_TILE : vt;
   for (int i = 0; i < c.k; ++i) {
     GemmCall g{};
-    if (transposed) {
-      g.tmW = &tm_x; g.x = c.W_out; g.ldx = c.r; g.M = c.Vd; g.n_out = c.B; g.mode = EPI_ARGMAX_T; g.bn = MARKOV_T_TILE;
-    } else {
-      g.tmW = c.tmW_out; g.x = x; g.ldx = c.r; g.M = c.B; g.n_out = c.Vd; g.mode = EPI_ARGMAX;
-    }
+    g.tmW = c.tmW_out; g.x = x; g.ldx = c.r; g.M = c.B; g.n_out = c.Vd; g.mode = EPI_ARGMAX;
     g.f16 = c.f16; g.K = c.r; g.splits = 1;
     g.addend = c.logits + size_t(i) * c.ld;                 // row b of this GEMM is row b * k + i of the block's logits
     g.ld_add = (long long)c.k * c.ld;
@@ -209,7 +194,7 @@ cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk
     if (e != cudaSuccess) return e;
     trk_begin(trk, "markov_reduce");
     launch_pdl(markov_reduce_gather_kernel, dim3((c.B + 7) / 8), dim3(1024), 0, stream, (const float*)part_val, (const int*)part_idx,
-               int(n_part), c.B, c.ids, c.k, i, c.id_map, reinterpret_cast<const uint16_t*>(c.W_in), x, c.r, int(i + 1 < c.k));
+               int(vt), c.B, c.ids, c.k, i, c.id_map, reinterpret_cast<const uint16_t*>(c.W_in), x, c.r, int(i + 1 < c.k));
     trk_end(trk);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

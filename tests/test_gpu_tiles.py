@@ -1,11 +1,17 @@
 """GPU tests at the sizes where a kernel's tiling or its dispatch changes: tile edges, remainders, ends of the range."""
-import numpy as np
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
 
-hs = pytest.importorskip("paper_2609_24197_b200")
+
+@pytest.fixture(scope="module")
+def hs():
+    import paper_2609_24197_b200 as m
+    from paper_2609_24197_b200 import build
+    build.build()
+    m.load_library()
+    return m
 
 
 def _rand(shape, seed, dtype=torch.float16, std=1.0):
@@ -19,7 +25,7 @@ def _rand(shape, seed, dtype=torch.float16, std=1.0):
 @pytest.mark.parametrize("M,n_out,K", [(256, 256, 64), (257, 300, 520), (289, 1000, 512), (430, 2048, 1024), (448, 2048, 1024),
                                        (449, 512, 2048), (549, 4096, 1024), (640, 19200, 256), (1153, 1111, 264)])
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
-def test_many_row_gemm_tile_widths(M, n_out, K, kind):
+def test_many_row_gemm_tile_widths(hs, M, n_out, K, kind):
     x, w = _rand((M, K), 1), _rand((n_out, K), 2, std=0.05)
     ref = x.double() @ w.double().t()
     y = torch.zeros((M, n_out), dtype=torch.float16 if kind == "f16" else torch.float32, device="cuda")
@@ -34,3 +40,34 @@ def test_many_row_gemm_tile_widths(M, n_out, K, kind):
     bound = K * 2.0 ** -24 * mag + (2.0 ** -11 * ref.abs() + 1e-7 if kind == "f16" else 0.0)
     worst = float(((y.double() - ref).abs() / bound).max())
     assert worst <= 1.0, worst
+
+
+# requests at the edges of the one-launch form's column chunks (32 per epilogue-warp chunk, 16 per MMA step) and of its range (128);
+# vocabularies of less than a tile, of a tile and a row, and of more tiles than SMs; ranks below, at and above a 64-column box
+@pytest.mark.parametrize("B,k,Vd,r", [(1, 1, 100, 8), (16, 3, 129, 64), (17, 4, 128, 72), (32, 2, 5000, 256), (33, 5, 19200, 256),
+                                      (64, 3, 257, 136), (65, 2, 40000, 256), (96, 4, 3001, 256), (97, 2, 900, 512), (128, 5, 21000, 256),
+                                      (129, 2, 300, 64)])
+@pytest.mark.parametrize("write", [True, False])
+def test_markov_head_chunks_and_tiles(hs, B, k, Vd, r, write):
+    g = torch.Generator().manual_seed(B * 1000 + k)
+    # logits on a grid of 2^-6 and factors on a grid of 2^-4 with |x| <= 1/2: every product and sum below is exact in fp32, so the
+    # ids (planted and natural ties included, lowest index first) and the logits must match exactly
+    logits = torch.randint(-256, 257, (B * k, Vd), generator=g).float() / 64
+    logits[:, Vd // 2] = logits.max() + 1
+    logits[:, Vd // 3] = logits[:, Vd // 2]
+    W_in = (torch.randint(-8, 9, (Vd, r), generator=g).float() / 16).half()
+    W_out = (torch.randint(-8, 9, (Vd, r), generator=g).float() / 16).half()
+    last = torch.randint(0, Vd, (B,), generator=g, dtype=torch.int32)
+    d_logits, ids = logits.cuda(), torch.full((B * k,), -1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(hs.hspec_markov_workspace_bytes(B, Vd, r), dtype=torch.uint8, device="cuda")
+    hs.hspec_op_markov_head(d_logits, W_in.cuda(), W_out.cuda(), last.cuda(), None, ids, B, k, write, ws)
+    prev, want, adj = last.long().cuda(), [], []
+    for i in range(k):
+        row = logits.view(B, k, Vd)[:, i].cuda().double() + W_in.cuda()[prev].double() @ W_out.cuda().double().t()
+        prev = torch.from_numpy(row.cpu().numpy().argmax(1)).cuda()          # numpy's arg-max takes the first of equal values
+        want.append(prev)
+        adj.append(row)
+    assert torch.equal(ids.view(B, k).long(), torch.stack(want, 1))
+    expect = torch.stack(adj, 1).view(B * k, Vd).float() if write else logits.cuda()
+    assert torch.equal(d_logits, expect)
+    assert hs.hspec_op_device_status()["rc"] == 0
