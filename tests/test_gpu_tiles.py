@@ -71,3 +71,35 @@ def test_markov_head_chunks_and_tiles(hs, B, k, Vd, r, write):
     expect = torch.stack(adj, 1).view(B * k, Vd).float() if write else logits.cuda()
     assert torch.equal(d_logits, expect)
     assert hs.hspec_op_device_status()["rc"] == 0
+
+
+# states of up to 16 values per channel: the kernel's register sizes (4, 16) and what they round up, head counts per group that give
+# one, two and four heads per block, head widths that leave threads idle, blocks of positions around its chunk of eight
+@pytest.mark.parametrize("B,k,H,P,N,G,d_conv", [(2, 1, 12, 64, 4, 1, 4), (3, 8, 12, 64, 4, 4, 4), (2, 9, 6, 24, 3, 2, 3), (1, 32, 5, 128, 16, 1, 4),
+                                                (2, 17, 8, 10, 5, 1, 1), (2, 7, 4, 64, 1, 2, 2)])
+@pytest.mark.parametrize("dt_given,state", [(True, True), (False, True), (False, False)])
+def test_scan_with_a_small_state(hs, B, k, H, P, N, G, d_conv, dt_given, state):
+    import numpy as np
+    from oracle import hspec_oracle as O
+    Di, d_xBC = H * P, H * P + 2 * G * N
+    ld = Di + d_xBC + (0 if dt_given else H)
+    f32 = torch.float32
+    zx, dt_raw = _rand((B * k, ld), 1, f32), _rand((B * k, H), 2, f32) if dt_given else None
+    s0 = _rand((B, H, P, N), 3, torch.float16, 1.5) if state else None
+    conv_w, conv_b = _rand((d_xBC, d_conv), 4, f32, 0.3), _rand((d_xBC,), 5, f32, 0.02)
+    A_log, dt_bias, D = _rand((H,), 6, f32).abs(), _rand((H,), 7, f32) - 4.0, 1 + _rand((H,), 8, f32, 0.1)
+    y = torch.full((B * k, Di), float("nan"), device="cuda")
+    hs.hspec_op_mamba_scan(zx, dt_raw, s0, conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, d_conv)
+    f64 = lambda t: t.double().cpu().numpy()
+    for b in range(B):
+        rows = f64(zx)[b * k:(b + 1) * k]
+        xBC = O.conv_silu(rows[:, Di:Di + d_xBC], f64(conv_w), f64(conv_b))
+        dt, a = O.discretise(f64(dt_raw)[b * k:(b + 1) * k] if dt_given else rows[:, Di + d_xBC:], f64(dt_bias), f64(A_log))
+        S = f64(s0)[b] if state else np.zeros((H, P, N))
+        yy, _ = O.scan_sequential(S, xBC[:, :Di].reshape(k, H, P), xBC[:, Di:Di + G * N].reshape(k, G, N),
+                                  xBC[:, Di + G * N:].reshape(k, G, N), dt, a, f64(D))
+        ref = yy.reshape(k, Di) * O.silu(rows[:, :Di])
+        got = f64(y)[b * k:(b + 1) * k]
+        # fp32 arithmetic over at most 32 positions and 16 state values, SiLU with the fast exponential and division (a few ulp
+        # each): 1e-5 of the output's RMS leaves an order of magnitude
+        assert np.abs(got - ref).max() <= 1e-5 * max(1.0, np.abs(ref).max()), np.abs(got - ref).max()
