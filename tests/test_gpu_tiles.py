@@ -103,3 +103,24 @@ def test_scan_with_a_small_state(hs, B, k, H, P, N, G, d_conv, dt_given, state):
         # fp32 arithmetic over at most 32 positions and 16 state values, SiLU with the fast exponential and division (a few ulp
         # each): 1e-5 of the output's RMS leaves an order of magnitude
         assert np.abs(got - ref).max() <= 1e-5 * max(1.0, np.abs(ref).max()), np.abs(got - ref).max()
+
+
+# rows that take clusters of 8, 4, 2 and 1 blocks; vocabularies below the split, at its edges, not a multiple of four (scalar tail, and
+# rows off the 16-byte boundary)
+@pytest.mark.parametrize("M", [1, 37, 74, 148, 296])
+@pytest.mark.parametrize("V", [1, 8191, 8192, 32768, 65535])
+def test_token_probs_row_splits(hs, M, V):
+    z = _rand((M, V), M + V, torch.float32, 3.0)
+    z[:, V // 2] += 8.0
+    z[0, 0] = float("-inf")
+    if V > 1:
+        z[M - 1, :V - 1] = float("-inf")                    # all of the mass in the last share
+    ids = torch.randint(0, V, (M,), device="cuda", dtype=torch.int32)
+    ids[M - 1] = V - 1
+    p = torch.full((M,), float("nan"), device="cuda")
+    hs.hspec_op_token_probs(z, ids, p)
+    ref = torch.softmax(z.double(), 1).gather(1, ids.long()[:, None])[:, 0]
+    if V == 1:
+        ref[0] = float("nan")                               # a row of -inf only has no probabilities
+    # exponentials to 2^-21 relative (argument below 2^5, two ulp), sums of positive terms
+    assert torch.allclose(p.double(), ref, rtol=2e-5, atol=1e-30, equal_nan=True)
