@@ -9,29 +9,6 @@ namespace hspec {
 
 namespace {
 
-// Block rows: row 0 of each request is the embedding of its last token, rows 1..k-1 the mask-token
-// embedding; no positional embedding is added (paper Sec. 3.3.1).
-__global__ void embed_rows_kernel(const __nv_bfloat16* __restrict__ embed, const int32_t* __restrict__ last_token,
-                                  int mask_id, float* __restrict__ X, int k, int D) {
-  pdl_wait();
-  pdl_trigger();
-  const int m = blockIdx.x;
-  const int b = m / k, i = m % k;
-  const int tok = (i == 0) ? last_token[b] : mask_id;
-  const __nv_bfloat16* src = embed + size_t(tok) * D;
-  float* dst = X + size_t(m) * D;
-  if ((D & 3) == 0 && ((reinterpret_cast<uintptr_t>(embed) | reinterpret_cast<uintptr_t>(X)) & 15) == 0) {
-    // four elements per thread and step: 8-byte loads, 16-byte stores
-    for (int d4 = threadIdx.x; d4 < D / 4; d4 += blockDim.x) {
-      const uint2 t = __ldg(reinterpret_cast<const uint2*>(src) + d4);
-      reinterpret_cast<float4*>(dst)[d4] = make_float4(__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u),
-                                                       __uint_as_float(t.y << 16), __uint_as_float(t.y & 0xffff0000u));
-    }
-    return;
-  }
-  for (int d = threadIdx.x; d < D; d += blockDim.x) dst[d] = __bfloat162float(src[d]);
-}
-
 __device__ __forceinline__ float block_sum(float v, float* red) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -46,6 +23,22 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   const float r = red[0];
   __syncthreads();
   return r;
+}
+
+// four normalised values x * inv * gain into a row of 16-bit values (a normalised value is at most sqrt(n) |w|; the saturating
+// convert still guards a huge gain or a NaN-free overflow of x * inv)
+__device__ __forceinline__ void store_norm4(uint16_t* row, int d4, const float4& v, float inv, const float4& g, int bf16_out, uint32_t* status) {
+  uint2 out;
+  if (bf16_out) {
+    out.x = pack_bf16(v.x * inv * g.x, v.y * inv * g.y);
+    out.y = pack_bf16(v.z * inv * g.z, v.w * inv * g.w);
+  } else {
+    const __half2 lo = __halves2half2(f16_sat(v.x * inv * g.x, status), f16_sat(v.y * inv * g.y, status));
+    const __half2 hi = __halves2half2(f16_sat(v.z * inv * g.z, status), f16_sat(v.w * inv * g.w, status));
+    out.x = *reinterpret_cast<const uint32_t*>(&lo);
+    out.y = *reinterpret_cast<const uint32_t*>(&hi);
+  }
+  reinterpret_cast<uint2*>(row)[d4] = out;
 }
 
 // y = x / sqrt(mean(x^2) + eps) * w, one CTA per row, fp16 (or bf16) out.  VPT = 16-byte vectors a thread keeps in
@@ -76,19 +69,7 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restr
       if (d4 < nv) {
         // (fetching the gains together with the row, before the block-wide sum, measured slower: 27 against 23 us)
         const float4 g = reinterpret_cast<const float4*>(w)[d4];
-        // (a normalised value is at most sqrt(n) |w|; the saturating convert still guards a huge gain or a NaN-free
-        // overflow of x * inv)
-        uint2 out;
-        if (bf16_out) {
-          out.x = pack_bf16(v[i].x * inv * g.x, v[i].y * inv * g.y);
-          out.y = pack_bf16(v[i].z * inv * g.z, v[i].w * inv * g.w);
-        } else {
-          const __half2 lo = __halves2half2(f16_sat(v[i].x * inv * g.x, status), f16_sat(v[i].y * inv * g.y, status));
-          const __half2 hi = __halves2half2(f16_sat(v[i].z * inv * g.z, status), f16_sat(v[i].w * inv * g.w, status));
-          out.x = *reinterpret_cast<const uint32_t*>(&lo);
-          out.y = *reinterpret_cast<const uint32_t*>(&hi);
-        }
-        reinterpret_cast<uint2*>(yr)[d4] = out;
+        store_norm4(yr, d4, v[i], inv, g, bf16_out, status);
       }
     }
     return;
@@ -98,6 +79,58 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restr
   const float tot = block_sum(ss, red);
   const float inv = rsqrtf(tot / float(n) + eps);
   for (int d = threadIdx.x; d < n; d += blockDim.x) store_act16(yr, d, xr[d] * inv * w[d], bf16_out != 0, status);
+}
+
+// Block rows: row 0 of each request is the embedding of its last token, rows 1..k-1 the mask-token embedding; no positional
+// embedding is added (paper Sec. 3.3.1).  X gets all B*k rows (the residual stream).  Rows 1..k-1 are the same for every
+// request, so the first layer's normalised input has only B + 1 different rows: u[b] for position 0 of request b, u[B] for the
+// rest.  One block per row of X; the B + 1 blocks that own a different row also write its norm.
+template <int VPT>
+__global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ embed, const int32_t* __restrict__ last_token, int mask_id,
+                                  const float* __restrict__ w, float* __restrict__ X, void* __restrict__ u, int B, int k, int D,
+                                  float eps, uint32_t* status, int bf16_out) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ float red[32];
+  const int m = blockIdx.x;
+  const int b = m / k, i = m % k;
+  const int tok = (i == 0) ? last_token[b] : mask_id;
+  const __nv_bfloat16* src = embed + size_t(tok) * D;
+  float* dst = X + size_t(m) * D;
+  const int urow = i == 0 ? b : (m == 1 ? B : -1);              // uniform over the block
+  uint16_t* ur = reinterpret_cast<uint16_t*>(u) + size_t(urow < 0 ? 0 : urow) * D;
+  if ((D & 3) == 0 && D <= 4 * VPT * int(blockDim.x)) {
+    // four elements per thread and step, kept in registers between the two passes
+    float4 v[VPT];
+    float ss = 0.f;
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) {
+      const int d4 = threadIdx.x + j * blockDim.x;
+      const uint2 t = d4 < D / 4 ? __ldg(reinterpret_cast<const uint2*>(src) + d4) : make_uint2(0u, 0u);
+      v[j] = make_float4(__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u), __uint_as_float(t.y << 16),
+                         __uint_as_float(t.y & 0xffff0000u));
+      if (d4 < D / 4) reinterpret_cast<float4*>(dst)[d4] = v[j];
+      ss += v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
+    }
+    if (urow < 0) return;
+    const float inv = rsqrtf(block_sum(ss, red) / float(D) + eps);
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) {
+      const int d4 = threadIdx.x + j * blockDim.x;
+      if (d4 < D / 4) store_norm4(ur, d4, v[j], inv, reinterpret_cast<const float4*>(w)[d4], bf16_out, status);
+    }
+    return;
+  }
+  float ss = 0.f;
+  for (int d = threadIdx.x; d < D; d += blockDim.x) {
+    const float v = __bfloat162float(src[d]);
+    dst[d] = v;
+    ss += v * v;
+  }
+  if (urow < 0) return;
+  const float inv = rsqrtf(block_sum(ss, red) / float(D) + eps);
+  for (int d = threadIdx.x; d < D; d += blockDim.x)
+    store_act16(ur, d, __bfloat162float(src[d]) * inv * w[d], bf16_out != 0, status);
 }
 
 // Per (row, head): optional RMSNorm over dh, then rotate-half RoPE at position ctx_len + i.
@@ -306,9 +339,11 @@ int grid_for(long long total, int threads) {
 
 }  // namespace
 
-cudaError_t embed_rows_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, float* X, int B, int k,
-                              int D, cudaStream_t stream) {
-  cudaError_t e = launch_pdl(embed_rows_kernel, dim3(B * k), dim3(256), 0, stream, (const __nv_bfloat16*)embed_bf16, last_token, mask_id, X, k, D);
+cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,
+                              int B, int k, int D, float eps, cudaStream_t stream, uint32_t* status, bool bf16_out) {
+  const int threads = D <= 4 * 6 * 256 ? 256 : 512;
+  cudaError_t e = launch_pdl(embed_norm_kernel<6>, dim3(B * k), dim3(threads), 0, stream, (const __nv_bfloat16*)embed_bf16, last_token,
+                             mask_id, norm_w, X, u_16, B, k, D, eps, status, bf16_out ? 1 : 0);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

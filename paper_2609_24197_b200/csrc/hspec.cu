@@ -94,8 +94,10 @@ Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
   auto upd = [&](size_t v) { if (v > sk) sk = v; };
   upd(splitk_need(B, c.r, c.n_fuse * c.D));
   upd(splitk_need(B, d.d_S, c.r));
-  upd(splitk_need(int(M), d.d_in_proj, c.D));
-  if (c.dt_rank > 0) upd(splitk_need(int(M), d.H, c.dt_rank));
+  for (int rows : {int(M), B + 1}) {                // (the first layer's in-projection has B + 1 rows)
+    upd(splitk_need(rows, d.d_in_proj, c.D));
+    if (c.dt_rank > 0) upd(splitk_need(rows, d.H, c.dt_rank));
+  }
   upd(splitk_need(int(M), c.D, c.Di));
   upd(splitk_need(int(M), d.d_qkv, c.D));
   upd(splitk_need(int(M), c.D, c.Hq * c.dh));
@@ -543,7 +545,12 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   // element-wise launches: bracket with the tracker (name, algorithmic bytes)
 #define EW(name, bytes, call) do { trk->begin(name, 0, bytes); cudaError_t e_ = (call); trk->end(); CUDA_TRY(h, e_); } while (0)
 
-  EW("embed_rows", Md * c.D * 6, embed_rows_launch(W("embed").data, in->last_token, c.mask_id, X, B, k, c.D, st));
+  // Before the first mixer a block has no more than B + 1 different rows (every position after the first carries the mask
+  // embedding): the first layer's in-projection runs on those, and the scan reads them through its row map.  At 128 requests x 16
+  // positions of the 32B-class shapes that GEMM goes from 2048 to 129 rows.
+  const int rows0 = k > 1 ? B + 1 : B;
+  EW("embed_norm", Md * c.D * 6, embed_norm_launch(W("embed").data, in->last_token, c.mask_id, fptr("layers.0.mamba.norm"), X, U, B, k, c.D,
+                                                   c.rms_eps, st, h->d_status, bf));
   // S_init = Proj_dS(Proj_r(concat h)): once per step, shared by all layers
   const void* lh_in = LH;
   if (bf && (reinterpret_cast<uintptr_t>(in->last_hidden) & 15) == 0) {
@@ -564,22 +571,24 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   for (int l = 0; l < c.L; ++l) {
     const std::string pre = "layers." + std::to_string(l) + ".";
     // ---- Mamba-2 mixer from the injected state
-    EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(pre + "mamba.norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
-    CUDA_TRY(h, gemm(pre + "mamba.in_proj", "gemm:in_proj", U, M, EPI_STORE_F32, BIG, d.d_in_proj));
+    const int rows = l == 0 ? rows0 : M;             // rows of the mixer's input projection
+    if (l > 0) EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(pre + "mamba.norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
+    CUDA_TRY(h, gemm(pre + "mamba.in_proj", "gemm:in_proj", U, rows, EPI_STORE_F32, BIG, d.d_in_proj));
     const float* dt_raw = nullptr;
     if (c.dt_rank > 0) {
-      trk->begin("cvt_dt_cols", 0, Md * c.dt_rank * 6);
-      cvt_cols_f16_kernel<<<(M * c.dt_rank + 255) / 256, 256, 0, st>>>(BIG, d.d_in_proj, c.Di + d.d_xBC, c.dt_rank, M,
+      trk->begin("cvt_dt_cols", 0, double(rows) * c.dt_rank * 6);
+      cvt_cols_f16_kernel<<<(rows * c.dt_rank + 255) / 256, 256, 0, st>>>(BIG, d.d_in_proj, c.Di + d.d_xBC, c.dt_rank, rows,
                                                                      DTL, h->d_status, bf ? 1 : 0);
       trk->end();
       CUDA_TRY(h, cudaGetLastError());
-      CUDA_TRY(h, gemm(pre + "mamba.dt_up", "gemm:dt_up", DTL, M, EPI_STORE_F32, DT, d.H));
+      CUDA_TRY(h, gemm(pre + "mamba.dt_up", "gemm:dt_up", DTL, rows, EPI_STORE_F32, DT, d.H));
       dt_raw = DT;
     }
     ScanCall sc{};
     sc.zxbcdt = BIG; sc.ld_in = d.d_in_proj; sc.dt_raw = dt_raw; sc.s_init = SINIT;
     sc.conv_w = fptr(pre + "mamba.conv_w"); sc.conv_b = fptr(pre + "mamba.conv_b");
     sc.dt_bias = fptr(pre + "mamba.dt_bias"); sc.A_log = fptr(pre + "mamba.A_log"); sc.Dskip = fptr(pre + "mamba.Dskip");
+    sc.shared_rows = l == 0 && k > 1;
     sc.y_gated = YG; sc.B = B; sc.k = k; sc.Di = c.Di; sc.P = c.P; sc.N = c.N; sc.G = c.G; sc.d_conv = c.d_conv;
     sc.ws = ws + p.SCAN; sc.ws_bytes = p.scan_bytes;
     CUDA_TRY(h, scan_launch(sc, st, trk, &errtxt));

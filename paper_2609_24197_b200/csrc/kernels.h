@@ -217,6 +217,7 @@ struct ScanCall {
   const float *conv_w, *conv_b, *dt_bias, *A_log, *Dskip;
   float* y_gated;                   // [B*k, Di]
   int B, k, Di, P, N, G, d_conv;
+  bool shared_rows;                 // zxbcdt and dt_raw have B + 1 rows: position 0 of every request, then one row for all later positions
   void* ws;                         // optional scratch (scan_workspace_bytes): enables the three-kernel fast path
   size_t ws_bytes;
 };
@@ -224,8 +225,8 @@ size_t scan_workspace_bytes(int B, int k, int Di, int N, int G);
 cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 
 // ---- element-wise kernels (elementwise.cu)
-cudaError_t embed_rows_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, float* X, int B, int k,
-                              int D, cudaStream_t stream);
+cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,
+                              int B, int k, int D, float eps, cudaStream_t stream, uint32_t* status, bool bf16_out);
 cudaError_t rmsnorm_launch(const float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
                            uint32_t* status, bool bf16_out = false);
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,

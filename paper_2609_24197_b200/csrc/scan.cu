@@ -24,6 +24,11 @@ struct ScanArgs {
   const float *conv_w, *conv_b, *dt_bias, *A_log, *Dskip;
   float* y;
   int B, k, Di, P, N, G, H, d_conv, d_xBC;
+  int shared_rows;  // zxbcdt (and dt_raw) hold B + 1 rows: row b is position 0 of request b, row B every later position
+  // row of zxbcdt / dt_raw that belongs to position i of request b
+  __device__ __forceinline__ size_t in_row(int b, int i) const {
+    return shared_rows ? size_t(i == 0 ? b : B) : size_t(b) * k + i;
+  }
   int NP;          // padded N (row pitch of the staged state in floats)
 };
 
@@ -59,7 +64,7 @@ mamba_scan_kernel(ScanArgs a) {
     float acc = a.conv_b[ch];
     for (int j = 0; j < a.d_conv; ++j) {
       const int src = i - (a.d_conv - 1) + j;
-      if (src >= 0) acc += a.conv_w[ch * a.d_conv + j] * a.zxbcdt[(row0 + src) * a.ld_in + a.Di + ch];
+      if (src >= 0) acc += a.conv_w[ch * a.d_conv + j] * a.zxbcdt[a.in_row(b, src) * a.ld_in + a.Di + ch];
     }
     const float v = silu_f(acc);
     if (cc < P) xs[i * P + cc] = v;
@@ -70,8 +75,8 @@ mamba_scan_kernel(ScanArgs a) {
   if (tid < 32) {
     float dt = 0.f, dA = 0.f;
     if (tid < k) {
-      const float raw = a.dt_raw ? a.dt_raw[(row0 + tid) * a.H + h]
-                                 : a.zxbcdt[(row0 + tid) * a.ld_in + a.Di + a.d_xBC + h];
+      const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, tid) * a.H + h]
+                                 : a.zxbcdt[a.in_row(b, tid) * a.ld_in + a.Di + a.d_xBC + h];
       dt = softplus_f(raw + a.dt_bias[h]);
       dA = dt * (-expf(a.A_log[h]));
     }
@@ -139,7 +144,7 @@ mamba_scan_kernel(ScanArgs a) {
         float y = dec[t] * acc[t] + Dh * xs[t * P + p];
         for (int s = 0; s <= t; ++s) y += Wm[t * KMAX + s] * xs[s * P + p];
         const size_t row = row0 + t;
-        const float z = a.zxbcdt[row * a.ld_in + h * P + p];
+        const float z = a.zxbcdt[a.in_row(b, t) * a.ld_in + h * P + p];
         a.y[row * a.Di + h * P + p] = y * silu_f(z);
       }
     }
@@ -175,7 +180,7 @@ scan_small_state_kernel(ScanArgs a, int hb) {
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
       const bool ok = act && t0 + i < k;
-      const float* row = a.zxbcdt + (row0 + (ok ? t0 + i : 0)) * a.ld_in;
+      const float* row = a.zxbcdt + a.in_row(b, ok ? t0 + i : 0) * a.ld_in;
       xr[i] = ok ? __ldg(row + a.Di + ch) : 0.f;
       zr[i] = ok ? __ldg(row + ch) : 0.f;
     }
@@ -195,7 +200,7 @@ scan_small_state_kernel(ScanArgs a, int hb) {
       float acc = a.conv_b[cb];
       for (int j = 0; j < a.d_conv; ++j) {
         const int src = i - (a.d_conv - 1) + j;
-        if (src >= 0) acc += a.conv_w[cb * a.d_conv + j] * a.zxbcdt[(row0 + src) * a.ld_in + a.Di + cb];
+        if (src >= 0) acc += a.conv_w[cb * a.d_conv + j] * a.zxbcdt[a.in_row(b, src) * a.ld_in + a.Di + cb];
       }
       v = silu_f(acc);
     }
@@ -203,7 +208,7 @@ scan_small_state_kernel(ScanArgs a, int hb) {
   }
   for (int idx = tid; idx < k * hb; idx += blockDim.x) {
     const int i = idx / hb, hh = h0 + idx % hb;
-    const float raw = a.dt_raw ? a.dt_raw[(row0 + i) * a.H + hh] : a.zxbcdt[(row0 + i) * a.ld_in + a.Di + a.d_xBC + hh];
+    const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, i) * a.H + hh] : a.zxbcdt[a.in_row(b, i) * a.ld_in + a.Di + a.d_xBC + hh];
     const float dt = softplus_f(raw + a.dt_bias[hh]);
     dts[idx] = dt;
     dec[idx] = expf(dt * (-expf(a.A_log[hh])));
@@ -281,7 +286,7 @@ mamba_scan_mma_kernel(ScanArgs a) {
       float acc = a.conv_b[ch];
       for (int j = 0; j < a.d_conv; ++j) {
         const int src = i - (a.d_conv - 1) + j;
-        if (src >= 0) acc += a.conv_w[ch * a.d_conv + j] * a.zxbcdt[(row0 + src) * a.ld_in + a.Di + ch];
+        if (src >= 0) acc += a.conv_w[ch * a.d_conv + j] * a.zxbcdt[a.in_row(b, src) * a.ld_in + a.Di + ch];
       }
       v = silu_f(acc);
     }
@@ -300,8 +305,8 @@ mamba_scan_mma_kernel(ScanArgs a) {
   {
     float dt = 0.f, dA = 0.f;
     if (lane < k) {
-      const float raw = a.dt_raw ? a.dt_raw[(row0 + lane) * a.H + h]
-                                 : a.zxbcdt[(row0 + lane) * a.ld_in + a.Di + a.d_xBC + h];
+      const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, lane) * a.H + h]
+                                 : a.zxbcdt[a.in_row(b, lane) * a.ld_in + a.Di + a.d_xBC + h];
       dt = softplus_f(raw + a.dt_bias[h]);
       dA = dt * (-expf(a.A_log[h]));
     }
@@ -401,7 +406,7 @@ mamba_scan_mma_kernel(ScanArgs a) {
 #pragma unroll
       for (int j = 0; j < NT; ++j) {
         const int col = h * P + j * 8 + tq * 2;
-        const float2 z = *reinterpret_cast<const float2*>(a.zxbcdt + row * a.ld_in + col);
+        const float2 z = *reinterpret_cast<const float2*>(a.zxbcdt + a.in_row(b, t) * a.ld_in + col);
         *reinterpret_cast<float2*>(a.y + row * a.Di + col) = make_float2(y[j][0] * silu_f(z.x), y[j][1] * silu_f(z.y));
       }
     }
@@ -457,7 +462,7 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
   for (int j = 0; j < CONV_ROWS + 3; ++j) {
     const int i = i0 - 3 + j;
     const bool ok = i >= 0 && i < a.k;
-    const float* src = a.zxbcdt + (row0 + (ok ? i : 0)) * a.ld_in + a.Di + ch;
+    const float* src = a.zxbcdt + a.in_row(b, ok ? i : 0) * a.ld_in + a.Di + ch;
     if (VEC == 4) {
       const float4 t = ok ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
       in[j][0] = t.x; in[j][VEC > 1 ? 1 : 0] = t.y; in[j][VEC > 1 ? 2 : 0] = t.z; in[j][VEC > 1 ? 3 : 0] = t.w;
@@ -579,7 +584,7 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
   // ---- dt, inclusive prefix sum of dt * A over the block positions (one warp shuffle scan per head)
   float dt = 0.f, dA = 0.f;
   if (lane < k) {
-    const float raw = a.dt_raw ? a.dt_raw[(row0 + lane) * a.H + h] : a.zxbcdt[(row0 + lane) * a.ld_in + a.Di + a.d_xBC + h];
+    const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, lane) * a.H + h] : a.zxbcdt[a.in_row(b, lane) * a.ld_in + a.Di + a.d_xBC + h];
     dt = softplus_f(raw + a.dt_bias[h]);
     dA = dt * (-expf(a.A_log[h]));
   }
@@ -689,7 +694,7 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
       const size_t row = row0 + t;
       float2 z[NT];
 #pragma unroll
-      for (int j = 0; j < NT; ++j) z[j] = *reinterpret_cast<const float2*>(a.zxbcdt + row * a.ld_in + h * P + j * 8 + tq * 2);
+      for (int j = 0; j < NT; ++j) z[j] = *reinterpret_cast<const float2*>(a.zxbcdt + a.in_row(b, t) * a.ld_in + h * P + j * 8 + tq * 2);
 #pragma unroll
       for (int j = 0; j < NT; ++j)
         *reinterpret_cast<float2*>(a.y + row * a.Di + h * P + j * 8 + tq * 2) =
@@ -726,6 +731,7 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   a.conv_w = c.conv_w; a.conv_b = c.conv_b; a.dt_bias = c.dt_bias; a.A_log = c.A_log; a.Dskip = c.Dskip;
   a.y = c.y_gated; a.B = c.B; a.k = c.k; a.Di = c.Di; a.P = c.P; a.N = c.N; a.G = c.G; a.H = c.Di / c.P;
   a.d_conv = c.d_conv; a.d_xBC = c.Di + 2 * c.G * c.N;
+  a.shared_rows = c.shared_rows ? 1 : 0;
   a.NP = c.N + 1;                                    // odd pitch: threads of a warp own consecutive p
   if (a.H % c.G) { if (err) *err = "scan: heads must divide into groups"; return cudaErrorInvalidValue; }
   // serving shapes: tensor-core path (needs 8-byte aligned rows for the float2 accesses)

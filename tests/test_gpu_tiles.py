@@ -124,3 +124,17 @@ def test_token_probs_row_splits(hs, M, V):
         ref[0] = float("nan")                               # a row of -inf only has no probabilities
     # exponentials to 2^-21 relative (argument below 2^5, two ulp), sums of positive terms
     assert torch.allclose(p.double(), ref, rtol=2e-5, atol=1e-30, equal_nan=True)
+
+
+# the first layer's in-projection runs on B + 1 rows: one request, a block of one position (no shared row), a row count that crosses
+# into the many-row kernel (257) while the block has more, low-rank dt
+@pytest.mark.parametrize("B,k,over", [(1, 2, dict()), (3, 1, dict()), (256, 2, dict()), (4, 3, dict(dt_rank=16, N=16)), (2, 4, dict(N=32))])
+def test_step_with_shared_first_layer_rows(hs, B, k, over):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(dict(D=256, n_fuse=1, r=256, L=2, has_attn=[1, 0], kv_slot=[0, -1], n_slots=1, Di=512, P=64, N=128, G=1,
+                                  d_conv=4, dt_rank=0, Hq=4, Hkv=2, dh=64, rope_theta=1.0e4, window=0, qk_norm=1, F=512, V=600,
+                                  rms_eps=1e-6, page_size=16, name="rows", B=B, k=k, ctx=("const", 20, 20)), **over))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[5 + (b % 30) for b in range(B)])
+    check_step(cfg, drafter, w, batch, k, requests=sorted({0, B // 2, B - 1}), what=f"rows {B} {k} {over}")
+    drafter.close()
