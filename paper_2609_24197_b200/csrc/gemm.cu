@@ -9,8 +9,14 @@
 //   warp 1 : allocates TMEM, issues tcgen05.mma (one elected thread), commits stages back
 //   warps 2..5 : epilogue, one TMEM lane quarter each: tcgen05.ld -> registers -> global
 //
-// Epilogues: fp32 / bf16 store, fp32 accumulate-into (residual), fp32 K-slice partial, and the
-// LM-head form that reduces each activation row's (max, index) over the CTA's 128 vocabulary rows.
+// Epilogues: fp32 / fp16 / bf16 store, fp32 accumulate-into (residual), SwiGLU, and the LM-head form that reduces each
+// activation row's (max, index) over the CTA's 128 vocabulary rows.
+//
+// K-slices: where a matrix has fewer tiles than the chip has SMs, the slices of a tile are the CTAs of one cluster.  Each leaves
+// its accumulator in its own shared memory (the ring is free by then), and each sums its share of the columns over all of them
+// through distributed shared memory, in slice order (deterministic), and applies the epilogue.  (Slices written to global memory and
+// summed by a second kernel cost a launch and a pass each: 11 of a one-request step's 51 launches.  16 rows, residual epilogue, back
+// to back: n_out 4096, K 4096 13.9 -> 11.0 us, K 14336 28.7 -> 21.6 us; 128 rows, K 8192 36.8 -> 20.2 us.)
 #include "common.cuh"
 #include "kernels.h"
 
@@ -50,7 +56,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile_m = blockIdx.x;            // activation-row tile (fastest: CTAs sharing a weight tile run together)
   const int tile_n = blockIdx.y;            // 128-row weight tile
-  const int split = blockIdx.z;
+  const int split = blockIdx.z, n_splits = gridDim.z;      // the slices of a tile form one cluster
   const int kt_begin = split * g.k_tiles_per_split;
   const int kt_end = min(g.k_tiles_total, kt_begin + g.k_tiles_per_split);
   const int n_kt = kt_end - kt_begin;       // >= 1 by construction of the grid
@@ -145,6 +151,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const int m0 = tile_m * g.BN;
     const int n = tile_n * TILE_W + q * 32 + lane;  // output feature (weight row) of this thread
     const bool n_ok = n < g.N_out;
+    if (n_splits > 1) {
+      // this slice's accumulator -> this CTA's shared memory, [column][128 weight rows] (every stage of the ring has been read)
+      float* mine = reinterpret_cast<float*>(smem) + q * 32 + lane;
+      for (int c0 = 0; c0 < g.BN; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(c0), r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) mine[(c0 + j) * TILE_W] = ok ? __uint_as_float(r[j]) : 0.f;
+      }
+    }
     // Addend of the arg-max epilogue (the causal-correction head): the loads of the next 16 columns are issued before
     // this batch is reduced.  Measured on that head's CTAs (K = 256, 128 requests): the epilogue
     // takes 23 000 of a CTA's 29 000 clocks - 10 000 with neither addend nor reduction, +6 000 for the reduction network,
@@ -161,30 +178,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool with_addend = g.mode == EPI_ARGMAX && g.addend != nullptr;
     if (with_addend && ok) load_addend(0);
 
-    for (int c0 = 0; c0 < g.BN && ok; c0 += 16) {
+    for (int c0 = 0; c0 < g.BN && ok && n_splits == 1; c0 += 16) {
       uint32_t r[16];
       tmem_ld16(tmem_acc + (uint32_t(q * 32) << 16) + uint32_t(c0), r);
       tmem_ld_wait();
-      if (g.mode == EPI_STORE_F32 || g.mode == EPI_PARTIAL_F32) {
-        float* out = reinterpret_cast<float*>(g.out) + (g.mode == EPI_PARTIAL_F32 ? size_t(split) * g.M * g.ldo : 0);
+      if (g.mode == EPI_STORE_F32) {
+        float* out = reinterpret_cast<float*>(g.out);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const int m = m0 + c0 + j;
           if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __uint_as_float(r[j]);
         }
       } else if (g.mode == EPI_ACCUM_F32) {
-        // read-modify-write of the residual stream: issue the 16 loads together, then add and store
+        // residual stream: y += acc as a reduction in the L2, no thread waits for the old value
         float* out = reinterpret_cast<float*>(g.out);
-        float old[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const int m = m0 + c0 + j;
-          old[j] = (n_ok && m < g.M) ? __ldcg(out + size_t(m) * g.ldo + n) : 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int m = m0 + c0 + j;
-          if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = old[j] + __uint_as_float(r[j]);
+          if (n_ok && m < g.M) red_add_f32(out + size_t(m) * g.ldo + n, __uint_as_float(r[j]));
         }
       } else if (g.mode == EPI_STORE_BF16) {
         __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(g.out);
@@ -243,60 +254,56 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
     tc_fence_before();
   }
-  __syncthreads();
+  if (n_splits > 1) {
+    cluster_sync_all();                             // every slice's accumulator lies in its CTA's shared memory
+    // CTA `split` finishes the columns split, split + n_splits, ...: four groups of 32 weight rows x the warps 2..5
+    if (warp >= 2) {
+      const int q = warp & 3;
+      const int n = tile_n * TILE_W + q * 32 + lane;
+      const bool n_ok = n < g.N_out;
+      const uint32_t base = smem_u32(smem) + uint32_t(q * 32 + lane) * 4;
+      constexpr int U = 4;                          // columns in flight
+      uint32_t peer[GEMM_MAX_SPLITS];
+#pragma unroll
+      for (int s = 0; s < GEMM_MAX_SPLITS; ++s) peer[s] = s < n_splits ? mapa_rank(base, uint32_t(s)) : 0u;
+      for (int c0 = split; c0 < g.BN && tile_m * g.BN + c0 < g.M; c0 += U * n_splits) {
+        float v[U][GEMM_MAX_SPLITS];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int s = 0; s < GEMM_MAX_SPLITS; ++s) {
+            const int c = c0 + u * n_splits;
+            v[u][s] = (s < n_splits && c < g.BN) ? ld_cluster_f32(peer[s] + uint32_t(c) * (TILE_W * 4)) : 0.f;
+          }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int c = c0 + u * n_splits, m = tile_m * g.BN + c;
+          if (c >= g.BN || m >= g.M) break;         // warp-uniform
+          float acc = v[u][0];
+#pragma unroll
+          for (int s = 1; s < GEMM_MAX_SPLITS; ++s)
+            if (s < n_splits) acc += v[u][s];
+          const size_t o = size_t(m) * g.ldo + n;
+          if (epi_is_swiglu(g.mode)) {
+            const float up = __shfl_xor_sync(0xffffffffu, acc, 16);       // lanes l and l + 16 hold gate and up of one feature
+            const int f = tile_n * 64 + q * 16 + lane;
+            if (lane < 16 && 2 * f < g.N_out) store_act16(g.out, size_t(m) * g.ldo + f, silu_f(acc) * up, g.mode == EPI_SWIGLU_BF16, g.status);
+          } else if (n_ok) {
+            if (g.mode == EPI_STORE_F32) reinterpret_cast<float*>(g.out)[o] = acc;
+            else if (g.mode == EPI_ACCUM_F32) red_add_f32(reinterpret_cast<float*>(g.out) + o, acc);
+            else if (g.mode == EPI_STORE_F16) reinterpret_cast<__half*>(g.out)[o] = f16_sat(acc, g.status);
+            else reinterpret_cast<__nv_bfloat16*>(g.out)[o] = __float2bfloat16_rn(acc);
+          }
+        }
+      }
+    }
+    cluster_sync_all();                             // no CTA leaves while another still reads its shared memory
+  } else {
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_acc, tmem_cols);
-  }
-}
-
-// Sum the K-slice partials in slice order (deterministic) and apply the final store.
-__global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, int M, int N, void* out,
-                                     long long ldo, int mode, uint32_t* status) {
-  pdl_wait();
-  pdl_trigger();
-  const long long total = (long long)M * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int m = int(i / N), n = int(i % N);
-    float acc = 0.f;
-    for (int s = 0; s < splits; ++s) acc += part[(size_t(s) * M + m) * N + n];
-    if (mode == EPI_STORE_F32) reinterpret_cast<float*>(out)[size_t(m) * ldo + n] = acc;
-    else if (mode == EPI_ACCUM_F32) reinterpret_cast<float*>(out)[size_t(m) * ldo + n] += acc;
-    else if (mode == EPI_STORE_F16) reinterpret_cast<__half*>(out)[size_t(m) * ldo + n] = f16_sat(acc, status);
-    else if (mode == EPI_SWIGLU_F16 || mode == EPI_SWIGLU_BF16) {
-      // n runs over interleaved rows; lower half of each 32-row block = gate, upper half = up of the same 16 features
-      if ((n & 31) < 16) {
-        float up = 0.f;
-        for (int s = 0; s < splits; ++s) up += part[(size_t(s) * M + m) * N + n + 16];
-        const int f = (n >> 5) * 16 + (n & 15);
-        store_act16(out, size_t(m) * ldo + f, silu_f(acc) * up, mode == EPI_SWIGLU_BF16, status);
-      }
-    }
-    else reinterpret_cast<__nv_bfloat16*>(out)[size_t(m) * ldo + n] = __float2bfloat16_rn(acc);
-  }
-}
-
-// The same for fp32 outputs whose row length and pitch are multiples of four: 16-byte loads and stores, one row
-// per blockIdx.y, every slice's load issued before the first add.
-template <int SPLITS>
-__global__ void splitk_reduce_f32x4_kernel(const float* __restrict__ part, int M, int N, float* __restrict__ out,
-                                           long long ldo, int accumulate) {
-  pdl_wait();
-  pdl_trigger();
-  const int m = blockIdx.y;
-  const size_t slice = size_t(M) * N;
-  for (int n4 = blockIdx.x * blockDim.x + threadIdx.x; n4 < (N >> 2); n4 += gridDim.x * blockDim.x) {
-    float4 v[SPLITS];
-#pragma unroll
-    for (int s = 0; s < SPLITS; ++s) v[s] = __ldcs(reinterpret_cast<const float4*>(part + s * slice + size_t(m) * N) + n4);
-    float4* dst = reinterpret_cast<float4*>(out + size_t(m) * ldo) + n4;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 old = accumulate ? *dst : acc;
-#pragma unroll
-    for (int s = 0; s < SPLITS; ++s) { acc.x += v[s].x; acc.y += v[s].y; acc.z += v[s].z; acc.w += v[s].w; }
-    if (accumulate) { acc.x = old.x + acc.x; acc.y = old.y + acc.y; acc.z = old.z + acc.z; acc.w = old.w + acc.w; }
-    *dst = acc;
   }
 }
 
@@ -395,15 +402,11 @@ int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode) {
   const int k_tiles = (K + TILE_K - 1) / TILE_K;
   const int tiles = ((n_out + TILE_W - 1) / TILE_W) * ((M + 255) / 256);
   if (tiles >= num_sms || k_tiles < 8) return 1;
-  int want = (2 * num_sms + tiles - 1) / tiles;
+  int want = 2 * num_sms / tiles;           // one wave of two CTAs per SM
   int max_by_k = k_tiles / 4;               // at least 4 K-tiles per slice
   int s = want < max_by_k ? want : max_by_k;
-  if (s > 16) s = 16;
+  if (s > GEMM_MAX_SPLITS) s = GEMM_MAX_SPLITS;
   return s < 1 ? 1 : s;
-}
-
-size_t gemm_splitk_bytes(int M, int n_out, int splits) {
-  return splits > 1 ? size_t(splits) * M * n_out * sizeof(float) : 0;
 }
 
 // Launches y = x W^T.  tmW must describe W with box rows 128; x is described here (box rows BN).
@@ -423,7 +426,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   g.M = c.M; g.N_out = c.n_out; g.K = c.K;
   g.BN = gemm_pick_bn(c.M);
   g.k_tiles_total = (c.K + TILE_K - 1) / TILE_K;
-  int splits = c.splits < 1 ? 1 : c.splits;
+  int splits = c.splits < 1 ? 1 : (c.splits > GEMM_MAX_SPLITS ? GEMM_MAX_SPLITS : c.splits);
   if (splits > g.k_tiles_total) splits = g.k_tiles_total;
   g.k_tiles_per_split = (g.k_tiles_total + splits - 1) / splits;
   splits = (g.k_tiles_total + g.k_tiles_per_split - 1) / g.k_tiles_per_split;   // no empty slice
@@ -446,52 +449,21 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   g.logits = c.logits; g.addend = c.addend; g.ld_add = c.ld_add; g.part_val = c.part_val; g.part_idx = c.part_idx;
   g.keep_w = c.keep_weights_in_l2 ? 1 : 0;
   g.ldo = c.ldo;
-  if (splits > 1) {
-    if (c.mode == EPI_ARGMAX) { if (err) *err = "LM-head epilogue cannot be K-sliced"; return cudaErrorInvalidValue; }
-    if (c.splitk_ws == nullptr || c.splitk_ws_bytes < gemm_splitk_bytes(c.M, c.n_out, splits)) {
-      if (err) *err = "K-slice workspace too small";
-      return cudaErrorInvalidValue;
-    }
-    g.mode = EPI_PARTIAL_F32; g.out = c.splitk_ws; g.ldo = c.n_out;
-  } else {
-    g.mode = c.mode; g.out = c.out;
+  if (splits > 1 && c.mode == EPI_ARGMAX) { if (err) *err = "LM-head epilogue cannot be K-sliced"; return cudaErrorInvalidValue; }
+  if (splits > 1 && size_t(stages) * stage_bytes < size_t(g.BN) * TILE_W * 4) {
+    if (err) *err = "K-slices: the accumulator does not fit where the pipeline was";
+    return cudaErrorInvalidValue;
   }
+  g.mode = c.mode; g.out = c.out;
   CUtensorMap tmB;
   if (!make_tmap_16bit_2d(&tmB, c.x, c.M, c.K, c.ldx, g.BN, c.f16, err)) return cudaErrorInvalidValue;
   dim3 grid((c.M + g.BN - 1) / g.BN, n_tiles_w, splits);
   const size_t smem = size_t(stages) * stage_bytes + fixed;
   trk_begin(trk, c.label ? c.label : "gemm", 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));
-  cudaError_t e = launch_pdl(gemm_tcgen05_kernel, grid, dim3(192), smem, stream, *c.tmW, tmB, g);
+  cudaError_t e = launch_pdl_cluster(gemm_tcgen05_kernel, grid, dim3(192), dim3(1, 1, splits), smem, stream, *c.tmW, tmB, g);
   trk_end(trk);
-  if (e == cudaSuccess) e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (splits > 1)
-    e = splitk_reduce_launch(reinterpret_cast<const float*>(c.splitk_ws), splits, c.M, c.n_out, c.out, c.ldo, c.mode, stream, trk,
-                             c.status);
-  return e;
-}
-
-cudaError_t splitk_reduce_launch(const float* part, int splits, int M, int N, void* out, long long ldo, int mode,
-                                 cudaStream_t stream, Tracker* trk, uint32_t* status) {
-  const long long total = (long long)M * N;
-  trk_begin(trk, "splitk_reduce", 0, double(splits + 1) * M * N * 4);
-  const bool f32 = mode == EPI_STORE_F32 || mode == EPI_ACCUM_F32;
-  if (f32 && (N & 3) == 0 && (ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0 && splits >= 2 && splits <= 4) {
-    // (the sum order s = 0, 1, ... and "old + sum" match the generic kernel bit for bit)
-    dim3 grid((N / 4 + 255) / 256, M);
-    float* o = reinterpret_cast<float*>(out);
-    const int acc = mode == EPI_ACCUM_F32;
-    if (splits == 2) launch_pdl(splitk_reduce_f32x4_kernel<2>, grid, dim3(256), 0, stream, part, M, N, o, ldo, acc);
-    else if (splits == 3) launch_pdl(splitk_reduce_f32x4_kernel<3>, grid, dim3(256), 0, stream, part, M, N, o, ldo, acc);
-    else launch_pdl(splitk_reduce_f32x4_kernel<4>, grid, dim3(256), 0, stream, part, M, N, o, ldo, acc);
-  } else {
-    int blocks = int((total + 255) / 256);
-    if (blocks > 148 * 8) blocks = 148 * 8;
-    launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, part, splits, M, N, out, ldo, mode, status);
-  }
-  trk_end(trk);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t argmax_reduce_launch(const float* pv, const int* pi, int n_tiles, int M, int* ids, cudaStream_t stream,

@@ -60,10 +60,7 @@ struct Plan {
   int attn_chunk, max_ctx;
 };
 
-size_t splitk_need(int M, int n_out, int K) {
-  if (gemm2_preferred(M, n_out)) return gemm2_tail_bytes();
-  return gemm_splitk_bytes(M, n_out, gemm_pick_splits(M, n_out, K, kNumSMs));
-}
+size_t splitk_need(int M, int n_out) { return gemm2_preferred(M, n_out) ? gemm2_tail_bytes() : 0; }
 
 Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
   const Dims d = dims_of(c);
@@ -92,17 +89,15 @@ Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
   p.ATT = take(p.att_bytes);
   size_t sk = 0;
   auto upd = [&](size_t v) { if (v > sk) sk = v; };
-  upd(splitk_need(B, c.r, c.n_fuse * c.D));
-  upd(splitk_need(B, d.d_S, c.r));
+  upd(splitk_need(B, c.r));
+  upd(splitk_need(B, d.d_S));
   for (int rows : {int(M), B + 1}) {                // (the first layer's in-projection has B + 1 rows)
-    upd(splitk_need(rows, d.d_in_proj, c.D));
-    if (c.dt_rank > 0) upd(splitk_need(rows, d.H, c.dt_rank));
+    upd(splitk_need(rows, d.d_in_proj));
+    if (c.dt_rank > 0) upd(splitk_need(rows, d.H));
   }
-  upd(splitk_need(int(M), c.D, c.Di));
-  upd(splitk_need(int(M), d.d_qkv, c.D));
-  upd(splitk_need(int(M), c.D, c.Hq * c.dh));
-  upd(splitk_need(int(M), 2 * c.F, c.D));
-  upd(splitk_need(int(M), c.D, c.F));
+  upd(splitk_need(int(M), c.D));
+  upd(splitk_need(int(M), d.d_qkv));
+  upd(splitk_need(int(M), 2 * c.F));
   p.splitk_bytes = sk;
   p.SPLITK = take(sk);
   const size_t vt = 2 * ((size_t(d.Vd) + 255) / 256);   // 128-row tiles, in pairs (the 2-SM kernel's indexing)
@@ -713,7 +708,7 @@ int hspec_get_profile(hspec_handle* h, hspec_prof_entry* out, int32_t max_entrie
   } while (0)
 
 size_t hspec_gemm_workspace_bytes(int32_t M, int32_t n_out, int32_t K) {
-  return gemm_splitk_bytes(M, n_out, 16) + gemm2_tail_bytes() + size_t((n_out + 127) / 128) * M * 8 + 2048;
+  return gemm2_tail_bytes() + size_t((n_out + 127) / 128) * M * 8 + 2048;
 }
 
 int hspec_op_gemm(const void* x, const void* Wt, int32_t in_dtype, void* y, int32_t M, int32_t n_out, int32_t K, int64_t ldy,

@@ -12,6 +12,7 @@
 namespace hspec {
 
 constexpr int GEMM_MAX_STAGES = 8;
+constexpr int GEMM_MAX_SPLITS = 8;       // K-slices of the one-CTA GEMM = CTAs of a cluster (8 is the portable limit)
 
 // Records the message hspec_last_error(NULL) returns (calling thread).
 void set_last_error(const std::string& msg);
@@ -91,17 +92,33 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// The same with the grid's CTAs in clusters of the given shape.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, dim3 cluster, size_t smem, cudaStream_t stream, Args&&... args) {
+  if (cluster.x * cluster.y * cluster.z == 1) return launch_pdl(kernel, grid, block, smem, stream, args...);
+  static const bool off = [] { const char* e = getenv("HSPEC_NO_PDL"); return e && e[0] == '1'; }();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = off ? 0 : 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster.x; at[1].val.clusterDim.y = cluster.y; at[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
 enum GemmEpilogue : int {
   EPI_STORE_F32 = 0,    // y fp32 = acc
   EPI_STORE_BF16 = 1,   // y bf16 = acc
   EPI_ACCUM_F32 = 2,    // y fp32 += acc   (residual)
-  EPI_PARTIAL_F32 = 3,  // K-slice partial (internal)
+  EPI_PARTIAL_F32 = 3,  // K-slice partial of the 2-SM kernel (internal)
   EPI_ARGMAX = 4,
   EPI_STORE_F16 = 5,    // y fp16 = acc
   EPI_SWIGLU_F16 = 6,   // weight rows interleaved in blocks of 16 (gate | up): h fp16 [M, n_out/2] = SiLU(gate) * up
   EPI_SWIGLU_BF16 = 7,  // the same with h stored as bf16
 };
-inline bool epi_is_swiglu(int mode) { return mode == EPI_SWIGLU_F16 || mode == EPI_SWIGLU_BF16; }
+__host__ __device__ inline bool epi_is_swiglu(int mode) { return mode == EPI_SWIGLU_F16 || mode == EPI_SWIGLU_BF16; }
 
 struct GemmArgs {       // kernel argument block
   int M, N_out, K;
@@ -148,13 +165,10 @@ bool make_tmap_16bit_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t
                        int box_rows, bool f16, std::string* err);
 int gemm_pick_bn(int M);
 int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode = EPI_STORE_F32);
-size_t gemm_splitk_bytes(int M, int n_out, int splits);
 cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool gemm2_preferred(int M, int n_out);        // many rows and at least one full round of cluster tiles
 size_t gemm2_tail_bytes();                     // scratch the 2-SM kernel's K-sliced tail wave may use
 void gemm2_pick(int M, int n_out, int K, int mode, int* bnt, int* splits);   // tile width and K-slices of the 2-SM kernel
-cudaError_t splitk_reduce_launch(const float* part, int splits, int M, int N, void* out, long long ldo, int mode,
-                                 cudaStream_t stream, Tracker* trk, uint32_t* status);
 cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 cudaError_t argmax_reduce_launch(const float* pv, const int* pi, int n_tiles, int M, int* ids, cudaStream_t stream,
                                  Tracker* trk, const int* id_map = nullptr);

@@ -138,3 +138,12 @@ def test_step_with_shared_first_layer_rows(hs, B, k, over):
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[5 + (b % 30) for b in range(B)])
     check_step(cfg, drafter, w, batch, k, requests=sorted({0, B // 2, B - 1}), what=f"rows {B} {k} {over}")
     drafter.close()
+
+
+# few rows: K-slices inside a cluster of 2 to 8 CTAs (slice counts that divide the k-steps and that do not, rows that leave some CTAs of
+# the cluster without a column), at the row counts where the tile width and the kernel change (16, 32, 128, 129)
+@pytest.mark.parametrize("M", [1, 7, 16, 17, 32, 33, 100, 128, 129, 255])
+@pytest.mark.parametrize("n_out,K", [(256, 4096), (130, 1000), (4096, 2048), (9000, 520), (17000, 640)])
+@pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
+def test_few_row_gemm_slices(hs, M, n_out, K, kind):
+    test_many_row_gemm_tile_widths(hs, M, n_out, K, kind)
