@@ -1,4 +1,4 @@
-// y = x W^T for many activation rows (M >= 256): the tensor-bound regime of the draft step.
+// y = x W^T for many activation rows (or, from 33 rows on, a large matrix).
 //
 // Two CTAs on two SMs form one MMA unit (tcgen05 cta_group::2): the pair owns a [256 weight rows x BNT
 // activation rows] tile of y^T.  Each CTA loads its own 128 weight rows and only HALF of the activation tile per
@@ -408,11 +408,13 @@ bool gemm2_preferred(int M, int n_out) {
   static const int min_m = [] { const char* e = getenv("HSPEC_GEMM2_MIN_M"); return e ? atoi(e) : 0; }();   // measurements only
   if (off) return false;
   if (min_m > 0) return M >= min_m;
-  // From 256 rows on the contractions are tensor-bound; even a partly filled wave of pair tiles beats the one-CTA
-  // kernel with K-slices and its reduction pass.  At 128..255 rows only a matrix of 2^18 weight rows or more (the
-  // state projection) goes this way: streaming it, the pair kernel measured 5.65 against 5.51 TB/s at 128 rows (at 64
-  // rows the one-CTA kernel wins, 6.24 against 6.01), and the step's small matrices keep the kernel they are tuned for.
-  return M >= 256 || (M >= 128 && n_out >= (1 << 18));
+  // Above 128 rows always: the one-CTA kernel's 256-wide accumulator leaves it one CTA per SM and half the weights in flight
+  // (us, one CTA / pair: 160 rows, n_out = K = 4096 35 / 22, n_out = 28672 68 / 51; 255 rows 46 / 21 and 87 / 65).  From 33 rows on
+  // for matrices of about a wave of pair tiles or more, where the pair kernel streams weights at least as fast (n_out = 17536:
+  // 16 rows 26.5 / 26.7, 48 rows 30.3 / 27.1, 128 rows 40.3 / 29.6; n_out = 262144: 316 / 324, 339 / 320, 434 / 370; the LM head of
+  // 152 064 rows, K = 5120, logits written: 246 / 239, 260 / 248, 328 / 291).  Smaller matrices keep the one-CTA kernel and its
+  // K-slices in a cluster (n_out = 4096, K = 14336: 21.5 / 25.1, 23.6 / 25.7, 27.9 / 28.0).
+  return M > 128 || (M > 32 && n_out >= 64 * 256);
 }
 
 // Tile width (activation rows per pair tile) and the number of K-slices for the tiles of the last, partly filled wave,
