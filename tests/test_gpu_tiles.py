@@ -147,3 +147,41 @@ def test_step_with_shared_first_layer_rows(hs, B, k, over):
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
 def test_few_row_gemm_slices(hs, M, n_out, K, kind):
     test_many_row_gemm_tile_widths(hs, M, n_out, K, kind)
+
+
+# query rows per KV head at the edges of the row copies (4 copies up to 32 rows, 2 up to 64, 1 above), contexts that end inside a copy's
+# part of a tile, a block that starts a tile of its own, single and several chunks, the window's leading edge inside a part
+@pytest.mark.parametrize("k,rep", [(1, 1), (8, 4), (11, 3), (32, 1), (16, 4), (32, 2), (13, 5), (16, 8)])
+@pytest.mark.parametrize("window,chunk", [(0, 0), (0, 256), (300, 0)])
+def test_attention_row_copies(hs, k, rep, window, chunk):
+    import numpy as np
+    Hkv, dh, ctx = 2, 128, [0, 1, 31, 97, 128, 500, 1111]
+    B, Hq = len(ctx), 2 * rep
+    pages = [(c + 15) // 16 for c in ctx]
+    perm = torch.randperm(sum(pages), generator=torch.Generator().manual_seed(3)).int()
+    table, at = torch.full((B, max(pages)), -1, dtype=torch.int32), 0
+    for b, n in enumerate(pages):
+        table[b, :n] = perm[at:at + n]
+        at += n
+    bf = torch.bfloat16
+    kp, vp = _rand((sum(pages), 16, Hkv, dh), 1, bf), _rand((sum(pages), 16, Hkv, dh), 2, bf)
+    q, kb, vb = _rand((B * k, Hq, dh), 4, bf), _rand((B * k, Hkv, dh), 5, bf), _rand((B * k, Hkv, dh), 6, bf)
+    o = torch.full((B * k, Hq * dh), float("nan"), dtype=torch.float16, device="cuda")
+    ws = torch.empty(hs.hspec_attention_workspace_bytes(B, k, Hq, Hkv, dh, max(ctx), window, chunk), dtype=torch.uint8, device="cuda")
+    hs.hspec_op_attention(q, kb, vb, kp, vp, table.cuda(), torch.tensor(ctx, dtype=torch.int32).cuda(), max(ctx), o, B, k, Hq, Hkv, dh, 16,
+                          window, chunk, ws)
+    for b, c in enumerate(ctx):
+        rows = table[b, :pages[b]].long().cuda()
+        K = torch.cat([kp[rows].reshape(-1, Hkv, dh)[:c], kb[b * k:(b + 1) * k]]).double()
+        V = torch.cat([vp[rows].reshape(-1, Hkv, dh)[:c], vb[b * k:(b + 1) * k]]).double()
+        pos_q, pos_k = torch.arange(c, c + k, device="cuda"), torch.arange(c + k, device="cuda")
+        d = pos_q[:, None] - pos_k[None, :]
+        vis = (d >= 0) & ((d < window) if window else torch.ones_like(d, dtype=torch.bool))
+        s = torch.einsum("ihrd,jhd->ihrj", q[b * k:(b + 1) * k].view(k, Hkv, rep, dh).double(), K) / np.sqrt(dh)
+        p = torch.softmax(s.masked_fill(~vis[:, None, None, :], float("-inf")), -1)
+        ref = torch.einsum("ihrj,jhd->ihrd", p, V).reshape(k, Hq * dh)
+        # softmax weights enter the product as bf16 (2^-9 relative each), the rest is fp32, the result fp16 (2^-11): relative to the sum of
+        # |weight x value|, with a factor 2 for the exponentials
+        mag = torch.einsum("ihrj,jhd->ihrd", p, V.abs()).reshape(k, Hq * dh)
+        err = (o[b * k:(b + 1) * k].double() - ref).abs()
+        assert bool((err <= 2.0 ** -8 * mag + 2.0 ** -11 * ref.abs() + 1e-6).all()), float((err / mag).max())
