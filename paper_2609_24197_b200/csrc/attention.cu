@@ -129,6 +129,7 @@ attn_partial_kernel(AttnArgs a) {
     cp_async_commit();
   }
 
+  const bool compute = warp * 16 < a.RT;                           // (the others only load)
   // rows of this thread inside the warp's 16-row slab
   const int g = lane >> 2, tq = lane & 3;
   const int r_lo = row0 + warp * 16 + g, r_hi = r_lo + 8;          // global row indices (may be >= R: padding)
@@ -145,6 +146,7 @@ attn_partial_kernel(AttnArgs a) {
     __syncthreads();
     if (t + NSTAGE - 1 < n_tiles) load_tile(t + NSTAGE - 1);
     cp_async_commit();
+    if (!compute) continue;
     if (!q_loaded) {                                   // Q landed with the first group
       q_loaded = true;
 #pragma unroll
@@ -228,8 +230,9 @@ attn_partial_kernel(AttnArgs a) {
     }
   }
   cp_async_wait<0>();
+  if (!compute) return;
 
-  // ---- partial (m, l, O) of this chunk
+  // ---- partial (m, l, O) of this chunk, or the finished rows of a request with a single one
   l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
   l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1); l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
   const size_t slab = (size_t(b) * a.Hkv + kvh) * a.max_chunks + c;
@@ -237,6 +240,16 @@ attn_partial_kernel(AttnArgs a) {
   for (int half = 0; half < 2; ++half) {
     const int r = half ? r_hi : r_lo;
     if (r >= a.R) continue;
+    if (n_chunks == 1) {
+      const float inv = 1.f / (half ? l_hi : l_lo);           // (the row's own block key is always visible: the sum is positive)
+      const size_t at = ((size_t(b) * a.k + r / a.rep) * a.Hq + kvh * a.rep + r % a.rep) * DH;
+#pragma unroll
+      for (int n = 0; n < DH / 8; ++n) {
+        store_act16(a.o, at + n * 8 + tq * 2, o[n][half * 2] * inv, a.o_bf16 != 0, a.status);
+        store_act16(a.o, at + n * 8 + tq * 2 + 1, o[n][half * 2 + 1] * inv, a.o_bf16 != 0, a.status);
+      }
+      continue;
+    }
     float* dst = a.ws_o + (slab * a.R + r) * DH;
 #pragma unroll
     for (int n = 0; n < DH / 8; ++n)
@@ -261,6 +274,7 @@ __global__ void attn_merge_kernel(AttnArgs a) {
   const int ctx = clamped_ctx(a, b);
   int lo0, n_chunks;
   visible_range(ctx, a.window, a.chunk, lo0, n_chunks);
+  if (n_chunks == 1) return;                       // finished by the first kernel
   const size_t slab0 = (size_t(b) * a.Hkv + kvh) * a.max_chunks;
   float m_tot = -INFINITY;
   for (int c = 0; c < n_chunks; ++c) m_tot = fmaxf(m_tot, a.ws_ml[((slab0 + c) * a.R + r) * 2]);
@@ -298,6 +312,22 @@ int attn_pick_chunk(int B, int Hkv, int max_ctx, int window, int num_sms) {
   // chunks for window + 15 tokens, or a request's last few tokens become a chunk (and a merge) of their own
   int lmax = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
   if (lmax < 1) lmax = 1;
+  if (window > 0 && lmax == window + 15) {
+    // Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
+    // Cost of a round in tiles: the chunk's own, three for an item's set-up and read-out, one more for a partial and its merge.
+    // 32 requests x 8 KV heads, window 2048 (256 items of 17 tiles on 148 SMs): one chunk 65.7 us, two 73.1, four 80.
+    long best = 0;
+    int best_chunk = 0;
+    for (int n = 1; n <= 32; ++n) {
+      const int chunk = (lmax + n * 128 - 1) / (n * 128) * 128;
+      if (chunk < 256 && n > 1) break;
+      const int pieces = (lmax + chunk - 1) / chunk;
+      const long rounds = (long(B) * Hkv * pieces + num_sms - 1) / num_sms;
+      const long cost = rounds * (chunk / 128 + (pieces > 1 ? 4 : 3));
+      if (best_chunk == 0 || cost < best) { best = cost; best_chunk = chunk; }
+    }
+    if (best_chunk <= 8192) return best_chunk < 256 ? 256 : best_chunk;
+  }
   int nsplit = (2 * num_sms + B * Hkv - 1) / (B * Hkv);
   if (nsplit < 1) nsplit = 1;
   if (nsplit > 32) nsplit = 32;
@@ -313,7 +343,7 @@ int attn_pick_chunk(int B, int Hkv, int max_ctx, int window, int num_sms) {
   return chunk;
 }
 
-static int max_chunks_of(int max_ctx, int window, int chunk) {
+int attn_max_chunks(int max_ctx, int window, int chunk) {
   // with a window the visible range may start up to 15 tokens earlier (page-aligned chunk grid of the tcgen05 path)
   int lmax = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
   int n = (lmax + chunk - 1) / chunk;
@@ -322,7 +352,7 @@ static int max_chunks_of(int max_ctx, int window, int chunk) {
 
 size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens) {
   const int R = k * (Hq / Hkv);
-  const size_t slabs = size_t(B) * Hkv * max_chunks_of(max_ctx, window, chunk_tokens);
+  const size_t slabs = size_t(B) * Hkv * attn_max_chunks(max_ctx, window, chunk_tokens);
   const size_t row_tiles = (size_t(R) + 127) / 128;
   return slabs * R * (dh + 2) * sizeof(float) + 256 + slabs * row_tiles * 16 + 64;   // partials + the tcgen05 path's work list
 }
@@ -337,7 +367,7 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   a.page_table_stride = c.page_table_stride;
   a.B = c.B; a.k = c.k; a.Hq = c.Hq; a.Hkv = c.Hkv; a.rep = c.Hq / c.Hkv;
   a.R = c.k * a.rep; a.RT = rows_per_cta(a.R); a.n_row_tiles = (a.R + a.RT - 1) / a.RT;
-  a.chunk = c.chunk_tokens; a.max_chunks = max_chunks_of(c.max_ctx, c.window, c.chunk_tokens);
+  a.chunk = c.chunk_tokens; a.max_chunks = attn_max_chunks(c.max_ctx, c.window, c.chunk_tokens);
   a.page_size = c.page_size; a.window = c.window;
   a.status = c.status;
   a.max_ctx = c.max_ctx < c.page_table_stride * c.page_size ? c.max_ctx : c.page_table_stride * c.page_size;
@@ -347,15 +377,15 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   const size_t need = attn_workspace_bytes(c.B, c.k, c.Hq, c.Hkv, c.dh, c.max_ctx, c.window, c.chunk_tokens);
   if (c.ws == nullptr || c.ws_bytes < need) { if (err) *err = "attention workspace too small"; return cudaErrorInvalidValue; }
   {
-    static const bool legacy = [] { const char* e = getenv("HSPEC_ATTN_MMA_SYNC"); return e && e[0] == '1'; }();
-    if (!legacy && attention_tc_supported(c)) return attention_tc_launch(c, a.max_chunks, stream, trk, err);
+    AttnPlan plan;
+    if (attention_plan(c, &plan)) return attention_tc_launch(c, a.max_chunks, stream, trk, err);
   }
   const size_t slabs = size_t(c.B) * c.Hkv * a.max_chunks;
   a.ws_o = reinterpret_cast<float*>(c.ws);
   a.ws_ml = a.ws_o + slabs * a.R * c.dh;
   const size_t smem = size_t(a.RT) * c.dh * 2 + size_t(2) * NSTAGE * KT * c.dh * 2;
   dim3 grid(a.max_chunks * a.n_row_tiles, c.Hkv, c.B);
-  const int threads = a.RT * 2;
+  const int threads = a.RT * 2 < 128 ? 128 : a.RT * 2;       // a warp per 16 rows; further warps only help with the loads
   static bool attr_done[MAX_DEVICES] = {};
   cudaError_t e = once_per_device(attr_done, [](int) {
     cudaError_t e2 = cudaFuncSetAttribute(attn_partial_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -364,15 +394,14 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   });
   if (e != cudaSuccess) return e;
   trk_begin(trk, "attn_partial");
-  if (c.dh == 128) attn_partial_kernel<128><<<grid, threads, smem, stream>>>(a);
-  else attn_partial_kernel<64><<<grid, threads, smem, stream>>>(a);
+  launch_pdl(c.dh == 128 ? attn_partial_kernel<128> : attn_partial_kernel<64>, grid, dim3(threads), smem, stream, a);
   trk_end(trk);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (a.max_chunks == 1) return e;                           // every request is one chunk, finished by the kernel itself
   dim3 mgrid(c.B * c.k, c.Hq);
   trk_begin(trk, "attn_merge");
-  if (c.dh == 128) attn_merge_kernel<128><<<mgrid, 128, 0, stream>>>(a);
-  else attn_merge_kernel<64><<<mgrid, 64, 0, stream>>>(a);
+  launch_pdl(c.dh == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>, mgrid, dim3(c.dh), 0, stream, a);
   trk_end(trk);
   return cudaGetLastError();
 }

@@ -29,16 +29,18 @@
 // then - so the next item's first scores are computed during the current item's last P V product and read-out
 // (another -3 % at 32B-class shapes, -5..8 % where the items are short).  Every wait is bounded; a timed-out role sets
 // a status word and the CTA unwinds.
+#include "attn_plan.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
 #include <cstdio>
+#include <cstdlib>
 
 namespace hspec {
 
 namespace {
 
-constexpr int KT = 128;            // keys per tile
+constexpr int KT = ATTN_KT;        // keys per tile
 constexpr int DH = 128;
 constexpr int NSK = 3, NSV = 3;    // slots of the K ring and of the V ring (7 x 32 KiB = all of shared memory)
 constexpr int NSB = 3;             // score buffers in tensor memory: the MMA warp runs two tiles of scores ahead of the softmax
@@ -187,37 +189,8 @@ __device__ __forceinline__ uint32_t idesc_bf16_128x128(bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// Geometry of one CTA's key range, computed identically by every role.
-struct Range {
-  int base;        // first position of the visible prefix, rounded down to a page boundary
-  int n_chunks;
-  int p_begin;     // first position of this chunk
-  int n_full;      // 128-key tiles fetched by TMA
-  int rem;         // valid prefix keys after the full tiles (only in the last chunk)
-  int n_manual;    // 0, 1 or 2 hand-loaded tiles (ragged end and/or the block's own keys)
-  int T;           // tiles in total
-  bool last;
-};
-
-__device__ __forceinline__ Range make_range(int ctx, int window, int chunk, int c, int k) {
-  Range g;
-  const int lo0 = (window > 0) ? max(0, ctx - window + 1) : 0;
-  g.base = lo0 & ~15;
-  const int len = ctx - g.base;
-  g.n_chunks = max(1, (len + chunk - 1) / chunk);
-  g.last = (c == g.n_chunks - 1);
-  g.p_begin = g.base + c * chunk;
-  const int p_end = min(ctx, g.p_begin + chunk);
-  const int span = max(0, p_end - g.p_begin);
-  g.n_full = span / KT;
-  g.rem = span - g.n_full * KT;
-  g.n_manual = g.last ? ((g.rem + k <= KT) ? 1 : 2) : 0;
-  g.T = g.n_full + g.n_manual;
-  return g;
-}
-
 // For manual tile index mi (0 or 1): how many prefix keys and block keys it holds, and where the prefix keys start.
-__device__ __forceinline__ void manual_tile(const Range& g, int mi, int k, int& n_prefix, int& prefix_start, int& n_block) {
+__device__ __forceinline__ void manual_tile(const AttnRange& g, int mi, int k, int& n_prefix, int& prefix_start, int& n_block) {
   prefix_start = g.p_begin + g.n_full * KT;
   if (g.n_manual == 1) { n_prefix = g.rem; n_block = k; }
   else if (mi == 0) { n_prefix = g.rem; n_block = 0; }
@@ -241,41 +214,13 @@ __device__ __forceinline__ int item_at(int n) {
   return n * G + ((n & 1) ? G - 1 - c : c);
 }
 
-// Work list: one item per (request, KV head, context chunk, 128-row tile), longest first (bucketed by tile count),
-// heads of one request and chunk next to each other so the CTAs that run them at the same time read neighbouring
-// bytes of the same pages.  The order inside a bucket depends on atomics; every item is computed independently, so
-// results do not.
-__global__ void attn_tc_plan_kernel(AttnTcArgs a, int* __restrict__ count, int4* __restrict__ items) {
+// The work list on its own, for calls that do not come with one.
+__global__ void __launch_bounds__(256) attn_tc_plan_kernel(AttnPlan a) {
   pdl_wait();
   pdl_trigger();
   __shared__ int bucket[64];
   __shared__ int offset[64];
-  const int per_chunk = a.Hkv * a.n_row_tiles;
-  const int pairs = a.B * a.max_chunks;            // one thread per (request, chunk slot); slots past n_chunks are skipped
-  for (int i = threadIdx.x; i < 64; i += blockDim.x) bucket[i] = 0;
-  __syncthreads();
-  for (int i = threadIdx.x; i < pairs; i += blockDim.x) {
-    const int b = i / a.max_chunks, c = i % a.max_chunks;
-    if (c == 0 && a.ctx_lens[b] != clamped_ctx(a, b)) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
-    const Range g = make_range(clamped_ctx(a, b), a.window, a.chunk, c, a.k);
-    if (c < g.n_chunks) atomicAdd(&bucket[min(g.T, 63)], per_chunk);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int off = 0;
-    for (int T = 63; T >= 0; --T) { offset[T] = off; off += bucket[T]; }
-    *count = off;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < pairs; i += blockDim.x) {
-    const int b = i / a.max_chunks, c = i % a.max_chunks;
-    const int ctx = clamped_ctx(a, b);
-    const Range g = make_range(ctx, a.window, a.chunk, c, a.k);
-    if (c >= g.n_chunks) continue;
-    int at = atomicAdd(&offset[min(g.T, 63)], per_chunk);
-    for (int kvh = 0; kvh < a.Hkv; ++kvh)
-      for (int rt = 0; rt < a.n_row_tiles; ++rt) items[at++] = make_int4(b, kvh | (rt << 16), c, ctx);
-  }
+  attn_build_plan(a, bucket, offset);
 }
 
 // One operand (K or V) of every tile of this CTA's items -> its own ring of 32 KiB slots.  K and V have separate
@@ -295,7 +240,7 @@ __device__ __forceinline__ void produce_operand(const AttnTcArgs& a, const CUten
     const Item wi = unpack_item(w_next);
     if (item_at(n + 1) < n_items) w_next = items[item_at(n + 1)];         // consumed one item later
     const int b = wi.b, kvh = wi.kvh;
-    const Range g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
+    const AttnRange g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
     const int32_t* ptab = a.page_table + size_t(b) * a.page_table_stride;
     // page ids are fetched one tile ahead (lanes 0..3, one page each): no dependent global load on the issue path
     int page_next = (lane < KT / 16 && g.n_full > 0) ? ptab[(g.p_begin >> 4) + lane] : 0;
@@ -505,7 +450,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       for (; item_at(int(n)) < n_items && ok; ++n) {
         const Item wi = unpack_item(w_next);
         if (item_at(int(n) + 1) < n_items) w_next = items[item_at(int(n) + 1)];
-        const Range g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
+        const AttnRange g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
         for (int t = 0; t < g.T && ok; ++t, ++gt) {
           // the scores of this tile must be under way (the softmax warps wait for them); the next two are issued as soon
           // as their K tile and, at an item's first tile, its Q tile are there
@@ -603,7 +548,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     for (; item_at(int(n)) < n_items && ok; ++n) {
       const Item wi = unpack_item(w_cur);
       const int b = wi.b, kvh = wi.kvh, c = wi.c, ctx = wi.ctx;
-      const Range g = make_range(ctx, a.window, a.chunk, c, a.k);
+      const AttnRange g = make_range(ctx, a.window, a.chunk, c, a.k);
       const int rg = wi.rt * 128 + r_item;          // row among the k * rep rows of this KV head
       const bool row_ok = rg < a.R;
       const int i_blk = rg / a.rep;                  // block position of the row
@@ -881,7 +826,7 @@ attn_tc_merge_kernel(AttnTcArgs a, uint16_t* __restrict__ o) {
   __shared__ __align__(16) uint8_t tile[32 * MERGE_ROW_BYTES];
   const int groups = (a.R + 31) / 32;
   const int b = blockIdx.x / (a.Hkv * groups), kvh = (blockIdx.x / groups) % a.Hkv, r0 = (blockIdx.x % groups) * 32;
-  const Range g = make_range(clamped_ctx(a, b), a.window, a.chunk, 0, a.k);
+  const AttnRange g = make_range(clamped_ctx(a, b), a.window, a.chunk, 0, a.k);
   if (g.n_chunks == 1) return;                     // finished by the attention kernel itself (uniform for the block)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int r = r0 + lane;
@@ -973,6 +918,22 @@ bool attention_tc_supported(const AttnCall& c) {
   return c.dh == 128 && c.page_size == 16 && c.num_pages > 0 && (c.chunk_tokens % KT) == 0 && c.k <= KT;
 }
 
+// The list (count + items) lies behind the partials in the workspace.
+bool attention_plan(const AttnCall& c, AttnPlan* plan) {
+  static const bool legacy = [] { const char* e = getenv("HSPEC_ATTN_MMA_SYNC"); return e && e[0] == '1'; }();
+  if (legacy || !attention_tc_supported(c)) return false;
+  const int R = c.k * (c.Hq / c.Hkv);
+  plan->ctx_lens = c.ctx_lens; plan->status = c.status;
+  plan->B = c.B; plan->k = c.k; plan->Hkv = c.Hkv; plan->n_row_tiles = (R + 127) / 128;
+  plan->chunk = c.chunk_tokens; plan->max_chunks = attn_max_chunks(c.max_ctx, c.window, c.chunk_tokens); plan->window = c.window;
+  plan->max_ctx = c.max_ctx < c.page_table_stride * 16 ? c.max_ctx : c.page_table_stride * 16;
+  const size_t slabs = size_t(c.B) * c.Hkv * plan->max_chunks;
+  float* end = reinterpret_cast<float*>(c.ws) + slabs * R * (c.dh + 2);
+  plan->count = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(end) + 15) & ~uintptr_t(15));
+  plan->items = reinterpret_cast<int4*>(plan->count + 4);
+  return true;
+}
+
 cudaError_t attention_tc_launch(const AttnCall& c, int max_chunks, cudaStream_t stream, Tracker* trk, std::string* err) {
   AttnTcArgs a{};
   a.q = (const __nv_bfloat16*)c.q; a.kb = (const __nv_bfloat16*)c.kb; a.vb = (const __nv_bfloat16*)c.vb;
@@ -1008,20 +969,25 @@ cudaError_t attention_tc_launch(const AttnCall& c, int max_chunks, cudaStream_t 
     if (e0 != cudaSuccess) return e0;
   }
   const int n_sms = sm_count[current_device()];
-  // work list (count + items) behind the partials in the workspace
-  int* count = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(a.ws_ml + slabs * a.R * 2) + 15) & ~uintptr_t(15));
-  int4* items = reinterpret_cast<int4*>(count + 4);
-  trk_begin(trk, "attn_plan");
-  launch_pdl(attn_tc_plan_kernel, dim3(1), dim3(256), 0, stream, a, count, items);
-  trk_end(trk);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  AttnPlan plan;
+  attention_plan(c, &plan);
+  cudaError_t e = cudaSuccess;
+  if (!c.planned) {
+    trk_begin(trk, "attn_plan");
+    launch_pdl(attn_tc_plan_kernel, dim3(1), dim3(256), 0, stream, plan);
+    trk_end(trk);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const int* count = plan.count;
+  const int4* items = plan.items;
   trk_begin(trk, "attn_partial");
   auto kernel = a.R <= 32 ? attn_tc_kernel<4> : (a.R <= 64 ? attn_tc_kernel<2> : attn_tc_kernel<1>);
-  launch_pdl(kernel, dim3(n_sms), dim3(352), smem, stream, tmK, tmV, a, (const int*)count, (const int4*)items);
+  launch_pdl(kernel, dim3(n_sms), dim3(352), smem, stream, tmK, tmV, a, count, items);
   trk_end(trk);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (max_chunks == 1) return e;                   // every request is one chunk, finished by the kernel itself
   trk_begin(trk, "attn_merge");
   launch_pdl(attn_tc_merge_kernel, dim3(c.B * c.Hkv * ((a.R + 31) / 32)), dim3(256), 0, stream, a, reinterpret_cast<uint16_t*>(c.o));
   trk_end(trk);

@@ -1,8 +1,10 @@
 // Row-wise and element-wise kernels of the draft step (all fp32 math; bf16 only where a tensor-core
 // operand is produced).
+#include "attn_plan.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
+#include <algorithm>
 #include <cstdlib>
 
 namespace hspec {
@@ -84,15 +86,27 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restr
 // Block rows: row 0 of each request is the embedding of its last token, rows 1..k-1 the mask-token embedding; no positional
 // embedding is added (paper Sec. 3.3.1).  X gets all B*k rows (the residual stream).  Rows 1..k-1 are the same for every
 // request, so the first layer's normalised input has only B + 1 different rows: u[b] for position 0 of request b, u[B] for the
-// rest.  One block per row of X; the B + 1 blocks that own a different row also write its norm.
+// rest.  One block per row of X; the B + 1 blocks that own a different row also write its norm.  The blocks behind them prepare
+// what else the step needs and nothing has to wait for (it was three launches of their own): one builds the attention's work list,
+// the others make the 16-bit copy of last_hidden.
 template <int VPT>
 __global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ embed, const int32_t* __restrict__ last_token, int mask_id,
                                   const float* __restrict__ w, float* __restrict__ X, void* __restrict__ u, int B, int k, int D,
-                                  float eps, uint32_t* status, int bf16_out) {
+                                  float eps, StepPrep prep, uint32_t* status, int bf16_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
   const int m = blockIdx.x;
+  if (m >= B * k) {
+    __shared__ int bucket[64], offset[64];
+    const int planners = prep.plan.items != nullptr ? 1 : 0;
+    if (m < B * k + planners) { attn_build_plan(prep.plan, bucket, offset); return; }
+    const __nv_bfloat16* lh = reinterpret_cast<const __nv_bfloat16*>(prep.lh_src);
+    const size_t stride = size_t(gridDim.x - B * k - planners) * blockDim.x;
+    for (size_t j = size_t(m - B * k - planners) * blockDim.x + threadIdx.x; j < prep.n_lh; j += stride)
+      store_act16(prep.lh_dst, j, __bfloat162float(lh[j]), bf16_out != 0, status);
+    return;
+  }
   const int b = m / k, i = m % k;
   const int tok = (i == 0) ? last_token[b] : mask_id;
   const __nv_bfloat16* src = embed + size_t(tok) * D;
@@ -340,10 +354,11 @@ int grid_for(long long total, int threads) {
 }  // namespace
 
 cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,
-                              int B, int k, int D, float eps, cudaStream_t stream, uint32_t* status, bool bf16_out) {
+                              int B, int k, int D, float eps, const StepPrep& prep, cudaStream_t stream, uint32_t* status, bool bf16_out) {
   const int threads = D <= 4 * 6 * 256 ? 256 : 512;
-  cudaError_t e = launch_pdl(embed_norm_kernel<6>, dim3(B * k), dim3(threads), 0, stream, (const __nv_bfloat16*)embed_bf16, last_token,
-                             mask_id, norm_w, X, u_16, B, k, D, eps, status, bf16_out ? 1 : 0);
+  const int lh_blocks = prep.lh_src ? int(std::min<size_t>((prep.n_lh + threads - 1) / threads, 148 * 4)) : 0;
+  cudaError_t e = launch_pdl(embed_norm_kernel<6>, dim3(B * k + (prep.plan.items ? 1 : 0) + lh_blocks), dim3(threads), 0, stream, (const __nv_bfloat16*)embed_bf16, last_token,
+                             mask_id, norm_w, X, u_16, B, k, D, eps, prep, status, bf16_out ? 1 : 0);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -308,13 +308,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 }
 
 // ids[m] = lowest index among the per-tile maxima (tiles are in ascending vocabulary order).
-// The partials are [tile][row]: a block takes eight consecutive rows, thread (r = tid % 8, tid / 8) walks every 32nd
-// tile of row r, so that eight neighbouring threads read one 32-byte sector (a block per row read 4 bytes of every
-// sector it touched: 33 us for 19 MB at M = 2048, V = 152 064).
+// The partials are [tile][row]: a block takes eight consecutive rows, thread (r = tid % 8, tid / 8) walks every 128th
+// tile of row r, so that eight neighbouring threads read one 32-byte sector, with the loads of four tiles in flight.  There are only
+// M / 8 blocks, so it is the length of a thread's chain that counts: with 256 threads and one tile at a time the 1 188 tiles of
+// a 152 064-token vocabulary were 38 dependent rounds (15 us at 16 and at 512 rows).
 __device__ __forceinline__ void argmax_take(float& v, int& idx, float ov, int oi) {
   if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
 }
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 argmax_reduce_kernel(const float* __restrict__ pv, const int* __restrict__ pi, int n_tiles, int M,
                      int* __restrict__ ids, const int* __restrict__ id_map) {
   pdl_wait();
@@ -323,20 +324,34 @@ argmax_reduce_kernel(const float* __restrict__ pv, const int* __restrict__ pi, i
   float v = -INFINITY;
   int idx = 0x7fffffff;
   if (m < M) {
-    for (int t = threadIdx.x >> 3; t < n_tiles; t += 32) argmax_take(v, idx, pv[size_t(t) * M + m], pi[size_t(t) * M + m]);
+    for (int t = threadIdx.x >> 3; t < n_tiles; t += 4 * 128) {
+      float tv[4];
+      int ti[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int tu = t + u * 128;
+        tv[u] = tu < n_tiles ? pv[size_t(tu) * M + m] : -INFINITY;
+        ti[u] = tu < n_tiles ? pi[size_t(tu) * M + m] : 0x7fffffff;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) argmax_take(v, idx, tv[u], ti[u]);
+    }
   }
   // lanes r, r + 8, r + 16, r + 24 of a warp hold the same row
   for (int off = 8; off < 32; off <<= 1)
     argmax_take(v, idx, __shfl_xor_sync(0xffffffffu, v, off), __shfl_xor_sync(0xffffffffu, idx, off));
-  __shared__ float sv[8][8];
-  __shared__ int si[8][8];
+  __shared__ float sv[32][8];
+  __shared__ int si[32][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane < 8) { sv[warp][lane] = v; si[warp][lane] = idx; }
   __syncthreads();
-  if (threadIdx.x < 8 && m < M) {
-    v = sv[0][r]; idx = si[0][r];
-    for (int w = 1; w < 8; ++w) argmax_take(v, idx, sv[w][r], si[w][r]);
-    ids[m] = id_map ? id_map[idx] : idx;                    // pruned drafter vocabulary: row index -> token id
+  if (warp < 8) {                                           // warp w: row w of the block, lane = the warp the value came from
+    v = sv[lane][warp]; idx = si[lane][warp];
+    for (int off = 16; off > 0; off >>= 1)
+      argmax_take(v, idx, __shfl_xor_sync(0xffffffffu, v, off), __shfl_xor_sync(0xffffffffu, idx, off));
+    const int mw = blockIdx.x * 8 + warp;
+    // (pruned drafter vocabulary: row index -> token id; a row without any maximum keeps its sentinel)
+    if (lane == 0 && mw < M) ids[mw] = id_map && idx != 0x7fffffff ? id_map[idx] : idx;
   }
 }
 
@@ -469,7 +484,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
 cudaError_t argmax_reduce_launch(const float* pv, const int* pi, int n_tiles, int M, int* ids, cudaStream_t stream,
                                  Tracker* trk, const int* id_map) {
   trk_begin(trk, "argmax_reduce", 0, double(n_tiles) * M * 8);
-  launch_pdl(argmax_reduce_kernel, dim3((M + 7) / 8), dim3(256), 0, stream, pv, pi, n_tiles, M, ids, id_map);
+  launch_pdl(argmax_reduce_kernel, dim3((M + 7) / 8), dim3(1024), 0, stream, pv, pi, n_tiles, M, ids, id_map);
   trk_end(trk);
   return cudaGetLastError();
 }

@@ -544,21 +544,27 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   // embedding): the first layer's in-projection runs on those, and the scan reads them through its row map.  At 128 requests x 16
   // positions of the 32B-class shapes that GEMM goes from 2048 to 129 rows.
   const int rows0 = k > 1 ? B + 1 : B;
-  EW("embed_norm", Md * c.D * 6, embed_norm_launch(W("embed").data, in->last_token, c.mask_id, fptr("layers.0.mamba.norm"), X, U, B, k, c.D,
-                                                   c.rms_eps, st, h->d_status, bf));
-  // S_init = Proj_dS(Proj_r(concat h)): once per step, shared by all layers
+  // everything of a layer's attention call but the pools; the work list is the same for all layers
+  auto attn_call = [&]() {
+    AttnCall a{};
+    a.q = Q; a.kb = KB; a.vb = VB;
+    a.num_pages = in->num_pages; a.status = h->d_status;
+    a.page_table = in->page_table; a.page_table_stride = in->page_table_stride; a.ctx_lens = in->ctx_lens;
+    a.max_ctx = max_ctx; a.o = U; a.o_bf16 = bf; a.B = B; a.k = k; a.Hq = c.Hq; a.Hkv = c.Hkv; a.dh = c.dh;
+    a.page_size = c.page_size; a.window = c.window; a.chunk_tokens = p.attn_chunk;
+    a.ws = ws + p.ATT; a.ws_bytes = p.att_bytes;
+    a.planned = true;
+    return a;
+  };
+  StepPrep prep{};
+  if (!any_attn || !attention_plan(attn_call(), &prep.plan)) prep.plan.items = nullptr;
   const void* lh_in = LH;
-  if (bf && (reinterpret_cast<uintptr_t>(in->last_hidden) & 15) == 0) {
-    lh_in = in->last_hidden;                       // already the operand type: read in place
-  } else {
-    const size_t n_lh = size_t(B) * c.n_fuse * c.D;
-    trk->begin("cvt_last_hidden", 0, double(n_lh) * 4);
-    if (bf) CUDA_TRY(h, cudaMemcpyAsync(LH, in->last_hidden, n_lh * 2, cudaMemcpyDeviceToDevice, st));
-    else bf16_to_f16_kernel<<<int(std::min<size_t>((n_lh + 255) / 256, 148 * 8)), 256, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(in->last_hidden), reinterpret_cast<__half*>(LH), n_lh, h->d_status);
-    trk->end();
-    CUDA_TRY(h, cudaGetLastError());
-  }
+  prep.n_lh = size_t(B) * c.n_fuse * c.D;
+  if (bf && (reinterpret_cast<uintptr_t>(in->last_hidden) & 15) == 0) lh_in = in->last_hidden;   // already the operand type: read in place
+  else { prep.lh_src = in->last_hidden; prep.lh_dst = LH; }
+  EW("embed_norm", Md * c.D * 6, embed_norm_launch(W("embed").data, in->last_token, c.mask_id, fptr("layers.0.mamba.norm"), X, U, B, k, c.D,
+                                                   c.rms_eps, prep, st, h->d_status, bf));
+  // S_init = Proj_dS(Proj_r(concat h)): once per step, shared by all layers
   CUDA_TRY(h, gemm("proj_r", "gemm:proj_r", lh_in, B, bf ? EPI_STORE_BF16 : EPI_STORE_F16, Fv, c.r));
   // (S_init is an output the scan consumes, not a GEMM operand: it stays fp16 in both modes)
   CUDA_TRY(h, gemm("proj_ds", "gemm:proj_ds", Fv, B, EPI_STORE_F16, SINIT, d.d_S));
@@ -596,14 +602,8 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
       EW("qk_norm_rope", Md * d.d_qkv * 6,
          qk_norm_rope_launch(BIG, fptr(pre + "attn.q_norm"), fptr(pre + "attn.k_norm"), in->ctx_lens, Q, KB, VB, B, k, c.Hq,
                              c.Hkv, c.dh, c.rope_theta, c.rms_eps, c.qk_norm, st));
-      AttnCall a{};
-      a.q = Q; a.kb = KB; a.vb = VB;
+      AttnCall a = attn_call();
       a.k_pool = in->k_pools[c.kv_slot[l]]; a.v_pool = in->v_pools[c.kv_slot[l]];
-      a.num_pages = in->num_pages; a.status = h->d_status;
-      a.page_table = in->page_table; a.page_table_stride = in->page_table_stride; a.ctx_lens = in->ctx_lens;
-      a.max_ctx = max_ctx; a.o = U; a.o_bf16 = bf; a.B = B; a.k = k; a.Hq = c.Hq; a.Hkv = c.Hkv; a.dh = c.dh;
-      a.page_size = c.page_size; a.window = c.window; a.chunk_tokens = p.attn_chunk;
-      a.ws = ws + p.ATT; a.ws_bytes = p.att_bytes;
       CUDA_TRY(h, attention_launch(a, st, trk, &errtxt));
       CUDA_TRY(h, gemm(pre + "attn.wo", "gemm:wo", U, M, EPI_ACCUM_F32, X, c.D));
     }

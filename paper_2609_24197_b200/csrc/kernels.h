@@ -212,13 +212,24 @@ struct AttnCall {
   bool o_bf16;
   int B, k, Hq, Hkv, dh, page_size, window;
   int chunk_tokens;                 // <= 0: choose
+  bool planned;                     // the work list is in the workspace already (built for the same lengths, chunk and row count)
   void* ws;
   size_t ws_bytes;
+};
+// The attention's work list (attn_plan.cuh): where it is built from and where it lies.
+struct AttnPlan {
+  const int32_t* ctx_lens;
+  uint32_t* status;
+  int B, k, Hkv, n_row_tiles, chunk, max_chunks, window, max_ctx;
+  int* count;
+  int4* items;
 };
 int attn_pick_chunk(int B, int Hkv, int max_ctx, int window, int num_sms);
 size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens);
 cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool attention_tc_supported(const AttnCall& c);
+bool attention_plan(const AttnCall& c, AttnPlan* plan);   // false: this call needs no work list (mma.sync path)
+int attn_max_chunks(int max_ctx, int window, int chunk);
 cudaError_t attention_tc_launch(const AttnCall& c, int max_chunks, cudaStream_t stream, Tracker* trk, std::string* err);
 cudaError_t gather_kv_launch(const void* pool, const int32_t* row, int ctx_len, int page_size, int Hkv, int dh,
                              void* dst, cudaStream_t stream);
@@ -239,8 +250,15 @@ size_t scan_workspace_bytes(int B, int k, int Di, int N, int G);
 cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 
 // ---- element-wise kernels (elementwise.cu)
+// What the first kernel of a step prepares next to the embedded rows: the 16-bit copy of last_hidden and the attention's work list.
+struct StepPrep {
+  const void* lh_src;               // bf16, n_lh values, copied to lh_dst as fp16 (or as they are when bf16_out); null: nothing to copy
+  void* lh_dst;
+  size_t n_lh;
+  AttnPlan plan;                    // plan.items null: no work list
+};
 cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,
-                              int B, int k, int D, float eps, cudaStream_t stream, uint32_t* status, bool bf16_out);
+                              int B, int k, int D, float eps, const StepPrep& prep, cudaStream_t stream, uint32_t* status, bool bf16_out);
 cudaError_t rmsnorm_launch(const float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
                            uint32_t* status, bool bf16_out = false);
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,
