@@ -417,7 +417,11 @@ int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode) {
   const int k_tiles = (K + TILE_K - 1) / TILE_K;
   const int tiles = ((n_out + TILE_W - 1) / TILE_W) * ((M + 255) / 256);
   if (tiles >= num_sms || k_tiles < 8) return 1;
-  int want = 2 * num_sms / tiles;           // one wave of two CTAs per SM
+  // One wave, two CTAs per SM - but a cluster lives in one GPC, and clusters stop fitting before the last of the 296 places is taken:
+  // 48 tiles (n_out = 6144, K = 4096, 16 rows) 5 slices 12.0 us, 6 17.3; 40 tiles (5120 x 5120, 96 rows) 6 17.1, 7 26.3; 64 tiles
+  // 4 17.6, 5 24.1; 96 tiles 2 23.8, 3 29.9.  Clusters of two still fit at 274 CTAs (137 tiles: 1 slice 26.9 us, 2 25.7, 3 31.7).
+  int want = 256 * num_sms / 148 / tiles;
+  if (want < 2 && 2 * tiles <= 276 * num_sms / 148) want = 2;
   int max_by_k = k_tiles / 4;               // at least 4 K-tiles per slice
   int s = want < max_by_k ? want : max_by_k;
   if (s > GEMM_MAX_SPLITS) s = GEMM_MAX_SPLITS;
