@@ -77,6 +77,11 @@ attn_partial_kernel(AttnArgs a) {
   uint8_t* sV = sK + NSTAGE * KT * DH * 2;
   constexpr int CPR = DH / 8;                        // 16-byte chunks per row
 
+  // A warp per 16 query rows computes.  Where those are fewer than four, the block's further warps do all the K/V loading, so that
+  // the few that compute never wait for a page id.
+  const bool compute = warp * 16 < a.RT;
+  const int n_loaders = nthr > a.RT * 2 ? nthr - a.RT * 2 : nthr, loader = nthr > a.RT * 2 ? tid - a.RT * 2 : tid;   // (loader < 0: none)
+
   // ---- Q rows of this tile -> shared (zero for padding rows)
   const int row0 = rt * a.RT;
   for (int idx = tid; idx < a.RT * CPR; idx += nthr) {
@@ -95,25 +100,36 @@ attn_partial_kernel(AttnArgs a) {
     const uint32_t dK = smem_u32(sK) + st * KT * DH * 2, dV = smem_u32(sV) + st * KT * DH * 2;
     if (t < n_pre) {
       const int base = p_begin + t * KT;
-      for (int idx = tid; idx < KT * CPR; idx += nthr) {
-        const int r = idx / CPR, ch = idx % CPR;
-        const int p = base + r;
-        bool ok = p < p_end;
-        size_t off = 0;
-        if (ok) {
-          const int page = ptab[p / a.page_size];
-          if (unsigned(page) >= unsigned(a.num_pages)) {     // never form an address from a bad id: zero row, counted once
-            ok = false;
-            if (ch == 0 && p % a.page_size == 0) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
-          } else {
-            off = ((size_t(page) * a.page_size + (p % a.page_size)) * a.Hkv + kvh) * DH + ch * 8;
-          }
+      constexpr int U = 4;                             // rows in flight per thread: their page ids are fetched together
+      for (int idx0 = loader; idx0 < KT * CPR; idx0 += U * n_loaders) {
+        int page[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int idx = idx0 + u * n_loaders, p = base + idx / CPR;
+          page[u] = (idx < KT * CPR && p < p_end) ? __ldg(ptab + p / a.page_size) : -1;
         }
-        cp_async16(dK + swz<DH>(r, ch * 8), a.k_pool + off, ok);
-        cp_async16(dV + swz<DH>(r, ch * 8), a.v_pool + off, ok);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int idx = idx0 + u * n_loaders;
+          if (idx >= KT * CPR) break;
+          const int r = idx / CPR, ch = idx % CPR;
+          const int p = base + r;
+          bool ok = p < p_end;
+          size_t off = 0;
+          if (ok) {
+            if (unsigned(page[u]) >= unsigned(a.num_pages)) {     // never form an address from a bad id: zero row, counted once
+              ok = false;
+              if (ch == 0 && p % a.page_size == 0) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
+            } else {
+              off = ((size_t(page[u]) * a.page_size + (p % a.page_size)) * a.Hkv + kvh) * DH + ch * 8;
+            }
+          }
+          cp_async16(dK + swz<DH>(r, ch * 8), a.k_pool + off, ok);
+          cp_async16(dV + swz<DH>(r, ch * 8), a.v_pool + off, ok);
+        }
       }
     } else {                                          // the block's own keys / values
-      for (int idx = tid; idx < KT * CPR; idx += nthr) {
+      for (int idx = loader; idx < KT * CPR; idx += n_loaders) {
         const int r = idx / CPR, ch = idx % CPR;
         const bool ok = r < a.k;
         const size_t off = ok ? ((size_t(b) * a.k + r) * a.Hkv + kvh) * DH + ch * 8 : 0;
@@ -125,11 +141,10 @@ attn_partial_kernel(AttnArgs a) {
 
 #pragma unroll
   for (int t = 0; t < NSTAGE - 1; ++t) {
-    if (t < n_tiles) load_tile(t);
+    if (t < n_tiles && loader >= 0) load_tile(t);
     cp_async_commit();
   }
 
-  const bool compute = warp * 16 < a.RT;                           // (the others only load)
   // rows of this thread inside the warp's 16-row slab
   const int g = lane >> 2, tq = lane & 3;
   const int r_lo = row0 + warp * 16 + g, r_hi = r_lo + 8;          // global row indices (may be >= R: padding)
@@ -144,7 +159,7 @@ attn_partial_kernel(AttnArgs a) {
   for (int t = 0; t < n_tiles; ++t) {
     cp_async_wait<NSTAGE - 2>();
     __syncthreads();
-    if (t + NSTAGE - 1 < n_tiles) load_tile(t + NSTAGE - 1);
+    if (t + NSTAGE - 1 < n_tiles && loader >= 0) load_tile(t + NSTAGE - 1);
     cp_async_commit();
     if (!compute) continue;
     if (!q_loaded) {                                   // Q landed with the first group
@@ -385,7 +400,7 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   a.ws_ml = a.ws_o + slabs * a.R * c.dh;
   const size_t smem = size_t(a.RT) * c.dh * 2 + size_t(2) * NSTAGE * KT * c.dh * 2;
   dim3 grid(a.max_chunks * a.n_row_tiles, c.Hkv, c.B);
-  const int threads = a.RT * 2 < 128 ? 128 : a.RT * 2;       // a warp per 16 rows; further warps only help with the loads
+  const int threads = a.RT * 2 < 128 ? a.RT * 2 + 96 : a.RT * 2;   // a warp per 16 rows, and three that only load where those are few
   static bool attr_done[MAX_DEVICES] = {};
   cudaError_t e = once_per_device(attr_done, [](int) {
     cudaError_t e2 = cudaFuncSetAttribute(attn_partial_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
