@@ -43,15 +43,29 @@ __device__ __forceinline__ void store_norm4(uint16_t* row, int d4, const float4&
   reinterpret_cast<uint2*>(row)[d4] = out;
 }
 
+// Four sums over the slices of a pending tail tile (slice order), for row m and columns n .. n + 3; zeros where the tile is not one.
+__device__ __forceinline__ float4 tail_sum4(const GemmTail& t, int m, int n) {
+  const int tm = m / t.BNT, tile = (n >> 8) * t.n_tiles_m + tm;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (tile < t.n_full_tiles) return acc;
+  const float* src = t.part + (size_t(tile - t.n_full_tiles) * t.splits * t.BNT + (m - tm * t.BNT)) * 256 + (n & 255);
+  for (int sp = 0; sp < t.splits; ++sp) {
+    const float4 v = __ldcs(reinterpret_cast<const float4*>(src + size_t(sp) * t.BNT * 256));
+    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+  }
+  return acc;
+}
+
 // y = x / sqrt(mean(x^2) + eps) * w, one CTA per row, fp16 (or bf16) out.  VPT = 16-byte vectors a thread keeps in
-// registers between the two passes.
-template <int VPT>
-__global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restrict__ w, void* __restrict__ y,
-                               int n, float eps, uint32_t* status, int bf16_out) {
+// registers between the two passes.  TAIL: the residual GEMM in front left the K-slices of its last wave's tiles unsummed; they are
+// added to x here, on the way (a launch of its own cost 6 us and a pass over x).
+template <int VPT, bool TAIL>
+__global__ void rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ w, void* __restrict__ y,
+                               int n, float eps, GemmTail tail, uint32_t* status, int bf16_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
-  const float* xr = x + size_t(blockIdx.x) * n;
+  float* xr = x + size_t(blockIdx.x) * n;
   uint16_t* yr = reinterpret_cast<uint16_t*>(y) + size_t(blockIdx.x) * n;      // a row of 16-bit values, either type
   if ((n & 3) == 0 && n <= 4 * VPT * int(blockDim.x)) {
     // 16-byte loads, the row stays in registers between the two passes
@@ -62,6 +76,11 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restr
     for (int i = 0; i < VPT; ++i) {
       const int d4 = threadIdx.x + i * blockDim.x;
       v[i] = d4 < nv ? reinterpret_cast<const float4*>(xr)[d4] : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (TAIL && d4 < nv) {
+        const float4 add = tail_sum4(tail, blockIdx.x, d4 * 4);
+        v[i].x += add.x; v[i].y += add.y; v[i].z += add.z; v[i].w += add.w;
+        reinterpret_cast<float4*>(xr)[d4] = v[i];
+      }
       ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
     }
     const float inv = rsqrtf(block_sum(ss, red) / float(n) + eps);
@@ -75,6 +94,15 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restr
       }
     }
     return;
+  }
+  if (TAIL) {                                       // (n is a multiple of four: the host sees to it)
+    for (int d4 = threadIdx.x; d4 < (n >> 2); d4 += blockDim.x) {
+      float4 v = reinterpret_cast<const float4*>(xr)[d4];
+      const float4 add = tail_sum4(tail, blockIdx.x, d4 * 4);
+      v.x += add.x; v.y += add.y; v.z += add.z; v.w += add.w;
+      reinterpret_cast<float4*>(xr)[d4] = v;
+    }
+    __syncthreads();
   }
   float ss = 0.f;
   for (int d = threadIdx.x; d < n; d += blockDim.x) { const float v = xr[d]; ss += v * v; }
@@ -362,12 +390,15 @@ cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token,
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t rmsnorm_launch(const float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
-                           uint32_t* status, bool bf16_out) {
+cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
+                           uint32_t* status, bool bf16_out, const GemmTail* tail) {
   // 256 threads with up to six vectors each as long as the row fits (n <= 6144), else 512: at n = 5120 the profiler
   // timed 16.5-17.1 us with 256 threads, 18.1-19.5 with 512, 19.6-21.0 with 128 (twelve vectors each)
   const int threads = n <= 4 * 6 * 256 ? 256 : 512;
-  cudaError_t e = launch_pdl(rmsnorm_kernel<6>, dim3(M), dim3(threads), 0, stream, x, w, y_16, n, eps, status, bf16_out ? 1 : 0);
+  const bool pending = tail != nullptr && tail->part != nullptr;
+  if (pending && (n & 3)) return cudaErrorInvalidValue;
+  cudaError_t e = launch_pdl(pending ? rmsnorm_kernel<6, true> : rmsnorm_kernel<6, false>, dim3(M), dim3(threads), 0, stream, x, w, y_16, n, eps,
+                             pending ? *tail : GemmTail{}, status, bf16_out ? 1 : 0);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -480,6 +480,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   const size_t smem = size_t(stages) * stage_bytes + fixed;
   trk_begin(trk, c.label ? c.label : "gemm", 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));
+  if (c.defer_tail) *c.defer_tail = GemmTail{};
   cudaError_t e = launch_pdl_cluster(gemm_tcgen05_kernel, grid, dim3(192), dim3(1, 1, splits), smem, stream, *c.tmW, tmB, g);
   trk_end(trk);
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -504,13 +504,21 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   const int clusters = total < 74 ? total : 74;
   const size_t smem = size_t(stages) * stage_bytes + fixed;
   // profile name "gemm2:<what>" tells this kernel's launches from the one-CTA kernel's "gemm:<what>"
-  std::string label = "gemm2:";
-  if (c.label) { const char* colon = strchr(c.label, ':'); label += colon ? colon + 1 : c.label; }
-  trk_begin(trk, label.c_str(), 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
+  char label[40] = "gemm2:";
+  if (c.label) {
+    const char* colon = strchr(c.label, ':');
+    strncat(label, colon ? colon + 1 : c.label, sizeof(label) - 7);
+  }
+  trk_begin(trk, label, 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));
   cudaError_t e = launch_pdl(gemm_2sm_kernel, dim3(2 * clusters), dim3(GEMM2_THREADS), smem, stream, *c.tmW, tmB, g);
   trk_end(trk);
   if (e == cudaSuccess) e = cudaGetLastError();
+  if (c.defer_tail) *c.defer_tail = GemmTail{};
+  if (e == cudaSuccess && splits > 1 && c.defer_tail && c.mode == EPI_ACCUM_F32) {
+    *c.defer_tail = GemmTail{g.part, g.n_full_tiles, g.n_tiles_m, g.BNT, splits};
+    return e;
+  }
   if (e == cudaSuccess && splits > 1) {
     trk_begin(trk, "gemm2_tail_reduce", 0, double(splits + 1) * tail * g.BNT * 256 * 4);
     launch_pdl(gemm2_tail_reduce_kernel, dim3(tail, g.BNT / TAIL_ROWS), dim3(256), 0, stream, g);

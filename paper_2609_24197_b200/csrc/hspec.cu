@@ -204,10 +204,23 @@ void Tracker::destroy() {
 
 }  // namespace hspec
 
+// The weights by role, so that a step does not build and look up about fifty names.
+struct StepWeights {
+  struct Layer {
+    const Weight *m_norm, *in_proj, *dt_up, *conv_w, *conv_b, *dt_bias, *A_log, *Dskip, *gnorm, *out_proj;
+    const Weight *a_norm, *wqkv, *q_norm, *k_norm, *wo;
+    const Weight *f_norm, *gate_up, *down;
+  };
+  const Weight *embed, *proj_r, *proj_ds, *final_norm, *lm_head, *vocab_map, *markov_in, *markov_out;
+  Layer layer[HSPEC_MAX_LAYERS];
+};
+
 struct hspec_handle {
   hspec_config cfg;
   Dims d;
   std::unordered_map<std::string, Weight> w;
+  StepWeights by_role;
+  bool complete = false;      // every tensor a step needs is loaded and by_role points at it (set by hspec_load_weights)
   std::string err;
   Tracker trk;
   uint32_t launches_last_step = 0;
@@ -284,6 +297,35 @@ std::vector<std::string> required_names(const hspec_config& c) {
       for (const char* s : {"attn.norm", "attn.wqkv", "attn.q_norm", "attn.k_norm", "attn.wo"}) n.push_back(p + s);
   }
   return n;
+}
+
+// First required tensor that is not loaded, or an empty string.
+std::string missing_tensor(const hspec_handle* h) {
+  for (const std::string& nm : required_names(h->cfg))
+    if (h->w.find(nm) == h->w.end()) return nm;
+  return std::string();
+}
+
+void resolve_weights(hspec_handle* h) {
+  h->complete = missing_tensor(h).empty();
+  if (!h->complete) return;
+  auto at = [&](const std::string& nm) -> const Weight* {
+    auto it = h->w.find(nm);
+    return it == h->w.end() ? nullptr : &it->second;
+  };
+  StepWeights& s = h->by_role;
+  s.embed = at("embed"); s.proj_r = at("proj_r"); s.proj_ds = at("proj_ds"); s.final_norm = at("final_norm"); s.lm_head = at("lm_head");
+  s.vocab_map = at("vocab_map"); s.markov_in = at("markov_in"); s.markov_out = at("markov_out");
+  for (int l = 0; l < h->cfg.L; ++l) {
+    const std::string p = "layers." + std::to_string(l) + ".";
+    StepWeights::Layer& y = s.layer[l];
+    y.m_norm = at(p + "mamba.norm"); y.in_proj = at(p + "mamba.in_proj"); y.dt_up = at(p + "mamba.dt_up");
+    y.conv_w = at(p + "mamba.conv_w"); y.conv_b = at(p + "mamba.conv_b"); y.dt_bias = at(p + "mamba.dt_bias");
+    y.A_log = at(p + "mamba.A_log"); y.Dskip = at(p + "mamba.Dskip"); y.gnorm = at(p + "mamba.gnorm"); y.out_proj = at(p + "mamba.out_proj");
+    y.a_norm = at(p + "attn.norm"); y.wqkv = at(p + "attn.wqkv"); y.q_norm = at(p + "attn.q_norm"); y.k_norm = at(p + "attn.k_norm");
+    y.wo = at(p + "attn.wo");
+    y.f_norm = at(p + "mlp.norm"); y.gate_up = at(p + "mlp.w_gate_up"); y.down = at(p + "mlp.w_down");
+  }
 }
 
 __global__ void bf16_to_f16_kernel(const __nv_bfloat16* __restrict__ src, __half* __restrict__ dst, size_t n,
@@ -366,6 +408,7 @@ size_t hspec_workspace_bytes(const hspec_config* cfg) {
 int hspec_load_weights(hspec_handle* h, const hspec_tensor* t, int32_t n) {
   if (!h || (!t && n > 0) || n < 0) return fail(h, HSPEC_ERR_INVALID_ARG, "hspec_load_weights: bad argument");
   std::string errtxt;
+  h->complete = false;                               // until every tensor of this call is in place
   int dev_count = 0;
   if (cudaGetDeviceCount(&dev_count) != cudaSuccess || dev_count < 1)
     return fail(h, HSPEC_ERR_CUDA, "hspec_load_weights: no CUDA device; this library has no CPU path");
@@ -423,6 +466,7 @@ int hspec_load_weights(hspec_handle* h, const hspec_tensor* t, int32_t n) {
     h->w[name] = w;
   }
   CUDA_TRY(h, cudaDeviceSynchronize());
+  resolve_weights(h);
   return HSPEC_OK;
 }
 
@@ -478,8 +522,8 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   }
   if (reinterpret_cast<uintptr_t>(in->workspace) & 1023)
     return fail(h, HSPEC_ERR_INVALID_ARG, "hspec_draft_block: workspace must be 1024-byte aligned");
-  for (const std::string& nm : required_names(c))
-    if (h->w.find(nm) == h->w.end()) return fail(h, HSPEC_ERR_NOT_LOADED, "hspec_draft_block: tensor '" + nm + "' was never loaded");
+  if (!h->complete) resolve_weights(h);              // (a load that failed half-way may still have left a complete set)
+  if (!h->complete) return fail(h, HSPEC_ERR_NOT_LOADED, "hspec_draft_block: tensor '" + missing_tensor(h) + "' was never loaded");
 
   const int B = in->B, k = in->k, M = B * k;
   int max_ctx = in->max_ctx > 0 ? in->max_ctx : in->page_table_stride * c.page_size;
@@ -524,17 +568,19 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   const double Md = double(M);
 
   const bool bf = c.act_bf16 != 0;                 // bf16 tensor-core operands instead of fp16
-  auto W = [&](const std::string& nm) -> const Weight& { return h->w.at(nm); };
-  auto fptr = [&](const std::string& nm) { return reinterpret_cast<const float*>(h->w.at(nm).data); };
-  auto gemm = [&](const std::string& wname, const char* label, const void* x, int rows, int mode, void* o,
-                  long long ldo) -> cudaError_t {
-    const Weight& w = W(wname);
+  const StepWeights& SW = h->by_role;
+  GemmTail tail{};                                 // what the last residual GEMM left for the norm behind it to add to X
+  auto fptr = [](const Weight* w) { return reinterpret_cast<const float*>(w->data); };
+  auto gemm = [&](const Weight* wp, const char* label, const void* x, int rows, int mode, void* o, long long ldo) -> cudaError_t {
+    const Weight& w = *wp;
+    if (mode == EPI_ACCUM_F32) tail = GemmTail{};
     GemmCall g{};
     g.tmW = &w.tm; g.x = x; g.f16 = !bf; g.ldx = w.cols; g.M = rows; g.n_out = int(w.rows); g.K = int(w.cols);
     g.mode = mode; g.out = o; g.ldo = ldo;
     g.splits = gemm_pick_splits(rows, g.n_out, g.K, kNumSMs, mode);
     g.splitk_ws = ws + p.SPLITK; g.splitk_ws_bytes = p.splitk_bytes;
     g.status = h->d_status; g.label = label;
+    g.defer_tail = mode == EPI_ACCUM_F32 ? &tail : nullptr;
     return gemm_launch(g, st, trk, &errtxt);
   };
   // element-wise launches: bracket with the tracker (name, algorithmic bytes)
@@ -562,19 +608,19 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   prep.n_lh = size_t(B) * c.n_fuse * c.D;
   if (bf && (reinterpret_cast<uintptr_t>(in->last_hidden) & 15) == 0) lh_in = in->last_hidden;   // already the operand type: read in place
   else { prep.lh_src = in->last_hidden; prep.lh_dst = LH; }
-  EW("embed_norm", Md * c.D * 6, embed_norm_launch(W("embed").data, in->last_token, c.mask_id, fptr("layers.0.mamba.norm"), X, U, B, k, c.D,
+  EW("embed_norm", Md * c.D * 6, embed_norm_launch(SW.embed->data, in->last_token, c.mask_id, fptr(SW.layer[0].m_norm), X, U, B, k, c.D,
                                                    c.rms_eps, prep, st, h->d_status, bf));
   // S_init = Proj_dS(Proj_r(concat h)): once per step, shared by all layers
-  CUDA_TRY(h, gemm("proj_r", "gemm:proj_r", lh_in, B, bf ? EPI_STORE_BF16 : EPI_STORE_F16, Fv, c.r));
+  CUDA_TRY(h, gemm(SW.proj_r, "gemm:proj_r", lh_in, B, bf ? EPI_STORE_BF16 : EPI_STORE_F16, Fv, c.r));
   // (S_init is an output the scan consumes, not a GEMM operand: it stays fp16 in both modes)
-  CUDA_TRY(h, gemm("proj_ds", "gemm:proj_ds", Fv, B, EPI_STORE_F16, SINIT, d.d_S));
+  CUDA_TRY(h, gemm(SW.proj_ds, "gemm:proj_ds", Fv, B, EPI_STORE_F16, SINIT, d.d_S));
 
   for (int l = 0; l < c.L; ++l) {
-    const std::string pre = "layers." + std::to_string(l) + ".";
+    const StepWeights::Layer& lw = SW.layer[l];
     // ---- Mamba-2 mixer from the injected state
     const int rows = l == 0 ? rows0 : M;             // rows of the mixer's input projection
-    if (l > 0) EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(pre + "mamba.norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
-    CUDA_TRY(h, gemm(pre + "mamba.in_proj", "gemm:in_proj", U, rows, EPI_STORE_F32, BIG, d.d_in_proj));
+    if (l > 0) EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.m_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
+    CUDA_TRY(h, gemm(lw.in_proj, "gemm:in_proj", U, rows, EPI_STORE_F32, BIG, d.d_in_proj));
     const float* dt_raw = nullptr;
     if (c.dt_rank > 0) {
       trk->begin("cvt_dt_cols", 0, double(rows) * c.dt_rank * 6);
@@ -582,62 +628,62 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
                                                                      DTL, h->d_status, bf ? 1 : 0);
       trk->end();
       CUDA_TRY(h, cudaGetLastError());
-      CUDA_TRY(h, gemm(pre + "mamba.dt_up", "gemm:dt_up", DTL, rows, EPI_STORE_F32, DT, d.H));
+      CUDA_TRY(h, gemm(lw.dt_up, "gemm:dt_up", DTL, rows, EPI_STORE_F32, DT, d.H));
       dt_raw = DT;
     }
     ScanCall sc{};
     sc.zxbcdt = BIG; sc.ld_in = d.d_in_proj; sc.dt_raw = dt_raw; sc.s_init = SINIT;
-    sc.conv_w = fptr(pre + "mamba.conv_w"); sc.conv_b = fptr(pre + "mamba.conv_b");
-    sc.dt_bias = fptr(pre + "mamba.dt_bias"); sc.A_log = fptr(pre + "mamba.A_log"); sc.Dskip = fptr(pre + "mamba.Dskip");
+    sc.conv_w = fptr(lw.conv_w); sc.conv_b = fptr(lw.conv_b);
+    sc.dt_bias = fptr(lw.dt_bias); sc.A_log = fptr(lw.A_log); sc.Dskip = fptr(lw.Dskip);
     sc.shared_rows = l == 0 && k > 1;
     sc.y_gated = YG; sc.B = B; sc.k = k; sc.Di = c.Di; sc.P = c.P; sc.N = c.N; sc.G = c.G; sc.d_conv = c.d_conv;
     sc.ws = ws + p.SCAN; sc.ws_bytes = p.scan_bytes;
     CUDA_TRY(h, scan_launch(sc, st, trk, &errtxt));
-    EW("rmsnorm_gated", Md * c.Di * 6, rmsnorm_launch(YG, fptr(pre + "mamba.gnorm"), U, M, c.Di, c.rms_eps, st, h->d_status, bf));
-    CUDA_TRY(h, gemm(pre + "mamba.out_proj", "gemm:out_proj", U, M, EPI_ACCUM_F32, X, c.D));
+    EW("rmsnorm_gated", Md * c.Di * 6, rmsnorm_launch(YG, fptr(lw.gnorm), U, M, c.Di, c.rms_eps, st, h->d_status, bf));
+    CUDA_TRY(h, gemm(lw.out_proj, "gemm:out_proj", U, M, EPI_ACCUM_F32, X, c.D));
     // ---- attention over the target's KV (in place) + the block
     if (c.has_attn[l]) {
-      EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(pre + "attn.norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
-      CUDA_TRY(h, gemm(pre + "attn.wqkv", "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv));
+      EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.a_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
+      CUDA_TRY(h, gemm(lw.wqkv, "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv));
       EW("qk_norm_rope", Md * d.d_qkv * 6,
-         qk_norm_rope_launch(BIG, fptr(pre + "attn.q_norm"), fptr(pre + "attn.k_norm"), in->ctx_lens, Q, KB, VB, B, k, c.Hq,
+         qk_norm_rope_launch(BIG, fptr(lw.q_norm), fptr(lw.k_norm), in->ctx_lens, Q, KB, VB, B, k, c.Hq,
                              c.Hkv, c.dh, c.rope_theta, c.rms_eps, c.qk_norm, st));
       AttnCall a = attn_call();
       a.k_pool = in->k_pools[c.kv_slot[l]]; a.v_pool = in->v_pools[c.kv_slot[l]];
       CUDA_TRY(h, attention_launch(a, st, trk, &errtxt));
-      CUDA_TRY(h, gemm(pre + "attn.wo", "gemm:wo", U, M, EPI_ACCUM_F32, X, c.D));
+      CUDA_TRY(h, gemm(lw.wo, "gemm:wo", U, M, EPI_ACCUM_F32, X, c.D));
     }
     // ---- SwiGLU MLP
-    EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(pre + "mlp.norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
+    EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.f_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
     if (c.F % 16 == 0) {
       // gate/up rows were interleaved at load: the GEMM epilogue applies SiLU(gate) * up and writes h directly.
       // U is both the GEMM's input (D columns) and h's home (F columns), so h goes to a second fp16 buffer.
-      CUDA_TRY(h, gemm(pre + "mlp.w_gate_up", "gemm:gate_up", U, M, bf ? EPI_SWIGLU_BF16 : EPI_SWIGLU_F16, U2, c.F));
+      CUDA_TRY(h, gemm(lw.gate_up, "gemm:gate_up", U, M, bf ? EPI_SWIGLU_BF16 : EPI_SWIGLU_F16, U2, c.F));
     } else {
-      CUDA_TRY(h, gemm(pre + "mlp.w_gate_up", "gemm:gate_up", U, M, EPI_STORE_F32, BIG, 2 * c.F));
+      CUDA_TRY(h, gemm(lw.gate_up, "gemm:gate_up", U, M, EPI_STORE_F32, BIG, 2 * c.F));
       EW("swiglu", Md * c.F * 10, swiglu_launch(BIG, U2, M, c.F, st, h->d_status, bf));
     }
-    CUDA_TRY(h, gemm(pre + "mlp.w_down", "gemm:down", U2, M, EPI_ACCUM_F32, X, c.D));
+    CUDA_TRY(h, gemm(lw.down, "gemm:down", U2, M, EPI_ACCUM_F32, X, c.D));
   }
-  if (out->hidden) EW("copy_hidden", Md * c.D * 8, copy_f32_launch(X, out->hidden, size_t(M) * c.D, st));
   // ---- final norm, LM head fused with the per-row arg-max
-  EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr("final_norm"), U, M, c.D, c.rms_eps, st, h->d_status, bf));
-  const int* id_map = c.V_draft > 0 ? reinterpret_cast<const int*>(W("vocab_map").data) : nullptr;
+  EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(SW.final_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
+  if (out->hidden) EW("copy_hidden", Md * c.D * 8, copy_f32_launch(X, out->hidden, size_t(M) * c.D, st));
+  const int* id_map = c.V_draft > 0 ? reinterpret_cast<const int*>(SW.vocab_map->data) : nullptr;
   if (c.markov_rank > 0) {
     // ---- LM head to fp32 logits, then the causal correction position by position (Sec. 3.3.3)
     float* logits = out->logits ? out->logits : reinterpret_cast<float*>(ws + p.LOGITS);
-    const Weight& w = W("lm_head");
+    const Weight& w = *SW.lm_head;
     GemmCall g{};
     g.tmW = &w.tm; g.x = U; g.f16 = !bf; g.ldx = c.D; g.M = M; g.n_out = d.Vd; g.K = c.D; g.mode = EPI_STORE_F32; g.splits = 1;
     g.out = logits; g.ldo = d.Vd; g.status = h->d_status; g.label = "gemm:lm_head";
     CUDA_TRY(h, gemm_launch(g, st, trk, &errtxt));
     MarkovCall mc{};
-    mc.logits = logits; mc.ld = d.Vd; mc.W_in = W("markov_in").data; mc.tmW_out = &W("markov_out").tm; mc.f16 = !bf;
+    mc.logits = logits; mc.ld = d.Vd; mc.W_in = SW.markov_in->data; mc.tmW_out = &SW.markov_out->tm; mc.f16 = !bf;
     mc.last_token = in->last_token; mc.id_map = id_map; mc.ids = out->draft_ids; mc.B = B; mc.k = k; mc.Vd = d.Vd;
     mc.r = c.markov_rank; mc.write_logits = out->logits != nullptr; mc.ws = ws + p.MARKOV; mc.status = h->d_status;
     CUDA_TRY(h, markov_launch(mc, st, trk, &errtxt));
   } else {
-    const Weight& w = W("lm_head");
+    const Weight& w = *SW.lm_head;
     GemmCall g{};
     g.tmW = &w.tm; g.x = U; g.f16 = !bf; g.ldx = c.D; g.M = M; g.n_out = d.Vd; g.K = c.D; g.mode = EPI_ARGMAX; g.splits = 1;
     g.logits = out->logits; g.ldo = d.Vd;
@@ -838,7 +884,8 @@ int hspec_op_markov_head(float* logits, int64_t ld, const void* W_in, const void
 int hspec_op_rmsnorm(const float* x, const float* w, void* y, int32_t M, int32_t n, float eps, void* stream) {
   if (!x || !w || !y || M < 1 || n < 1) return fail(nullptr, HSPEC_ERR_INVALID_ARG, "hspec_op_rmsnorm: bad argument");
   std::string errtxt;
-  OP_TRY(rmsnorm_launch(x, w, y, M, n, eps, reinterpret_cast<cudaStream_t>(stream), global_status()));
+  // (without a pending tail x is only read)
+  OP_TRY(rmsnorm_launch(const_cast<float*>(x), w, y, M, n, eps, reinterpret_cast<cudaStream_t>(stream), global_status()));
   return HSPEC_OK;
 }
 

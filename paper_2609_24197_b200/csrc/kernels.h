@@ -139,6 +139,12 @@ struct GemmArgs {       // kernel argument block
   uint32_t* status;
 };
 
+// Partial tiles of a 2-SM GEMM whose K-sliced tail wave has not been summed yet: [tail tile][slice][activation row][256 weight rows].
+struct GemmTail {
+  const float* part;        // null: nothing pending
+  int n_full_tiles, n_tiles_m, BNT, splits;
+};
+
 struct GemmCall {       // host-side description of one y = x W^T
   const CUtensorMap* tmW;   // weights [n_out, K], box 128 x 64
   const void* x;            // [M, K] in the same 16-bit type as the weights, row pitch ldx elements
@@ -159,6 +165,7 @@ struct GemmCall {       // host-side description of one y = x W^T
   int* part_idx;
   uint32_t* status;
   const char* label;        // profile name (may be null)
+  GemmTail* defer_tail;     // EPI_ACCUM_F32: the caller adds the sliced tail tiles itself (their description is left here); may be null
 };
 
 bool make_tmap_16bit_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld_elems,
@@ -259,8 +266,9 @@ struct StepPrep {
 };
 cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,
                               int B, int k, int D, float eps, const StepPrep& prep, cudaStream_t stream, uint32_t* status, bool bf16_out);
-cudaError_t rmsnorm_launch(const float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
-                           uint32_t* status, bool bf16_out = false);
+// tail: the last GEMM's tail tiles are still to be added to x (x is then written as well); null or empty: x is only read.
+cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, float eps, cudaStream_t stream,
+                           uint32_t* status, bool bf16_out = false, const GemmTail* tail = nullptr);
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,
                                 void* kb, void* vb, int B, int k, int Hq, int Hkv, int dh, float theta, float eps,
                                 int qk_norm, cudaStream_t stream);

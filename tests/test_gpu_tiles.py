@@ -185,3 +185,17 @@ def test_attention_row_copies(hs, k, rep, window, chunk):
         mag = torch.einsum("ihrj,jhd->ihrd", p, V.abs()).reshape(k, Hq * dh)
         err = (o[b * k:(b + 1) * k].double() - ref).abs()
         assert bool((err <= 2.0 ** -8 * mag + 2.0 ** -11 * ref.abs() + 1e-6).all()), float((err / mag).max())
+
+
+# the norm behind a residual GEMM adds the GEMM's K-sliced tail tiles: row counts with a whole-wave part and a tail, all tail, and no tail,
+# widths above and below what the norm keeps in registers (6 x 4 x 256 and 6 x 4 x 512 floats), hidden state asked for
+@pytest.mark.parametrize("D,F,B,k", [(512, 4096, 9, 32), (4096, 2048, 20, 13), (7168, 1024, 9, 30), (12544, 512, 10, 26)])
+def test_residual_tail_is_added_by_the_norm(hs, D, F, B, k):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(D=D, n_fuse=1, r=64, L=1, has_attn=[0], kv_slot=[-1], n_slots=0, Di=1024, P=64, N=4, G=1, d_conv=4, dt_rank=0,
+                             Hq=2, Hkv=1, dh=64, rope_theta=1.0e4, window=0, qk_norm=1, F=F, V=300, rms_eps=1e-6, page_size=16, name="tail",
+                             B=B, k=k, ctx=("const", 16, 16)))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[16] * B)
+    check_step(cfg, drafter, w, batch, k, requests=[0, B - 1], what=f"tail {D} {F}")
+    drafter.close()
