@@ -5,7 +5,8 @@
 // 152 064 and rank 256; it stays in the L2 for the next position) and the batch's logits rows (read, and written back when the
 // caller wants them).  As one GEMM and one reduction launch per position it took 47.6 + 8.9 us at 32 requests and that
 // vocabulary and 44 + 9.8 us at 96 requests and 32 000 rows: CTAs too short to fill their pipelines, a reduction network per
-// 16 columns, and a launch boundary on each side.  As one launch for all positions: 22 and 23 us per position.
+// 16 columns, and a launch boundary on each side.  As one launch for all positions: 21 and 14 us per position (and 52 against 72 at
+// 128 requests and 152 064 rows, logits not written).
 //
 // Here one cooperative kernel (one CTA per SM) walks the positions with a grid barrier between them:
 //   warp 16       producer: 64-column boxes of W_out (128 vocabulary rows each) through a ring of 16 KB stages; it does not
@@ -194,25 +195,35 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&tail->x_ready));
     };
-    float add[NCH * 8];
+    // Logits on their way: AQ chunks (of the NCH a tile has), refilled as they are used.  With four chunks of maxima 96 registers have
+    // room for one: a spilled logit waits for its load on the spot (us per position at 128 requests, V = 152 064: one chunk 62.8,
+    // two 77.5, four 93.8).
+    constexpr int AQ = NCH == 4 ? 1 : NCH;
+    float add[AQ * 8];
     const size_t req_stride = size_t(a.k) * a.ld;                // from request to request in the block's logits
+    // (the empty asm keeps the walk a chain of additions: as base + j x stride the offsets of all columns were kept in registers
+    // across the tiles, and the logits spilled: 18.8 -> 14.0 us per position at 96 requests, 119 -> 94 at 128)
+    auto step_row = [&](auto*& p) { p += req_stride; asm volatile("" : "+l"(p)); };
     auto load_add = [&](int u, int pos, int t) {                 // chunk u of this CTA's t-th tile at position pos
       const int n = (cta + t * grid) * TILE_W + row_in_tile, c0 = (u * 4 + cg) * 8;
       const float* src = a.logits + size_t(pos) * a.ld + n + size_t(c0) * req_stride;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) add[u * 8 + j] = (n < a.Vd && c0 + j < a.B) ? __ldcs(src + j * req_stride) : 0.f;
+      for (int j = 0; j < 8; ++j) {
+        add[u % AQ * 8 + j] = (n < a.Vd && c0 + j < a.B) ? __ldcs(src) : 0.f;
+        step_row(src);
+      }
     };
 #pragma unroll
-    for (int u = 0; u < NCH; ++u) load_add(u, 0, 0);
+    for (int u = 0; u < AQ; ++u) load_add(u, 0, 0);
     gather([&](int b) { return a.last_token[b]; });
 
     for (int pos = 0; pos < a.k; ++pos) {
       float best[NCH * 8];
-      uint32_t ord[NCH * 4];                                     // ordinal of the best tile, two 16-bit values per register
+      uint32_t ord[NCH * 2];                                     // ordinal of the best tile, four 8-bit values per register
 #pragma unroll
       for (int j = 0; j < NCH * 8; ++j) best[j] = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < NCH * 4; ++j) ord[j] = 0;
+      for (int j = 0; j < NCH * 2; ++j) ord[j] = 0;
       for (int t = 0; t < n_my; ++t, ++gt) {
         const uint32_t acc = gt & 1;
         const int n = (cta + t * grid) * TILE_W + row_in_tile;
@@ -235,17 +246,19 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
           float* dst = a.logits + size_t(pos) * a.ld + n + size_t(c0) * req_stride;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float v = __uint_as_float(r[j]) + add[u * 8 + j];
+            const float v = __uint_as_float(r[j]) + add[u % AQ * 8 + j];
             if (n_ok && c0 + j < a.B) {
-              if (a.write_logits) __stcs(dst + j * req_stride, v);
+              if (a.write_logits) __stcs(dst, v);
               if (v > best[u * 8 + j]) {                         // ascending tiles, strict: the lowest index wins ties
                 best[u * 8 + j] = v;
-                uint32_t& o = ord[(u * 8 + j) >> 1];
-                o = (j & 1) ? ((o & 0xffffu) | (uint32_t(t) << 16)) : ((o & 0xffff0000u) | uint32_t(t));
+                uint32_t& o = ord[(u * 8 + j) >> 2];             // byte j % 4 becomes t
+                o = __byte_perm(o, uint32_t(t), j % 4 == 0 ? 0x3214 : j % 4 == 1 ? 0x3240 : j % 4 == 2 ? 0x3410 : 0x4210);
               }
             }
+            step_row(dst);
           }
-          if (more) load_add(u, pos2, t2);
+          if (u + AQ < NCH) load_add(u + AQ, pos, t);
+          else if (more) load_add(u + AQ - NCH, pos2, t2);
         }
         tc_fence_before();
         __syncwarp();
@@ -259,7 +272,7 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
         unsigned long long v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const uint32_t o = (ord[(u * 8 + j) >> 1] >> ((j & 1) * 16)) & 0xffffu;
+          const uint32_t o = (ord[(u * 8 + j) >> 2] >> ((j & 3) * 8)) & 0xffu;
           const int n = (cta + int(o) * grid) * TILE_W + row_in_tile;
           v[j] = n < a.Vd ? order_key(best[u * 8 + j], uint32_t(n)) : 0ull;
         }
@@ -353,7 +366,7 @@ size_t markov_chain_bytes(int B) { return size_t(3) * B * 8 + 16; }
 // Up to 128 requests whose factor rows leave room for at least four stages of W_out (rank 256 at 128 requests does).
 bool markov_chain_supported(int B, int Vd, int r) {
   const size_t x = size_t((r + TILE_K - 1) / TILE_K) * ((B + 15) / 16 * 16) * 128;
-  return B <= MAX_B && x <= 128 * 1024 && Vd <= (1 << 24);
+  return B <= MAX_B && x <= 128 * 1024 && Vd <= (1 << 21);         // (at 128 SMs or more: a tile's ordinal within its CTA fits a byte)
 }
 
 cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk) {
@@ -379,6 +392,7 @@ cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracke
   // a full SM's shared memory, so that one CTA sits on each SM
   const size_t smem = fixed + size_t(a.stages) * W_STAGE;
   const int grid = a.n_tiles < g_chain_sms[dev] ? a.n_tiles : g_chain_sms[dev];
+  if ((a.n_tiles + grid - 1) / grid > 255) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaMemsetAsync(c.ws, 0, markov_chain_bytes(c.B), stream);
   if (e != cudaSuccess) return e;
   trk_begin(trk, "markov_chain", 2.0 * c.B * c.k * double(c.Vd) * c.r, double(c.k) * c.Vd * c.r * 2,

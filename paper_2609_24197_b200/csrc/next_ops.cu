@@ -212,8 +212,9 @@ size_t markov_workspace_bytes(int B, int Vd, int r) {
   return round_up(size_t(B) * r * 2, 256) + 2 * round_up(vt * B * 4, 256) + round_up(markov_chain_bytes(B), 256) + 256;
 }
 
-// Up to 128 requests all positions run in one launch (markov_chain.cu: 176 us against 452 for 8 positions at 32 requests and
-// V = 151 936, 375 against 861 for 16 positions at 96 requests and V = 32 000); above that one GEMM and one reduction per position.
+// Up to 128 requests all positions run in one launch (markov_chain.cu; us per position with the logits written, GEMM + reduction against
+// it: 32 requests, V = 151 936 48 / 21, 96, 32 000 34 / 14, 64, 152 064 69 / 30, 1, 32 000 10.4 / 7.6); above that one GEMM and one
+// reduction per position.
 cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk, std::string* err) {
   if (markov_chain_supported(c.B, c.Vd, c.r)) return markov_chain_launch(c, stream, trk);
   const size_t vt = (size_t(c.Vd) + 127) / 128;
