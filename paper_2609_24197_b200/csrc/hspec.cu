@@ -624,8 +624,9 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     const float* dt_raw = nullptr;
     if (c.dt_rank > 0) {
       trk->begin("cvt_dt_cols", 0, double(rows) * c.dt_rank * 6);
-      cvt_cols_f16_kernel<<<(rows * c.dt_rank + 255) / 256, 256, 0, st>>>(BIG, d.d_in_proj, c.Di + d.d_xBC, c.dt_rank, rows,
-                                                                     DTL, h->d_status, bf ? 1 : 0);
+      // (a plain launch between overlapped ones held the host up for 20 us)
+      CUDA_TRY(h, launch_pdl(cvt_cols_f16_kernel, dim3((rows * c.dt_rank + 255) / 256), dim3(256), 0, st, (const float*)BIG, (long long)d.d_in_proj,
+                             c.Di + d.d_xBC, c.dt_rank, rows, DTL, h->d_status, bf ? 1 : 0));
       trk->end();
       CUDA_TRY(h, cudaGetLastError());
       CUDA_TRY(h, gemm(lw.dt_up, "gemm:dt_up", DTL, rows, EPI_STORE_F32, DT, d.H));

@@ -783,8 +783,7 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     }
     dim3 grid_f(a.H / 4, c.B);
     trk_begin(trk, "mamba_scan", 2.0 * c.B * c.k * a.H * c.P * c.N, double(c.B) * a.H * c.P * c.N * 2);
-    if (two) mamba_scan_mma_kernel<64, 128, 2><<<grid_f, 128, smem_f, stream>>>(a);
-    else mamba_scan_mma_kernel<64, 128, 1><<<grid_f, 128, smem_f, stream>>>(a);
+    launch_pdl(two ? mamba_scan_mma_kernel<64, 128, 2> : mamba_scan_mma_kernel<64, 128, 1>, grid_f, dim3(128), smem_f, stream, a);
     trk_end(trk);
     return cudaGetLastError();
   }
@@ -818,7 +817,7 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   }
   dim3 grid(a.H, c.B);
   trk_begin(trk, "mamba_scan", 0, double(c.B) * a.H * c.P * c.N * 2);
-  mamba_scan_kernel<<<grid, SCAN_THREADS, smem, stream>>>(a);
+  launch_pdl(mamba_scan_kernel, grid, dim3(SCAN_THREADS), smem, stream, a);
   trk_end(trk);
   return cudaGetLastError();
 }
