@@ -10,6 +10,7 @@
 #include "common.cuh"
 #include "kernels.h"
 
+#include <algorithm>
 #include <cstdlib>
 
 namespace hspec {
@@ -322,11 +323,19 @@ int rows_per_cta(int R) { int rt = ((R + 15) / 16) * 16; return rt > 128 ? 128 :
 
 }  // namespace
 
-int attn_pick_chunk(int B, int Hkv, int max_ctx, int window, int num_sms) {
+int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms) {
   // with a window the visible range starts on a page boundary, up to 15 tokens before the window itself: size the
   // chunks for window + 15 tokens, or a request's last few tokens become a chunk (and a merge) of their own
   int lmax = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
   if (lmax < 1) lmax = 1;
+  if (dh != 128) {
+    // The mma.sync kernel walks its 64-key tiles one after the other, about 4 us each when few rows share a KV head, so a context is cut
+    // down to single tiles as long as that gives no more than four CTAs per SM (test-sized drafter, us per step, 256-token chunks / two /
+    // four / eight CTAs per SM: one request of 256 tokens 84.5 / 76.6 / 76.6 / 76.6, 64 of 1000..4096 with 32 positions 264 / 264 / 221 / 224,
+    // 30 of 500..4096 with a 2048-token window 162 / 136 / 130 / 137).
+    const int n = std::min(32, (4 * num_sms + B * Hkv - 1) / (B * Hkv));
+    return std::min(8192, std::max(KT, (lmax + n * KT - 1) / (n * KT) * KT));
+  }
   if (window > 0 && lmax == window + 15) {
     // Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
     // Cost of a round in tiles: the chunk's own, three for an item's set-up and read-out, one more for a partial and its merge.

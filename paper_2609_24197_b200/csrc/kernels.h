@@ -231,7 +231,7 @@ struct AttnPlan {
   int* count;
   int4* items;
 };
-int attn_pick_chunk(int B, int Hkv, int max_ctx, int window, int num_sms);
+int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms);
 size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens);
 cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool attention_tc_supported(const AttnCall& c);
