@@ -41,7 +41,7 @@ constexpr uint32_t A_BYTES = 128 * TILE_K * 2;     // 16 KiB: this CTA's 128 wei
 
 struct Gemm2Args {
   int M, N_out, K;
-  int BNT;                 // activation rows per cluster tile (a multiple of 32, at most 256); each CTA stages BNT/2
+  int BNT;                 // activation rows per cluster tile (a multiple of 16, at most 256); each CTA stages BNT/2
   uint32_t acc_cols;       // TMEM columns per accumulator: BNT rounded up to a power of two
   int k_tiles, stages;
   int ksub;                // 64-column k-steps per pipeline stage (1 or 2): one barrier round per stage
@@ -421,7 +421,7 @@ bool gemm2_preferred(int M, int n_out) {
 // by a simple model: full waves of the 74 SM pairs x k-steps x cost of a k-step, plus the tail wave (k-steps / slices),
 // a fixed cost per wave (pipeline fill, the last epilogue) and, with slices, the pass that sums the partial tiles.
 // One cost unit ~ 2.2 ns (a k-step of a 256-wide pair tile = 256 units ~ 0.56 us).
-// The rows are spread evenly over the tiles, so that the last one is not mostly padding: 549 rows are three tiles of 192
+// The rows are spread evenly over the tiles, in steps of 16, so that the last one is not mostly padding: 549 rows are three tiles of 192
 // and not of 256 (n_out = 28672, K = 4096: 134 -> 122 us; n_out = 4096, K = 14336: 70 -> 66 us).
 void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out) {
   const int tw = (n_out + 255) / 256;
@@ -431,7 +431,7 @@ void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out
   int best_bnt = 256, best_s = 1;
   for (int widest = 256; widest >= 128; widest -= 32) {
     const int nm = (M + widest - 1) / widest;
-    const int bnt = ((M + nm - 1) / nm + 31) / 32 * 32;
+    const int bnt = ((M + nm - 1) / nm + 15) / 16 * 16;
     const int tiles = tw * nm;
     const int full_waves = tiles / 74, tail = tiles % 74;
     // a k-step fills 16 KB of weights and BNT x 64 bytes of activations per SM: below 256 rows it is this fill that sets the
