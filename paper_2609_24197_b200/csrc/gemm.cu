@@ -81,14 +81,21 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_acc = tail->tmem_base;
-  pdl_wait();                                   // set-up done: now the previous kernel's results may be read
-  pdl_trigger();
 
   if (warp == 0) {
     if (elect_one()) {
       // weights are streamed once per step, unless the caller runs the same matrix again right away
       const uint64_t pol_w = g.keep_w ? policy_evict_last() : policy_evict_first();
       const uint64_t pol_x = policy_evict_last();    // activations are re-read by every weight tile
+      // The weights do not depend on the kernels in front: the first stages' boxes are requested while those still run.
+      int early = 0;
+      for (; g.early_w && early < n_kt && early < g.stages; ++early) {
+        const uint32_t full = smem_u32(&tail->full[early]);
+        mbar_expect_tx(full, stage_bytes);
+        tma_load_2d(smem_u32(smem + size_t(early) * stage_bytes), &tmA, (kt_begin + early) * TILE_K, tile_n * TILE_W, full, pol_w);
+      }
+      pdl_wait();
+      pdl_trigger();
       for (int i = 0; i < n_kt; ++i) {
         const int s = i % g.stages;
         const uint32_t round = i / g.stages;
@@ -98,9 +105,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           break;
         }
         const uint32_t full = smem_u32(&tail->full[s]);
-        mbar_expect_tx(full, stage_bytes);
         uint8_t* sa = smem + size_t(s) * stage_bytes;
-        tma_load_2d(smem_u32(sa), &tmA, (kt_begin + i) * TILE_K, tile_n * TILE_W, full, pol_w);
+        if (i >= early) {
+          mbar_expect_tx(full, stage_bytes);
+          tma_load_2d(smem_u32(sa), &tmA, (kt_begin + i) * TILE_K, tile_n * TILE_W, full, pol_w);
+        }
         tma_load_2d(smem_u32(sa + A_STAGE_BYTES), &tmB, (kt_begin + i) * TILE_K, tile_m * g.BN, full, pol_x);
       }
     }
@@ -134,6 +143,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else {
     // ---------------------------------------------------------------- epilogue
     const int q = warp & 3;                         // TMEM lane quarter this warp may read
+    pdl_wait();                                     // nothing else is read or written before the kernels in front have finished
     if (g.addend != nullptr && g.mode == EPI_ARGMAX) {
       // the addend rows of this tile do not depend on the accumulator: pull this warp's 128-byte piece of every
       // row into L2 while the main loop runs (one line per lane and pass)
@@ -467,6 +477,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   g.f16 = c.f16 ? 1 : 0;
   g.logits = c.logits; g.addend = c.addend; g.ld_add = c.ld_add; g.part_val = c.part_val; g.part_idx = c.part_idx;
   g.keep_w = c.keep_weights_in_l2 ? 1 : 0;
+  g.early_w = c.w_stable ? 1 : 0;
   g.ldo = c.ldo;
   if (splits > 1 && c.mode == EPI_ARGMAX) { if (err) *err = "LM-head epilogue cannot be K-sliced"; return cudaErrorInvalidValue; }
   if (splits > 1 && size_t(stages) * stage_bytes < size_t(g.BN) * TILE_W * 4) {

@@ -52,6 +52,7 @@ struct Gemm2Args {
   int n_full_tiles, tail_splits, k_tiles_per_split;
   float* part;
   int f16, mode;
+  int early_w;             // the weights may be read before the previous kernel of the stream has finished
   void* out;
   long long ldo;
   float* logits;
@@ -162,8 +163,6 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = tail->tmem_base;
   volatile uint32_t* abort_flag = &tail->abort_flag;
-  pdl_wait();                                   // set-up done: now the previous kernel's results may be read
-  pdl_trigger();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -173,6 +172,22 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       // 13.5 vs 13.75 ms per step at conc128_32b.
       // (With a single activation tile nobody shares a weight tile: the weights stream through once, evict-first.)
       const uint64_t pol_w = g.n_tiles_m == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
+      // The weights do not depend on the kernels in front: the first stages' boxes are requested while those still run.
+      uint32_t early = 0;
+      if (g.early_w) {
+        int tile, sp, kt_begin, kt_end;
+        decode(cluster_id, tile, sp, kt_begin, kt_end);
+        for (int kt = kt_begin; kt < kt_end && early < uint32_t(g.stages); kt += g.ksub, ++early) {
+          const int n_sub = min(g.ksub, kt_end - kt);
+          const uint32_t full = smem_u32(&tail->full[early]);
+          if (rank == 0) mbar_expect_tx(full, 2 * uint32_t(n_sub) * sub_bytes);
+          for (int sub = 0; sub < n_sub; ++sub)
+            tma_load_2d_pair(smem_u32(smem + size_t(early) * stage_bytes + size_t(sub) * sub_bytes), &tmA, (kt + sub) * TILE_K,
+                             (tile / g.n_tiles_m) * 256 + int(rank) * 128, full, pol_w);
+        }
+      }
+      pdl_wait();
+      pdl_trigger();
       uint32_t it = 0;
       bool ok = true;
       for (int unit = cluster_id; unit < total_units && ok; unit += n_clusters) {
@@ -190,10 +205,10 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           }
           const int n_sub = min(g.ksub, kt_end - kt);
           const uint32_t full = smem_u32(&tail->full[s]);
-          if (rank == 0) mbar_expect_tx(full, 2 * uint32_t(n_sub) * sub_bytes);   // both CTAs' bytes land on the leader's barrier
+          if (rank == 0 && it >= early) mbar_expect_tx(full, 2 * uint32_t(n_sub) * sub_bytes);   // both CTAs' bytes land on the leader's barrier
           for (int sub = 0; sub < n_sub; ++sub) {
             uint8_t* sa = smem + size_t(s) * stage_bytes + size_t(sub) * sub_bytes;
-            tma_load_2d_pair(smem_u32(sa), &tmA, (kt + sub) * TILE_K, tn * 256 + int(rank) * 128, full, pol_w);
+            if (it >= early) tma_load_2d_pair(smem_u32(sa), &tmA, (kt + sub) * TILE_K, tn * 256 + int(rank) * 128, full, pol_w);
             tma_load_2d_pair(smem_u32(sa + A_BYTES), &tmB, (kt + sub) * TILE_K, tm * g.BNT + int(rank) * (g.BNT / 2), full, pol_x);
           }
         }
@@ -234,6 +249,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
   } else {
     // ---------------------------------------------------------------- epilogue (both CTAs)
+    pdl_wait();                                  // nothing is read or written before the kernels in front have finished
     const int q = warp & 3;
     uint32_t tile_count = 0;
     bool ok = true;
@@ -487,6 +503,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   g.tail_splits = splits;
   g.n_full_tiles = splits > 1 ? tiles - tail : tiles;
   g.part = reinterpret_cast<float*>(c.splitk_ws);
+  g.early_w = c.w_stable ? 1 : 0;
   g.f16 = c.f16 ? 1 : 0; g.mode = c.mode; g.out = c.out; g.ldo = c.ldo;
   if (c.addend != nullptr) { if (err) *err = "the 2-SM kernel has no addend epilogue"; return cudaErrorInvalidValue; }
   g.logits = c.logits; g.part_val = c.part_val; g.part_idx = c.part_idx; g.status = c.status;

@@ -580,6 +580,7 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     g.splits = gemm_pick_splits(rows, g.n_out, g.K, kNumSMs, mode);
     g.splitk_ws = ws + p.SPLITK; g.splitk_ws_bytes = p.splitk_bytes;
     g.status = h->d_status; g.label = label;
+    g.w_stable = true;                             // library copies, or borrowed unchanged for the handle's life
     g.defer_tail = mode == EPI_ACCUM_F32 ? &tail : nullptr;
     return gemm_launch(g, st, trk, &errtxt);
   };
@@ -677,6 +678,7 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     GemmCall g{};
     g.tmW = &w.tm; g.x = U; g.f16 = !bf; g.ldx = c.D; g.M = M; g.n_out = d.Vd; g.K = c.D; g.mode = EPI_STORE_F32; g.splits = 1;
     g.out = logits; g.ldo = d.Vd; g.status = h->d_status; g.label = "gemm:lm_head";
+    g.w_stable = true;
     CUDA_TRY(h, gemm_launch(g, st, trk, &errtxt));
     MarkovCall mc{};
     mc.logits = logits; mc.ld = d.Vd; mc.W_in = SW.markov_in->data; mc.tmW_out = &SW.markov_out->tm; mc.f16 = !bf;
@@ -690,6 +692,7 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     g.logits = out->logits; g.ldo = d.Vd;
     g.part_val = reinterpret_cast<float*>(ws + p.AMAXV); g.part_idx = reinterpret_cast<int*>(ws + p.AMAXI);
     g.status = h->d_status; g.label = "gemm:lm_head_argmax";
+    g.w_stable = true;
     CUDA_TRY(h, gemm_launch(g, st, trk, &errtxt));
     CUDA_TRY(h, argmax_reduce_launch(g.part_val, g.part_idx, (d.Vd + 127) / 128, M, out->draft_ids, st, trk, id_map));
   }

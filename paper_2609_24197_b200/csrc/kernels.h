@@ -134,6 +134,7 @@ struct GemmArgs {       // kernel argument block
   const float* addend;  // EPI_ARGMAX only (one-CTA kernel): value = acc + addend[m * ld_add + n] (may be null)
   long long ld_add;
   int keep_w;           // weights loaded evict-last instead of evict-first
+  int early_w;          // the weights may be read before the previous kernel of the stream has finished
   float* part_val;
   int* part_idx;
   uint32_t* status;
@@ -163,6 +164,7 @@ struct GemmCall {       // host-side description of one y = x W^T
   bool keep_weights_in_l2;  // one-CTA kernel: the same W is used again by the next launch (keep it in L2 if it fits)
   float* part_val;
   int* part_idx;
+  bool w_stable;            // nothing that may still be running on the stream writes the weights: they may be fetched early
   uint32_t* status;
   const char* label;        // profile name (may be null)
   GemmTail* defer_tail;     // EPI_ACCUM_F32: the caller adds the sliced tail tiles itself (their description is left here); may be null
