@@ -199,6 +199,7 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
     // room for one: a spilled logit waits for its load on the spot (us per position at 128 requests, V = 152 064: one chunk 62.8,
     // two 77.5, four 93.8).
     constexpr int AQ = NCH == 4 ? 1 : NCH;
+    static_assert(AQ == NCH || AQ == 1, "the refill below knows these two");
     float add[AQ * 8];
     const size_t req_stride = size_t(a.k) * a.ld;                // from request to request in the block's logits
     // (the empty asm keeps the walk a chain of additions: as base + j x stride the offsets of all columns were kept in registers
@@ -257,8 +258,15 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
             }
             step_row(dst);
           }
-          if (u + AQ < NCH) load_add(u + AQ, pos, t);
-          else if (more) load_add(u + AQ - NCH, pos2, t2);
+          // refill: the chunk's own successor in the next tile, or, with a single chunk in flight, the next one this warp has (a warp's last
+          // chunk can lie past the batch: 112 columns are 14 chunks for 4 x 4 places)
+          if (AQ == NCH) {
+            if (more) load_add(u, pos2, t2);
+          } else if (u + 1 < NCH && c0 + 32 < a.BN) {
+            load_add(u + 1, pos, t);
+          } else if (more) {
+            load_add(0, pos2, t2);
+          }
         }
         tc_fence_before();
         __syncwarp();

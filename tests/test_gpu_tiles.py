@@ -45,7 +45,7 @@ def test_many_row_gemm_tile_widths(hs, M, n_out, K, kind):
 # requests at the edges of the one-launch form's column chunks (32 per epilogue-warp chunk, 16 per MMA step) and of its range (128);
 # vocabularies of less than a tile, of a tile and a row, and of more tiles than SMs; ranks below, at and above a 64-column box
 @pytest.mark.parametrize("B,k,Vd,r", [(1, 1, 100, 8), (16, 3, 129, 64), (17, 4, 128, 72), (32, 2, 5000, 256), (33, 5, 19200, 256),
-                                      (64, 3, 257, 136), (65, 2, 40000, 256), (96, 4, 3001, 256), (97, 2, 900, 512), (128, 5, 21000, 256),
+                                      (64, 3, 257, 136), (65, 2, 40000, 256), (96, 4, 3001, 256), (97, 2, 900, 512), (100, 3, 41000, 256), (112, 3, 700, 64), (113, 3, 700, 64), (128, 5, 21000, 256),
                                       (129, 2, 300, 64)])
 @pytest.mark.parametrize("write", [True, False])
 def test_markov_head_chunks_and_tiles(hs, B, k, Vd, r, write):
