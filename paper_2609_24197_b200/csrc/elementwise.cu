@@ -43,28 +43,35 @@ __device__ __forceinline__ void store_norm4(uint16_t* row, int d4, const float4&
   reinterpret_cast<uint2*>(row)[d4] = out;
 }
 
-// Four sums over the slices of a pending tail tile (slice order), for row m and columns n .. n + 3; zeros where the tile is not one.
-__device__ __forceinline__ float4 tail_sum4(const GemmTail& t, int m, int n) {
-  const int tm = m / t.BNT, tile = (n >> 8) * t.n_tiles_m + tm;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (tile < t.n_full_tiles) return acc;
-  const float* src = t.part + (size_t(tile - t.n_full_tiles) * t.splits * t.BNT + (m - tm * t.BNT)) * 256 + (n & 255);
-  for (int sp = 0; sp < t.splits; ++sp) {
-    const float4 v = __ldcs(reinterpret_cast<const float4*>(src + size_t(sp) * t.BNT * 256));
-    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+// A row's view of a pending tail: weight tile tn of the row is tile first + tn * step of the walk, its partials start at `row` inside a slice.
+struct TailRow {
+  int first, step, row;
+  __device__ TailRow() : first(0), step(0), row(0) {}
+  __device__ TailRow(const GemmTail& t, int m) {
+    const int tm = m / t.BNT;
+    first = t.raster.index_of(0, tm);
+    step = t.raster.index_of(1, tm) - first;
+    row = m - tm * t.BNT;
   }
-  return acc;
+};
+// Where the first slice of columns n .. n + 3 of the row lies; null where their tile is not a tail tile.
+__device__ __forceinline__ const float4* tail_src(const GemmTail& t, const TailRow& r, int n) {
+  const int tile = r.first + (n >> 8) * r.step - t.n_full_tiles;
+  if (tile < 0) return nullptr;
+  return reinterpret_cast<const float4*>(t.part + (size_t(tile) * t.splits * t.BNT + r.row) * 256 + (n & 255));
 }
+__device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 
 // y = x / sqrt(mean(x^2) + eps) * w, one CTA per row, fp16 (or bf16) out.  VPT = 16-byte vectors a thread keeps in
 // registers between the two passes.  TAIL: the residual GEMM in front left the K-slices of its last wave's tiles unsummed; they are
 // added to x here, on the way (a launch of its own cost 6 us and a pass over x).
 template <int VPT, bool TAIL>
-__global__ void rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ w, void* __restrict__ y,
+__global__ void __launch_bounds__(512, 2) rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ w, void* __restrict__ y,
                                int n, float eps, GemmTail tail, uint32_t* status, int bf16_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
+  const TailRow tail_row = TAIL ? TailRow(tail, blockIdx.x) : TailRow();
   float* xr = x + size_t(blockIdx.x) * n;
   uint16_t* yr = reinterpret_cast<uint16_t*>(y) + size_t(blockIdx.x) * n;      // a row of 16-bit values, either type
   if ((n & 3) == 0 && n <= 4 * VPT * int(blockDim.x)) {
@@ -76,12 +83,39 @@ __global__ void rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ 
     for (int i = 0; i < VPT; ++i) {
       const int d4 = threadIdx.x + i * blockDim.x;
       v[i] = d4 < nv ? reinterpret_cast<const float4*>(xr)[d4] : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (TAIL && d4 < nv) {
-        const float4 add = tail_sum4(tail, blockIdx.x, d4 * 4);
-        v[i].x += add.x; v[i].y += add.y; v[i].z += add.z; v[i].w += add.w;
-        reinterpret_cast<float4*>(xr)[d4] = v[i];
-      }
+      if (TAIL) continue;
       ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+    }
+    if (TAIL) {
+      // three vectors at a time (64 registers: four blocks per SM), slice after slice with the three loads of a slice in flight
+      // together; each element is (0 + slice 0 + slice 1 ..) added to x
+      static_assert(VPT % 3 == 0, "vectors are taken in threes");
+#pragma unroll
+      for (int i0 = 0; i0 < VPT; i0 += 3) {
+        const float4* src[3];
+        float4 acc[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const int d4 = threadIdx.x + (i0 + i) * blockDim.x;
+          src[i] = d4 < nv ? tail_src(tail, tail_row, d4 * 4) : nullptr;
+          acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int sp = 0; sp < tail.splits; ++sp) {
+          float4 part[3];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) part[i] = src[i] ? __ldcs(src[i] + size_t(sp) * tail.BNT * 64) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) add4(acc[i], part[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const int d4 = threadIdx.x + (i0 + i) * blockDim.x;
+          float4& x4 = v[i0 + i];
+          add4(x4, acc[i]);
+          if (d4 < nv) reinterpret_cast<float4*>(xr)[d4] = x4;
+          ss += x4.x * x4.x + x4.y * x4.y + x4.z * x4.z + x4.w * x4.w;
+        }
+      }
     }
     const float inv = rsqrtf(block_sum(ss, red) / float(n) + eps);
 #pragma unroll
@@ -98,8 +132,11 @@ __global__ void rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ 
   if (TAIL) {                                       // (n is a multiple of four: the host sees to it)
     for (int d4 = threadIdx.x; d4 < (n >> 2); d4 += blockDim.x) {
       float4 v = reinterpret_cast<const float4*>(xr)[d4];
-      const float4 add = tail_sum4(tail, blockIdx.x, d4 * 4);
-      v.x += add.x; v.y += add.y; v.z += add.z; v.w += add.w;
+      if (const float4* src = tail_src(tail, tail_row, d4 * 4)) {
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int sp = 0; sp < tail.splits; ++sp) add4(acc, __ldcs(src + size_t(sp) * tail.BNT * 64));
+        add4(v, acc);
+      }
       reinterpret_cast<float4*>(xr)[d4] = v;
     }
     __syncthreads();

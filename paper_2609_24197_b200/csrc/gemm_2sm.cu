@@ -45,7 +45,7 @@ struct Gemm2Args {
   uint32_t acc_cols;       // TMEM columns per accumulator: BNT rounded up to a power of two
   int k_tiles, stages;
   int ksub;                // 64-column k-steps per pipeline stage (1 or 2): one barrier round per stage
-  int n_tiles_w, n_tiles_m;
+  GemmRaster raster;
   // Work units: the first n_full_tiles tiles run whole (full waves of the SM pairs); each of the remaining "tail" tiles
   // is cut into tail_splits K-slices so that the last, partly filled wave keeps every pair busy.  A slice stores an
   // fp32 partial tile to `part` ([tail tile][slice][activation row][256 weight rows]); a second kernel sums them.
@@ -127,7 +127,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  const int total_tiles = g.n_tiles_w * g.n_tiles_m;
+  const int total_tiles = g.raster.n_tiles_w * g.raster.n_tiles_m;
   const int total_units = g.n_full_tiles + (total_tiles - g.n_full_tiles) * g.tail_splits;
   // unit u < n_full_tiles: tile u, all of K; else tail tile n_full_tiles + v / tail_splits, K-slice v % tail_splits
   auto decode = [&](int u, int& tile, int& sp, int& kt_begin, int& kt_end) {
@@ -171,19 +171,21 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       // drift apart and fetch it again), and in a long power-capped step the extra DRAM traffic costs clock:
       // 13.5 vs 13.75 ms per step at conc128_32b.
       // (With a single activation tile nobody shares a weight tile: the weights stream through once, evict-first.)
-      const uint64_t pol_w = g.n_tiles_m == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
+      const uint64_t pol_w = g.raster.n_tiles_m == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
       // The weights do not depend on the kernels in front: the first stages' boxes are requested while those still run.
       uint32_t early = 0;
       if (g.early_w) {
         int tile, sp, kt_begin, kt_end;
         decode(cluster_id, tile, sp, kt_begin, kt_end);
+        int tn, tm;
+        g.raster.tile_at(tile, tn, tm);
         for (int kt = kt_begin; kt < kt_end && early < uint32_t(g.stages); kt += g.ksub, ++early) {
           const int n_sub = min(g.ksub, kt_end - kt);
           const uint32_t full = smem_u32(&tail->full[early]);
           if (rank == 0) mbar_expect_tx(full, 2 * uint32_t(n_sub) * sub_bytes);
           for (int sub = 0; sub < n_sub; ++sub)
             tma_load_2d_pair(smem_u32(smem + size_t(early) * stage_bytes + size_t(sub) * sub_bytes), &tmA, (kt + sub) * TILE_K,
-                             (tile / g.n_tiles_m) * 256 + int(rank) * 128, full, pol_w);
+                             tn * 256 + int(rank) * 128, full, pol_w);
         }
       }
       pdl_wait();
@@ -193,7 +195,8 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       for (int unit = cluster_id; unit < total_units && ok; unit += n_clusters) {
         int tile, sp, kt_begin, kt_end;
         decode(unit, tile, sp, kt_begin, kt_end);
-        const int tn = tile / g.n_tiles_m, tm = tile % g.n_tiles_m;
+        int tn, tm;
+        g.raster.tile_at(tile, tn, tm);
         for (int kt = kt_begin; kt < kt_end; kt += g.ksub, ++it) {
           const int s = it % g.stages;
           const uint32_t lap = it / g.stages;
@@ -258,7 +261,8 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     for (int unit = cluster_id; unit < total_units && ok; unit += n_clusters, ++tile_count) {
       int tile, sp, kt_begin, kt_end;
       decode(unit, tile, sp, kt_begin, kt_end);
-      const int tn = tile / g.n_tiles_m, tm = tile % g.n_tiles_m;
+      int tn, tm;
+      g.raster.tile_at(tile, tn, tm);
       const int mode = sp >= 0 ? EPI_PARTIAL_F32 : g.mode;
       const uint32_t acc = tile_count & 1, use = tile_count >> 1;
       if (!mbar_wait(smem_u32(&tail->tmem_full[acc]), use & 1)) {
@@ -377,7 +381,8 @@ gemm2_tail_reduce_kernel(Gemm2Args g) {
   pdl_wait();
   pdl_trigger();
   const int tail = blockIdx.x, tile = g.n_full_tiles + tail;
-  const int tn = tile / g.n_tiles_m, tm = tile % g.n_tiles_m;
+  int tn, tm;
+  g.raster.tile_at(tile, tn, tm);
   const int n = tn * 256 + threadIdx.x;
   const int m_base = tm * g.BNT + blockIdx.y * TAIL_ROWS;
   if (m_base >= g.M) return;
@@ -488,9 +493,16 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   gemm2_pick(c.M, c.n_out, c.K, c.mode, &g.BNT, &splits);
   g.acc_cols = g.BNT > 128 ? 256 : (g.BNT > 64 ? 128 : 64);
   g.k_tiles = (c.K + TILE_K - 1) / TILE_K;
-  g.n_tiles_w = (c.n_out + 255) / 256;
-  g.n_tiles_m = (c.M + g.BNT - 1) / g.BNT;
-  const int tiles = g.n_tiles_w * g.n_tiles_m;
+  g.raster.n_tiles_w = (c.n_out + 255) / 256;
+  g.raster.n_tiles_m = (c.M + g.BNT - 1) / g.BNT;
+  // Groups of at most 16 activation tiles, evenly: with all 32 of M = 8192 inside one weight tile a wave was 32 x 2.3 tiles, its activations
+  // (67 MB at K = 4096) did not stay in the L2 - 1.5 GB read from DRAM where 0.2 were needed - and the power that took came off the
+  // clock.  us (burst / sustained), 32 tiles together, groups of 16, 11, 8: n_out 28672, K 4096 1531 / 1780, 1413 / 1557, 1417 / 1551,
+  // 1442 / 1618; n_out 4096, K 14336 846 / 956, 779 / 882, 762 / 911, 756 / 895.  M = 4096 (16 tiles): whole 699 / 776, two groups of
+  // eight 717 / 796.
+  const int n_groups = (g.raster.n_tiles_m + 15) / 16;
+  g.raster.group = (g.raster.n_tiles_m + n_groups - 1) / n_groups;
+  const int tiles = g.raster.n_tiles_w * g.raster.n_tiles_m;
   const int tail = tiles % 74;
   if (c.splits > 0) splits = c.splits;                    // the caller fixed the number of K-slices (of the tail tiles)
   if (c.mode == EPI_ARGMAX || tail == 0) splits = 1;
@@ -533,7 +545,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   if (e == cudaSuccess) e = cudaGetLastError();
   if (c.defer_tail) *c.defer_tail = GemmTail{};
   if (e == cudaSuccess && splits > 1 && c.defer_tail && c.mode == EPI_ACCUM_F32) {
-    *c.defer_tail = GemmTail{g.part, g.n_full_tiles, g.n_tiles_m, g.BNT, splits};
+    *c.defer_tail = GemmTail{g.part, g.raster, g.n_full_tiles, g.BNT, splits};
     return e;
   }
   if (e == cudaSuccess && splits > 1) {

@@ -140,10 +140,30 @@ struct GemmArgs {       // kernel argument block
   uint32_t* status;
 };
 
+// Order in which the 2-SM GEMM walks its tiles (weight tile tn, activation tile tm): groups of `group` activation tiles, inside a group
+// the weight tiles one after the other, inside a weight tile the group's activation tiles.
+struct GemmRaster {
+  int n_tiles_w, n_tiles_m, group;
+  __host__ __device__ void tile_at(int i, int& tn, int& tm) const {
+    if (group >= n_tiles_m) { tn = i / n_tiles_m; tm = i - tn * n_tiles_m; return; }     // (one group: one division)
+    const int g = i / (n_tiles_w * group), r = i - g * n_tiles_w * group;
+    const int size = group < n_tiles_m - g * group ? group : n_tiles_m - g * group;
+    tn = r / size;
+    tm = g * group + r % size;
+  }
+  __host__ __device__ int index_of(int tn, int tm) const {
+    if (group >= n_tiles_m) return tn * n_tiles_m + tm;
+    const int g = tm / group;
+    const int size = group < n_tiles_m - g * group ? group : n_tiles_m - g * group;
+    return g * n_tiles_w * group + tn * size + tm - g * group;
+  }
+};
+
 // Partial tiles of a 2-SM GEMM whose K-sliced tail wave has not been summed yet: [tail tile][slice][activation row][256 weight rows].
 struct GemmTail {
   const float* part;        // null: nothing pending
-  int n_full_tiles, n_tiles_m, BNT, splits;
+  GemmRaster raster;
+  int n_full_tiles, BNT, splits;
 };
 
 struct GemmCall {       // host-side description of one y = x W^T

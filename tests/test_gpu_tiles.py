@@ -21,9 +21,10 @@ def _rand(shape, seed, dtype=torch.float16, std=1.0):
 
 
 # rows that make the 2-SM kernel take tiles of 256, 224, 192, 160 and 128 rows, full and with a remainder, whole waves and tail
-# waves; weight rows that end inside a tile of the pair
+# waves; weight rows that end inside a tile of the pair; more activation tiles than one group of the walk holds
 @pytest.mark.parametrize("M,n_out,K", [(256, 256, 64), (257, 300, 520), (289, 1000, 512), (430, 2048, 1024), (448, 2048, 1024),
-                                       (449, 512, 2048), (549, 4096, 1024), (640, 19200, 256), (1153, 1111, 264)])
+                                       (449, 512, 2048), (549, 4096, 1024), (640, 19200, 256), (1153, 1111, 264),
+                                       (4500, 1200, 2048)])
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
 def test_many_row_gemm_tile_widths(hs, M, n_out, K, kind):
     x, w = _rand((M, K), 1), _rand((n_out, K), 2, std=0.05)
@@ -189,7 +190,7 @@ def test_attention_row_copies(hs, k, rep, window, chunk):
 
 # the norm behind a residual GEMM adds the GEMM's K-sliced tail tiles: row counts with a whole-wave part and a tail, all tail, and no tail,
 # widths above and below what the norm keeps in registers (6 x 4 x 256 and 6 x 4 x 512 floats), hidden state asked for
-@pytest.mark.parametrize("D,F,B,k", [(512, 4096, 9, 32), (4096, 2048, 20, 13), (7168, 1024, 9, 30), (12544, 512, 10, 26)])
+@pytest.mark.parametrize("D,F,B,k", [(512, 4096, 9, 32), (4096, 2048, 20, 13), (7168, 1024, 9, 30), (12544, 512, 10, 26), (1280, 1024, 141, 32)])
 def test_residual_tail_is_added_by_the_norm(hs, D, F, B, k):
     import synth
     from harness import check_step, cuda_setup
