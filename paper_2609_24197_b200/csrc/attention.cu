@@ -53,8 +53,11 @@ __device__ __forceinline__ uint32_t swz(int row, int col) {   // byte offset of 
   return uint32_t(row * DH * 2 + ((((col >> 3) ^ (row & 7))) << 4) + ((col & 7) << 1));
 }
 
-template <int DH>
-__global__ void __launch_bounds__(256)
+// KS: how many warps share 16 query rows.  Each of them takes KT / KS keys of every tile with a softmax of its own (running maximum, sum
+// and O), merged through shared memory when the chunk is done.  With one warp per 16 rows a call with few rows was one warp's
+// dependent chain, 4 us per tile; four warps also run a quarter of the code, which a step always finds cold in the instruction cache.
+template <int DH, int KS>
+__global__ void __launch_bounds__(KS > 1 ? 352 : 256)
 attn_partial_kernel(AttnArgs a) {
   pdl_wait();
   pdl_trigger();
@@ -77,11 +80,13 @@ attn_partial_kernel(AttnArgs a) {
   uint8_t* sK = sQ + a.RT * DH * 2;
   uint8_t* sV = sK + NSTAGE * KT * DH * 2;
   constexpr int CPR = DH / 8;                        // 16-byte chunks per row
+  constexpr int KW = KT / KS;                        // keys of a tile per warp
 
-  // A warp per 16 query rows computes.  Where those are fewer than four, the block's further warps do all the K/V loading, so that
-  // the few that compute never wait for a page id.
-  const bool compute = warp * 16 < a.RT;
-  const int n_loaders = nthr > a.RT * 2 ? nthr - a.RT * 2 : nthr, loader = nthr > a.RT * 2 ? tid - a.RT * 2 : tid;   // (loader < 0: none)
+  // KS warps per 16 query rows compute.  The block's further warps, where it has any, do all the K/V loading, so that those that
+  // compute never wait for a page id.
+  const int n_compute = a.RT * 2 * KS, slab16 = warp / KS, part = warp % KS;     // (threads; the warp's rows; its part of the keys)
+  const bool compute = tid < n_compute;
+  const int n_loaders = nthr > n_compute ? nthr - n_compute : nthr, loader = nthr > n_compute ? tid - n_compute : tid;   // (loader < 0: none)
 
   // ---- Q rows of this tile -> shared (zero for padding rows)
   const int row0 = rt * a.RT;
@@ -107,7 +112,7 @@ attn_partial_kernel(AttnArgs a) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int idx = idx0 + u * n_loaders, p = base + idx / CPR;
-          page[u] = (idx < KT * CPR && p < p_end) ? __ldg(ptab + p / a.page_size) : -1;
+          page[u] = (idx < KT * CPR && p < p_end) ? ptab[p / a.page_size] : -1;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -148,7 +153,7 @@ attn_partial_kernel(AttnArgs a) {
 
   // rows of this thread inside the warp's 16-row slab
   const int g = lane >> 2, tq = lane & 3;
-  const int r_lo = row0 + warp * 16 + g, r_hi = r_lo + 8;          // global row indices (may be >= R: padding)
+  const int r_lo = row0 + slab16 * 16 + g, r_hi = r_lo + 8;          // global row indices (may be >= R: padding)
   const int i_lo = r_lo / a.rep, i_hi = r_hi / a.rep;              // block position of the row
   float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
   float o[DH / 8][4];
@@ -167,21 +172,21 @@ attn_partial_kernel(AttnArgs a) {
       q_loaded = true;
 #pragma unroll
       for (int ks = 0; ks < DH / 16; ++ks)
-        ldmatrix_x4(qf[ks], smem_u32(sQ) + swz<DH>(warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, ks * 16 + (lane >> 4) * 8));
+        ldmatrix_x4(qf[ks], smem_u32(sQ) + swz<DH>(slab16 * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, ks * 16 + (lane >> 4) * 8));
     }
     const int st = t % NSTAGE;
     const uint32_t bK = smem_u32(sK) + st * KT * DH * 2, bV = smem_u32(sV) + st * KT * DH * 2;
 
-    // ---- S = Q K^T for 64 keys
-    float s[KT / 8][4];
+    // ---- S = Q K^T for this warp's KW keys
+    float s[KW / 8][4];
 #pragma unroll
-    for (int n = 0; n < KT / 8; ++n) { s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f; }
+    for (int n = 0; n < KW / 8; ++n) { s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f; }
 #pragma unroll
     for (int ks = 0; ks < DH / 16; ++ks) {
 #pragma unroll
-      for (int n2 = 0; n2 < KT / 16; ++n2) {
+      for (int n2 = 0; n2 < KW / 16; ++n2) {
         uint32_t kf[4];
-        ldmatrix_x4(kf, bK + swz<DH>(n2 * 16 + (lane & 7) + (lane >> 4) * 8, ks * 16 + ((lane >> 3) & 1) * 8));
+        ldmatrix_x4(kf, bK + swz<DH>(part * KW + n2 * 16 + (lane & 7) + (lane >> 4) * 8, ks * 16 + ((lane >> 3) & 1) * 8));
         mma_bf16_16816(s[2 * n2], qf[ks], kf[0], kf[1]);
         mma_bf16_16816(s[2 * n2 + 1], qf[ks], kf[2], kf[3]);
       }
@@ -194,12 +199,12 @@ attn_partial_kernel(AttnArgs a) {
     const bool need_mask = is_block || (key0 + KT > p_end) || (a.window > 0 && key0 < lo0 + a.k);
     float mx_lo = -INFINITY, mx_hi = -INFINITY;
 #pragma unroll
-    for (int n = 0; n < KT / 8; ++n) {
+    for (int n = 0; n < KW / 8; ++n) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         float v = s[n][e] * a.scale_log2;
         if (need_mask) {
-          const int kk = n * 8 + tq * 2 + (e & 1);
+          const int kk = part * KW + n * 8 + tq * 2 + (e & 1);
           const int i = (e < 2) ? i_lo : i_hi;
           bool vis;
           if (is_block) vis = (kk <= i) && (kk < a.k) && (a.window <= 0 || i - kk < a.window);
@@ -220,9 +225,9 @@ attn_partial_kernel(AttnArgs a) {
     const float al_lo = exp2f(m_lo - ref_lo), al_hi = exp2f(m_hi - ref_hi);   // m = -inf -> 0
     m_lo = mn_lo; m_hi = mn_hi;
     float sum_lo = 0.f, sum_hi = 0.f;
-    uint32_t pf[KT / 16][4];
+    uint32_t pf[KW / 16][4];
 #pragma unroll
-    for (int n = 0; n < KT / 8; ++n) {
+    for (int n = 0; n < KW / 8; ++n) {
       const float p0 = exp2f(s[n][0] - ref_lo), p1 = exp2f(s[n][1] - ref_lo);
       const float p2 = exp2f(s[n][2] - ref_hi), p3 = exp2f(s[n][3] - ref_hi);
       sum_lo += p0 + p1; sum_hi += p2 + p3;
@@ -235,23 +240,74 @@ attn_partial_kernel(AttnArgs a) {
 
     // ---- O += P V
 #pragma unroll
-    for (int kt = 0; kt < KT / 16; ++kt) {
+    for (int kt = 0; kt < KW / 16; ++kt) {
 #pragma unroll
       for (int d2 = 0; d2 < DH / 16; ++d2) {
         uint32_t vf[4];
-        ldmatrix_x4_trans(vf, bV + swz<DH>(kt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, d2 * 16 + (lane >> 4) * 8));
+        ldmatrix_x4_trans(vf, bV + swz<DH>(part * KW + kt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, d2 * 16 + (lane >> 4) * 8));
         mma_bf16_16816(o[2 * d2], pf[kt], vf[0], vf[1]);
         mma_bf16_16816(o[2 * d2 + 1], pf[kt], vf[2], vf[3]);
       }
     }
   }
   cp_async_wait<0>();
-  if (!compute) return;
+  if (KS == 1 && !compute) return;
 
   // ---- partial (m, l, O) of this chunk, or the finished rows of a request with a single one
   l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
   l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1); l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
   const size_t slab = (size_t(b) * a.Hkv + kvh) * a.max_chunks + c;
+  if constexpr (KS > 1) {
+    // the parts of a row: (maximum, sum, O) to shared memory over the K/V ring, then a thread per four columns of a row adds them up in
+    // part order
+    constexpr int LD = DH + 8;                         // row pitch in floats: the quads' 8-byte stores fall on different banks
+    float* so = reinterpret_cast<float*>(sK);          // [KS][RT][LD]
+    float* sml = so + KS * a.RT * LD;                  // [KS][RT][2]
+    __syncthreads();                                   // every warp is done with the ring
+    if (compute) {
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int rl = part * a.RT + slab16 * 16 + g + half * 8;
+#pragma unroll
+        for (int n = 0; n < DH / 8; ++n)
+          *reinterpret_cast<float2*>(so + rl * LD + n * 8 + tq * 2) = make_float2(o[n][half * 2], o[n][half * 2 + 1]);
+        if (tq == 0) { sml[rl * 2] = half ? m_hi : m_lo; sml[rl * 2 + 1] = half ? l_hi : l_lo; }
+      }
+    }
+    __syncthreads();
+    for (int idx = tid; idx < a.RT * (DH / 4); idx += nthr) {
+      const int rl = idx / (DH / 4), d = idx % (DH / 4) * 4, r = row0 + rl;
+      if (r >= a.R) break;                             // (rows ascend with idx)
+      float m = -INFINITY;
+#pragma unroll
+      for (int q = 0; q < KS; ++q) m = fmaxf(m, sml[(q * a.RT + rl) * 2]);
+      const float ref = m == -INFINITY ? 0.f : m;
+      float l = 0.f;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        const float w = exp2f(sml[(q * a.RT + rl) * 2] - ref);
+        const float4 x = *reinterpret_cast<const float4*>(so + (q * a.RT + rl) * LD + d);
+        l += sml[(q * a.RT + rl) * 2 + 1] * w;
+        v.x += x.x * w; v.y += x.y * w; v.z += x.z * w; v.w += x.w * w;
+      }
+      if (n_chunks == 1) {
+        const float inv = 1.f / l;                     // (the row's own block key is always visible: the sum is positive)
+        const size_t at = ((size_t(b) * a.k + r / a.rep) * a.Hq + kvh * a.rep + r % a.rep) * DH + d;
+        store_act16(a.o, at, v.x * inv, a.o_bf16 != 0, a.status);
+        store_act16(a.o, at + 1, v.y * inv, a.o_bf16 != 0, a.status);
+        store_act16(a.o, at + 2, v.z * inv, a.o_bf16 != 0, a.status);
+        store_act16(a.o, at + 3, v.w * inv, a.o_bf16 != 0, a.status);
+        continue;
+      }
+      *reinterpret_cast<float4*>(a.ws_o + (slab * a.R + r) * DH + d) = v;
+      if (d == 0) {
+        float* ml = a.ws_ml + (slab * a.R + r) * 2;
+        ml[0] = m;
+        ml[1] = l;
+      }
+    }
+  } else {
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     const int r = half ? r_hi : r_lo;
@@ -275,6 +331,7 @@ attn_partial_kernel(AttnArgs a) {
       ml[0] = half ? m_hi : m_lo;
       ml[1] = half ? l_hi : l_lo;
     }
+  }
   }
 }
 
@@ -407,18 +464,25 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   const size_t slabs = size_t(c.B) * c.Hkv * a.max_chunks;
   a.ws_o = reinterpret_cast<float*>(c.ws);
   a.ws_ml = a.ws_o + slabs * a.R * c.dh;
-  const size_t smem = size_t(a.RT) * c.dh * 2 + size_t(2) * NSTAGE * KT * c.dh * 2;
+  static bool attr_done[2][3][MAX_DEVICES] = {};
   dim3 grid(a.max_chunks * a.n_row_tiles, c.Hkv, c.B);
-  const int threads = a.RT * 2 < 128 ? a.RT * 2 + 96 : a.RT * 2;   // a warp per 16 rows, and three that only load where those are few
-  static bool attr_done[MAX_DEVICES] = {};
-  cudaError_t e = once_per_device(attr_done, [](int) {
-    cudaError_t e2 = cudaFuncSetAttribute(attn_partial_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e2 != cudaSuccess) return e2;
-    return cudaFuncSetAttribute(attn_partial_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  // Sharing rows shortens a CTA's chain but costs work (each part rescales its own O and keeps its own sums), so it stops where the
+  // CTAs fill the chip anyway.  Test-sized drafter, us per step, one warp per 16 rows / shared: 16 or 32 rows with four warps, up to
+  // four CTAs per SM: 8 CTAs 73.1 / 66.3, 256 88.8 / 81.3, 544 115.2 / 110.5, 540 121.4 / 119.6; 640 148 / 169.  64 rows with two warps,
+  // up to one CTA per SM: 144 CTAs 116.6 / 112.4; 384 113.7 / 119.0, 512 121.4 / 127.2.
+  const long long ctas = (long long)grid.x * grid.y * grid.z;
+  const int ks = a.RT <= 32 && ctas <= 4 * 148 ? 4 : (a.RT <= 64 && ctas <= 148 ? 2 : 1);
+  const size_t ring = size_t(2) * NSTAGE * KT * c.dh * 2, parts = ks > 1 ? size_t(ks) * a.RT * (c.dh + 10) * 4 : 0;
+  const size_t smem = size_t(a.RT) * c.dh * 2 + std::max(ring, parts);
+  const int threads = a.RT * 2 * ks + (ks > 1 || a.RT < 64 ? 96 : 0);      // three more warps that only load where few compute
+  auto kernel = c.dh == 128 ? (ks == 4 ? attn_partial_kernel<128, 4> : ks == 2 ? attn_partial_kernel<128, 2> : attn_partial_kernel<128, 1>)
+                            : (ks == 4 ? attn_partial_kernel<64, 4> : ks == 2 ? attn_partial_kernel<64, 2> : attn_partial_kernel<64, 1>);
+  cudaError_t e = once_per_device(attr_done[c.dh == 128][ks / 2], [kernel](int) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   });
   if (e != cudaSuccess) return e;
   trk_begin(trk, "attn_partial");
-  launch_pdl(c.dh == 128 ? attn_partial_kernel<128> : attn_partial_kernel<64>, grid, dim3(threads), smem, stream, a);
+  launch_pdl(kernel, grid, dim3(threads), smem, stream, a);
   trk_end(trk);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

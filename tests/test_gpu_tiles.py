@@ -151,13 +151,15 @@ def test_few_row_gemm_slices(hs, M, n_out, K, kind):
 
 
 # query rows per KV head at the edges of the row copies (4 copies up to 32 rows, 2 up to 64, 1 above), contexts that end inside a copy's
-# part of a tile, a block that starts a tile of its own, single and several chunks, the window's leading edge inside a part
+# part of a tile, a block that starts a tile of its own, single and several chunks, the window's leading edge inside a part; head width
+# 64 and chunks of 64 tokens: the other kernel, four, two and one warps per 16 rows, and more CTAs than the shared form takes
 @pytest.mark.parametrize("k,rep", [(1, 1), (8, 4), (11, 3), (32, 1), (16, 4), (32, 2), (13, 5), (16, 8)])
-@pytest.mark.parametrize("window,chunk", [(0, 0), (0, 256), (300, 0)])
-def test_attention_row_copies(hs, k, rep, window, chunk):
+@pytest.mark.parametrize("window,chunk", [(0, 0), (0, 256), (300, 0), (0, 64)])
+@pytest.mark.parametrize("dh,Hkv", [(128, 2), (64, 2), (64, 8)])
+def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
     import numpy as np
-    Hkv, dh, ctx = 2, 128, [0, 1, 31, 97, 128, 500, 1111]
-    B, Hq = len(ctx), 2 * rep
+    ctx = [0, 1, 31, 97, 128, 500, 1111]
+    B, Hq = len(ctx), Hkv * rep
     pages = [(c + 15) // 16 for c in ctx]
     perm = torch.randperm(sum(pages), generator=torch.Generator().manual_seed(3)).int()
     table, at = torch.full((B, max(pages)), -1, dtype=torch.int32), 0
