@@ -623,7 +623,8 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     if (l > 0) EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.m_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
     CUDA_TRY(h, gemm(lw.in_proj, "gemm:in_proj", U, rows, EPI_STORE_F32, BIG, d.d_in_proj));
     const float* dt_raw = nullptr;
-    if (c.dt_rank > 0) {
+    const bool dt_in_scan = c.dt_rank > 0 && scan_expands_dt(B, k, d.H, c.dt_rank);
+    if (c.dt_rank > 0 && !dt_in_scan) {
       trk->begin("cvt_dt_cols", 0, double(rows) * c.dt_rank * 6);
       // (a plain launch between overlapped ones held the host up for 20 us)
       CUDA_TRY(h, launch_pdl(cvt_cols_f16_kernel, dim3((rows * c.dt_rank + 255) / 256), dim3(256), 0, st, (const float*)BIG, (long long)d.d_in_proj,
@@ -635,13 +636,15 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     }
     ScanCall sc{};
     sc.zxbcdt = BIG; sc.ld_in = d.d_in_proj; sc.dt_raw = dt_raw; sc.s_init = SINIT;
+    if (dt_in_scan) { sc.dt_w = lw.dt_up->data; sc.dt_rank = c.dt_rank; sc.dt_bf16 = bf; }
     sc.conv_w = fptr(lw.conv_w); sc.conv_b = fptr(lw.conv_b);
     sc.dt_bias = fptr(lw.dt_bias); sc.A_log = fptr(lw.A_log); sc.Dskip = fptr(lw.Dskip);
-    sc.shared_rows = l == 0 && k > 1;
+    sc.shared_rows = l == 0 && k > 1; sc.w_stable = true;
     sc.y_gated = YG; sc.B = B; sc.k = k; sc.Di = c.Di; sc.P = c.P; sc.N = c.N; sc.G = c.G; sc.d_conv = c.d_conv;
     sc.ws = ws + p.SCAN; sc.ws_bytes = p.scan_bytes;
+    sc.norm_w = fptr(lw.gnorm); sc.u_16 = U; sc.norm_eps = c.rms_eps; sc.bf16_out = bf; sc.status = h->d_status;
     CUDA_TRY(h, scan_launch(sc, st, trk, &errtxt));
-    EW("rmsnorm_gated", Md * c.Di * 6, rmsnorm_launch(YG, fptr(lw.gnorm), U, M, c.Di, c.rms_eps, st, h->d_status, bf));
+    if (!scan_does_norm(sc)) EW("rmsnorm_gated", Md * c.Di * 6, rmsnorm_launch(YG, fptr(lw.gnorm), U, M, c.Di, c.rms_eps, st, h->d_status, bf));
     CUDA_TRY(h, gemm(lw.out_proj, "gemm:out_proj", U, M, EPI_ACCUM_F32, X, c.D));
     // ---- attention over the target's KV (in place) + the block
     if (c.has_attn[l]) {

@@ -267,14 +267,25 @@ cudaError_t gather_kv_launch(const void* pool, const int32_t* row, int ctx_len, 
 struct ScanCall {
   const float* zxbcdt; long long ld_in;
   const float* dt_raw;              // [B*k, H] or null (then the dt columns of zxbcdt)
+  const void* dt_w;                 // with dt_raw null: [H, dt_rank] fp16 / bf16, the dt columns are dt_rank wide and expanded by the scan; or null
+  int dt_rank;
+  bool dt_bf16;
   const void* s_init;               // fp16 [B, H, P, N] or null
   const float *conv_w, *conv_b, *dt_bias, *A_log, *Dskip;
-  float* y_gated;                   // [B*k, Di]
+  float* y_gated;                   // [B*k, Di]; not written when the scan does the norm as well (scan_does_norm)
+  const float* norm_w;              // gated norm behind the scan, its 16-bit result and what it needs; null: no norm asked for
+  void* u_16;
+  float norm_eps;
+  bool bf16_out;
+  uint32_t* status;
   int B, k, Di, P, N, G, d_conv;
+  bool w_stable;                    // nothing that may still be running on the stream writes the weights: they may be fetched early
   bool shared_rows;                 // zxbcdt and dt_raw have B + 1 rows: position 0 of every request, then one row for all later positions
   void* ws;                         // optional scratch (scan_workspace_bytes): enables the three-kernel fast path
   size_t ws_bytes;
 };
+bool scan_does_norm(const ScanCall& c);
+bool scan_expands_dt(int B, int k, int H, int dt_rank);
 size_t scan_workspace_bytes(int B, int k, int Di, int N, int G);
 cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 

@@ -20,6 +20,9 @@ constexpr int KMAX = 32;
 struct ScanArgs {
   const float* zxbcdt; long long ld_in;
   const float* dt_raw;
+  const uint16_t* dt_w;   // [H, dt_rank] fp16 (or bf16): the dt columns of zxbcdt are dt_rank wide and expanded here; null: they are not
+  int dt_rank, dt_bf16;
+  int w_stable;           // no kernel in front writes the weights: they may be read before it has finished
   const __half* s_init;
   const float *conv_w, *conv_b, *dt_bias, *A_log, *Dskip;
   float* y;
@@ -29,7 +32,28 @@ struct ScanArgs {
   __device__ __forceinline__ size_t in_row(int b, int i) const {
     return shared_rows ? size_t(i == 0 ? b : B) : size_t(b) * k + i;
   }
+  // dt of head h before the bias, at position i of request b
+  __device__ __forceinline__ float dt_pre(int b, int i, int h) const {
+    const size_t row = in_row(b, i);
+    if (dt_raw) return dt_raw[row * H + h];
+    const float* x = zxbcdt + row * ld_in + Di + d_xBC;
+    if (!dt_w) return x[h];
+    const uint16_t* wr = dt_w + size_t(h) * dt_rank;
+    float s = 0.f;
+#pragma unroll 16
+    for (int r = 0; r < dt_rank; ++r) s += x[r] * (dt_bf16 ? __uint_as_float(uint32_t(wr[r]) << 16) : __half2float(__ushort_as_half(wr[r])));
+    return s;
+  }
   int NP;          // padded N (row pitch of the staged state in floats)
+};
+
+// The gated norm behind the scan, where one kernel does both.
+struct ScanNorm {
+  const float* w;      // [Di]
+  uint16_t* u;         // [B * k, Di] fp16 or bf16
+  float eps;
+  int bf16_out;
+  uint32_t* status;
 };
 
 __device__ __forceinline__ float softplus_f(float v) { return v > 20.f ? v : log1pf(expf(v)); }
@@ -75,8 +99,7 @@ mamba_scan_kernel(ScanArgs a) {
   if (tid < 32) {
     float dt = 0.f, dA = 0.f;
     if (tid < k) {
-      const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, tid) * a.H + h]
-                                 : a.zxbcdt[a.in_row(b, tid) * a.ld_in + a.Di + a.d_xBC + h];
+      const float raw = a.dt_pre(b, tid, h);
       dt = softplus_f(raw + a.dt_bias[h]);
       dA = dt * (-expf(a.A_log[h]));
     }
@@ -158,11 +181,15 @@ mamba_scan_kernel(ScanArgs a) {
 // are computed once per block into shared memory while the threads' own inputs (x and z of eight positions) are in flight.
 // The operands are a few MB, so latency is what counts: the general kernel above takes 33 us at the paper's shape
 // (32 requests, 48 heads, 8 positions), this one 5.  (Event times less the 6 us an empty pair of events reads: 39.4 -> 10.8.)
-template <int NMAX>
-__global__ void __launch_bounds__(256)
-scan_small_state_kernel(ScanArgs a, int hb) {
-  pdl_wait();
-  pdl_trigger();
+// NORM: the gated RMSNorm over all Di channels behind the scan happens here too, without a launch of its own and without the fp32 rows
+// in between: a request's blocks are one cluster (eight at most) and add up their rows' sums of squares through distributed
+// shared memory, in a fixed order.  Together with the dt expansion (dt_pre) this takes three launches out of a step of the test-sized
+// drafter and one per layer out of the paper's: 69.1 -> 67.4 and 1507 -> 1495 us per step; before the wait for the kernels in front
+// the block already reads what the layer's weights give.
+template <int NMAX, bool NORM>
+__global__ void __launch_bounds__(512)
+scan_small_state_kernel(ScanArgs a, int hb, ScanNorm nm) {
+  if (!a.w_stable) { pdl_wait(); pdl_trigger(); }
   extern __shared__ __align__(16) float sm[];
   const int k = a.k, P = a.P, N = a.N, tid = threadIdx.x;
   const int h0 = blockIdx.x * hb, b = blockIdx.y, g = h0 / (a.H / a.G);
@@ -170,54 +197,75 @@ scan_small_state_kernel(ScanArgs a, int hb) {
   float* Cs = Bs + k * NMAX;         // [k][NMAX]
   float* dts = Cs + k * NMAX;        // [k][hb]
   float* dec = dts + k * hb;         // [k][hb]
+  float* part = dec + k * hb;        // NORM: [k] this block's sums of squares, then ys
+  float* ys = part + k;              // NORM: [k][hb * P] the gated outputs
   const size_t row0 = size_t(b) * k;
   const int hl = tid / P, p = tid % P, h = h0 + hl;
   const bool act = hl < hb;
   constexpr int CH = 8;              // positions whose inputs are in flight together
   const int ch = act ? h * P + p : 0;
-  float xr[CH], zr[CH], w[4], S[NMAX];
+  // ---- what the layer's weights give, before the kernels in front have finished: the taps of the thread's own channel and of the B or C
+  // channel it convolves below (always the same one: the block is a multiple of 2 NMAX wide)
+  const int is_c = tid % (2 * NMAX) / NMAX, nb_c = tid % NMAX;
+  const int cb = a.Di + is_c * a.G * N + g * N + (nb_c < N ? nb_c : 0);    // channel inside xBC
+  float w[4], wb[4];                 // right-aligned taps
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const bool tap = j >= 4 - a.d_conv;
+    w[j] = tap ? a.conv_w[ch * a.d_conv + j - (4 - a.d_conv)] : 0.f;
+    wb[j] = tap ? a.conv_w[cb * a.d_conv + j - (4 - a.d_conv)] : 0.f;
+  }
+  const float bias = a.conv_b[ch], bias_b = a.conv_b[cb];
+  const float gain = NORM ? nm.w[ch] : 0.f;
+  const float Dh = a.Dskip[act ? h : h0];
+  const float dtb = a.dt_bias[h0 + tid % hb], Ah = -expf(a.A_log[h0 + tid % hb]);   // (of the first dt the thread computes)
+  if (a.w_stable) { pdl_wait(); pdl_trigger(); }
+  // (plain loads from here on: the read-only form __ldg may be moved up past the wait, and did)
+  float xr[CH], zr[CH], S[NMAX];
   auto fetch = [&](int t0) {
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
       const bool ok = act && t0 + i < k;
       const float* row = a.zxbcdt + a.in_row(b, ok ? t0 + i : 0) * a.ld_in;
-      xr[i] = ok ? __ldg(row + a.Di + ch) : 0.f;
-      zr[i] = ok ? __ldg(row + ch) : 0.f;
+      xr[i] = ok ? row[a.Di + ch] : 0.f;
+      zr[i] = ok ? row[ch] : 0.f;
     }
   };
   fetch(0);
+  {
+    const __half* s0 = a.s_init + ((size_t(b) * a.H + (act ? h : h0)) * P + p) * N;
+    const bool have = act && a.s_init != nullptr;
+    if (N == NMAX && (reinterpret_cast<uintptr_t>(a.s_init) & 7) == 0) {   // whole rows of 8 or 32 bytes
 #pragma unroll
-  for (int j = 0; j < 4; ++j) w[j] = (j >= 4 - a.d_conv) ? a.conv_w[ch * a.d_conv + j - (4 - a.d_conv)] : 0.f;   // right-aligned taps
-  const float bias = a.conv_b[ch];
-#pragma unroll
-  for (int n = 0; n < NMAX; ++n)
-    S[n] = (act && a.s_init != nullptr && n < N) ? __half2float(a.s_init[((size_t(b) * a.H + h) * P + p) * N + n]) : 0.f;
-  for (int idx = tid; idx < k * 2 * NMAX; idx += blockDim.x) {
-    const int i = idx / (2 * NMAX), rest = idx % (2 * NMAX), is_c = rest / NMAX, n = rest % NMAX;
-    float v = 0.f;
-    if (n < N) {
-      const int cb = a.Di + is_c * a.G * N + g * N + n;            // channel inside xBC
-      float acc = a.conv_b[cb];
-      for (int j = 0; j < a.d_conv; ++j) {
-        const int src = i - (a.d_conv - 1) + j;
-        if (src >= 0) acc += a.conv_w[cb * a.d_conv + j] * a.zxbcdt[a.in_row(b, src) * a.ld_in + a.Di + cb];
+      for (int n = 0; n < NMAX; n += 4) {
+        const uint2 v = have ? *reinterpret_cast<const uint2*>(s0 + n) : make_uint2(0, 0);
+        const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&v.x)), hi = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
+        S[n] = lo.x; S[n + 1] = lo.y; S[n + 2] = hi.x; S[n + 3] = hi.y;
       }
-      v = silu_f(acc);
+    } else {
+#pragma unroll
+      for (int n = 0; n < NMAX; ++n) S[n] = have && n < N ? __half2float(s0[n]) : 0.f;
     }
-    (is_c ? Cs : Bs)[i * NMAX + n] = v;
+  }
+  for (int idx = tid; idx < k * 2 * NMAX; idx += blockDim.x) {
+    const int i = idx / (2 * NMAX);
+    float x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = i - 3 + j >= 0 ? a.zxbcdt[a.in_row(b, i - 3 + j) * a.ld_in + a.Di + cb] : 0.f;
+    const float v = silu_f(bias_b + wb[0] * x[0] + wb[1] * x[1] + wb[2] * x[2] + wb[3] * x[3]);
+    (is_c ? Cs : Bs)[i * NMAX + nb_c] = nb_c < N ? v : 0.f;
   }
   for (int idx = tid; idx < k * hb; idx += blockDim.x) {
     const int i = idx / hb, hh = h0 + idx % hb;
-    const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, i) * a.H + hh] : a.zxbcdt[a.in_row(b, i) * a.ld_in + a.Di + a.d_xBC + hh];
-    const float dt = softplus_f(raw + a.dt_bias[hh]);
+    const bool first = idx == tid;
+    const float dt = softplus_f(a.dt_pre(b, i, hh) + (first ? dtb : a.dt_bias[hh]));
     dts[idx] = dt;
-    dec[idx] = expf(dt * (-expf(a.A_log[hh])));
+    dec[idx] = expf(dt * (first ? Ah : -expf(a.A_log[hh])));
   }
   __syncthreads();
-  if (!act) return;
-  const float Dh = a.Dskip[h];
+  if (!NORM && !act) return;
   float c1 = 0.f, c2 = 0.f, c3 = 0.f;                              // the three rows before this one (zero left context)
-  for (int t0 = 0; t0 < k; t0 += CH) {
+  for (int t0 = 0; act && t0 < k; t0 += CH) {
     if (t0 > 0) fetch(t0);
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
@@ -226,14 +274,45 @@ scan_small_state_kernel(ScanArgs a, int hb) {
       const float x = silu_f(bias + w[0] * c3 + w[1] * c2 + w[2] * c1 + w[3] * xr[i]);
       c3 = c2; c2 = c1; c1 = xr[i];
       const float at = dec[t * hb + hl], dx = dts[t * hb + hl] * x;
-      float y = Dh * x;
+      float y[4] = {Dh * x, 0.f, 0.f, 0.f};                        // (four sums: one would be a chain of N products)
 #pragma unroll
-      for (int n = 0; n < NMAX; ++n) {
-        S[n] = at * S[n] + dx * Bs[t * NMAX + n];
-        y += S[n] * Cs[t * NMAX + n];
+      for (int n = 0; n < NMAX; n += 4) {
+        const float4 bv = *reinterpret_cast<const float4*>(Bs + t * NMAX + n), cv = *reinterpret_cast<const float4*>(Cs + t * NMAX + n);
+        S[n] = at * S[n] + dx * bv.x;             y[0] += S[n] * cv.x;
+        S[n + 1] = at * S[n + 1] + dx * bv.y;     y[1] += S[n + 1] * cv.y;
+        S[n + 2] = at * S[n + 2] + dx * bv.z;     y[2] += S[n + 2] * cv.z;
+        S[n + 3] = at * S[n + 3] + dx * bv.w;     y[3] += S[n + 3] * cv.w;
       }
-      a.y[(row0 + t) * a.Di + ch] = y * silu_f(zr[i]);
+      const float out = ((y[0] + y[1]) + (y[2] + y[3])) * silu_f(zr[i]);
+      if (NORM) ys[t * hb * P + tid] = out;
+      else a.y[(row0 + t) * a.Di + ch] = out;
     }
+  }
+  if constexpr (NORM) {
+    __syncthreads();
+    const int lane = tid & 31, nb = int(gridDim.x), n = hb * P;
+    for (int t = tid >> 5; t < k; t += blockDim.x >> 5) {
+      float ss = 0.f;
+      for (int d = lane; d < n; d += 32) ss += ys[t * n + d] * ys[t * n + d];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      if (lane == 0) part[t] = ss;
+    }
+    if (nb > 1) cluster_sync_all(); else __syncthreads();
+    float* inv = dec;                                              // [k]; the decays are no longer needed
+    // eight lanes per row, one per block of the cluster
+    for (int idx = tid; idx < (k * 8 + 31) / 32 * 32; idx += blockDim.x) {
+      const int t = min(idx >> 3, k - 1), r = idx & 7;
+      float v = r >= nb ? 0.f : nb > 1 ? ld_cluster_f32(mapa_rank(smem_u32(part + t), r)) : part[t];
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (r == 0) inv[t] = rsqrtf(v / float(a.Di) + nm.eps);
+    }
+    if (nb > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // this block has read the others' sums
+    __syncthreads();
+    if (act)
+      for (int t = 0; t < k; ++t) store_act16(nm.u + (row0 + t) * a.Di, ch, ys[t * n + tid] * inv[t] * gain, nm.bf16_out != 0, nm.status);
+    if (nb > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // no block leaves while another reads its sums
   }
 }
 
@@ -305,8 +384,7 @@ mamba_scan_mma_kernel(ScanArgs a) {
   {
     float dt = 0.f, dA = 0.f;
     if (lane < k) {
-      const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, lane) * a.H + h]
-                                 : a.zxbcdt[a.in_row(b, lane) * a.ld_in + a.Di + a.d_xBC + h];
+      const float raw = a.dt_pre(b, lane, h);
       dt = softplus_f(raw + a.dt_bias[h]);
       dA = dt * (-expf(a.A_log[h]));
     }
@@ -356,7 +434,7 @@ mamba_scan_mma_kernel(ScanArgs a) {
       uint4 sv[NT];
 #pragma unroll
       for (int j = 0; j < NT; ++j)
-        sv[j] = __ldg(reinterpret_cast<const uint4*>(S + size_t(j * 8 + gq) * N + kp * 32 + tq * 8));
+        sv[j] = *reinterpret_cast<const uint4*>(S + size_t(j * 8 + gq) * N + kp * 32 + tq * 8);
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt) {
         const uint4 c_lo = *reinterpret_cast<const uint4*>(C16 + (mt * 16 + gq) * N + kp * 32 + tq * 8);
@@ -441,7 +519,7 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
 #pragma unroll
   for (int v = 0; v < VEC; ++v) {
     if (VEC == 4 && a.d_conv == 4) {                         // a channel's four taps in one 16-byte load
-      const float4 t = __ldg(reinterpret_cast<const float4*>(a.conv_w) + ch + v);
+      const float4 t = reinterpret_cast<const float4*>(a.conv_w)[ch + v];
       w[v][0] = t.x; w[v][1] = t.y; w[v][2] = t.z; w[v][3] = t.w;
     } else {
 #pragma unroll
@@ -449,7 +527,7 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
     }
   }
   if (VEC == 4) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(a.conv_b + ch));
+    const float4 t = *reinterpret_cast<const float4*>(a.conv_b + ch);
     bias[0] = t.x; bias[VEC > 1 ? 1 : 0] = t.y; bias[VEC > 1 ? 2 : 0] = t.z; bias[VEC > 1 ? 3 : 0] = t.w;
   } else {
     bias[0] = a.conv_b[ch];
@@ -464,10 +542,10 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
     const bool ok = i >= 0 && i < a.k;
     const float* src = a.zxbcdt + a.in_row(b, ok ? i : 0) * a.ld_in + a.Di + ch;
     if (VEC == 4) {
-      const float4 t = ok ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 t = ok ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
       in[j][0] = t.x; in[j][VEC > 1 ? 1 : 0] = t.y; in[j][VEC > 1 ? 2 : 0] = t.z; in[j][VEC > 1 ? 3 : 0] = t.w;
     } else {
-      in[j][0] = ok ? __ldg(src) : 0.f;
+      in[j][0] = ok ? *src : 0.f;
     }
   }
 #pragma unroll
@@ -584,7 +662,7 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
   // ---- dt, inclusive prefix sum of dt * A over the block positions (one warp shuffle scan per head)
   float dt = 0.f, dA = 0.f;
   if (lane < k) {
-    const float raw = a.dt_raw ? a.dt_raw[a.in_row(b, lane) * a.H + h] : a.zxbcdt[a.in_row(b, lane) * a.ld_in + a.Di + a.d_xBC + h];
+    const float raw = a.dt_pre(b, lane, h);
     dt = softplus_f(raw + a.dt_bias[h]);
     dA = dt * (-expf(a.A_log[h]));
   }
@@ -723,15 +801,40 @@ size_t scan_workspace_bytes(int B, int k, int Di, int N, int G) {
   return M * d_xBC * 4 + size_t(B) * G * KMAX * KMAX * 4 + M * 2 * size_t(G) * N * 2 + 256;
 }
 
+namespace {
+constexpr size_t SMALL_STATE_SMEM = sizeof(float) * KMAX * (2 * (16 + 8) + 1 + 512);   // the most a call with the norm can ask for
+// Heads per block of the small-state kernel: heads of one group share a block while they fit 256 threads; when the norm follows, up to
+// eight heads and 512 threads, so that a request's blocks fit a cluster of eight.
+int small_state_heads(const ScanCall& c) {
+  const int H = c.Di / c.P, hpg = H / c.G;
+  int hb = 1;
+  while (hb < 4 && hpg % (2 * hb) == 0 && 2 * hb * c.P <= 256) hb *= 2;
+  if (c.norm_w != nullptr)
+    for (int n = hb; n <= 8 && n * c.P <= 512; ++n)
+      if (hpg % n == 0 && H / n <= 8) return n;
+  return hb;
+}
+}  // namespace
+
+bool scan_does_norm(const ScanCall& c) {
+  return c.norm_w != nullptr && c.N <= 16 && c.Di / c.P / small_state_heads(c) <= 8;
+}
+
+// An expansion of the dt columns inside the scan reads every column once per head through the L1; past a few million products the
+// tensor-core GEMM is the better one although it takes two launches more.
+bool scan_expands_dt(int B, int k, int H, int dt_rank) { return dt_rank <= 64 && (long long)B * k * H * dt_rank <= (1 << 22); }
+
 cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, std::string* err) {
   if (c.k < 1 || c.k > KMAX) { if (err) *err = "scan: k out of range"; return cudaErrorInvalidValue; }
   if (c.Di % c.P) { if (err) *err = "scan: Di must be a multiple of P"; return cudaErrorInvalidValue; }
   ScanArgs a{};
-  a.zxbcdt = c.zxbcdt; a.ld_in = c.ld_in; a.dt_raw = c.dt_raw; a.s_init = (const __half*)c.s_init;
+  a.zxbcdt = c.zxbcdt; a.ld_in = c.ld_in; a.dt_raw = c.dt_raw; a.dt_w = (const uint16_t*)c.dt_w; a.dt_rank = c.dt_rank; a.dt_bf16 = c.dt_bf16 ? 1 : 0;
+  a.s_init = (const __half*)c.s_init;
   a.conv_w = c.conv_w; a.conv_b = c.conv_b; a.dt_bias = c.dt_bias; a.A_log = c.A_log; a.Dskip = c.Dskip;
   a.y = c.y_gated; a.B = c.B; a.k = c.k; a.Di = c.Di; a.P = c.P; a.N = c.N; a.G = c.G; a.H = c.Di / c.P;
   a.d_conv = c.d_conv; a.d_xBC = c.Di + 2 * c.G * c.N;
   a.shared_rows = c.shared_rows ? 1 : 0;
+  a.w_stable = c.w_stable ? 1 : 0;
   a.NP = c.N + 1;                                    // odd pitch: threads of a warp own consecutive p
   if (a.H % c.G) { if (err) *err = "scan: heads must divide into groups"; return cudaErrorInvalidValue; }
   // serving shapes: tensor-core path (needs 8-byte aligned rows for the float2 accesses)
@@ -788,16 +891,22 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     return cudaGetLastError();
   }
   if (c.N <= 16) {
-    // a state of up to 16 values per channel lives in registers; heads of one group share a block while they fit 256 threads
-    int hb = 1;
-    while (hb < 4 && (a.H / c.G) % (2 * hb) == 0 && 2 * hb * c.P <= 256) hb *= 2;
-    const int threads = (hb * c.P + 31) / 32 * 32;
-    const int nmax = c.N <= 4 ? 4 : 16;
-    const size_t smem_n = sizeof(float) * size_t(c.k) * 2 * (nmax + hb);
+    const int hb = small_state_heads(c), threads = (hb * c.P + 31) / 32 * 32, nmax = c.N <= 4 ? 4 : 16;
+    const bool norm = scan_does_norm(c);
+    const size_t smem_n = sizeof(float) * (size_t(c.k) * 2 * (nmax + hb) + (norm ? size_t(c.k) * (1 + hb * c.P) : 0));
     const dim3 grid_n(a.H / hb, c.B);
-    trk_begin(trk, "mamba_scan", 0, double(c.B) * a.H * c.P * c.N * 2);
-    cudaError_t e = nmax == 4 ? launch_pdl(scan_small_state_kernel<4>, grid_n, dim3(threads), smem_n, stream, a, hb)
-                              : launch_pdl(scan_small_state_kernel<16>, grid_n, dim3(threads), smem_n, stream, a, hb);
+    const ScanNorm nm{c.norm_w, (uint16_t*)c.u_16, c.norm_eps, c.bf16_out ? 1 : 0, c.status};
+    auto kernel = nmax == 4 ? (norm ? scan_small_state_kernel<4, true> : scan_small_state_kernel<4, false>)
+                            : (norm ? scan_small_state_kernel<16, true> : scan_small_state_kernel<16, false>);
+    if (norm) {
+      static bool nset[2][MAX_DEVICES] = {};
+      const cudaError_t e = once_per_device(nset[nmax == 4 ? 0 : 1], [kernel](int) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMALL_STATE_SMEM));
+      });
+      if (e != cudaSuccess) return e;
+    }
+    trk_begin(trk, norm ? "mamba_scan_norm" : "mamba_scan", 0, double(c.B) * a.H * c.P * c.N * 2);
+    cudaError_t e = launch_pdl_cluster(kernel, grid_n, dim3(threads), dim3(norm ? grid_n.x : 1), smem_n, stream, a, hb, nm);
     trk_end(trk);
     return e != cudaSuccess ? e : cudaGetLastError();
   }

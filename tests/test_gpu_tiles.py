@@ -202,3 +202,17 @@ def test_residual_tail_is_added_by_the_norm(hs, D, F, B, k):
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[16] * B)
     check_step(cfg, drafter, w, batch, k, requests=[0, B - 1], what=f"tail {D} {F}")
     drafter.close()
+
+# small states: the gated norm runs in the scan's own kernel as long as a request's blocks fit a cluster of eight (here one to eight blocks,
+# head counts per group that are no power of two, and one too many: 9 blocks), low-rank dt up to the width where a GEMM expands it instead
+@pytest.mark.parametrize("Di,P,N,G,dt_rank,B,k", [(256, 64, 16, 1, 16, 1, 1), (3072, 64, 4, 4, 0, 3, 8), (1152, 64, 4, 9, 0, 2, 5), (2048, 64, 16, 8, 64, 2, 32),
+                                                  (2304, 64, 3, 36, 0, 2, 4), (640, 32, 8, 5, 40, 3, 9), (512, 64, 16, 2, 72, 2, 3), (960, 120, 4, 1, 8, 2, 17)])
+def test_small_state_scan_with_norm(hs, Di, P, N, G, dt_rank, B, k):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(D=256, n_fuse=1, r=64, L=2, has_attn=[0, 0], kv_slot=[-1, -1], n_slots=0, Di=Di, P=P, N=N, G=G, d_conv=4, dt_rank=dt_rank,
+                             Hq=4, Hkv=2, dh=64, rope_theta=1.0e4, window=0, qk_norm=1, F=512, V=600, rms_eps=1e-6, page_size=16, name="small",
+                             B=B, k=k, ctx=("const", 20, 20)))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[20] * B)
+    check_step(cfg, drafter, w, batch, k, requests=list(range(B)), what=f"small {Di} {P} {N} {G} {dt_rank}")
+    drafter.close()
