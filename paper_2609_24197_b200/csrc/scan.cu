@@ -492,29 +492,23 @@ mamba_scan_mma_kernel(ScanArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Three-kernel form of the fast path (used when the caller provides scratch): the small per-position
+// Two-kernel form of the fast path (used when the caller provides scratch): the small per-position
 // operands are prepared once per request and group, so the kernel that streams S_init has no
 // block-wide phases in front of its loads.
-//   scan_conv_kernel   causal depthwise conv + SiLU of every xBC channel (thread = 4 channels x 4 positions);
-//                      C is also written as fp16 head + fp16 remainder for the tensor-core contraction
-//   scan_cb_kernel     CB[b, g, t, s] = C_t . B_s for s <= t
+//   scan_conv_kernel   causal depthwise conv + SiLU of every xBC channel (thread = 4 channels x 4 positions); for the B and C channels
+//                      of a group one block does all positions, writes C as fp16 head + fp16 remainder for the tensor-core
+//                      contraction and CB[b, g, t, s] = C_t . B_s for s <= t
 //   mamba_scan_stream_kernel  one warp per head: everything it needs is fetched up front (cp.async for the
-//                      shared operands, 16-byte loads of S_init straight into the MMA fragments)
+//                      shared operands, 32-byte loads of S_init straight into the MMA fragments)
 constexpr int CONV_ROWS = 4;                                 // block positions per thread
 // thread = (VEC adjacent channels, group of four block positions): the filter reads raw inputs only, so the groups are
 // independent; a thread's seven (vector) loads are in flight together and it needs few registers.  VEC = 4 (16-byte
 // loads and stores) when every channel offset and row stride is a multiple of four, else 1.  (One thread per channel
 // walking all k rows held 72 registers, three blocks per SM, and reached 25 % of the DRAM peak with its warps waiting
 // on loads; one channel and four rows per thread was bound by the instruction issue, 85 %, most of it set-up.)
+// conv + SiLU of channels ch .. ch + VEC - 1 at positions i0 .. i0 + CONV_ROWS - 1 (those past the block are left as they come)
 template <int VEC>
-__global__ void __launch_bounds__(256)
-scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16) {
-  pdl_wait();
-  pdl_trigger();
-  const int ch = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
-  const int n_grp = (a.k + CONV_ROWS - 1) / CONV_ROWS;
-  const int b = blockIdx.y / n_grp, i0 = (blockIdx.y % n_grp) * CONV_ROWS;
-  if (ch >= a.d_xBC) return;
+__device__ __forceinline__ void conv_rows(const ScanArgs& a, int b, int i0, int ch, float (&out)[CONV_ROWS][VEC]) {
   float w[VEC][4], bias[VEC];
 #pragma unroll
   for (int v = 0; v < VEC; ++v) {
@@ -532,9 +526,6 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
   } else {
     bias[0] = a.conv_b[ch];
   }
-  const size_t row0 = size_t(b) * a.k;
-  const int GN = a.G * a.N;
-  const int c_col = ch - a.Di - GN;                          // >= 0 for C channels
   float in[CONV_ROWS + 3][VEC];                              // rows i0 - 3 .. i0 + 3 (zero left context before the block)
 #pragma unroll
   for (int j = 0; j < CONV_ROWS + 3; ++j) {
@@ -549,55 +540,70 @@ scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16)
     }
   }
 #pragma unroll
-  for (int r = 0; r < CONV_ROWS; ++r) {
-    const int i = i0 + r;
-    if (i >= a.k) break;
-    float o[VEC];
+  for (int r = 0; r < CONV_ROWS; ++r)
 #pragma unroll
     for (int v = 0; v < VEC; ++v)
-      o[v] = silu_f(bias[v] + w[v][0] * in[r][v] + w[v][1] * in[r + 1][v] + w[v][2] * in[r + 2][v] + w[v][3] * in[r + 3][v]);
-    float* dst = xact + (row0 + i) * a.d_xBC + ch;
-    if (VEC == 4) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[VEC > 1 ? 1 : 0], o[VEC > 1 ? 2 : 0], o[VEC > 1 ? 3 : 0]);
-    else dst[0] = o[0];
-    if (c_col >= 0) {
-      __half hi[VEC], lo[VEC];
+      out[r][v] = silu_f(bias[v] + w[v][0] * in[r][v] + w[v][1] * in[r + 1][v] + w[v][2] * in[r + 2][v] + w[v][3] * in[r + 3][v]);
+}
+
+// Blocks x < G: the B and C channels of one group and, from shared memory, their products CB (a launch of its own before that read
+// both back from memory: conv 8 us + CB 4 us at 32 requests of the 8B-class shapes, k = 16).  The rows are padded by four floats
+// so that the 16-byte reads of a warp's threads spread over the banks.  Blocks x >= G: 256 VEC channels of x at CONV_ROWS positions.
+template <int VEC>
+__global__ void __launch_bounds__(256)
+scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16, float* __restrict__ cb) {
+  pdl_wait();
+  pdl_trigger();
+  const int k = a.k, N = a.N, n_grp = (k + CONV_ROWS - 1) / CONV_ROWS;
+  const int b = blockIdx.y / n_grp, grp = blockIdx.y % n_grp;
+  const size_t row0 = size_t(b) * k;
+  float o[CONV_ROWS][VEC];
+  if (int(blockIdx.x) >= a.G) {
+    const int ch = ((blockIdx.x - a.G) * 256 + threadIdx.x) * VEC, i0 = grp * CONV_ROWS;
+    if (ch >= a.Di) return;
+    conv_rows<VEC>(a, b, i0, ch, o);
 #pragma unroll
-      for (int v = 0; v < VEC; ++v) { hi[v] = __float2half_rn(o[v]); lo[v] = __float2half_rn(o[v] - __half2float(hi[v])); }
-      __half* d_hi = c16 + ((row0 + i) * 2 + 0) * GN + c_col;
-      __half* d_lo = c16 + ((row0 + i) * 2 + 1) * GN + c_col;
-      if (VEC == 4) {
-        *reinterpret_cast<uint2*>(d_hi) = *reinterpret_cast<const uint2*>(hi);
-        *reinterpret_cast<uint2*>(d_lo) = *reinterpret_cast<const uint2*>(lo);
-      } else {
-        d_hi[0] = hi[0];
-        d_lo[0] = lo[0];
+    for (int r = 0; r < CONV_ROWS; ++r) {
+      if (i0 + r >= k) break;
+      float* dst = xact + (row0 + i0 + r) * a.Di + ch;
+      if (VEC == 4) *reinterpret_cast<float4*>(dst) = make_float4(o[r][0], o[r][VEC > 1 ? 1 : 0], o[r][VEC > 1 ? 2 : 0], o[r][VEC > 1 ? 3 : 0]);
+      else dst[0] = o[r][0];
+    }
+    return;
+  }
+  if (grp != 0) return;
+  extern __shared__ __align__(16) float cb_sm[];
+  const int g = blockIdx.x, ldr = N + 4, GN = a.G * N;
+  float* Bs = cb_sm;                 // [k][N + 4]
+  float* Cs = cb_sm + k * ldr;       // [k][N + 4]
+  for (int idx = threadIdx.x; idx < n_grp * (2 * N / VEC); idx += 256) {
+    const int i0 = idx / (2 * N / VEC) * CONV_ROWS, c = idx % (2 * N / VEC) * VEC, is_c = c >= N, n = is_c ? c - N : c;
+    conv_rows<VEC>(a, b, i0, a.Di + is_c * GN + g * N + n, o);
+#pragma unroll
+    for (int r = 0; r < CONV_ROWS; ++r) {
+      const int i = i0 + r;
+      if (i >= k) break;
+      float* dst = (is_c ? Cs : Bs) + i * ldr + n;
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) dst[v] = o[r][v];
+      if (is_c) {
+        __half hi[VEC], lo[VEC];
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) { hi[v] = __float2half_rn(o[r][v]); lo[v] = __float2half_rn(o[r][v] - __half2float(hi[v])); }
+        __half* d_hi = c16 + ((row0 + i) * 2 + 0) * GN + g * N + n;
+        __half* d_lo = c16 + ((row0 + i) * 2 + 1) * GN + g * N + n;
+        if (VEC == 4) {
+          *reinterpret_cast<uint2*>(d_hi) = *reinterpret_cast<const uint2*>(hi);
+          *reinterpret_cast<uint2*>(d_lo) = *reinterpret_cast<const uint2*>(lo);
+        } else {
+          d_hi[0] = hi[0];
+          d_lo[0] = lo[0];
+        }
       }
     }
   }
-}
-
-// CB[b, g, t, s] = C_t . B_s for s <= t.  One block per (request, group): the block's B and C rows are staged in shared
-// memory (rows padded by four floats so that the 16-byte reads of a warp's threads spread over the banks), each thread
-// takes (t, s) pairs with float4 dot products in the order n = 0 .. N - 1 of the scalar loop it replaces (that loop read
-// both rows from global memory one float at a time and ran at the L1's limit).
-__global__ void __launch_bounds__(256)
-scan_cb_kernel(ScanArgs a, const float* __restrict__ xact, float* __restrict__ cb) {
-  pdl_wait();
-  pdl_trigger();
-  extern __shared__ __align__(16) float cb_sm[];
-  const int g = blockIdx.x, b = blockIdx.y;
-  const int k = a.k, N = a.N, ldr = N + 4;
-  const size_t row0 = size_t(b) * k;
-  const int GN = a.G * N;
-  float* Bs = cb_sm;                 // [k][N + 4]
-  float* Cs = cb_sm + k * ldr;       // [k][N + 4]
-  for (int idx = threadIdx.x; idx < 2 * k * (N / 4); idx += blockDim.x) {
-    const int which = idx / (k * (N / 4)), rem = idx % (k * (N / 4)), r = rem / (N / 4), c4 = rem % (N / 4);
-    const float4 v = *reinterpret_cast<const float4*>(xact + (row0 + r) * a.d_xBC + a.Di + which * GN + g * N + c4 * 4);
-    *reinterpret_cast<float4*>((which ? Cs : Bs) + r * ldr + c4 * 4) = v;
-  }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < k * k; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < k * k; idx += 256) {
     const int t = idx / k, s2 = idx % k;
     float dot = 0.f;
     if (s2 <= t) {
@@ -616,8 +622,6 @@ template <int P, int N, int MT>
 __global__ void __launch_bounds__(128, MT == 1 ? 4 : 3)
 mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __half* __restrict__ c16,
                          const float* __restrict__ cb) {
-  pdl_wait();
-  pdl_trigger();
   constexpr int HPC = 4, NT = P / 8, ROWS = MT * 16;
   constexpr int XS = P + 8;                                    // floats per x row in shared memory (padded: the fragment reads
                                                                // of rows tq and columns gq then fall on 32 different banks)
@@ -635,7 +639,8 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
   float* xs = CB + ROWS * ROWS + warp * (ROWS * XS);           // per warp [ROWS][XS]
   float* Wh = CB + ROWS * ROWS + HPC * ROWS * XS + warp * ROWS * (ROWS + 1);   // per warp [ROWS][ROWS+1]
 
-  // ---- state fragments of the first two k-step pairs: issued before anything else
+  // ---- state fragments of the first two k-step pairs: issued before anything else, and before the wait for the kernel in front: that
+  // kernel (the conv) started its dependents only once everything ahead of it, the state's producer included, had finished
   const int gq = lane >> 2, tq = lane & 3;
   const __half* S = a.s_init ? a.s_init + (size_t(b) * a.H + h) * P * N : nullptr;
   // (32-byte loads: the four lanes of a row then cover a whole 128-byte line per instruction; with 16-byte loads every
@@ -645,6 +650,8 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
 #pragma unroll
     for (int j = 0; j < NT; ++j) ldg_nc_32B(S + size_t(j * 8 + gq) * N + tq * 16, sv0[j][0], sv0[j][1]);
   }
+  pdl_wait();
+  pdl_trigger();
   // ---- shared operands (C halves, CB) and this head's x rows: cp.async, zero fill for the padding rows
   for (int idx = tid; idx < ROWS * 2 * N / 8; idx += 128) {
     const int r = idx / (2 * N / 8), rest = idx % (2 * N / 8), half = rest / (N / 8), c8 = rest % (N / 8);
@@ -656,7 +663,7 @@ mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __hal
   }
   for (int idx = lane; idx < ROWS * P / 4; idx += 32) {
     const int r = idx / (P / 4), c4 = idx % (P / 4);
-    cp_async16(smem_u32(xs + r * XS + c4 * 4), xact + (row0 + min(r, k - 1)) * a.d_xBC + h * P + c4 * 4, r < k);
+    cp_async16(smem_u32(xs + r * XS + c4 * 4), xact + (row0 + min(r, k - 1)) * a.Di + h * P + c4 * 4, r < k);
   }
   cp_async_commit();
   // ---- dt, inclusive prefix sum of dt * A over the block positions (one warp shuffle scan per head)
@@ -846,16 +853,13 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     float* xact = reinterpret_cast<float*>(c.ws);
     float* cbw = xact + M * a.d_xBC;
     __half* c16 = reinterpret_cast<__half*>(cbw + size_t(c.B) * c.G * KMAX * KMAX);
-    trk_begin(trk, "scan_conv", 0, double(M) * a.d_xBC * 8);
+    trk_begin(trk, "scan_conv", 0, double(M) * (a.d_xBC + a.Di) * 4);
     const bool vec4 = a.Di % 4 == 0 && (c.G * c.N) % 4 == 0 && a.ld_in % 4 == 0 &&
                       ((reinterpret_cast<uintptr_t>(a.zxbcdt) | reinterpret_cast<uintptr_t>(c.ws) | reinterpret_cast<uintptr_t>(a.conv_w) |
                         reinterpret_cast<uintptr_t>(a.conv_b)) & 15) == 0;
-    const dim3 grid_c((a.d_xBC / (vec4 ? 4 : 1) + 255) / 256, c.B * ((c.k + CONV_ROWS - 1) / CONV_ROWS));
-    if (vec4) launch_pdl(scan_conv_kernel<4>, grid_c, dim3(256), 0, stream, a, xact, c16);
-    else launch_pdl(scan_conv_kernel<1>, grid_c, dim3(256), 0, stream, a, xact, c16);
-    trk_end(trk);
-    trk_begin(trk, "scan_cb", 0, 0);
-    launch_pdl(scan_cb_kernel, dim3(c.G, c.B), dim3(256), size_t(2) * c.k * (c.N + 4) * sizeof(float), stream, a, xact, (float*)cbw);
+    const dim3 grid_c(c.G + (a.Di / (vec4 ? 4 : 1) + 255) / 256, c.B * ((c.k + CONV_ROWS - 1) / CONV_ROWS));
+    const size_t smem_c = size_t(2) * c.k * (c.N + 4) * sizeof(float);
+    launch_pdl(vec4 ? scan_conv_kernel<4> : scan_conv_kernel<1>, grid_c, dim3(256), smem_c, stream, a, xact, c16, cbw);
     trk_end(trk);
     const size_t smem_s = two ? scan_stream_smem<2>() : scan_stream_smem<1>();
     static bool sset[2][MAX_DEVICES] = {};
