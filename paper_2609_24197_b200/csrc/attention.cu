@@ -33,6 +33,8 @@ struct AttnArgs {
   int B, k, Hq, Hkv, rep, R, RT, n_row_tiles;
   int chunk, max_chunks, page_size, window;
   int max_ctx;       // host bound on the context lengths: a length outside [0, max_ctx] is clamped and counted
+  int early;         // nothing on the stream that may still be running writes the context's keys, values or lengths: the first tile of them
+                     // is fetched before the kernel in front (which writes q and the block's own rows) has finished
   int num_pages;     // a page id outside [0, num_pages) is read as zeros and counted
   float scale_log2;
 };
@@ -59,8 +61,7 @@ __device__ __forceinline__ uint32_t swz(int row, int col) {   // byte offset of 
 template <int DH, int KS>
 __global__ void __launch_bounds__(KS > 1 ? 352 : 256)
 attn_partial_kernel(AttnArgs a) {
-  pdl_wait();
-  pdl_trigger();
+  if (!a.early) { pdl_wait(); pdl_trigger(); }
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
   const int b = blockIdx.z, kvh = blockIdx.y;
@@ -69,7 +70,10 @@ attn_partial_kernel(AttnArgs a) {
   if (tid == 0 && blockIdx.x == 0 && kvh == 0 && ctx != a.ctx_lens[b]) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
   int lo0, n_chunks;
   visible_range(ctx, a.window, a.chunk, lo0, n_chunks);
-  if (c >= n_chunks) return;
+  if (c >= n_chunks) {
+    if (a.early) pdl_wait();
+    return;
+  }
   const bool last = (c == n_chunks - 1);
   const int p_begin = lo0 + c * a.chunk;
   const int p_end = min(ctx, p_begin + a.chunk);
@@ -87,18 +91,6 @@ attn_partial_kernel(AttnArgs a) {
   const int n_compute = a.RT * 2 * KS, slab16 = warp / KS, part = warp % KS;     // (threads; the warp's rows; its part of the keys)
   const bool compute = tid < n_compute;
   const int n_loaders = nthr > n_compute ? nthr - n_compute : nthr, loader = nthr > n_compute ? tid - n_compute : tid;   // (loader < 0: none)
-
-  // ---- Q rows of this tile -> shared (zero for padding rows)
-  const int row0 = rt * a.RT;
-  for (int idx = tid; idx < a.RT * CPR; idx += nthr) {
-    const int r = idx / CPR, ch = idx % CPR;
-    const int rg = row0 + r;
-    const bool ok = rg < a.R;
-    const int i = ok ? rg / a.rep : 0, gq = ok ? rg % a.rep : 0;
-    const __nv_bfloat16* src = a.q + ((size_t(b) * a.k + i) * a.Hq + kvh * a.rep + gq) * DH + ch * 8;
-    cp_async16(smem_u32(sQ) + swz<DH>(r, ch * 8), src, ok);
-  }
-  cp_async_commit();
 
   const int32_t* ptab = a.page_table + size_t(b) * a.page_table_stride;
   auto load_tile = [&](int t) {
@@ -145,8 +137,24 @@ attn_partial_kernel(AttnArgs a) {
     }
   };
 
+  // the first group holds tile 0 and the Q rows
+  const bool tile0_early = a.early && n_pre > 0;
+  if (tile0_early && loader >= 0) load_tile(0);
+  if (a.early) { pdl_wait(); pdl_trigger(); }
+  // ---- Q rows of this tile -> shared (zero for padding rows)
+  const int row0 = rt * a.RT;
+  for (int idx = tid; idx < a.RT * CPR; idx += nthr) {
+    const int r = idx / CPR, ch = idx % CPR;
+    const int rg = row0 + r;
+    const bool ok = rg < a.R;
+    const int i = ok ? rg / a.rep : 0, gq = ok ? rg % a.rep : 0;
+    const __nv_bfloat16* src = a.q + ((size_t(b) * a.k + i) * a.Hq + kvh * a.rep + gq) * DH + ch * 8;
+    cp_async16(smem_u32(sQ) + swz<DH>(r, ch * 8), src, ok);
+  }
+  if (!tile0_early && n_tiles > 0 && loader >= 0) load_tile(0);
+  cp_async_commit();
 #pragma unroll
-  for (int t = 0; t < NSTAGE - 1; ++t) {
+  for (int t = 1; t < NSTAGE - 1; ++t) {
     if (t < n_tiles && loader >= 0) load_tile(t);
     cp_async_commit();
   }
@@ -451,6 +459,7 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   a.chunk = c.chunk_tokens; a.max_chunks = attn_max_chunks(c.max_ctx, c.window, c.chunk_tokens);
   a.page_size = c.page_size; a.window = c.window;
   a.status = c.status;
+  a.early = c.planned ? 1 : 0;
   a.max_ctx = c.max_ctx < c.page_table_stride * c.page_size ? c.max_ctx : c.page_table_stride * c.page_size;
   a.num_pages = int(c.num_pages < 0x7fffffff ? c.num_pages : 0x7fffffff);
   a.scale_log2 = 1.4426950408889634f / sqrtf(float(c.dh));

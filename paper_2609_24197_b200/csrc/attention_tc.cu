@@ -63,6 +63,8 @@ struct AttnTcArgs {
   int B, k, Hq, Hkv, rep, R, n_row_tiles;
   int chunk, max_chunks, window;
   int max_ctx;           // host bound on the context lengths: a length outside [0, max_ctx] is clamped and counted
+  int early;             // the work list was there before the kernel in front started: the context's keys and values are fetched while
+                         // that kernel still runs (nothing on the stream writes them), only q and the block's own rows wait for it
   int num_pages;         // pages in each pool: a page id outside [0, num_pages) is read as zeros and counted
   float scale_log2;
 };
@@ -267,6 +269,7 @@ __device__ __forceinline__ void produce_operand(const AttnTcArgs& a, const CUten
       } else {
         int n_prefix, prefix_start, n_block;
         manual_tile(g, t - g.n_full, a.k, n_prefix, prefix_start, n_block);
+        if (a.early && n_block > 0) pdl_wait();        // (the block's rows come from the kernel in front)
         const int full_pages = n_prefix >> 4;
         const int tma_rows = full_pages << 4;
         if (lane == 0 && full_pages > 0) mbar_expect_tx_only(bar, full_pages * 4096);
@@ -320,8 +323,7 @@ template <int DUP>
 __global__ void __launch_bounds__(352, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnTcArgs a,
                const int* __restrict__ count, const int4* __restrict__ items) {
-  pdl_wait();
-  pdl_trigger();
+  if (!a.early) { pdl_wait(); pdl_trigger(); }
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sQ = smem;                               // Q tile, 32 KiB
   uint8_t* sKV = smem + KV_BYTES;                   // K ring (NSK x 32 KiB), then V ring (NSV x 32 KiB)
@@ -329,7 +331,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_items = *count;
-  if (item_at(0) >= n_items) return;                // uniform for the whole CTA
+  if (item_at(0) >= n_items) {                      // uniform for the whole CTA
+    if (a.early) pdl_wait();
+    return;
+  }
   if (smem_u32(smem) & 1023) {                      // the swizzled operand tiles need a 1 KiB-aligned base
     if (tid == 0) atomicExch(a.status, STATUS_BAD_SMEM_BASE);
     return;
@@ -543,6 +548,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     };
     int4 w_cur = items[item_at(0)];
     int4 w_next = (item_at(1) < n_items) ? items[item_at(1)] : w_cur;
+    // (dependents start only from here: what they and their dependents rely on is that everything ahead of this kernel has finished)
+    if (a.early) { pdl_wait(); pdl_trigger(); }
     q_copy_issue(unpack_item(w_cur));
     q_copy_finish();
     for (; item_at(int(n)) < n_items && ok; ++n) {
@@ -940,6 +947,7 @@ cudaError_t attention_tc_launch(const AttnCall& c, int max_chunks, cudaStream_t 
   a.k_pool = (const __nv_bfloat16*)c.k_pool; a.v_pool = (const __nv_bfloat16*)c.v_pool;
   a.page_table = c.page_table; a.ctx_lens = c.ctx_lens; a.page_table_stride = c.page_table_stride;
   a.status = c.status;
+  a.early = c.planned ? 1 : 0;
   a.B = c.B; a.k = c.k; a.Hq = c.Hq; a.Hkv = c.Hkv; a.rep = c.Hq / c.Hkv; a.R = c.k * a.rep;
   a.n_row_tiles = (a.R + 127) / 128;
   a.chunk = c.chunk_tokens; a.max_chunks = max_chunks; a.window = c.window;
