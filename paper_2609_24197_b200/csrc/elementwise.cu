@@ -260,37 +260,57 @@ __global__ void qk_norm_rope_kernel(const float* __restrict__ qkv, const float* 
 // memory and serve all Hq + Hkv heads (a warp per head recomputed them 72 times per row at the 32B-class shapes), a
 // warp takes every eighth head with 8-byte loads, the loads of ROPE_HB heads in flight together.  The arithmetic per
 // element is that of the kernel above.
+// TAIL: the QKV projection in front left the K-slices of its last wave's tiles unsummed; they are added up here, in slice order, on the
+// way (a head's columns lie in one 256-wide weight tile).  early: the context lengths are not written by anything that may still run,
+// so the sines and cosines are ready before the wait.
 constexpr int ROPE_HB = 5;
+template <bool TAIL>
 __global__ void __launch_bounds__(256)
 qk_norm_rope_row_kernel(const float* __restrict__ qkv, const float* __restrict__ qw, const float* __restrict__ kw,
                         const float* __restrict__ inv_freq, const int32_t* __restrict__ ctx_lens,
                         __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ kb, __nv_bfloat16* __restrict__ vb,
-                        int k, int Hq, int Hkv, int dh, float eps, int qk_norm) {
-  pdl_wait();
-  pdl_trigger();
+                        int k, int Hq, int Hkv, int dh, float eps, int qk_norm, int early, GemmTail tail) {
+  if (!early) { pdl_wait(); pdl_trigger(); }
   __shared__ __align__(8) float cs_s[64], sn_s[64];
   const int m = blockIdx.x, half = dh / 2, heads = Hq + 2 * Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float pos = float(ctx_lens[m / k] + m % k);
   for (int j = threadIdx.x; j < half; j += blockDim.x) sincosf(pos * inv_freq[j], &sn_s[j], &cs_s[j]);
+  if (early) { pdl_wait(); pdl_trigger(); }
   __syncthreads();
   const float* row = qkv + size_t(m) * heads * dh;
+  const TailRow tail_row = TAIL ? TailRow(tail, m) : TailRow();
   // dh <= 128: a lane's share of a head is one pair of rotation pairs, j = 2 lane and 2 lane + 1 (lanes past dh / 4
   // hold zeros and store nothing, but take part in the warp reduction)
   const int j2 = lane;
   const bool act = j2 < half / 2;
   for (int h0 = warp; h0 < heads; h0 += 8 * ROPE_HB) {
     float2 a[ROPE_HB], b[ROPE_HB];
+    const float* src[ROPE_HB];                              // TAIL: the head's columns in the first slice; null: not in a tail tile
 #pragma unroll
     for (int u = 0; u < ROPE_HB; ++u) {
       const int hh = h0 + u * 8;
-      if (hh < heads && act) {
+      src[u] = TAIL && hh < heads ? reinterpret_cast<const float*>(tail_src(tail, tail_row, hh * dh)) : nullptr;
+      if (hh < heads && act && src[u] == nullptr) {
         a[u] = *reinterpret_cast<const float2*>(row + size_t(hh) * dh + 2 * j2);
         b[u] = *reinterpret_cast<const float2*>(row + size_t(hh) * dh + half + 2 * j2);
       } else {
         a[u] = b[u] = make_float2(0.f, 0.f);
       }
     }
+    if (TAIL)
+      for (int sp = 0; sp < tail.splits; ++sp) {
+        float2 pa[ROPE_HB], pb[ROPE_HB];
+#pragma unroll
+        for (int u = 0; u < ROPE_HB; ++u) {
+          const bool on = src[u] != nullptr && act;
+          const float* p = src[u] + size_t(sp) * tail.BNT * 256 + 2 * j2;
+          pa[u] = on ? *reinterpret_cast<const float2*>(p) : make_float2(0.f, 0.f);
+          pb[u] = on ? *reinterpret_cast<const float2*>(p + half) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < ROPE_HB; ++u) { a[u].x += pa[u].x; a[u].y += pa[u].y; b[u].x += pb[u].x; b[u].y += pb[u].y; }
+      }
 #pragma unroll
     for (int u = 0; u < ROPE_HB; ++u) {
       const int hh = h0 + u * 8;
@@ -439,17 +459,22 @@ cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, f
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+bool qk_norm_rope_takes_tail(int dh) { return dh == 64 || dh == 128; }
+
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,
                                 void* kb, void* vb, int B, int k, int Hq, int Hkv, int dh, float theta, float eps,
-                                int qk_norm, cudaStream_t stream) {
+                                int qk_norm, cudaStream_t stream, bool early, const GemmTail* tail) {
   if (dh > 256 || (dh & 1)) return cudaErrorInvalidValue;
+  const bool pending = tail != nullptr && tail->part != nullptr;
   const float* tab = rope_table(theta, dh);
   if (!tab) return cudaErrorMemoryAllocation;
   if ((dh & 3) == 0 && dh <= 128) {
-    cudaError_t e = launch_pdl(qk_norm_rope_row_kernel, dim3(B * k), dim3(256), 0, stream, qkv, qw, kw, tab, ctx_lens,
-                               (__nv_bfloat16*)q, (__nv_bfloat16*)kb, (__nv_bfloat16*)vb, k, Hq, Hkv, dh, eps, qk_norm);
+    cudaError_t e = launch_pdl(pending ? qk_norm_rope_row_kernel<true> : qk_norm_rope_row_kernel<false>, dim3(B * k), dim3(256), 0, stream, qkv,
+                               qw, kw, tab, ctx_lens, (__nv_bfloat16*)q, (__nv_bfloat16*)kb, (__nv_bfloat16*)vb, k, Hq, Hkv, dh, eps, qk_norm,
+                               early ? 1 : 0, pending ? *tail : GemmTail{});
     return e != cudaSuccess ? e : cudaGetLastError();
   }
+  if (pending) return cudaErrorInvalidValue;       // (qk_norm_rope_takes_tail said no)
   const int n_pairs = B * k * (Hq + 2 * Hkv);
   cudaError_t e = launch_pdl(qk_norm_rope_kernel, dim3((n_pairs + 7) / 8), dim3(256), 0, stream, qkv, qw, kw, tab, ctx_lens,
                              (__nv_bfloat16*)q, (__nv_bfloat16*)kb, (__nv_bfloat16*)vb, k, Hq, Hkv, dh, eps, qk_norm, n_pairs);

@@ -544,7 +544,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   trk_end(trk);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (c.defer_tail) *c.defer_tail = GemmTail{};
-  if (e == cudaSuccess && splits > 1 && c.defer_tail && c.mode == EPI_ACCUM_F32) {
+  if (e == cudaSuccess && splits > 1 && c.defer_tail && (c.mode == EPI_ACCUM_F32 || c.mode == EPI_STORE_F32)) {
     *c.defer_tail = GemmTail{g.part, g.raster, g.n_full_tiles, g.BNT, splits};
     return e;
   }

@@ -571,7 +571,8 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   const StepWeights& SW = h->by_role;
   GemmTail tail{};                                 // what the last residual GEMM left for the norm behind it to add to X
   auto fptr = [](const Weight* w) { return reinterpret_cast<const float*>(w->data); };
-  auto gemm = [&](const Weight* wp, const char* label, const void* x, int rows, int mode, void* o, long long ldo) -> cudaError_t {
+  auto gemm = [&](const Weight* wp, const char* label, const void* x, int rows, int mode, void* o, long long ldo,
+                  GemmTail* store_tail = nullptr) -> cudaError_t {
     const Weight& w = *wp;
     if (mode == EPI_ACCUM_F32) tail = GemmTail{};
     GemmCall g{};
@@ -581,7 +582,7 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     g.splitk_ws = ws + p.SPLITK; g.splitk_ws_bytes = p.splitk_bytes;
     g.status = h->d_status; g.label = label;
     g.w_stable = true;                             // library copies, or borrowed unchanged for the handle's life
-    g.defer_tail = mode == EPI_ACCUM_F32 ? &tail : nullptr;
+    g.defer_tail = mode == EPI_ACCUM_F32 ? &tail : store_tail;
     return gemm_launch(g, st, trk, &errtxt);
   };
   // element-wise launches: bracket with the tracker (name, algorithmic bytes)
@@ -649,10 +650,11 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     // ---- attention over the target's KV (in place) + the block
     if (c.has_attn[l]) {
       EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.a_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
-      CUDA_TRY(h, gemm(lw.wqkv, "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv));
+      GemmTail qkv_tail{};
+      CUDA_TRY(h, gemm(lw.wqkv, "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv, qk_norm_rope_takes_tail(c.dh) ? &qkv_tail : nullptr));
       EW("qk_norm_rope", Md * d.d_qkv * 6,
          qk_norm_rope_launch(BIG, fptr(lw.q_norm), fptr(lw.k_norm), in->ctx_lens, Q, KB, VB, B, k, c.Hq,
-                             c.Hkv, c.dh, c.rope_theta, c.rms_eps, c.qk_norm, st));
+                             c.Hkv, c.dh, c.rope_theta, c.rms_eps, c.qk_norm, st, true, &qkv_tail));
       AttnCall a = attn_call();
       a.k_pool = in->k_pools[c.kv_slot[l]]; a.v_pool = in->v_pools[c.kv_slot[l]];
       CUDA_TRY(h, attention_launch(a, st, trk, &errtxt));

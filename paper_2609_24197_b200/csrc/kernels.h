@@ -187,7 +187,7 @@ struct GemmCall {       // host-side description of one y = x W^T
   bool w_stable;            // nothing that may still be running on the stream writes the weights: they may be fetched early
   uint32_t* status;
   const char* label;        // profile name (may be null)
-  GemmTail* defer_tail;     // EPI_ACCUM_F32: the caller adds the sliced tail tiles itself (their description is left here); may be null
+  GemmTail* defer_tail;     // EPI_ACCUM_F32 or EPI_STORE_F32: the caller adds the sliced tail tiles itself (their description is left here); may be null
 };
 
 bool make_tmap_16bit_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld_elems,
@@ -304,7 +304,8 @@ cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, f
                            uint32_t* status, bool bf16_out = false, const GemmTail* tail = nullptr);
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,
                                 void* kb, void* vb, int B, int k, int Hq, int Hkv, int dh, float theta, float eps,
-                                int qk_norm, cudaStream_t stream);
+                                int qk_norm, cudaStream_t stream, bool early = false, const GemmTail* tail = nullptr);
+bool qk_norm_rope_takes_tail(int dh);   // whether the launch can add up a tail that the projection in front left
 cudaError_t swiglu_launch(const float* gu, void* h_16, int M, int F, cudaStream_t stream, uint32_t* status, bool bf16_out = false);
 cudaError_t copy_f32_launch(const float* src, float* dst, size_t n, cudaStream_t stream);
 

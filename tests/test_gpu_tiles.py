@@ -216,3 +216,17 @@ def test_small_state_scan_with_norm(hs, Di, P, N, G, dt_rank, B, k):
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[20] * B)
     check_step(cfg, drafter, w, batch, k, requests=list(range(B)), what=f"small {Di} {P} {N} {G} {dt_rank}")
     drafter.close()
+
+
+# the QK norm behind the QKV projection adds that GEMM's K-sliced tail tiles: all tail, and a whole wave with a tail behind it, heads of a
+# quarter and of half a weight tile, a last weight tile that is only part full
+@pytest.mark.parametrize("dh,Hq,Hkv,B,k", [(64, 16, 4, 9, 32), (128, 8, 2, 9, 32), (128, 6, 1, 20, 13), (64, 14, 2, 141, 32)])
+def test_qkv_tail_is_added_by_the_qk_norm(hs, dh, Hq, Hkv, B, k):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(D=1024, n_fuse=1, r=64, L=1, has_attn=[1], kv_slot=[0], n_slots=1, Di=1024, P=64, N=4, G=1, d_conv=4, dt_rank=0,
+                             Hq=Hq, Hkv=Hkv, dh=dh, rope_theta=1.0e4, window=0, qk_norm=1, F=512, V=600, rms_eps=1e-6, page_size=16, name="qkvtail",
+                             B=B, k=k, ctx=("const", 20, 20)))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[b % 40 for b in range(B)])
+    check_step(cfg, drafter, w, batch, k, requests=sorted({0, 1, B // 2, B - 1}), what=f"qkv tail {dh} {B}")
+    drafter.close()
