@@ -238,8 +238,8 @@ int hspec_op_lm_head_argmax(const void* x, const void* W, int32_t in_dtype, int3
 /* The same LM head + arg-max for callers that cannot allocate device memory at the point where they draft: an engine
  * whose KV-cache pool already owns every free byte of HBM (a later cudaMalloc fails), a decode loop that cannot take the
  * device synchronisation and driver lock of an allocation, a plug-in that is handed pointers but no allocator.  (The
- * paper has no counterpart; this is a deployment aid.)  The per-tile (max, index) partials and the status word live in
- * a fixed array inside the library's device image: 8 MiB + 256 B on every GPU that loads the library, held until the
+ * paper has no counterpart; this is a deployment aid.)  The per-row (value, index) keys and the status word live in
+ * a fixed array inside the library's device image: 4.3 KiB on every GPU that loads the library, held until the
  * process exits.  Limits: M <= 512 rows, V <= 262144; larger sizes are rejected with HSPEC_ERR_BAD_SHAPE.
  * The call allocates nothing (no cudaMalloc / cudaFree, no allocating library routine).  Its FIRST call on a device
  * resolves the array's device address (cudaGetSymbolAddress, with that device current) and, with CUDA's lazy module

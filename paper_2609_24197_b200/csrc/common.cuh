@@ -364,4 +364,11 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// (value, index) as one unsigned number: the larger key has the larger value, at equal values the lower index.  Any value beats the zero
+// key, NaN never gets this far.
+__device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
+  uint32_t u = __float_as_uint(v + 0.f);                    // (-0 compares equal to +0)
+  u = (u & 0x80000000u) ? ~u : u | 0x80000000u;
+  return (static_cast<unsigned long long>(u) << 32) | (0xffffffffu - uint32_t(idx));
+}
 }  // namespace hspec

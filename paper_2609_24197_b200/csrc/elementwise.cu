@@ -162,6 +162,7 @@ __global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ embed, const
   pdl_trigger();
   __shared__ float red[32];
   const int m = blockIdx.x;
+  if (prep.keys != nullptr && threadIdx.x == 0 && m < B * k) prep.keys[m] = 0;
   if (m >= B * k) {
     __shared__ int bucket[64], offset[64];
     const int planners = prep.plan.items != nullptr ? 1 : 0;

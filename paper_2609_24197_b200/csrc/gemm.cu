@@ -258,6 +258,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
         }
         if (!ok) { v = -INFINITY; idx = 0x7fffffff; }
+        if (g.keys != nullptr) {
+          if (idx != 0x7fffffff) atomicMax(g.keys + m, argmax_key(v, idx));
+          continue;
+        }
         g.part_val[size_t(tile_n) * g.M + m] = v;
         g.part_idx[size_t(tile_n) * g.M + m] = idx;
       }
@@ -317,52 +321,26 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   }
 }
 
-// ids[m] = lowest index among the per-tile maxima (tiles are in ascending vocabulary order).
-// The partials are [tile][row]: a block takes eight consecutive rows, thread (r = tid % 8, tid / 8) walks every 128th
-// tile of row r, so that eight neighbouring threads read one 32-byte sector, with the loads of four tiles in flight.  There are only
-// M / 8 blocks, so it is the length of a thread's chain that counts: with 256 threads and one tile at a time the 1 188 tiles of
-// a 152 064-token vocabulary were 38 dependent rounds (15 us at 16 and at 512 rows).
-__device__ __forceinline__ void argmax_take(float& v, int& idx, float ov, int oi) {
-  if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-}
-__global__ void __launch_bounds__(1024)
-argmax_reduce_kernel(const float* __restrict__ pv, const int* __restrict__ pi, int n_tiles, int M,
-                     int* __restrict__ ids, const int* __restrict__ id_map) {
+__global__ void __launch_bounds__(256)
+argmax_init_kernel(unsigned long long* keys, int M) {
   pdl_wait();
   pdl_trigger();
-  const int r = threadIdx.x & 7, m = blockIdx.x * 8 + r;
-  float v = -INFINITY;
-  int idx = 0x7fffffff;
-  if (m < M) {
-    for (int t = threadIdx.x >> 3; t < n_tiles; t += 4 * 128) {
-      float tv[4];
-      int ti[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int tu = t + u * 128;
-        tv[u] = tu < n_tiles ? pv[size_t(tu) * M + m] : -INFINITY;
-        ti[u] = tu < n_tiles ? pi[size_t(tu) * M + m] : 0x7fffffff;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) argmax_take(v, idx, tv[u], ti[u]);
-    }
-  }
-  // lanes r, r + 8, r + 16, r + 24 of a warp hold the same row
-  for (int off = 8; off < 32; off <<= 1)
-    argmax_take(v, idx, __shfl_xor_sync(0xffffffffu, v, off), __shfl_xor_sync(0xffffffffu, idx, off));
-  __shared__ float sv[32][8];
-  __shared__ int si[32][8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane < 8) { sv[warp][lane] = v; si[warp][lane] = idx; }
-  __syncthreads();
-  if (warp < 8) {                                           // warp w: row w of the block, lane = the warp the value came from
-    v = sv[lane][warp]; idx = si[lane][warp];
-    for (int off = 16; off > 0; off >>= 1)
-      argmax_take(v, idx, __shfl_xor_sync(0xffffffffu, v, off), __shfl_xor_sync(0xffffffffu, idx, off));
-    const int mw = blockIdx.x * 8 + warp;
-    // (pruned drafter vocabulary: row index -> token id; a row without any maximum keeps its sentinel)
-    if (lane == 0 && mw < M) ids[mw] = id_map && idx != 0x7fffffff ? id_map[idx] : idx;
-  }
+  const int m = blockIdx.x * 256 + threadIdx.x;
+  if (m < M) keys[m] = 0;
+}
+
+// A row without any maximum keeps its sentinel.  (Before, the tiles' (value, index) pairs went to memory and this kernel reduced them: the
+// LM head of 152 064 rows, 77 requests 282 -> 279 us.  Letting the GEMM's last CTA write the ids instead costs a fence, a ticket
+// and a read-back at its end, more than this launch: test-sized drafter 65.3 -> 66.6 us per step.)
+__global__ void __launch_bounds__(256)
+argmax_ids_kernel(const unsigned long long* keys, int M, int* ids, const int* id_map) {
+  pdl_wait();
+  pdl_trigger();
+  const int m = blockIdx.x * 256 + threadIdx.x;
+  if (m >= M) return;
+  const unsigned long long key = keys[m];
+  const int idx = key ? int(0xffffffffu - uint32_t(key)) : 0x7fffffff;
+  ids[m] = id_map && idx != 0x7fffffff ? id_map[idx] : idx;
 }
 
 // ------------------------------------------------------------------ host side
@@ -475,7 +453,7 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   g.stages = stages;
   g.status = c.status;
   g.f16 = c.f16 ? 1 : 0;
-  g.logits = c.logits; g.addend = c.addend; g.ld_add = c.ld_add; g.part_val = c.part_val; g.part_idx = c.part_idx;
+  g.logits = c.logits; g.addend = c.addend; g.ld_add = c.ld_add; g.keys = c.keys; g.part_val = c.part_val; g.part_idx = c.part_idx;
   g.keep_w = c.keep_weights_in_l2 ? 1 : 0;
   g.early_w = c.w_stable ? 1 : 0;
   g.ldo = c.ldo;
@@ -497,12 +475,16 @@ cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, st
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t argmax_reduce_launch(const float* pv, const int* pi, int n_tiles, int M, int* ids, cudaStream_t stream,
-                                 Tracker* trk, const int* id_map) {
-  trk_begin(trk, "argmax_reduce", 0, double(n_tiles) * M * 8);
-  launch_pdl(argmax_reduce_kernel, dim3((M + 7) / 8), dim3(1024), 0, stream, pv, pi, n_tiles, M, ids, id_map);
+cudaError_t argmax_init_launch(unsigned long long* keys, int M, cudaStream_t stream) {
+  const cudaError_t e = launch_pdl(argmax_init_kernel, dim3((M + 255) / 256), dim3(256), 0, stream, keys, M);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t argmax_ids_launch(const unsigned long long* keys, int M, int* ids, const int* id_map, cudaStream_t stream, Tracker* trk) {
+  trk_begin(trk, "argmax_ids", 0, double(M) * 12);
+  const cudaError_t e = launch_pdl(argmax_ids_kernel, dim3((M + 255) / 256), dim3(256), 0, stream, keys, M, ids, id_map);
   trk_end(trk);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace hspec

@@ -56,8 +56,7 @@ struct Gemm2Args {
   void* out;
   long long ldo;
   float* logits;
-  float* part_val;
-  int* part_idx;
+  unsigned long long* keys;
   uint32_t* status;
 };
 
@@ -357,8 +356,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int oi = tail->red_idx[qq][c];
             if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
           }
-          g.part_val[size_t(tile_n128) * g.M + m] = v;
-          g.part_idx[size_t(tile_n128) * g.M + m] = idx;
+          if (idx != 0x7fffffff) atomicMax(g.keys + m, argmax_key(v, idx));
         }
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");        // red_* is reused by the next tile
       }
@@ -518,7 +516,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   g.early_w = c.w_stable ? 1 : 0;
   g.f16 = c.f16 ? 1 : 0; g.mode = c.mode; g.out = c.out; g.ldo = c.ldo;
   if (c.addend != nullptr) { if (err) *err = "the 2-SM kernel has no addend epilogue"; return cudaErrorInvalidValue; }
-  g.logits = c.logits; g.part_val = c.part_val; g.part_idx = c.part_idx; g.status = c.status;
+  g.logits = c.logits; g.keys = c.keys; g.status = c.status;
   static const int ksub_env = [] { const char* e = getenv("HSPEC_GEMM2_KSUB"); return e ? atoi(e) : 0; }();   // measurements only
   g.ksub = (ksub_env == 1 || ksub_env == 2) ? ksub_env : 2;
   const size_t stage_bytes = size_t(g.ksub) * (A_BYTES + size_t(g.BNT / 2) * TILE_K * 2);

@@ -55,7 +55,7 @@ int imax(int a, int b) { return a > b ? a : b; }
 
 // Offsets of the step's scratch buffers inside the caller's workspace.
 struct Plan {
-  size_t X, U, U2, BIG, LH, Fv, SINIT, SCAN, scan_bytes, DTL, DT, YG, Q, KB, VB, ATT, SPLITK, AMAXV, AMAXI, LOGITS, MARKOV, total;
+  size_t X, U, U2, BIG, LH, Fv, SINIT, SCAN, scan_bytes, DTL, DT, YG, Q, KB, VB, ATT, SPLITK, KEYS, LOGITS, MARKOV, total;
   size_t att_bytes, splitk_bytes;
   int attn_chunk, max_ctx;
 };
@@ -100,9 +100,7 @@ Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
   upd(splitk_need(int(M), 2 * c.F));
   p.splitk_bytes = sk;
   p.SPLITK = take(sk);
-  const size_t vt = 2 * ((size_t(d.Vd) + 255) / 256);   // 128-row tiles, in pairs (the 2-SM kernel's indexing)
-  p.AMAXV = take(vt * M * 4);
-  p.AMAXI = take(vt * M * 4);
+  p.KEYS = take(M * 8);                                 // the LM head's arg-max: a key per row
   if (c.markov_rank > 0) {
     // the causal-correction head works on materialised fp32 logits of the whole block
     p.LOGITS = take(M * size_t(d.Vd) * 4);
@@ -606,6 +604,8 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   };
   StepPrep prep{};
   if (!any_attn || !attention_plan(attn_call(), &prep.plan)) prep.plan.items = nullptr;
+  const int* id_map = c.V_draft > 0 ? reinterpret_cast<const int*>(SW.vocab_map->data) : nullptr;
+  if (c.markov_rank == 0) prep.keys = reinterpret_cast<unsigned long long*>(ws + p.KEYS);
   const void* lh_in = LH;
   prep.n_lh = size_t(B) * c.n_fuse * c.D;
   if (bf && (reinterpret_cast<uintptr_t>(in->last_hidden) & 15) == 0) lh_in = in->last_hidden;   // already the operand type: read in place
@@ -675,7 +675,6 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
   // ---- final norm, LM head fused with the per-row arg-max
   EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(SW.final_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
   if (out->hidden) EW("copy_hidden", Md * c.D * 8, copy_f32_launch(X, out->hidden, size_t(M) * c.D, st));
-  const int* id_map = c.V_draft > 0 ? reinterpret_cast<const int*>(SW.vocab_map->data) : nullptr;
   if (c.markov_rank > 0) {
     // ---- LM head to fp32 logits, then the causal correction position by position (Sec. 3.3.3)
     float* logits = out->logits ? out->logits : reinterpret_cast<float*>(ws + p.LOGITS);
@@ -695,11 +694,11 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     GemmCall g{};
     g.tmW = &w.tm; g.x = U; g.f16 = !bf; g.ldx = c.D; g.M = M; g.n_out = d.Vd; g.K = c.D; g.mode = EPI_ARGMAX; g.splits = 1;
     g.logits = out->logits; g.ldo = d.Vd;
-    g.part_val = reinterpret_cast<float*>(ws + p.AMAXV); g.part_idx = reinterpret_cast<int*>(ws + p.AMAXI);
+    g.keys = prep.keys;
     g.status = h->d_status; g.label = "gemm:lm_head_argmax";
     g.w_stable = true;
     CUDA_TRY(h, gemm_launch(g, st, trk, &errtxt));
-    CUDA_TRY(h, argmax_reduce_launch(g.part_val, g.part_idx, (d.Vd + 127) / 128, M, out->draft_ids, st, trk, id_map));
+    CUDA_TRY(h, argmax_ids_launch(g.keys, M, out->draft_ids, id_map, st, trk));
   }
 #undef EW
   h->launches_last_step = uint32_t(trk->launches - launches0);
@@ -799,13 +798,13 @@ int hspec_op_lm_head_argmax(const void* x, const void* Wt, int32_t in_dtype, int
   GemmCall g{};
   g.tmW = &tm; g.x = x; g.f16 = (in_dtype == HSPEC_F16); g.ldx = K; g.M = M; g.n_out = V; g.K = K; g.mode = EPI_ARGMAX; g.splits = 1;
   g.logits = logits; g.ldo = V;
-  g.part_val = reinterpret_cast<float*>(workspace);
-  g.part_idx = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(workspace) + align_up(vt * M * 4, 256));
+  g.keys = reinterpret_cast<unsigned long long*>(align_up(reinterpret_cast<uintptr_t>(workspace), 256));
   g.status = global_status();
   if (!g.status) return fail(nullptr, HSPEC_ERR_CUDA, "hspec_op_lm_head_argmax: cannot allocate the status word");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  OP_TRY(argmax_init_launch(g.keys, M, st));
   OP_TRY(gemm_launch(g, st, nullptr, &errtxt));
-  OP_TRY(argmax_reduce_launch(g.part_val, g.part_idx, int(vt), M, ids, st, nullptr));
+  OP_TRY(argmax_ids_launch(g.keys, M, ids, nullptr, st, nullptr));
   return HSPEC_OK;
 }
 

@@ -135,6 +135,7 @@ struct GemmArgs {       // kernel argument block
   long long ld_add;
   int keep_w;           // weights loaded evict-last instead of evict-first
   int early_w;          // the weights may be read before the previous kernel of the stream has finished
+  unsigned long long* keys;
   float* part_val;
   int* part_idx;
   uint32_t* status;
@@ -182,7 +183,9 @@ struct GemmCall {       // host-side description of one y = x W^T
   const float* addend;      // EPI_ARGMAX, one-CTA kernel only: fp32 [M, ld_add] added before the arg-max (may be null)
   long long ld_add;
   bool keep_weights_in_l2;  // one-CTA kernel: the same W is used again by the next launch (keep it in L2 if it fits)
-  float* part_val;
+  unsigned long long* keys; // EPI_ARGMAX: [M], zero when the launch starts; every tile raises its rows' keys (value and index in 64 bits,
+                            // common.cuh), argmax_ids_launch turns them into ids.  Null (one-CTA kernel only): partials instead
+  float* part_val;          // EPI_ARGMAX with keys null: per-tile (max, lowest index), [tile][row]
   int* part_idx;
   bool w_stable;            // nothing that may still be running on the stream writes the weights: they may be fetched early
   uint32_t* status;
@@ -199,8 +202,9 @@ bool gemm2_preferred(int M, int n_out);        // many rows and at least one ful
 size_t gemm2_tail_bytes();                     // scratch the 2-SM kernel's K-sliced tail wave may use
 void gemm2_pick(int M, int n_out, int K, int mode, int* bnt, int* splits);   // tile width and K-slices of the 2-SM kernel
 cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
-cudaError_t argmax_reduce_launch(const float* pv, const int* pi, int n_tiles, int M, int* ids, cudaStream_t stream,
-                                 Tracker* trk, const int* id_map = nullptr);
+// Zeroes the keys, for callers that have no kernel of their own in front to do it; ids from the keys (id_map: vocabulary row -> token id).
+cudaError_t argmax_init_launch(unsigned long long* keys, int M, cudaStream_t stream);
+cudaError_t argmax_ids_launch(const unsigned long long* keys, int M, int* ids, const int* id_map, cudaStream_t stream, Tracker* trk);
 
 // ---- steps next to the draft block (next_ops.cu)
 struct MarkovCall {
@@ -295,6 +299,7 @@ struct StepPrep {
   const void* lh_src;               // bf16, n_lh values, copied to lh_dst as fp16 (or as they are when bf16_out); null: nothing to copy
   void* lh_dst;
   size_t n_lh;
+  unsigned long long* keys;         // [B * k] zeroed for the LM head's arg-max; null: none
   AttnPlan plan;                    // plan.items null: no work list
 };
 cudaError_t embed_norm_launch(const void* embed_bf16, const int32_t* last_token, int mask_id, const float* norm_w, float* X, void* u_16,

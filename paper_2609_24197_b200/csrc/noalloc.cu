@@ -3,13 +3,13 @@
 // Some hosts of this library cannot call cudaMalloc at the point where they draft: a serving engine that has
 // already handed every free byte of HBM to its KV-cache pool (a later allocation simply fails), a latency-critical
 // decode loop that cannot afford the implicit device synchronisation and driver lock an allocation takes, or a
-// plug-in that is given device pointers but no allocator.  For them the per-tile (max, index) partials of the fused
+// plug-in that is given device pointers but no allocator.  For them the per-row (value, index) keys of the fused
 // arg-max — the scratch that hspec_op_lm_head_argmax takes from a caller-allocated workspace — live in a fixed
 // array inside the library's own device image, together with the status word for bounded waits.
 //
 // The array is part of every process image that loads the library: each GPU that loads it holds these bytes until
 // the process exits.  All calls share it, so two calls that overlap on the GPU (different streams) race on the
-// partials; the contents left by one call are garbage to the next, which overwrites every slot it reads.
+// keys; the contents left by one call are garbage to the next, which zeroes what it uses first.
 #include "../../include/hspec.h"
 
 #include <mutex>
@@ -26,11 +26,10 @@ constexpr int NA_MAX_DEVICES = 64;
 struct NoAllocScratch {
   uint32_t status[64];                                   // word 0: bounded-wait status (must start at zero: it does,
                                                          // and only a give-up ever writes it)
-  float part_val[size_t(NA_MAX_TILES) * NA_MAX_ROWS];
-  int part_idx[size_t(NA_MAX_TILES) * NA_MAX_ROWS];
+  unsigned long long keys[NA_MAX_ROWS];                  // the arg-max's key per row, zeroed by every call
 };
 
-// 8 MiB + 256 B per GPU.  In HOST code this name is only a handle for cudaGetSymbolAddress, not a device address.
+// 4.3 KiB per GPU.  In HOST code this name is only a handle for cudaGetSymbolAddress, not a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
 std::mutex g_setup_mutex;
@@ -81,7 +80,7 @@ extern "C" int hspec_op_lm_head_argmax_noalloc(const void* x, const void* W, int
   using namespace hspec;
   if (!x || !W || !ids || M < 1 || V < 1 || K < 8 || K % 8) return na_fail(HSPEC_ERR_INVALID_ARG, "bad argument");
   if (in_dtype != HSPEC_BF16 && in_dtype != HSPEC_F16) return na_fail(HSPEC_ERR_INVALID_ARG, "x and W must both be bf16 or both fp16");
-  const int tiles = 2 * ((V + 255) / 256);               // 128-row tiles, counted in pairs as the 2-SM kernel indexes them
+  const int tiles = 2 * ((V + 255) / 256);               // 128-row tiles, in pairs
   if (M > NA_MAX_ROWS || tiles > NA_MAX_TILES)
     return na_fail(HSPEC_ERR_BAD_SHAPE, "the built-in scratch holds at most " + std::to_string(NA_MAX_ROWS) + " rows and a vocabulary of " +
                                             std::to_string(NA_MAX_TILES * 128) + " (got M=" + std::to_string(M) + ", V=" + std::to_string(V) +
@@ -94,13 +93,15 @@ extern "C" int hspec_op_lm_head_argmax_noalloc(const void* x, const void* W, int
   GemmCall g{};
   g.tmW = &tm; g.x = x; g.f16 = (in_dtype == HSPEC_F16); g.ldx = K; g.M = M; g.n_out = V; g.K = K; g.mode = EPI_ARGMAX; g.splits = 1;
   g.logits = logits; g.ldo = V;
-  g.part_val = s->part_val; g.part_idx = s->part_idx;     // device addresses obtained above, never the symbol itself
+  g.keys = s->keys;                                       // device addresses obtained above, never the symbol itself
   g.status = s->status;
   g.label = "gemm:lm_head_argmax";
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  cudaError_t e = gemm_launch(g, st, nullptr, &why);
+  cudaError_t e = argmax_init_launch(g.keys, M, st);
+  if (e != cudaSuccess) return na_fail(HSPEC_ERR_CUDA, cudaGetErrorString(e));
+  e = gemm_launch(g, st, nullptr, &why);
   if (e != cudaSuccess) return na_fail(HSPEC_ERR_CUDA, std::string(cudaGetErrorString(e)) + (why.empty() ? "" : " (" + why + ")"));
-  e = argmax_reduce_launch(g.part_val, g.part_idx, (V + 127) / 128, M, ids, st, nullptr);
+  e = argmax_ids_launch(g.keys, M, ids, nullptr, st, nullptr);
   if (e != cudaSuccess) return na_fail(HSPEC_ERR_CUDA, cudaGetErrorString(e));
   return HSPEC_OK;
 }

@@ -230,3 +230,32 @@ def test_qkv_tail_is_added_by_the_qk_norm(hs, dh, Hq, Hkv, B, k):
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[b % 40 for b in range(B)])
     check_step(cfg, drafter, w, batch, k, requests=sorted({0, 1, B // 2, B - 1}), what=f"qkv tail {dh} {B}")
     drafter.close()
+
+
+# the arg-max across tiles: equal values in one tile, in neighbouring and in distant ones (lowest index wins), +0 against -0, rows of negative
+# values only; one-CTA kernel and pair kernel, one activation tile and several, a single vocabulary row
+@pytest.mark.parametrize("M", [1, 9, 128, 129, 600])
+@pytest.mark.parametrize("V", [1, 127, 300, 20000])
+@pytest.mark.parametrize("alloc", [True, False])
+def test_lm_head_argmax_ties(hs, M, V, alloc):
+    K = 64
+    if not alloc and M > 512:
+        pytest.skip("more rows than the built-in scratch takes")
+    x, W = _rand((M, K), 1, torch.float16), _rand((V, K), 2, torch.float16)
+    W[V // 2] = W[0]                                          # a tie far away
+    W[min(V - 1, 3)] = W[0]
+    x[M // 2] = -x[M // 2].abs()
+    x[0] = 0.                                                 # every logit is +0 or -0: index 0
+    ids = torch.full((M,), -1, dtype=torch.int32, device="cuda")
+    logits = torch.empty((M, V), device="cuda")
+    for _ in range(2):                                        # the second call starts from what the first one left
+        ids.fill_(-1)
+        if alloc:
+            ws = torch.full((((V + 127) // 128) * M * 8 + 1024,), 255, dtype=torch.uint8, device="cuda")
+            hs.hspec_op_lm_head_argmax(x, W, ids, logits, ws)
+        else:
+            hs.hspec_op_lm_head_argmax_noalloc(x, W, ids, logits=logits)
+        z = logits.clone()
+        best = z.max(1, keepdim=True).values
+        first = torch.where(z == best, torch.arange(V, device="cuda"), V).min(1).values.int()     # exact: the kernel's own logits
+        assert torch.equal(ids, first)
