@@ -208,6 +208,19 @@ __device__ __forceinline__ Item unpack_item(const int4 w) {
   return it;
 }
 
+// Loads of what the kernel in front may still be writing.  They must stay behind the wait, which is under a condition here: a load through
+// a const __restrict__ pointer (or __ldg) counts as read-only and is moved up past it.
+__device__ __forceinline__ int load_after_wait(const int* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int4 load_item(const int4* p) {
+  int4 v;
+  asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 // The n-th item of this CTA.  The list is sorted longest first; handing round n out in ascending CTA order for even n and
 // in descending order for odd n evens out the CTAs' shares (plain round-robin gives CTA 0 the longest item of every
 // round).  Once an index falls past the end of the list, every later one does too.
@@ -234,13 +247,13 @@ __global__ void __launch_bounds__(256) attn_tc_plan_kernel(AttnPlan a) {
 //   cp.async with zero fill for every unused row, so nothing that is not a real key or value is ever multiplied.
 __device__ __forceinline__ void produce_operand(const AttnTcArgs& a, const CUtensorMap* tm, const __nv_bfloat16* pool,
                                                 const __nv_bfloat16* blk, uint8_t* ring, uint64_t* full, uint64_t* empty,
-                                                volatile uint32_t* abort_flag, const int4* __restrict__ items, int n_items,
+                                                volatile uint32_t* abort_flag, const int4* items, int n_items,
                                                 int lane, int ns) {
   uint32_t gt = 0;                                 // tiles issued so far, across items
-  int4 w_next = items[item_at(0)];
+  int4 w_next = load_item(items + item_at(0));
   for (int n = 0; item_at(n) < n_items; ++n) {
     const Item wi = unpack_item(w_next);
-    if (item_at(n + 1) < n_items) w_next = items[item_at(n + 1)];         // consumed one item later
+    if (item_at(n + 1) < n_items) w_next = load_item(items + item_at(n + 1));         // consumed one item later
     const int b = wi.b, kvh = wi.kvh;
     const AttnRange g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
     const int32_t* ptab = a.page_table + size_t(b) * a.page_table_stride;
@@ -322,7 +335,7 @@ __device__ __forceinline__ void produce_operand(const AttnTcArgs& a, const CUten
 template <int DUP>
 __global__ void __launch_bounds__(352, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnTcArgs a,
-               const int* __restrict__ count, const int4* __restrict__ items) {
+               const int* count, const int4* items) {
   if (!a.early) { pdl_wait(); pdl_trigger(); }
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sQ = smem;                               // Q tile, 32 KiB
@@ -330,7 +343,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
   AttnTcBars* bars = reinterpret_cast<AttnTcBars*>(sKV + (NSK + NSV) * KV_BYTES);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_items = *count;
+  const int n_items = load_after_wait(count);
   if (item_at(0) >= n_items) {                      // uniform for the whole CTA
     if (a.early) pdl_wait();
     return;
@@ -405,13 +418,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       // thread issued earlier; the tensor pipe runs one thread's MMAs in issue order.
       uint32_t gts = 0, n_s = 0;
       int t_s = 0;
-      int4 ws_next = items[item_at(0)];
+      int4 ws_next = load_item(items + item_at(0));
       bool s_valid = true;
       int T_s;
       {
         const Item w0 = unpack_item(ws_next);
         T_s = make_range(w0.ctx, a.window, a.chunk, w0.c, a.k).T;
-        if (item_at(1) < n_items) ws_next = items[item_at(1)];
+        if (item_at(1) < n_items) ws_next = load_item(items + item_at(1));
       }
       // returns 1 = issued, 0 = the item's Q tile is not there yet (only when it may come back later), -1 = timed out
       auto issue_s = [&](bool must) -> int {
@@ -444,17 +457,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
           if (item_at(int(n_s)) < n_items) {
             const Item wn = unpack_item(ws_next);
             T_s = make_range(wn.ctx, a.window, a.chunk, wn.c, a.k).T;
-            if (item_at(int(n_s) + 1) < n_items) ws_next = items[item_at(int(n_s) + 1)];
+            if (item_at(int(n_s) + 1) < n_items) ws_next = load_item(items + item_at(int(n_s) + 1));
           } else {
             s_valid = false;
           }
         }
         return 1;
       };
-      int4 w_next = items[item_at(0)];
+      int4 w_next = load_item(items + item_at(0));
       for (; item_at(int(n)) < n_items && ok; ++n) {
         const Item wi = unpack_item(w_next);
-        if (item_at(int(n) + 1) < n_items) w_next = items[item_at(int(n) + 1)];
+        if (item_at(int(n) + 1) < n_items) w_next = load_item(items + item_at(int(n) + 1));
         const AttnRange g = make_range(wi.ctx, a.window, a.chunk, wi.c, a.k);
         for (int t = 0; t < g.T && ok; ++t, ++gt) {
           // the scores of this tile must be under way (the softmax warps wait for them); the next two are issued as soon
@@ -546,8 +559,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->q_ready));
     };
-    int4 w_cur = items[item_at(0)];
-    int4 w_next = (item_at(1) < n_items) ? items[item_at(1)] : w_cur;
+    int4 w_cur = load_item(items + item_at(0));
+    int4 w_next = (item_at(1) < n_items) ? load_item(items + item_at(1)) : w_cur;
     // (dependents start only from here: what they and their dependents rely on is that everything ahead of this kernel has finished)
     if (a.early) { pdl_wait(); pdl_trigger(); }
     q_copy_issue(unpack_item(w_cur));
@@ -561,7 +574,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       const int i_blk = rg / a.rep;                  // block position of the row
       const bool has_next = item_at(int(n) + 1) < n_items;
       int4 w_next2 = w_next;                         // the descriptor is fetched two items ahead
-      if (item_at(int(n) + 2) < n_items) w_next2 = items[item_at(int(n) + 2)];
+      if (item_at(int(n) + 2) < n_items) w_next2 = load_item(items + item_at(int(n) + 2));
       if (has_next) prefetch_q(unpack_item(w_next));
       float m_ref = NEG, l_sum = 0.f;
       // a warp all of whose 32 rows are padding (fewer than 128 query rows share the KV head) only keeps the

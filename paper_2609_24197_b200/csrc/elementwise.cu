@@ -263,12 +263,13 @@ __global__ void qk_norm_rope_kernel(const float* __restrict__ qkv, const float* 
 // element is that of the kernel above.
 // TAIL: the QKV projection in front left the K-slices of its last wave's tiles unsummed; they are added up here, in slice order, on the
 // way (a head's columns lie in one 256-wide weight tile).  early: the context lengths are not written by anything that may still run,
-// so the sines and cosines are ready before the wait.
+// so the sines and cosines are ready before the wait.  (qkv and ctx_lens are no __restrict__ pointers: read-only loads may be moved up past a
+// wait that stands under a condition.)
 constexpr int ROPE_HB = 5;
 template <bool TAIL>
 __global__ void __launch_bounds__(256)
-qk_norm_rope_row_kernel(const float* __restrict__ qkv, const float* __restrict__ qw, const float* __restrict__ kw,
-                        const float* __restrict__ inv_freq, const int32_t* __restrict__ ctx_lens,
+qk_norm_rope_row_kernel(const float* qkv, const float* __restrict__ qw, const float* __restrict__ kw,
+                        const float* __restrict__ inv_freq, const int32_t* ctx_lens,
                         __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ kb, __nv_bfloat16* __restrict__ vb,
                         int k, int Hq, int Hkv, int dh, float eps, int qk_norm, int early, GemmTail tail) {
   if (!early) { pdl_wait(); pdl_trigger(); }

@@ -171,10 +171,14 @@ def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
     q, kb, vb = _rand((B * k, Hq, dh), 4, bf), _rand((B * k, Hkv, dh), 5, bf), _rand((B * k, Hkv, dh), 6, bf)
     o = torch.full((B * k, Hq * dh), float("nan"), dtype=torch.float16, device="cuda")
     ws = torch.empty(hs.hspec_attention_workspace_bytes(B, k, Hq, Hkv, dh, max(ctx), window, chunk), dtype=torch.uint8, device="cuda")
-    hs.hspec_op_attention(q, kb, vb, kp, vp, table.cuda(), torch.tensor(ctx, dtype=torch.int32).cuda(), max(ctx), o, B, k, Hq, Hkv, dh, 16,
-                          window, chunk, ws)
+    table, lens = table.cuda(), torch.tensor(ctx, dtype=torch.int32).cuda()
+    for _ in range(3):            # a work list read before it is written is an empty one here, and leaves NaN
+        ws.zero_()
+        o.fill_(float("nan"))
+        hs.hspec_op_attention(q, kb, vb, kp, vp, table, lens, max(ctx), o, B, k, Hq, Hkv, dh, 16, window, chunk, ws)
+        assert not bool(o.isnan().any())
     for b, c in enumerate(ctx):
-        rows = table[b, :pages[b]].long().cuda()
+        rows = table[b, :pages[b]].long()
         K = torch.cat([kp[rows].reshape(-1, Hkv, dh)[:c], kb[b * k:(b + 1) * k]]).double()
         V = torch.cat([vp[rows].reshape(-1, Hkv, dh)[:c], vb[b * k:(b + 1) * k]]).double()
         pos_q, pos_k = torch.arange(c, c + k, device="cuda"), torch.arange(c + k, device="cuda")
