@@ -328,7 +328,7 @@ __device__ __forceinline__ void produce_operand(const AttnTcArgs& a, const CUten
 // DUP: how often every query row lies in the 128-row tile.  The softmax owns rows (TMEM lanes), so with 64 or fewer rows per KV head
 // half of its lanes or more had nothing to do while the others set the kernel's pace.  With DUP = 2 (at most 64 rows) or 4 (at
 // most 32) a row is there DUP times, and copy p takes the exponentials of the p-th part of the tile's keys only (its P is zero
-// elsewhere): an independent partial softmax, merged with the other copies' by shuffles when the item is read out.  A copy's
+// elsewhere), with the row's one reference maximum; the copies' sums meet by shuffles when the item is read out.  A copy's
 // lane is in the same warp, 32 / DUP lanes on, so all four lane quarters (= schedulers) get the same share.  Plan, kernel and merge,
 // DUP = 1 -> 2 / 4: 32 requests of 512..8192 tokens, 64 rows 124.3 -> 119.2 us; 61 requests, 2048-token window, 36 rows 132 -> 121;
 // 32 requests, the same window, 32 rows 78.8 -> 73.2.
@@ -645,7 +645,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
           mx4[2] = fmaxf(mx4[2], s[j + 2]); mx4[3] = fmaxf(mx4[3], s[j + 3]);
         }
         // both threads of the row then hold the same two values and take the same decision below
-        const float mx_own = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+        float mx_own = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+        // (and over the row's copies: with one reference for all of them the bf16 weights are those of a row that is there once)
+        if (DUP > 1) {
+#pragma unroll
+          for (int off = 16; off >= LR; off >>= 1) mx_own = fmaxf(mx_own, __shfl_xor_sync(0xffffffffu, mx_own, off));
+        }
         TCLK(2)
         bars->xmax[gt & 1][hf][r_local] = mx_own;
         __syncwarp();
@@ -723,17 +728,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       TCLK(6)
       const size_t slab = (size_t(b) * a.Hkv + kvh) * a.max_chunks + c;
       const bool whole = g.n_chunks == 1;            // the request's only chunk: normalise and finish here
-      // the row's copies meet: common reference, weights, row sum (copies past the visible keys carry weight 0)
-      float m_row = m_ref, w_copy = 1.f, l_all = l_row;
+      // the row's copies meet
+      float l_all = l_row;
       if (DUP > 1) {
-#pragma unroll
-        for (int off = 16; off >= LR; off >>= 1) m_row = fmaxf(m_row, __shfl_xor_sync(0xffffffffu, m_row, off));
-        w_copy = ex2_ftz(m_ref - m_row);
-        l_all = l_row * w_copy;
 #pragma unroll
         for (int off = 16; off >= LR; off >>= 1) l_all += __shfl_xor_sync(0xffffffffu, l_all, off);
       }
-      // 32 columns of the accumulator, weighted and summed over the copies: copy p is left with OC = 32 / DUP of them, the ones from
+      // 32 columns of the accumulator, summed over the copies: copy p is left with OC = 32 / DUP of them, the ones from
       // p * OC on (every round a lane hands half of its columns to its partner)
       constexpr int OC = 32 / DUP;
       auto read_o = [&](int j, float (&v)[OC]) {
@@ -742,7 +743,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
         tmem_wait_ld32(o);
         float f[32];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) f[e] = DUP == 1 ? __uint_as_float(o[e]) : __uint_as_float(o[e]) * w_copy;
+        for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(o[e]);
         if (DUP >= 2) {
           const bool up = (lane & 16) != 0;
 #pragma unroll
@@ -812,7 +813,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
       if (lane == 0) mbar_arrive(smem_u32(&bars->o_free));
       if (row_ok && hf == 0 && part == 0 && !whole) {
         float* ml = a.ws_ml + (slab * a.R + rg) * 2;
-        ml[0] = (m_row == NEG) ? -INFINITY : m_row;
+        ml[0] = (m_ref == NEG) ? -INFINITY : m_ref;
         ml[1] = l_all;
       }
       w_cur = w_next;
