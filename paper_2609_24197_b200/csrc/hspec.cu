@@ -651,7 +651,7 @@ int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* ou
     if (c.has_attn[l]) {
       EW("rmsnorm", Md * c.D * 6, rmsnorm_launch(X, fptr(lw.a_norm), U, M, c.D, c.rms_eps, st, h->d_status, bf, &tail));
       GemmTail qkv_tail{};
-      CUDA_TRY(h, gemm(lw.wqkv, "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv, qk_norm_rope_takes_tail(c.dh) ? &qkv_tail : nullptr));
+      CUDA_TRY(h, gemm(lw.wqkv, "gemm:wqkv", U, M, EPI_STORE_F32, BIG, d.d_qkv, qk_norm_rope_takes_tail(M, c.dh) ? &qkv_tail : nullptr));
       EW("qk_norm_rope", Md * d.d_qkv * 6,
          qk_norm_rope_launch(BIG, fptr(lw.q_norm), fptr(lw.k_norm), in->ctx_lens, Q, KB, VB, B, k, c.Hq,
                              c.Hkv, c.dh, c.rope_theta, c.rms_eps, c.qk_norm, st, true, &qkv_tail));

@@ -310,7 +310,7 @@ cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, f
 cudaError_t qk_norm_rope_launch(const float* qkv, const float* qw, const float* kw, const int32_t* ctx_lens, void* q,
                                 void* kb, void* vb, int B, int k, int Hq, int Hkv, int dh, float theta, float eps,
                                 int qk_norm, cudaStream_t stream, bool early = false, const GemmTail* tail = nullptr);
-bool qk_norm_rope_takes_tail(int dh);   // whether the launch can add up a tail that the projection in front left
+bool qk_norm_rope_takes_tail(int rows, int dh);   // whether the launch adds up a tail that the projection in front left
 cudaError_t swiglu_launch(const float* gu, void* h_16, int M, int F, cudaStream_t stream, uint32_t* status, bool bf16_out = false);
 cudaError_t copy_f32_launch(const float* src, float* dst, size_t n, cudaStream_t stream);
 

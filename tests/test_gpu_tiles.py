@@ -222,9 +222,9 @@ def test_small_state_scan_with_norm(hs, Di, P, N, G, dt_rank, B, k):
     drafter.close()
 
 
-# the QK norm behind the QKV projection adds that GEMM's K-sliced tail tiles: all tail, and a whole wave with a tail behind it, heads of a
-# quarter and of half a weight tile, a last weight tile that is only part full
-@pytest.mark.parametrize("dh,Hq,Hkv,B,k", [(64, 16, 4, 9, 32), (128, 8, 2, 9, 32), (128, 6, 1, 20, 13), (64, 14, 2, 141, 32)])
+# the QK norm behind the QKV projection adds that GEMM's K-sliced tail tiles up to 512 rows (here 260 to 512; 513 and a whole wave with a tail behind
+# it take the pass of their own): heads of a quarter and of half a weight tile, a last weight tile that is only part full
+@pytest.mark.parametrize("dh,Hq,Hkv,B,k", [(64, 16, 4, 9, 32), (128, 8, 2, 9, 32), (128, 6, 1, 20, 13), (128, 8, 2, 16, 32), (64, 14, 2, 27, 19), (64, 14, 2, 141, 32)])
 def test_qkv_tail_is_added_by_the_qk_norm(hs, dh, Hq, Hkv, B, k):
     import synth
     from harness import check_step, cuda_setup
