@@ -185,7 +185,8 @@ typedef struct {
 
 /* Validates the config, creates the handle (host memory only; no weights yet).  Sec. 3.3 / App. B.1. */
 int hspec_init(const hspec_config* cfg, hspec_handle** out);
-/* Device scratch bytes a step of up to (max_batch, max_k, max_pages_per_req) needs. */
+/* Device scratch bytes a step of up to (max_batch, max_k, max_pages_per_req) needs, whatever its own batch, block and
+ * context bound. */
 size_t hspec_workspace_bytes(const hspec_config* cfg);
 /* Copies n named device tensors into library-owned device memory (may be called several times; synchronises the
  * device).  Shapes are checked against the config. */
@@ -194,7 +195,7 @@ int hspec_load_weights(hspec_handle* h, const hspec_tensor* tensors, int32_t n);
  * device builds a small RoPE table (one allocation, one copy) and sets kernel attributes; every later call only
  * launches kernels on the stream, so a warmed-up step may be captured in a CUDA graph and replayed: the replay reads
  * the current contents of the same input buffers.  The workspace must hold hspec_workspace_bytes(cfg) bytes, which
- * covers every (B, k) up to (max_batch, max_k). */
+ * covers every (B, k) up to (max_batch, max_k) and every page_table_stride and max_ctx. */
 int hspec_draft_block(hspec_handle* h, const hspec_step* in, const hspec_out* out);
 /* Frees the handle and its weight copies.  Pools and the workspace stay the caller's. */
 int hspec_destroy(hspec_handle* h);
@@ -326,6 +327,7 @@ int hspec_op_attention(const void* q, const void* kb, const void* vb, const void
                        int32_t max_ctx, void* o, int32_t B, int32_t k, int32_t Hq, int32_t Hkv, int32_t dh,
                        int32_t page_size, int32_t window, int32_t chunk_tokens, void* workspace,
                        size_t workspace_bytes, void* stream);
+/* Scratch for one batch shape; with chunk_tokens <= 0 it covers every bound up to max_ctx. */
 size_t hspec_attention_workspace_bytes(int32_t B, int32_t k, int32_t Hq, int32_t Hkv, int32_t dh, int32_t max_ctx,
                                        int32_t window, int32_t chunk_tokens);
 /* Contiguous copy of one request's prefix out of a paged pool: dst bf16 [ctx_len, Hkv, dh] (pure data movement,

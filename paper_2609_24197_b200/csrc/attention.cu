@@ -388,20 +388,47 @@ int rows_per_cta(int R) { int rt = ((R + 15) / 16) * 16; return rt > 128 ? 128 :
 
 }  // namespace
 
-int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms) {
-  // with a window the visible range starts on a page boundary, up to 15 tokens before the window itself: size the
-  // chunks for window + 15 tokens, or a request's last few tokens become a chunk (and a merge) of their own
-  int lmax = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
-  if (lmax < 1) lmax = 1;
+namespace {
+
+// A visible range of l tokens is cut into chunks of l / pieces tokens, rounded up to `step` and kept within [least, most].
+struct ChunkRule {
+  int pieces, least, most, step;
+  int chunk(int l) const {
+    const int c = ((l + pieces - 1) / pieces + step - 1) / step * step;
+    return c < least ? least : c > most ? most : c;
+  }
+  // The most chunks any range of up to l tokens is cut into: a chunk below `most` makes at most `pieces` of them, and none is below `least`.
+  int max_chunks(int l) const { return std::max(std::min(pieces, (l + least - 1) / least), (l + most - 1) / most); }
+};
+
+ChunkRule chunk_rule(int B, int Hkv, int dh, int num_sms) {
   if (dh != 128) {
     // The mma.sync kernel walks its 64-key tiles one after the other, about 4 us each when few rows share a KV head, so a context is cut
     // down to single tiles as long as that gives no more than four CTAs per SM (test-sized drafter, us per step, 256-token chunks / two /
     // four / eight CTAs per SM: one request of 256 tokens 84.5 / 76.6 / 76.6 / 76.6, 64 of 1000..4096 with 32 positions 264 / 264 / 221 / 224,
     // 30 of 500..4096 with a 2048-token window 162 / 136 / 130 / 137).
-    const int n = std::min(32, (4 * num_sms + B * Hkv - 1) / (B * Hkv));
-    return std::min(8192, std::max(KT, (lmax + n * KT - 1) / (n * KT) * KT));
+    return {std::min(32, (4 * num_sms + B * Hkv - 1) / (B * Hkv)), KT, 8192, KT};
   }
-  if (window > 0 && lmax == window + 15) {
+  // long chunks mean fewer partials to write and merge and fewer item boundaries; past 8192 tokens the work list gets
+  // too uneven.  Measured at 8, 16, 32 and 64 requests x 8 KV heads with contexts up to 16k and 32k: a cap of 8192 is
+  // 3-11 % faster than 4096 wherever it binds and never slower; 16384 loses 5-9 %.
+  static const int cap_env = [] { const char* e = getenv("HSPEC_ATTN_CHUNK_CAP"); return e ? atoi(e) : 0; }();   // measurements only
+  return {std::min(32, (2 * num_sms + B * Hkv - 1) / (B * Hkv)), 256, cap_env >= 256 ? cap_env : 8192, 128};
+}
+
+// Tokens a request of up to max_ctx can see.  With a window the visible range starts on a page boundary, up to 15 tokens before the
+// window itself: chunks are sized for window + 15 tokens, or a request's last few tokens become a chunk (and a merge) of their own.
+int visible_tokens(int max_ctx, int window) {
+  const int l = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
+  return l < 1 ? 1 : l;
+}
+
+}  // namespace
+
+int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms) {
+  const int lmax = visible_tokens(max_ctx, window);
+  const ChunkRule rule = chunk_rule(B, Hkv, dh, num_sms);
+  if (dh == 128 && window > 0 && lmax == window + 15) {
     // Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
     // Cost of a round in tiles: the chunk's own, three for an item's set-up and read-out, one more for a partial and its merge.
     // 32 requests x 8 KV heads, window 2048 (256 items of 17 tiles on 148 SMs): one chunk 65.7 us, two 73.1, four 80.
@@ -417,33 +444,30 @@ int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms
     }
     if (best_chunk <= 8192) return best_chunk < 256 ? 256 : best_chunk;
   }
-  int nsplit = (2 * num_sms + B * Hkv - 1) / (B * Hkv);
-  if (nsplit < 1) nsplit = 1;
-  if (nsplit > 32) nsplit = 32;
-  int chunk = (lmax + nsplit - 1) / nsplit;
-  chunk = ((chunk + 127) / 128) * 128;
-  if (chunk < 256) chunk = 256;
-  // long chunks mean fewer partials to write and merge and fewer item boundaries; past 8192 tokens the work list gets
-  // too uneven.  Measured at 8, 16, 32 and 64 requests x 8 KV heads with contexts up to 16k and 32k: a cap of 8192 is
-  // 3-11 % faster than 4096 wherever it binds and never slower; 16384 loses 5-9 %.
-  static const int cap_env = [] { const char* e = getenv("HSPEC_ATTN_CHUNK_CAP"); return e ? atoi(e) : 0; }();   // measurements only
-  const int cap = cap_env >= 256 ? cap_env : 8192;
-  if (chunk > cap) chunk = cap;
-  return chunk;
+  return rule.chunk(lmax);
 }
 
-int attn_max_chunks(int max_ctx, int window, int chunk) {
-  // with a window the visible range may start up to 15 tokens earlier (page-aligned chunk grid of the tcgen05 path)
-  int lmax = (window > 0 && window + 15 < max_ctx) ? window + 15 : max_ctx;
-  int n = (lmax + chunk - 1) / chunk;
-  return n < 1 ? 1 : n;
-}
+int attn_max_chunks(int max_ctx, int window, int chunk) { return (visible_tokens(max_ctx, window) + chunk - 1) / chunk; }
 
-size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens) {
+namespace {
+size_t attn_bytes(int B, int k, int Hq, int Hkv, int dh, int max_chunks) {
   const int R = k * (Hq / Hkv);
-  const size_t slabs = size_t(B) * Hkv * attn_max_chunks(max_ctx, window, chunk_tokens);
+  const size_t slabs = size_t(B) * Hkv * max_chunks;
   const size_t row_tiles = (size_t(R) + 127) / 128;
   return slabs * R * (dh + 2) * sizeof(float) + 256 + slabs * row_tiles * 16 + 64;   // partials + the tcgen05 path's work list
+}
+}  // namespace
+
+size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens) {
+  return attn_bytes(B, k, Hq, Hkv, dh, attn_max_chunks(max_ctx, window, chunk_tokens));
+}
+
+// A call with a smaller bound on its contexts can be cut into more chunks than one with the largest: below the window the rule is
+// another one, and a range of pieces x least tokens makes more chunks than a longer one whose chunks have grown.
+size_t attn_workspace_bytes_any_ctx(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int num_sms) {
+  const int chunk = attn_pick_chunk(B, Hkv, dh, max_ctx, window, num_sms);
+  const int n = std::max(attn_max_chunks(max_ctx, window, chunk), chunk_rule(B, Hkv, dh, num_sms).max_chunks(visible_tokens(max_ctx, window)));
+  return attn_bytes(B, k, Hq, Hkv, dh, n);
 }
 
 cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* trk, std::string* err) {

@@ -62,7 +62,8 @@ struct Plan {
 
 size_t splitk_need(int M, int n_out) { return gemm2_preferred(M, n_out) ? gemm2_tail_bytes() : 0; }
 
-Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
+// any_ctx: room for the attention of every bound up to max_ctx and not only of this one.
+Plan make_plan(const hspec_config& c, int B, int k, int max_ctx, bool any_ctx = false) {
   const Dims d = dims_of(c);
   const size_t M = size_t(B) * k;
   Plan p{};
@@ -85,7 +86,8 @@ Plan make_plan(const hspec_config& c, int B, int k, int max_ctx) {
   p.VB = take(M * size_t(c.Hkv) * c.dh * 2);
   p.max_ctx = max_ctx;
   p.attn_chunk = attn_pick_chunk(B, c.Hkv, c.dh, max_ctx, c.window, kNumSMs);
-  p.att_bytes = attn_workspace_bytes(B, k, c.Hq, c.Hkv, c.dh, max_ctx, c.window, p.attn_chunk);
+  p.att_bytes = any_ctx ? attn_workspace_bytes_any_ctx(B, k, c.Hq, c.Hkv, c.dh, max_ctx, c.window, kNumSMs)
+                        : attn_workspace_bytes(B, k, c.Hq, c.Hkv, c.dh, max_ctx, c.window, p.attn_chunk);
   p.ATT = take(p.att_bytes);
   size_t sk = 0;
   auto upd = [&](size_t v) { if (v > sk) sk = v; };
@@ -390,14 +392,14 @@ int hspec_init(const hspec_config* cfg, hspec_handle** out) {
 
 size_t hspec_workspace_bytes(const hspec_config* cfg) {
   if (!cfg || check_config(*cfg)) return 0;
-  // The layout of a step depends on its own (B, k): how the contexts are cut into chunks and how many K-slices a GEMM
-  // uses change at thresholds, so a smaller step can need MORE of some scratch buffer than the largest one.  The
-  // size handed out covers every (B, k) the handle accepts.
+  // The layout of a step depends on its own (B, k) and context bound: how the contexts are cut into chunks and how many
+  // K-slices a GEMM uses change at thresholds, so a smaller step can need MORE of some scratch buffer than the largest
+  // one.  The size handed out covers every (B, k, bound) the handle accepts.
   const int max_ctx = cfg->max_pages_per_req * cfg->page_size;
   size_t total = 0;
   for (int B = 1; B <= cfg->max_batch; ++B)
     for (int k = 1; k <= cfg->max_k; ++k) {
-      const size_t t = make_plan(*cfg, B, k, max_ctx).total;
+      const size_t t = make_plan(*cfg, B, k, max_ctx, true).total;
       if (t > total) total = t;
     }
   return total;
@@ -936,6 +938,7 @@ static int resolve_chunk(int B, int Hkv, int dh, int max_ctx, int window, int ch
 
 size_t hspec_attention_workspace_bytes(int32_t B, int32_t k, int32_t Hq, int32_t Hkv, int32_t dh, int32_t max_ctx,
                                        int32_t window, int32_t chunk_tokens) {
+  if (chunk_tokens <= 0) return attn_workspace_bytes_any_ctx(B, k, Hq, Hkv, dh, max_ctx, window, kNumSMs);
   return attn_workspace_bytes(B, k, Hq, Hkv, dh, max_ctx, window, resolve_chunk(B, Hkv, dh, max_ctx, window, chunk_tokens));
 }
 

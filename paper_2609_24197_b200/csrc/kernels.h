@@ -259,6 +259,8 @@ struct AttnPlan {
 };
 int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms);
 size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens);
+// The most any call with a bound of at most max_ctx and a chunk picked by the library needs.
+size_t attn_workspace_bytes_any_ctx(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int num_sms);
 cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool attention_tc_supported(const AttnCall& c);
 bool attention_plan(const AttnCall& c, AttnPlan* plan);   // false: this call needs no work list (mma.sync path)

@@ -52,6 +52,21 @@ def test_workspace_grows_with_batch(lib):
     assert 0 < small < large
 
 
+# heads of 128 and of 64, with and without a window, batches that are cut into many chunks, a few and one, bounds on both sides of the
+# window and of the longest chunk; one token per page, so that a page count is a bound
+@pytest.mark.parametrize("name,window", [("serving_8b", 0), ("serving_8b", 512), ("serving_8b", 2048), ("tiny", 0), ("tiny", 512), ("tiny", 2048)])
+@pytest.mark.parametrize("B,k", [(1, 16), (4, 8), (32, 8), (61, 9)])
+def test_workspace_covers_every_smaller_context_bound(lib, name, window, B, k):
+    import synth
+    cfg = dict(synth.get_config(name), window=window, page_size=1)
+    bounds = sorted({b for c in (64, 128, 256, 512, 1024, 1984, 2048, 2112, 4096, 8192, 16384, 32768)
+                     for b in (c - 1, c, c + 1, c + 15, c + 16)} | {2000, 3000, 5000, 12345, 40000})
+    sizes = [hs.hspec_workspace_bytes(hs.make_config(cfg, B, k, b)) for b in bounds]
+    assert sizes == sorted(sizes)
+    att = [hs.hspec_attention_workspace_bytes(B, k, cfg["Hq"], cfg["Hkv"], cfg["dh"], b, window) for b in range(1, 4200, 3)]
+    assert att == sorted(att)
+
+
 def test_no_cpu_path(lib):
     import torch
     if torch.cuda.is_available():

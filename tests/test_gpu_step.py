@@ -267,3 +267,21 @@ def test_smaller_batch_than_planned_fits_the_workspace():
     r = check_step(cfg, drafter, w, batch, 16, requests=[0, 72], what="B=73 of 128")
     assert r["ids_compared"] > 0
     drafter.close()
+
+
+# a handle made for the longest context a server takes, drafting for a batch of short ones: a window (below it another chunk rule holds), heads of
+# 64 without one; the bound given by max_ctx, and by the page table's width alone
+@pytest.mark.parametrize("over,top", [(dict(Hq=8, Hkv=8, window=2048, B=32), 32768), (dict(dh=64, Hq=4, Hkv=2, B=4), 2112)])
+def test_smaller_context_bound_than_planned_fits_the_workspace(over, top):
+    import paper_2609_24197_b200 as hs
+    cfg = synth.derived(dict(MID, k=8, **over))
+    w = synth.make_weights(cfg, device="cuda")
+    batch = synth.make_request_batch(cfg, ctx_lens=[2000 - 37 * b for b in range(cfg["B"])], device="cuda")
+    drafter = hs.Drafter(cfg, w, cfg["B"], 8, top)
+    check_step(cfg, drafter, w, batch, 8, requests=[0, cfg["B"] - 1], what=f"bound 2000 of {top}")
+    own = drafter.draft(batch, 8, max_ctx=2000)[0]
+    assert batch["page_table"].shape[1] * 16 < top
+    by_table = drafter.draft(batch, 8)[0]
+    torch.cuda.synchronize()
+    assert torch.equal(own, by_table)
+    drafter.close()
