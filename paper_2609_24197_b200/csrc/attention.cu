@@ -425,20 +425,24 @@ int visible_tokens(int max_ctx, int window) {
 
 }  // namespace
 
-int attn_pick_chunk(int B, int Hkv, int dh, int max_ctx, int window, int num_sms) {
+int attn_pick_chunk(int B, int Hkv, int dh, int rows, int max_ctx, int window, int num_sms) {
   const int lmax = visible_tokens(max_ctx, window);
   const ChunkRule rule = chunk_rule(B, Hkv, dh, num_sms);
   if (dh == 128 && window > 0 && lmax == window + 15) {
     // Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
     // Cost of a round in tiles: the chunk's own, three for an item's set-up and read-out, one more for a partial and its merge.
-    // 32 requests x 8 KV heads, window 2048 (256 items of 17 tiles on 148 SMs): one chunk 65.7 us, two 73.1, four 80.
+    // 32 requests x 8 KV heads, window 2048 (256 items of 17 tiles on 148 SMs): one chunk 65.7 us, two 73.1, four 80.  Over windows of 512,
+    // 2048 and 4096 tokens, 1 to 128 requests and 32 to 256 rows per KV head, the chunk this picks was the best of nine or within 13 %
+    // of it (calls of less than 40 us: within 20 %).
+    // More than 128 rows per KV head are several items each (256 rows, window 2048: 24 requests in one chunk 113.6 us, in two 144.4).
+    const long per_piece = long(B) * Hkv * ((rows + 127) / 128);
     long best = 0;
     int best_chunk = 0;
     for (int n = 1; n <= 32; ++n) {
       const int chunk = (lmax + n * 128 - 1) / (n * 128) * 128;
       if (chunk < 256 && n > 1) break;
       const int pieces = (lmax + chunk - 1) / chunk;
-      const long rounds = (long(B) * Hkv * pieces + num_sms - 1) / num_sms;
+      const long rounds = (per_piece * pieces + num_sms - 1) / num_sms;
       const long cost = rounds * (chunk / 128 + (pieces > 1 ? 4 : 3));
       if (best_chunk == 0 || cost < best) { best = cost; best_chunk = chunk; }
     }
@@ -465,7 +469,7 @@ size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, 
 // A call with a smaller bound on its contexts can be cut into more chunks than one with the largest: below the window the rule is
 // another one, and a range of pieces x least tokens makes more chunks than a longer one whose chunks have grown.
 size_t attn_workspace_bytes_any_ctx(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int num_sms) {
-  const int chunk = attn_pick_chunk(B, Hkv, dh, max_ctx, window, num_sms);
+  const int chunk = attn_pick_chunk(B, Hkv, dh, k * (Hq / Hkv), max_ctx, window, num_sms);
   const int n = std::max(attn_max_chunks(max_ctx, window, chunk), chunk_rule(B, Hkv, dh, num_sms).max_chunks(visible_tokens(max_ctx, window)));
   return attn_bytes(B, k, Hq, Hkv, dh, n);
 }

@@ -67,6 +67,16 @@ def test_workspace_covers_every_smaller_context_bound(lib, name, window, B, k):
     assert att == sorted(att)
 
 
+# under a window a call is cut so that its work items fill the SMs; 256 query rows per KV head are two items where 128 are one, so half the
+# requests with twice the rows are cut alike (the choice is made on the host, in a function that is called by its C++ name here)
+@pytest.mark.parametrize("window", [512, 2048, 4096])
+@pytest.mark.parametrize("B", [1, 2, 4, 8, 12, 24, 37])
+def test_chunks_under_a_window_count_row_tiles(lib, B, window):
+    chunk = lambda b, rows: lib._ZN5hspec15attn_pick_chunkEiiiiiii(b, 8, 128, rows, 20000, window, 148)
+    assert chunk(B, 256) == chunk(2 * B, 128) == chunk(2 * B, 7)
+    assert chunk(B, 129) == chunk(B, 256)
+
+
 def test_no_cpu_path(lib):
     import torch
     if torch.cuda.is_available():
