@@ -170,6 +170,14 @@ __device__ __forceinline__ void warp_argmax16(float (&v)[16], int (&idx)[16], in
   row = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
+// The value and index a lane brings into an arg-max.  A NaN is never chosen, and neither is a row past the matrix (on = false): both
+// come as (-inf, no index), which loses against every number, -inf included.
+__device__ __forceinline__ void argmax_candidate(float x, int n, bool on, float& v, int& idx) {
+  on = on && x == x;
+  v = on ? x : -INFINITY;
+  idx = on ? n : 0x7fffffff;
+}
+
 // ------------------------------------------------------------------ TMA (no multicast anywhere)
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
@@ -365,7 +373,7 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // (value, index) as one unsigned number: the larger key has the larger value, at equal values the lower index.  Any value beats the zero
-// key, NaN never gets this far.
+// key.  Not for NaN: a NaN is no candidate of an arg-max (argmax_candidate).
 __device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
   uint32_t u = __float_as_uint(v + 0.f);                    // (-0 compares equal to +0)
   u = (u & 0x80000000u) ? ~u : u | 0x80000000u;

@@ -234,9 +234,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const int m = m0 + c0 + j;
-          v[j] = n_ok ? __uint_as_float(r[j]) + add[j] : -INFINITY;
-          vi[j] = n;
-          if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = v[j];
+          const float x = __uint_as_float(r[j]) + add[j];
+          if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
+          argmax_candidate(x, n, n_ok, v[j], vi[j]);
         }
         int row = 0;
         warp_argmax16(v, vi, lane, row);

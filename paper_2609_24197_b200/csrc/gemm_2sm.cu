@@ -327,9 +327,9 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int m = m0 + c0 + j;
-            v[j] = n_ok ? __uint_as_float(r[j]) : -INFINITY;
-            vi[j] = n;
-            if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = v[j];
+            const float x = __uint_as_float(r[j]);
+            if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
+            argmax_candidate(x, n, n_ok, v[j], vi[j]);
           }
           // (The network costs the LM head 4 % - 2.34 -> 2.24 ms per step without it - mostly as clock under the power cap.
           // One redux.sync maximum + ballot per column instead of the shuffle rounds: 2.56 ms.)

@@ -64,12 +64,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); }
 
-// (value, index) as one unsigned key: larger value first, then the lower index (-0 counts as +0)
-__device__ __forceinline__ unsigned long long order_key(float v, uint32_t idx) {
-  const uint32_t u = __float_as_uint(v + 0.0f);
-  const uint32_t o = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return (static_cast<unsigned long long>(o) << 32) | (0xffffffffu - idx);
-}
 __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int off) {
   const uint32_t lo = __shfl_xor_sync(0xffffffffu, uint32_t(v), off), hi = __shfl_xor_sync(0xffffffffu, uint32_t(v >> 32), off);
   return (static_cast<unsigned long long>(hi) << 32) | lo;
@@ -250,7 +244,7 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
             const float v = __uint_as_float(r[j]) + add[u % AQ * 8 + j];
             if (n_ok && c0 + j < a.B) {
               if (a.write_logits) __stcs(dst, v);
-              if (v > best[u * 8 + j]) {                         // ascending tiles, strict: the lowest index wins ties
+              if (v > best[u * 8 + j]) {                         // ascending tiles, strict: the lowest index wins ties, NaN never does
                 best[u * 8 + j] = v;
                 uint32_t& o = ord[(u * 8 + j) >> 2];             // byte j % 4 becomes t
                 o = __byte_perm(o, uint32_t(t), j % 4 == 0 ? 0x3214 : j % 4 == 1 ? 0x3240 : j % 4 == 2 ? 0x3410 : 0x4210);
@@ -282,7 +276,7 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
         for (int j = 0; j < 8; ++j) {
           const uint32_t o = (ord[(u * 8 + j) >> 2] >> ((j & 3) * 8)) & 0xffu;
           const int n = (cta + int(o) * grid) * TILE_W + row_in_tile;
-          v[j] = n < a.Vd ? order_key(best[u * 8 + j], uint32_t(n)) : 0ull;
+          v[j] = n < a.Vd ? argmax_key(best[u * 8 + j], n) : 0ull;
         }
         int col;
         const unsigned long long m = max_over_lanes8(v, lane, col);

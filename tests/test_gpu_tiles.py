@@ -263,3 +263,64 @@ def test_lm_head_argmax_ties(hs, M, V, alloc):
         best = z.max(1, keepdim=True).values
         first = torch.where(z == best, torch.arange(V, device="cuda"), V).min(1).values.int()     # exact: the kernel's own logits
         assert torch.equal(ids, first)
+
+
+# NaN logits are never chosen: one NaN at the first and the last row of a tile and of the matrix, next to and away from the maximum, a row
+# that is all NaN (no id), +inf (chosen), -inf; one-CTA kernel and pair kernel, a last tile that is part full
+@pytest.mark.parametrize("M", [5, 40, 200])
+@pytest.mark.parametrize("V", [130, 300, 20000])
+def test_lm_head_argmax_leaves_nan_out(hs, M, V):
+    K = 64
+    x, W = _rand((M, K), 1, torch.float16), _rand((V, K), 2, torch.float16)
+    x[:, 0] = 1.0
+    x[1, 0] = -1.0
+    x[2] = float("nan")
+    nan, inf = float("nan"), float("inf")
+    for v in {0, 31, 32, 127, 128, V // 2, V - 1}:
+        W[v, 1] = nan
+    ids = torch.empty(M, dtype=torch.int32, device="cuda")
+    logits = torch.empty((M, V), device="cuda")
+    ws = torch.empty(((V + 127) // 128) * M * 8 + 1024, dtype=torch.uint8, device="cuda")
+    for big in (None, 5, V - 2):                              # (+inf in every row but row 1, where it is -inf)
+        if big is not None:
+            W[big, 0] = inf
+        ids.fill_(-1)
+        hs.hspec_op_lm_head_argmax(x, W, ids, logits, ws)
+        z = logits.nan_to_num(nan=-inf, posinf=inf, neginf=-inf)
+        first = torch.where((z == z.max(1, keepdim=True).values) & ~logits.isnan(), torch.arange(V, device="cuda"), 0x7fffffff).min(1).values.int()
+        assert bool(logits[2].isnan().all()) and bool((logits[0].isnan().sum() >= 6).item())
+        assert torch.equal(ids, first) and int(ids[2]) == 0x7fffffff
+        hs.hspec_op_lm_head_argmax_noalloc(x, W, ids.fill_(-1), logits=logits)
+        assert torch.equal(ids, first)
+
+
+# the same for the causal-correction head, in one launch (up to 128 requests) and position by position, with and without a pruned vocabulary
+@pytest.mark.parametrize("B", [3, 100, 131])
+@pytest.mark.parametrize("pruned", [False, True])
+def test_markov_head_leaves_nan_out(hs, B, pruned):
+    k, Vd, r, V = 4, 19300, 64, 25000
+    g = torch.Generator().manual_seed(B)
+    logits = (torch.randint(-256, 257, (B, k, Vd), generator=g).float() / 64).cuda()
+    nan, inf = float("nan"), float("inf")
+    logits[:, :, [0, 31, 32, 128, Vd // 2, Vd - 1]] = nan
+    logits[0, 1] = nan                                        # row 0, and the next position goes on from it
+    logits[1, 0] = -inf
+    logits[1, 2, 700] = inf
+    logits[2, 3, 500] = -inf
+    W_in = (torch.randint(-8, 9, (V, r), generator=g).float() / 16).half().cuda()
+    W_out = (torch.randint(-8, 9, (Vd, r), generator=g).float() / 16).half().cuda()
+    id_map = torch.sort(torch.randperm(V, generator=g)[:Vd])[0].int().cuda() if pruned else None
+    last = torch.randint(0, V, (B,), generator=g, dtype=torch.int32).cuda()
+    ids = torch.full((B * k,), -1, dtype=torch.int32, device="cuda")
+    out = logits.clone().view(B * k, Vd)
+    ws = torch.empty(hs.hspec_markov_workspace_bytes(B, Vd, r), dtype=torch.uint8, device="cuda")
+    hs.hspec_op_markov_head(out, W_in, W_out, last, id_map, ids, B, k, True, ws)
+    prev = last.long()
+    for i in range(k):                                        # (exact in fp32, as in the test above)
+        row = logits[:, i].double() + W_in[prev].double() @ W_out.double().t()
+        assert torch.equal(out.view(B, k, Vd)[:, i].nan_to_num(nan=777.0), row.float().nan_to_num(nan=777.0))
+        row = row.nan_to_num(nan=-inf, posinf=inf, neginf=-inf)
+        best = torch.where(row == row.max(1, keepdim=True).values, torch.arange(Vd, device="cuda"), Vd).min(1).values
+        prev = id_map[best].long() if pruned else best
+        assert torch.equal(ids.view(B, k)[:, i].long(), prev), i
+    assert hs.hspec_op_device_status()["rc"] == 0
