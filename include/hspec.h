@@ -283,7 +283,8 @@ int hspec_op_token_probs(const float* logits, int64_t ld, const int32_t* ids, fl
  *   ids      device int32 [B*k] out: chosen token ids
  *   workspace >= hspec_markov_workspace_bytes(B, Vd, r), 256-byte aligned.
  * Up to 128 requests all positions run in one cooperative launch on `stream` (behind a memset of the workspace's head); above
- * that, 2k + 1 launches (one rank-r product with arg-max per position). */
+ * that, and where a cooperative launch of one block per SM is refused (a context that owns part of the SMs), 2k + 1
+ * launches (one rank-r product with arg-max per position). */
 int hspec_op_markov_head(float* logits, int64_t ld, const void* W_in, const void* W_out, int32_t w_dtype, const int32_t* last_token,
                          const int32_t* id_map, int32_t* ids, int32_t B, int32_t k, int32_t Vd, int32_t r, int32_t write_logits,
                          void* workspace, size_t workspace_bytes, void* stream);

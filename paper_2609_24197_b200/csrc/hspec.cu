@@ -196,6 +196,11 @@ void Tracker::end() {
   ++used;
 }
 
+void Tracker::drop_last() {
+  --launches;
+  if (profiling) --used;
+}
+
 void Tracker::destroy() {
   for (Entry& e : entries) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
   entries.clear();

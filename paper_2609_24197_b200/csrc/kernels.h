@@ -59,6 +59,7 @@ struct Tracker {
   void begin_step(cudaStream_t st) { used = 0; stream = st; }
   void begin(const char* name, double flops = 0, double bytes = 0, double io_bytes = 0);   // call right before a launch
   void end();                                                         // call right after it
+  void drop_last();                                                   // the launch was refused: it did not happen
   void destroy();
 };
 inline void trk_begin(Tracker* t, const char* name, double flops = 0, double bytes = 0, double io_bytes = 0) {
@@ -229,6 +230,8 @@ size_t markov_workspace_bytes(int B, int Vd, int r);
 cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool markov_chain_supported(int B, int Vd, int r);      // all positions in one launch (markov_chain.cu)
 size_t markov_chain_bytes(int B);
+// Needs one CTA on every SM at once: cudaErrorCooperativeLaunchTooLarge or cudaErrorNotSupported where that cannot be had (a context that owns
+// part of the SMs; HSPEC_NO_COOPERATIVE=1 in the environment has the same effect), with nothing enqueued but the workspace's memset.
 cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk);
 
 // ---- attention (attention.cu)

@@ -22,6 +22,8 @@
 #include "common.cuh"
 #include "kernels.h"
 
+#include <cstdlib>
+
 namespace hspec {
 
 namespace {
@@ -361,24 +363,35 @@ cudaError_t chain_launch_n(const CUtensorMap* tm, const ChainArgs& a, int grid, 
 
 bool g_chain_dev[MAX_DEVICES] = {};
 
+// Shared memory and SMs of the current device, looked up once.  (The SM count is the context's where a limit is set from outside.)
+cudaError_t chain_device(int* dev) {
+  const cudaError_t e = once_per_device(g_chain_dev, [](int d) {
+    cudaError_t e2 = cudaDeviceGetAttribute(&g_chain_smem[d], cudaDevAttrMaxSharedMemoryPerBlockOptin, d);
+    if (e2 == cudaSuccess) e2 = cudaDeviceGetAttribute(&g_chain_sms[d], cudaDevAttrMultiProcessorCount, d);
+    return e2;
+  });
+  *dev = current_device();
+  return e == cudaSuccess && *dev < 0 ? cudaErrorInvalidDevice : e;
+}
+
 }  // namespace
 
 size_t markov_chain_bytes(int B) { return size_t(3) * B * 8 + 16; }
 
-// Up to 128 requests whose factor rows leave room for at least four stages of W_out (rank 256 at 128 requests does).
+// Up to 128 requests whose factor rows leave room for at least four stages of W_out (rank 256 at 128 requests does), up to 2^21 vocabulary
+// rows, and no more tiles per CTA than their ordinals' byte counts.
 bool markov_chain_supported(int B, int Vd, int r) {
   const size_t x = size_t((r + TILE_K - 1) / TILE_K) * ((B + 15) / 16 * 16) * 128;
-  return B <= MAX_B && x <= 128 * 1024 && Vd <= (1 << 21);         // (at 128 SMs or more: a tile's ordinal within its CTA fits a byte)
+  int dev = -1;
+  return B <= MAX_B && x <= 128 * 1024 && Vd <= (1 << 21) && chain_device(&dev) == cudaSuccess && (Vd + TILE_W - 1) / TILE_W <= 255 * g_chain_sms[dev];
 }
 
 cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk) {
-  const cudaError_t e0 = once_per_device(g_chain_dev, [](int dev) {
-    cudaError_t e = cudaDeviceGetAttribute(&g_chain_smem[dev], cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_chain_sms[dev], cudaDevAttrMultiProcessorCount, dev);
-    return e;
-  });
+  static const bool refuse = [] { const char* e = getenv("HSPEC_NO_COOPERATIVE"); return e && e[0] == '1'; }();
+  if (refuse) return cudaErrorCooperativeLaunchTooLarge;
+  int dev = -1;
+  const cudaError_t e0 = chain_device(&dev);
   if (e0 != cudaSuccess) return e0;
-  const int dev = current_device();
   ChainArgs a{};
   a.logits = c.logits; a.ld = c.ld; a.W_in = reinterpret_cast<const uint16_t*>(c.W_in); a.last_token = c.last_token;
   a.id_map = c.id_map; a.ids = c.ids; a.status = c.status;
@@ -394,7 +407,6 @@ cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracke
   // a full SM's shared memory, so that one CTA sits on each SM
   const size_t smem = fixed + size_t(a.stages) * W_STAGE;
   const int grid = a.n_tiles < g_chain_sms[dev] ? a.n_tiles : g_chain_sms[dev];
-  if ((a.n_tiles + grid - 1) / grid > 255) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaMemsetAsync(c.ws, 0, markov_chain_bytes(c.B), stream);
   if (e != cudaSuccess) return e;
   trk_begin(trk, "markov_chain", 2.0 * c.B * c.k * double(c.Vd) * c.r, double(c.k) * c.Vd * c.r * 2,
@@ -404,6 +416,10 @@ cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracke
   else if (a.BN <= 96) e = chain_launch_n<3>(c.tmW_out, a, grid, smem, stream);
   else e = chain_launch_n<4>(c.tmW_out, a, grid, smem, stream);
   trk_end(trk);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();                                          // nothing was enqueued, the context is as it was
+    if (trk) trk->drop_last();
+  }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

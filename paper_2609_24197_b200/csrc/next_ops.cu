@@ -214,10 +214,13 @@ size_t markov_workspace_bytes(int B, int Vd, int r) {
 }
 
 // Up to 128 requests all positions run in one launch (markov_chain.cu; us per position with the logits written, GEMM + reduction against
-// it: 32 requests, V = 151 936 48 / 21, 96, 32 000 34 / 14, 64, 152 064 69 / 30, 1, 32 000 10.4 / 7.6); above that one GEMM and one
-// reduction per position.
+// it: 32 requests, V = 151 936 48 / 21, 96, 32 000 34 / 14, 64, 152 064 69 / 30, 1, 32 000 10.4 / 7.6); above that, and where that launch
+// is refused, one GEMM and one reduction per position.
 cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk, std::string* err) {
-  if (markov_chain_supported(c.B, c.Vd, c.r)) return markov_chain_launch(c, stream, trk);
+  if (markov_chain_supported(c.B, c.Vd, c.r)) {
+    const cudaError_t e = markov_chain_launch(c, stream, trk);
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return e;
+  }
   const size_t vt = (size_t(c.Vd) + 127) / 128;
   uint8_t* ws = reinterpret_cast<uint8_t*>(c.ws);
   uint16_t* x = reinterpret_cast<uint16_t*>(ws);

@@ -324,3 +324,15 @@ def test_markov_head_leaves_nan_out(hs, B, pruned):
         prev = id_map[best].long() if pruned else best
         assert torch.equal(ids.view(B, k)[:, i].long(), prev), i
     assert hs.hspec_op_device_status()["rc"] == 0
+
+
+def test_markov_head_where_cooperative_launches_are_refused():
+    """The tests of the one-launch form again, in a process in which that launch is refused: same ids, same logits, position by position."""
+    import os
+    import subprocess
+    import sys
+    res = subprocess.run([sys.executable, "-m", "pytest", "-q", "-x", "-p", "no:cacheprovider", __file__, "-k",
+                          "test_markov_head_chunks_and_tiles or test_markov_head_leaves_nan_out"],
+                         env=dict(os.environ, HSPEC_NO_COOPERATIVE="1"), capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert res.returncode == 0 and " passed" in res.stdout, res.stdout[-3000:] + res.stderr[-1000:]
