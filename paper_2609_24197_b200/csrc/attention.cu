@@ -519,16 +519,15 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   });
   if (e != cudaSuccess) return e;
   trk_begin(trk, "attn_partial");
-  launch_pdl(kernel, grid, dim3(threads), smem, stream, a);
+  e = launch_pdl(kernel, grid, dim3(threads), smem, stream, a);
   trk_end(trk);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.max_chunks == 1) return e;                           // every request is one chunk, finished by the kernel itself
   dim3 mgrid(c.B * c.k, c.Hq);
   trk_begin(trk, "attn_merge");
-  launch_pdl(c.dh == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>, mgrid, dim3(c.dh), 0, stream, a);
+  e = launch_pdl(c.dh == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>, mgrid, dim3(c.dh), 0, stream, a);
   trk_end(trk);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t gather_kv_launch(const void* pool, const int32_t* row, int ctx_len, int page_size, int Hkv, int dh,

@@ -996,24 +996,22 @@ cudaError_t attention_tc_launch(const AttnCall& c, int max_chunks, cudaStream_t 
   cudaError_t e = cudaSuccess;
   if (!c.planned) {
     trk_begin(trk, "attn_plan");
-    launch_pdl(attn_tc_plan_kernel, dim3(1), dim3(256), 0, stream, plan);
+    e = launch_pdl(attn_tc_plan_kernel, dim3(1), dim3(256), 0, stream, plan);
     trk_end(trk);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const int* count = plan.count;
   const int4* items = plan.items;
   trk_begin(trk, "attn_partial");
   auto kernel = a.R <= 32 ? attn_tc_kernel<4> : (a.R <= 64 ? attn_tc_kernel<2> : attn_tc_kernel<1>);
-  launch_pdl(kernel, dim3(n_sms), dim3(352), smem, stream, tmK, tmV, a, count, items);
+  e = launch_pdl(kernel, dim3(n_sms), dim3(352), smem, stream, tmK, tmV, a, count, items);
   trk_end(trk);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (max_chunks == 1) return e;                   // every request is one chunk, finished by the kernel itself
   trk_begin(trk, "attn_merge");
-  launch_pdl(attn_tc_merge_kernel, dim3(c.B * c.Hkv * ((a.R + 31) / 32)), dim3(256), 0, stream, a, reinterpret_cast<uint16_t*>(c.o));
+  e = launch_pdl(attn_tc_merge_kernel, dim3(c.B * c.Hkv * ((a.R + 31) / 32)), dim3(256), 0, stream, a, reinterpret_cast<uint16_t*>(c.o));
   trk_end(trk);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace hspec

@@ -548,9 +548,8 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   }
   if (e == cudaSuccess && splits > 1) {
     trk_begin(trk, "gemm2_tail_reduce", 0, double(splits + 1) * tail * g.BNT * 256 * 4);
-    launch_pdl(gemm2_tail_reduce_kernel, dim3(tail, g.BNT / TAIL_ROWS), dim3(256), 0, stream, g);
+    e = launch_pdl(gemm2_tail_reduce_kernel, dim3(tail, g.BNT / TAIL_ROWS), dim3(256), 0, stream, g);
     trk_end(trk);
-    e = cudaGetLastError();
   }
   return e;
 }

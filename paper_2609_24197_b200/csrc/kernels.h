@@ -90,7 +90,9 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = off ? 0 : 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  if (e != cudaSuccess) cudaGetLastError();        // (the code is returned; left behind, the next call would find it)
+  return e;
 }
 
 // The same with the grid's CTAs in clusters of the given shape.
@@ -106,7 +108,9 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = cluster.x; at[1].val.clusterDim.y = cluster.y; at[1].val.clusterDim.z = cluster.z;
   cfg.attrs = at; cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  if (e != cudaSuccess) cudaGetLastError();        // (the code is returned; left behind, the next call would find it)
+  return e;
 }
 
 enum GemmEpilogue : int {

@@ -416,10 +416,8 @@ cudaError_t markov_chain_launch(const MarkovCall& c, cudaStream_t stream, Tracke
   else if (a.BN <= 96) e = chain_launch_n<3>(c.tmW_out, a, grid, smem, stream);
   else e = chain_launch_n<4>(c.tmW_out, a, grid, smem, stream);
   trk_end(trk);
-  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
-    cudaGetLastError();                                          // nothing was enqueued, the context is as it was
-    if (trk) trk->drop_last();
-  }
+  if (e != cudaSuccess) cudaGetLastError();                      // (the code is returned; left behind, the next call would find it)
+  if ((e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) && trk) trk->drop_last();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -245,10 +245,9 @@ cudaError_t markov_launch(const MarkovCall& c, cudaStream_t stream, Tracker* trk
     e = gemm_launch(g, stream, trk, err);
     if (e != cudaSuccess) return e;
     trk_begin(trk, "markov_reduce");
-    launch_pdl(markov_reduce_gather_kernel, dim3((c.B + 7) / 8), dim3(1024), 0, stream, (const float*)part_val, (const int*)part_idx,
-               int(vt), c.B, c.ids, c.k, i, c.id_map, reinterpret_cast<const uint16_t*>(c.W_in), x, c.r, int(i + 1 < c.k));
+    e = launch_pdl(markov_reduce_gather_kernel, dim3((c.B + 7) / 8), dim3(1024), 0, stream, (const float*)part_val, (const int*)part_idx,
+                   int(vt), c.B, c.ids, c.k, i, c.id_map, reinterpret_cast<const uint16_t*>(c.W_in), x, c.r, int(i + 1 < c.k));
     trk_end(trk);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -859,8 +859,9 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
                         reinterpret_cast<uintptr_t>(a.conv_b)) & 15) == 0;
     const dim3 grid_c(c.G + (a.Di / (vec4 ? 4 : 1) + 255) / 256, c.B * ((c.k + CONV_ROWS - 1) / CONV_ROWS));
     const size_t smem_c = size_t(2) * c.k * (c.N + 4) * sizeof(float);
-    launch_pdl(vec4 ? scan_conv_kernel<4> : scan_conv_kernel<1>, grid_c, dim3(256), smem_c, stream, a, xact, c16, cbw);
+    const cudaError_t e_conv = launch_pdl(vec4 ? scan_conv_kernel<4> : scan_conv_kernel<1>, grid_c, dim3(256), smem_c, stream, a, xact, c16, cbw);
     trk_end(trk);
+    if (e_conv != cudaSuccess) return e_conv;        // (the stream kernel reads the state early on the strength of this launch in front of it)
     const size_t smem_s = two ? scan_stream_smem<2>() : scan_stream_smem<1>();
     static bool sset[2][MAX_DEVICES] = {};
     {
@@ -872,10 +873,10 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     }
     dim3 grid_s(a.H / 4, c.B);
     trk_begin(trk, "mamba_scan", 2.0 * c.B * c.k * a.H * c.P * c.N, double(c.B) * a.H * c.P * c.N * 2);
-    if (two) launch_pdl(mamba_scan_stream_kernel<64, 128, 2>, grid_s, dim3(128), smem_s, stream, a, (const float*)xact, (const __half*)c16, (const float*)cbw);
-    else launch_pdl(mamba_scan_stream_kernel<64, 128, 1>, grid_s, dim3(128), smem_s, stream, a, (const float*)xact, (const __half*)c16, (const float*)cbw);
+    const cudaError_t e = launch_pdl(two ? mamba_scan_stream_kernel<64, 128, 2> : mamba_scan_stream_kernel<64, 128, 1>, grid_s, dim3(128), smem_s, stream, a,
+                                     (const float*)xact, (const __half*)c16, (const float*)cbw);
     trk_end(trk);
-    return cudaGetLastError();
+    return e;
   }
   if (c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ld_in % 2 == 0 && c.Di % 2 == 0) {
     const bool two = c.k > 16;
@@ -890,9 +891,9 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     }
     dim3 grid_f(a.H / 4, c.B);
     trk_begin(trk, "mamba_scan", 2.0 * c.B * c.k * a.H * c.P * c.N, double(c.B) * a.H * c.P * c.N * 2);
-    launch_pdl(two ? mamba_scan_mma_kernel<64, 128, 2> : mamba_scan_mma_kernel<64, 128, 1>, grid_f, dim3(128), smem_f, stream, a);
+    const cudaError_t e = launch_pdl(two ? mamba_scan_mma_kernel<64, 128, 2> : mamba_scan_mma_kernel<64, 128, 1>, grid_f, dim3(128), smem_f, stream, a);
     trk_end(trk);
-    return cudaGetLastError();
+    return e;
   }
   if (c.N <= 16) {
     const int hb = small_state_heads(c), threads = (hb * c.P + 31) / 32 * 32, nmax = c.N <= 4 ? 4 : 16;
@@ -930,9 +931,9 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   }
   dim3 grid(a.H, c.B);
   trk_begin(trk, "mamba_scan", 0, double(c.B) * a.H * c.P * c.N * 2);
-  launch_pdl(mamba_scan_kernel, grid, dim3(SCAN_THREADS), smem, stream, a);
+  const cudaError_t e = launch_pdl(mamba_scan_kernel, grid, dim3(SCAN_THREADS), smem, stream, a);
   trk_end(trk);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace hspec

@@ -143,3 +143,22 @@ def test_peaked_target_keys_in_a_whole_step(hs):
     st = drafter.stats()
     assert st["rc"] == 0 and st["attn_rescales"] > 0, st
     drafter.close()
+
+
+def test_scan_whose_first_launch_is_refused_launches_nothing(hs):
+    """A scan of more requests than a grid holds rows of blocks for its conv is refused; nothing may run behind the launch that failed, and
+    the next call must not find its error."""
+    B, k, Di, P, N, G = 17000, 16, 256, 64, 128, 1
+    ld = Di + Di + 2 * G * N + Di // P
+    zx = torch.zeros((B * k, ld), device="cuda")
+    vec = lambda n: torch.zeros(n, device="cuda")
+    args = (None, None, vec((Di + 2 * G * N) * 4), vec(Di + 2 * G * N), vec(Di // P), vec(Di // P), vec(Di // P))
+    y = torch.full((B * k, Di), 7.0, device="cuda")
+    ws = torch.zeros(hs.hspec_scan_workspace_bytes(B, k, Di, N, G), dtype=torch.uint8, device="cuda")
+    with pytest.raises(hs.HSpecError, match="invalid configuration"):
+        hs.hspec_op_mamba_scan(zx, *args, y, B, k, Di, P, N, G, 4, ws)
+    torch.cuda.synchronize()
+    assert bool((y == 7.0).all())
+    hs.hspec_op_mamba_scan(zx, *args, y, 100, k, Di, P, N, G, 4, ws)
+    torch.cuda.synchronize()
+    assert bool((y[:1600] == 0.0).all()) and bool((y[1600:] == 7.0).all())
