@@ -285,3 +285,33 @@ def test_smaller_context_bound_than_planned_fits_the_workspace(over, top):
     torch.cuda.synchronize()
     assert torch.equal(own, by_table)
     drafter.close()
+
+
+# a step with the causal-correction head holds a memset and, up to 128 requests, a cooperative launch: captured and replayed like the rest
+@pytest.mark.parametrize("B,V_draft", [(3, 0), (130, 1200)])
+def test_step_with_the_causal_correction_head_replays_bit_exactly(B, V_draft):
+    cfg = synth.derived(dict(MID, B=B, markov_rank=64, V_draft=V_draft))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[(41 * b) % 700 for b in range(B)], poison_tail=False)
+    k = 5
+    direct = [t.clone() for t in drafter.draft(batch, k, want_logits=True)[:2]]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            replayed = drafter.draft(batch, k, want_logits=True)[:2]
+    for _ in range(2):
+        torch.cuda.synchronize()
+        replayed[0].fill_(-1)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(replayed[0], direct[0]) and torch.equal(replayed[1], direct[1])
+    batch["last_token"].copy_((batch["last_token"] + 7) % cfg["V"])
+    batch["last_hidden"].copy_(batch["last_hidden"].flip(0))
+    graph.replay()
+    torch.cuda.synchronize()
+    fresh = drafter.draft(batch, k, want_logits=True)[:2]
+    torch.cuda.synchronize()
+    assert torch.equal(replayed[0], fresh[0]) and torch.equal(replayed[1], fresh[1])
+    assert not torch.equal(fresh[0], direct[0]) and drafter.stats()["device_status"] == 0
+    drafter.close()

@@ -150,24 +150,17 @@ def test_few_row_gemm_slices(hs, M, n_out, K, kind):
     test_many_row_gemm_tile_widths(hs, M, n_out, K, kind)
 
 
-# query rows per KV head at the edges of the row copies (4 copies up to 32 rows, 2 up to 64, 1 above), contexts that end inside a copy's
-# part of a tile, a block that starts a tile of its own, single and several chunks, the window's leading edge inside a part; head width
-# 64 and chunks of 64 tokens: the other kernel, four, two and one warps per 16 rows, and more CTAs than the shared form takes
-@pytest.mark.parametrize("k,rep", [(1, 1), (8, 4), (11, 3), (32, 1), (16, 4), (32, 2), (13, 5), (16, 8)])
-@pytest.mark.parametrize("window,chunk", [(0, 0), (0, 256), (300, 0), (0, 64)])
-@pytest.mark.parametrize("dh,Hkv", [(128, 2), (64, 2), (64, 8)])
-def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
+def _attention_against_fp64(hs, ctx, k, rep, window, chunk, dh, Hkv, page=16):
     import numpy as np
-    ctx = [0, 1, 31, 97, 128, 500, 1111]
     B, Hq = len(ctx), Hkv * rep
-    pages = [(c + 15) // 16 for c in ctx]
+    pages = [(c + page - 1) // page for c in ctx]
     perm = torch.randperm(sum(pages), generator=torch.Generator().manual_seed(3)).int()
     table, at = torch.full((B, max(pages)), -1, dtype=torch.int32), 0
     for b, n in enumerate(pages):
         table[b, :n] = perm[at:at + n]
         at += n
     bf = torch.bfloat16
-    kp, vp = _rand((sum(pages), 16, Hkv, dh), 1, bf), _rand((sum(pages), 16, Hkv, dh), 2, bf)
+    kp, vp = _rand((sum(pages), page, Hkv, dh), 1, bf), _rand((sum(pages), page, Hkv, dh), 2, bf)
     q, kb, vb = _rand((B * k, Hq, dh), 4, bf), _rand((B * k, Hkv, dh), 5, bf), _rand((B * k, Hkv, dh), 6, bf)
     o = torch.full((B * k, Hq * dh), float("nan"), dtype=torch.float16, device="cuda")
     ws = torch.empty(hs.hspec_attention_workspace_bytes(B, k, Hq, Hkv, dh, max(ctx), window, chunk), dtype=torch.uint8, device="cuda")
@@ -175,7 +168,7 @@ def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
     for _ in range(3):            # a work list read before it is written is an empty one here, and leaves NaN
         ws.zero_()
         o.fill_(float("nan"))
-        hs.hspec_op_attention(q, kb, vb, kp, vp, table, lens, max(ctx), o, B, k, Hq, Hkv, dh, 16, window, chunk, ws)
+        hs.hspec_op_attention(q, kb, vb, kp, vp, table, lens, max(ctx), o, B, k, Hq, Hkv, dh, page, window, chunk, ws)
         assert not bool(o.isnan().any())
     for b, c in enumerate(ctx):
         rows = table[b, :pages[b]].long()
@@ -192,6 +185,25 @@ def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
         mag = torch.einsum("ihrj,jhd->ihrd", p, V.abs()).reshape(k, Hq * dh)
         err = (o[b * k:(b + 1) * k].double() - ref).abs()
         assert bool((err <= 2.0 ** -8 * mag + 2.0 ** -11 * ref.abs() + 1e-6).all()), float((err / mag).max())
+
+
+# query rows per KV head at the edges of the row copies (4 copies up to 32 rows, 2 up to 64, 1 above), contexts that end inside a copy's
+# part of a tile, a block that starts a tile of its own, single and several chunks, the window's leading edge inside a part; head width
+# 64: the other kernel, four and two warps per 16 rows, and one above 64 rows
+@pytest.mark.parametrize("k,rep", [(1, 1), (8, 4), (11, 3), (32, 1), (16, 4), (32, 2), (13, 5), (16, 8)])
+@pytest.mark.parametrize("window,chunk", [(0, 0), (0, 256), (300, 0), (0, 64)])
+@pytest.mark.parametrize("dh,Hkv", [(128, 2), (64, 2), (64, 8)])
+def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
+    _attention_against_fp64(hs, [0, 1, 31, 97, 128, 500, 1111], k, rep, window, chunk, dh, Hkv)
+
+
+# the mma.sync kernel's forms: four, two and one warps per 16 query rows, with and without warps that only load, on either side of the CTA counts
+# that choose between them (592 with up to 32 rows, 148 with up to 64); heads of 128 come here with pages that are not 16 tokens
+@pytest.mark.parametrize("dh,page,B,Hkv,k,rep", [(64, 16, 74, 8, 8, 4), (64, 16, 75, 8, 8, 4), (64, 16, 75, 8, 1, 1), (64, 16, 18, 8, 16, 4), (64, 16, 19, 8, 16, 4),
+                                                 (128, 32, 3, 2, 4, 4), (128, 8, 3, 2, 16, 4), (128, 8, 75, 8, 8, 4), (128, 5, 2, 2, 16, 8), (128, 1, 1, 1, 32, 16)])
+@pytest.mark.parametrize("window", [0, 40])
+def test_attention_warps_per_row(hs, dh, page, B, Hkv, k, rep, window):
+    _attention_against_fp64(hs, [(37 * b + 61) % 129 for b in range(B)], k, rep, window, 256, dh, Hkv, page)
 
 
 # the norm behind a residual GEMM adds the GEMM's K-sliced tail tiles: row counts with a whole-wave part and a tail, all tail, and no tail,
@@ -336,3 +348,18 @@ def test_markov_head_where_cooperative_launches_are_refused():
                          env=dict(os.environ, HSPEC_NO_COOPERATIVE="1"), capture_output=True, text=True, timeout=300,
                          cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert res.returncode == 0 and " passed" in res.stdout, res.stdout[-3000:] + res.stderr[-1000:]
+
+
+# low-rank dt that the scan expands itself, at the states the other scan kernels take: the stream kernel (N = 128, one and two tiles of 16
+# positions), the generic one (N = 32), on either side of the product count (2^22) and of the rank (64) above which a GEMM does it; bf16 operands
+@pytest.mark.parametrize("Di,N,G,dt_rank,B,k,bf16", [(512, 128, 1, 16, 2, 16, 0), (512, 128, 2, 64, 3, 17, 0), (512, 128, 2, 64, 3, 32, 1), (512, 128, 1, 72, 2, 5, 0),
+                                                     (768, 32, 1, 16, 2, 9, 0), (768, 32, 3, 64, 2, 32, 0), (4096, 128, 4, 64, 32, 32, 0), (4096, 128, 4, 64, 33, 32, 0)])
+def test_low_rank_dt_in_the_scan(hs, Di, N, G, dt_rank, B, k, bf16):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(D=256, n_fuse=1, r=64, L=2, has_attn=[0, 0], kv_slot=[-1, -1], n_slots=0, Di=Di, P=64, N=N, G=G, d_conv=4, dt_rank=dt_rank,
+                             Hq=4, Hkv=2, dh=64, rope_theta=1.0e4, window=0, qk_norm=1, F=512, V=600, rms_eps=1e-6, page_size=16, name="lowrank",
+                             act_bf16=bf16, B=B, k=k, ctx=("const", 20, 20)))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[20] * B)
+    check_step(cfg, drafter, w, batch, k, requests=[0, B - 1], what=f"low rank {Di} {N} {dt_rank} {B}", **(dict(tol=5e-2) if bf16 else {}))
+    drafter.close()
