@@ -349,6 +349,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ 
     return;
   }
   if (smem_u32(smem) & 1023) {                      // the swizzled operand tiles need a 1 KiB-aligned base
+    if (a.early) pdl_wait();
     if (tid == 0) atomicExch(a.status, STATUS_BAD_SMEM_BASE);
     return;
   }
