@@ -60,10 +60,18 @@ __device__ __forceinline__ void store_act16(void* base, size_t idx, float v, boo
 }
 
 // ------------------------------------------------------------------ programmatic dependent launch
-// A kernel launched with launch_pdl() may start while the kernel before it on the stream is still running: its CTAs
-// run their set-up and then block in pdl_wait() until that kernel has finished and its writes are visible.  Nothing
-// produced by an earlier kernel may be read, and nothing may be written to global memory, before pdl_wait().
-// pdl_trigger() lets the NEXT kernel on the stream start launching once every CTA of this one has called it.
+// A kernel launched with launch_pdl() may start while the kernel before it on the stream is still running; pdl_wait() blocks until that
+// kernel has finished and its writes are visible.  pdl_trigger() lets the NEXT kernel on the stream start once every CTA of this one has
+// called it.  Every kernel keeps to this:
+//   * pdl_trigger() comes behind the kernel's own pdl_wait().  When a kernel starts, its predecessor has therefore seen the end of its own,
+//     and everything up to two kernels back has finished.  One kernel that triggers before it has waited breaks the reads below in the
+//     kernels behind it, and nothing would show it but wrong numbers.
+//   * Before pdl_wait() nothing is written to global memory, and only this is read: what kernels at least two back have written (the
+//     step's work list, the scan's injected state), and what no kernel of the step writes (weights, where the caller says that they are
+//     stable; the target's cache, its page table and lengths, which are there before the step's first kernel has waited).
+//   * No CTA ends without a thread of it having waited: the kernel behind takes this one's end for the end of those in front.
+//   * What is read behind a wait that stands under a condition goes through plain, volatile or asynchronous loads: a read-only load (__ldg,
+//     const __restrict__) may be moved up past it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -226,7 +234,8 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
-// fp32 addition in the L2; nothing is returned
+// fp32 addition in the L2; nothing is returned.  One rounding, like an addition in registers, but subnormal operands and results (below
+// 2^-126) are taken as zero.
 __device__ __forceinline__ void red_add_f32(float* p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
@@ -234,7 +243,7 @@ __device__ __forceinline__ void red_add_f32(float* p, float v) {
 // ------------------------------------------------------------------ tcgen05 / TMEM
 // True in exactly one lane of a converged warp.  A role that one thread plays is entered through this and not through
 // lane == 0: with it the compiler knows that a single thread is active around the MMA instructions.
-// 2-SM GEMM, M = 2048, K = 5120: n_out = 51200 818 -> 770 us, n_out = 21664 356 -> 335 us.
+// 2-SM GEMM, M = 2048, K = 5120: n_out = 51200 818 -> 763 us, n_out = 21664 356 -> 336 us.
 __device__ __forceinline__ bool elect_one() {
   uint32_t r;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));

@@ -329,9 +329,9 @@ argmax_init_kernel(unsigned long long* keys, int M) {
   if (m < M) keys[m] = 0;
 }
 
-// A row without any maximum keeps its sentinel.  (Before, the tiles' (value, index) pairs went to memory and this kernel reduced them: the
-// LM head of 152 064 rows, 77 requests 282 -> 279 us.  Letting the GEMM's last CTA write the ids instead costs a fence, a ticket
-// and a read-back at its end, more than this launch: test-sized drafter 65.3 -> 66.6 us per step.)
+// A row without any number (all NaN, or a wait that gave up) has no id: 0x7fffffff.  (A key per row against (value, index) pairs per tile and row
+// that a kernel reduces: LM head of 152 064 rows, 77 requests 279 against 282 us.  Letting the GEMM's last CTA write the ids instead
+// costs a fence, a ticket and a read-back at its end, more than this launch: test-sized drafter 65.3 -> 66.6 us per step.)
 __global__ void __launch_bounds__(256)
 argmax_ids_kernel(const unsigned long long* keys, int M, int* ids, const int* id_map) {
   pdl_wait();

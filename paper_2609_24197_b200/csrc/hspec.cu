@@ -797,6 +797,7 @@ int hspec_op_lm_head_argmax(const void* x, const void* Wt, int32_t in_dtype, int
                             void* workspace, size_t workspace_bytes, void* stream) {
   if (!x || !Wt || !ids || !workspace || M < 1 || V < 1 || K < 8 || K % 8)
     return fail(nullptr, HSPEC_ERR_INVALID_ARG, "hspec_op_lm_head_argmax: bad argument");
+  // (only M keys are used; the size that the entry point asks for is the one callers know, and covers them)
   const size_t vt = (size_t(V) + 127) / 128;
   if (workspace_bytes < vt * M * 8 + 1024) return fail(nullptr, HSPEC_ERR_WORKSPACE_TOO_SMALL, "hspec_op_lm_head_argmax: workspace too small");
   std::string errtxt;

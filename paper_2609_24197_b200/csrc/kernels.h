@@ -80,7 +80,8 @@ inline double gemm_io_bytes(int M, int n_out, int K, int mode, bool logits) {
 }
 inline void trk_end(Tracker* t) { if (t) t->end(); }
 
-// Launch with programmatic stream serialisation: the kernel MUST call pdl_wait() before it touches global data.
+// Launch with programmatic stream serialisation: the kernel keeps to the rules in common.cuh about what it may do before pdl_wait() and when it
+// may call pdl_trigger().
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
   static const bool off = [] { const char* e = getenv("HSPEC_NO_PDL"); return e && e[0] == '1'; }();
@@ -294,7 +295,7 @@ struct ScanCall {
   int B, k, Di, P, N, G, d_conv;
   bool w_stable;                    // nothing that may still be running on the stream writes the weights: they may be fetched early
   bool shared_rows;                 // zxbcdt and dt_raw have B + 1 rows: position 0 of every request, then one row for all later positions
-  void* ws;                         // optional scratch (scan_workspace_bytes): enables the three-kernel fast path
+  void* ws;                         // optional scratch (scan_workspace_bytes): enables the two-kernel fast path
   size_t ws_bytes;
 };
 bool scan_does_norm(const ScanCall& c);

@@ -196,16 +196,7 @@ cudaError_t token_probs_launch(const float* logits, long long ld, const int* ids
   // enough blocks for two per SM, as long as a block still has a few KB to read
   int S = 1;
   while (S < 8 && M * S < 2 * 148 && V / (2 * S) >= 4096) S *= 2;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(unsigned(M) * S); cfg.blockDim = dim3(512); cfg.stream = stream;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = 2;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, token_probs_kernel, logits, ld, ids, p, V, S);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return launch_pdl_cluster(token_probs_kernel, dim3(unsigned(M) * S), dim3(512), dim3(S), 0, stream, logits, ld, ids, p, V, S);
 }
 
 size_t markov_workspace_bytes(int B, int Vd, int r) {

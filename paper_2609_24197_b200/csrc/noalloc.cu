@@ -20,7 +20,7 @@
 namespace {
 
 constexpr int NA_MAX_ROWS = 512;        // activation rows per call
-constexpr int NA_MAX_TILES = 2048;      // 128-row vocabulary tiles: V <= 262144
+constexpr int NA_MAX_V = 262144;        // the call's documented limit; nothing in the scratch depends on the vocabulary
 constexpr int NA_MAX_DEVICES = 64;
 
 struct NoAllocScratch {
@@ -80,10 +80,9 @@ extern "C" int hspec_op_lm_head_argmax_noalloc(const void* x, const void* W, int
   using namespace hspec;
   if (!x || !W || !ids || M < 1 || V < 1 || K < 8 || K % 8) return na_fail(HSPEC_ERR_INVALID_ARG, "bad argument");
   if (in_dtype != HSPEC_BF16 && in_dtype != HSPEC_F16) return na_fail(HSPEC_ERR_INVALID_ARG, "x and W must both be bf16 or both fp16");
-  const int tiles = 2 * ((V + 255) / 256);               // 128-row tiles, in pairs
-  if (M > NA_MAX_ROWS || tiles > NA_MAX_TILES)
-    return na_fail(HSPEC_ERR_BAD_SHAPE, "the built-in scratch holds at most " + std::to_string(NA_MAX_ROWS) + " rows and a vocabulary of " +
-                                            std::to_string(NA_MAX_TILES * 128) + " (got M=" + std::to_string(M) + ", V=" + std::to_string(V) +
+  if (M > NA_MAX_ROWS || V > NA_MAX_V)
+    return na_fail(HSPEC_ERR_BAD_SHAPE, "the built-in scratch holds at most " + std::to_string(NA_MAX_ROWS) + " rows, and the vocabulary may have " +
+                                            std::to_string(NA_MAX_V) + " (got M=" + std::to_string(M) + ", V=" + std::to_string(V) +
                                             "); use hspec_op_lm_head_argmax with a workspace instead");
   std::string why;
   NoAllocScratch* s = nullptr;
