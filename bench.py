@@ -9,7 +9,8 @@ One "step" = one call of hspec_draft_block (the whole hot path) over one batch o
 The headline workload is the concurrency-128 configuration (32B-class shapes, B = 128, k = 16, contexts
 log-uniform in [1024, 32768]); the concurrency-1 and concurrency-32 configurations, the two serving workloads with
 the paper's 2048-token window, and the 18 cells of the concurrency x block-size sweep are measured in the same run
-and reported under "by_concurrency", "window_2048" and "sweep".  Prints ONE JSON line (rank 0).
+and reported under "by_concurrency", "window_2048" and "sweep".  Rank 0 prints those tables as "[bench] name: {...}" lines and
+then, last, ONE JSON line with the headline.
 
 Timing: W warm-up steps, then untimed steps for --settle-s seconds (so the GPU sits at the clocks it keeps under its
 power cap, the condition the tensor peak was measured in), then --repeats timed regions of exactly K steps each, every
@@ -762,6 +763,22 @@ def main_case(args):
 
 # ----------------------------------------------------------------------------- entry points
 
+# What is measured beside the headline, in the order in which it is printed.
+TABLES = ("dtype_note", "timing", "peaks", "step", "rooflines", "attention", "gemm", "kernels", "kv_injection_counterexample",
+          "by_concurrency", "window_2048", "bf16_operands", "sweep")
+
+
+def print_result(line):
+    """The tables, a line of their own each (not JSON lines: "[bench] name: {...}"), then the ONE JSON line with the headline."""
+    for name in TABLES:
+        if name in line:
+            print(f"[bench] {name}: {json.dumps(line[name])}")
+    head = {k: v for k, v in line.items() if k not in TABLES}
+    if "roofline" in head:                         # (its notes are in the rooflines table)
+        head["roofline"] = {k: v for k, v in head["roofline"].items() if "note" not in k and not isinstance(v, dict)}
+    print(json.dumps(head), flush=True)
+
+
 def main_ours(args):
     rank, local_rank, world = dist_info()
     if not torch.cuda.is_available():
@@ -780,12 +797,12 @@ def main_ours(args):
         sw = run_sweep(args.steps, args.warmup, peaks, rank)
         if rank == 0:
             head = next(c for c in sw["cells"] if c["B"] == 128 and c["k"] == 16)
-            print(json.dumps({"metric": METRIC, "value": head["draft_tokens_per_s"], "unit": "draft tokens/s", "n_gpus": world,
-                              "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": head["ms_per_step"],
-                              "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f16",
-                              "data": "synthetic", "config": {"workload": "sweep_8b_B128_k16", "note": "value = the B = 128, "
-                                                              "k = 16 cell; every cell under `sweep`"},
-                              "sweep": sw, "peaks": peaks}))
+            print_result({"metric": METRIC, "value": head["draft_tokens_per_s"], "unit": "draft tokens/s", "n_gpus": world,
+                          "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": head["ms_per_step"],
+                          "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f16",
+                          "data": "synthetic", "config": {"workload": "sweep_8b_B128_k16", "note": "value = the B = 128, "
+                                                          "k = 16 cell; every cell under `sweep`"},
+                          "sweep": sw, "peaks": peaks})
         return
     head = run_workload(args.workload, args.steps, args.warmup, rank, clock_gpu=torch.cuda.current_device(),
                         lean=args.lean, repeats=args.repeats, settle_s=args.settle_s)
@@ -880,7 +897,7 @@ def main_ours(args):
                 print(f"[bench] sweep skipped: {exc}", file=sys.stderr)
             torch.cuda.empty_cache()
     if rank == 0:
-        print(json.dumps(line))
+        print_result(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

@@ -90,3 +90,24 @@ def test_reference_arm_prints_one_contract_line_on_cpu():
     assert line["cpu_baseline"]["kind"] == "oracle" and line["cpu_baseline"]["cores"] >= 1
     assert line["e2e"]["h2d_bytes_per_step"] == 0 and line["e2e"]["d2h_bytes_per_step"] == 0
     assert line["config"]["workload"] == "tiny"
+
+
+def test_result_ends_with_one_short_json_line(capsys):
+    """Whoever reads the bench's output takes its last line, and may have only the last few thousand characters of the output."""
+    import json
+    line = {"metric": bench.METRIC, "value": 177000.1, "unit": "draft tokens/s", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": 11.5,
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f16", "data": "synthetic",
+            "config": {"workload": "conc128_32b", "l2": "inputs larger than L2: 26.8 GB touched per step, no flush"},
+            "e2e": {"value": 1.0, "unit": "draft tokens/s", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 1}, "gpu_launches": 820,
+            "clocks": {"sm_mhz": 1300.0, "sm_max_mhz": 1965.0, "reasons": ["sw_power_cap"]},
+            "roofline": {"kernel": "gemm_2sm_kernel", "frac": 0.97, "note": "n" * 400, "traffic_note": "t" * 400, "per_clock": {"frac": 1.0}},
+            "cpu_baseline": {"value": 0.665, "unit": "draft tokens/s", "cores": 16, "kind": "oracle", "sample": "s" * 80}}
+    tables = {name: [{"cell": i, "note": "x" * 80} for i in range(40)] for name in bench.TABLES}
+    bench.print_result(dict(line, **tables))
+    out = capsys.readouterr().out.splitlines()
+    last = json.loads(out[-1])
+    assert len(out[-1]) < 1500 and sum(o.startswith("{") for o in out) == 1
+    for key in set(line) - {"roofline"}:
+        assert last[key] == line[key], key
+    assert last["roofline"] == {"kernel": "gemm_2sm_kernel", "frac": 0.97}
+    assert {o.split(":")[0] for o in out[:-1]} == {f"[bench] {name}" for name in bench.TABLES}
