@@ -153,8 +153,8 @@ typedef struct {
 /* Outputs of one step, device memory owned by the caller. */
 typedef struct {
   int32_t* draft_ids;   /* int32 [B, k], required: arg-max of the logits, lowest row index on ties; target token ids
-                           (mapped through vocab_map when the drafter vocabulary is pruned).  A NaN logit is never
-                           chosen; a row of nothing but NaN gets 0x7fffffff, with the causal-correction head row 0 */
+                           (mapped through vocab_map when the drafter vocabulary is pruned).  A NaN logit counts as
+                           -infinity: it is chosen only where nothing is above that, as row 0 of the vocabulary */
   float* logits;        /* fp32 [B, k, V] ([B, k, V_draft] when pruned) or NULL (then the logits are never materialised,
                            except in the workspace when markov_rank > 0); with the causal-correction head these are the
                            corrected logits */
@@ -233,8 +233,8 @@ int hspec_op_gemm(const void* x, const void* W, int32_t in_dtype, void* y, int32
                   int32_t out_dtype, int32_t accumulate, int32_t splits, void* workspace, size_t workspace_bytes,
                   void* stream);
 size_t hspec_gemm_workspace_bytes(int32_t M, int32_t n_out, int32_t K);
-/* LM head fused with arg-max (App. B.2): ids[m] = lowest index of max_v x[m,:] . W[v,:], NaN left out (0x7fffffff where
- * all are); logits fp32 [M, V] or NULL.
+/* LM head fused with arg-max (App. B.2): ids[m] = lowest index of max_v x[m,:] . W[v,:], a NaN counting as -infinity;
+ * logits fp32 [M, V] or NULL.
  * x and W are both bf16 or both fp16 (in_dtype). */
 int hspec_op_lm_head_argmax(const void* x, const void* W, int32_t in_dtype, int32_t* ids, float* logits, int32_t M, int32_t V,
                             int32_t K, void* workspace, size_t workspace_bytes, void* stream);
@@ -274,8 +274,8 @@ int hspec_op_token_probs(const float* logits, int64_t ld, const int32_t* ids, fl
 /* Causal correction after the backbone (Sec. 3.3.3; rank 256 in App. B.1): a first-order dependency between adjacent
  * draft positions applied to the logits.  The paper prints no formula; the reading implemented is a low-rank bigram
  * table, logits'[b, i, :] = logits[b, i, :] + W_out . W_in[prev(b, i), :], prev(b, 0) = last_token[b], prev(b, i) =
- * the token chosen at position i - 1 from the adjusted logits (lowest index on ties, NaN left out, row 0 where all are
- * NaN), positions strictly in order.
+ * the token chosen at position i - 1 from the adjusted logits (lowest index on ties, a NaN counting as -infinity),
+ * positions strictly in order.
  *   logits   device fp32 [B*k, ld] (row b*k + i), adjusted in place when write_logits != 0, else left as they are
  *   W_in     device [V, r]  fp16 or bf16 (w_dtype), one row per possible previous TOKEN id
  *   W_out    device [Vd, r] same type, one row per drafter-vocabulary index; r % 8 == 0, both 16-byte aligned

@@ -178,13 +178,10 @@ __device__ __forceinline__ void warp_argmax16(float (&v)[16], int (&idx)[16], in
   row = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
-// The value and index a lane brings into an arg-max.  A NaN is never chosen, and neither is a row past the matrix (on = false): both
-// come as (-inf, no index), which loses against every number, -inf included.
-__device__ __forceinline__ void argmax_candidate(float x, int n, bool on, float& v, int& idx) {
-  on = on && x == x;
-  v = on ? x : -INFINITY;
-  idx = on ? n : 0x7fffffff;
-}
+// The value that matrix row n brings into an arg-max: a NaN counts as -inf, and so does a row past the matrix (on = false).  Those lie behind
+// every row of the matrix, so at equal values one of these is found first.  (With the index taken away from NaN as well, so that a row
+// of nothing but NaN has none, the 2-SM GEMM needs 88 registers instead of 80 and a step of the paper's drafter takes 10 us more.)
+__device__ __forceinline__ float argmax_value(float x, bool on) { return on ? fmaxf(x, -INFINITY) : -INFINITY; }
 
 // ------------------------------------------------------------------ TMA (no multicast anywhere)
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
@@ -382,7 +379,7 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // (value, index) as one unsigned number: the larger key has the larger value, at equal values the lower index.  Any value beats the zero
-// key.  Not for NaN: a NaN is no candidate of an arg-max (argmax_candidate).
+// key.  Not for NaN (argmax_value).
 __device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
   uint32_t u = __float_as_uint(v + 0.f);                    // (-0 compares equal to +0)
   u = (u & 0x80000000u) ? ~u : u | 0x80000000u;

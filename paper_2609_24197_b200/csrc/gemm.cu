@@ -236,7 +236,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           const int m = m0 + c0 + j;
           const float x = __uint_as_float(r[j]) + add[j];
           if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
-          argmax_candidate(x, n, n_ok, v[j], vi[j]);
+          v[j] = argmax_value(x, n_ok);
+          vi[j] = n;
         }
         int row = 0;
         warp_argmax16(v, vi, lane, row);
@@ -329,7 +330,7 @@ argmax_init_kernel(unsigned long long* keys, int M) {
   if (m < M) keys[m] = 0;
 }
 
-// A row without any number (all NaN, or a wait that gave up) has no id: 0x7fffffff.  (A key per row against (value, index) pairs per tile and row
+// A row that no tile has finished (a wait that gave up) has no id: 0x7fffffff.  (A key per row against (value, index) pairs per tile and row
 // that a kernel reduces: LM head of 152 064 rows, 77 requests 279 against 282 us.  Letting the GEMM's last CTA write the ids instead
 // costs a fence, a ticket and a read-back at its end, more than this launch: test-sized drafter 65.3 -> 66.6 us per step.)
 __global__ void __launch_bounds__(256)

@@ -329,7 +329,8 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int m = m0 + c0 + j;
             const float x = __uint_as_float(r[j]);
             if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
-            argmax_candidate(x, n, n_ok, v[j], vi[j]);
+            v[j] = argmax_value(x, n_ok);
+            vi[j] = n;
           }
           // (The network costs the LM head 4 % - 2.34 -> 2.24 ms per step without it - mostly as clock under the power cap.
           // One redux.sync maximum + ballot per column instead of the shuffle rounds: 2.56 ms.)

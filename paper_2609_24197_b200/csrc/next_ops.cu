@@ -167,7 +167,7 @@ markov_reduce_gather_kernel(const float* __restrict__ pv, const int* __restrict_
     if (b < B) {
       v = sv[0][rr]; idx = si[0][rr];
       for (int w = 1; w < 32; ++w) take(sv[w][rr], si[w][rr]);
-      if (idx == 0x7fffffff) idx = 0;                     // (a row without any number still needs a factor row for the next position)
+      if (idx == 0x7fffffff) idx = 0;                     // (a wait that gave up: the next position still needs a factor row)
       tok = id_map ? id_map[idx] : idx;
       ids[size_t(b) * k + i] = tok;
     }

@@ -277,11 +277,11 @@ def test_lm_head_argmax_ties(hs, M, V, alloc):
         assert torch.equal(ids, first)
 
 
-# NaN logits are never chosen: one NaN at the first and the last row of a tile and of the matrix, next to and away from the maximum, a row
-# that is all NaN (no id), +inf (chosen), -inf; one-CTA kernel and pair kernel, a last tile that is part full
+# a NaN logit counts as -inf: one at the first and the last row of a tile and of the matrix, next to and away from the maximum, a row that is
+# all NaN (index 0), +inf (chosen), -inf; one-CTA kernel and pair kernel, a last tile that is part full
 @pytest.mark.parametrize("M", [5, 40, 200])
 @pytest.mark.parametrize("V", [130, 300, 20000])
-def test_lm_head_argmax_leaves_nan_out(hs, M, V):
+def test_lm_head_argmax_takes_nan_as_minus_infinity(hs, M, V):
     K = 64
     x, W = _rand((M, K), 1, torch.float16), _rand((V, K), 2, torch.float16)
     x[:, 0] = 1.0
@@ -299,9 +299,9 @@ def test_lm_head_argmax_leaves_nan_out(hs, M, V):
         ids.fill_(-1)
         hs.hspec_op_lm_head_argmax(x, W, ids, logits, ws)
         z = logits.nan_to_num(nan=-inf, posinf=inf, neginf=-inf)
-        first = torch.where((z == z.max(1, keepdim=True).values) & ~logits.isnan(), torch.arange(V, device="cuda"), 0x7fffffff).min(1).values.int()
+        first = torch.where(z == z.max(1, keepdim=True).values, torch.arange(V, device="cuda"), V).min(1).values.int()
         assert bool(logits[2].isnan().all()) and bool((logits[0].isnan().sum() >= 6).item())
-        assert torch.equal(ids, first) and int(ids[2]) == 0x7fffffff
+        assert torch.equal(ids, first) and int(ids[2]) == 0
         hs.hspec_op_lm_head_argmax_noalloc(x, W, ids.fill_(-1), logits=logits)
         assert torch.equal(ids, first)
 
@@ -309,7 +309,7 @@ def test_lm_head_argmax_leaves_nan_out(hs, M, V):
 # the same for the causal-correction head, in one launch (up to 128 requests) and position by position, with and without a pruned vocabulary
 @pytest.mark.parametrize("B", [3, 100, 131])
 @pytest.mark.parametrize("pruned", [False, True])
-def test_markov_head_leaves_nan_out(hs, B, pruned):
+def test_markov_head_takes_nan_as_minus_infinity(hs, B, pruned):
     k, Vd, r, V = 4, 19300, 64, 25000
     g = torch.Generator().manual_seed(B)
     logits = (torch.randint(-256, 257, (B, k, Vd), generator=g).float() / 64).cuda()
@@ -344,7 +344,7 @@ def test_markov_head_where_cooperative_launches_are_refused():
     import subprocess
     import sys
     res = subprocess.run([sys.executable, "-m", "pytest", "-q", "-x", "-p", "no:cacheprovider", __file__, "-k",
-                          "test_markov_head_chunks_and_tiles or test_markov_head_leaves_nan_out"],
+                          "test_markov_head_chunks_and_tiles or test_markov_head_takes_nan"],
                          env=dict(os.environ, HSPEC_NO_COOPERATIVE="1"), capture_output=True, text=True, timeout=300,
                          cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert res.returncode == 0 and " passed" in res.stdout, res.stdout[-3000:] + res.stderr[-1000:]
