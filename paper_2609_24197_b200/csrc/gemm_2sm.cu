@@ -20,7 +20,8 @@
 //
 // On M = 2048, n_out = 25600, K = 5120, SM clocks per 256 x 256 x 16
 // instruction (the arithmetic needs 128): MMA issue alone, no barrier at all 128; one k-step per stage 167 alone and
-// 182 with loads and read-out; two k-steps per stage 146 and 160.
+// 182 with loads and read-out; two k-steps per stage 146 and 160 (with eight epilogue warps and elect.sync: 145, the tensor pipe
+// 92 % busy).
 #include "common.cuh"
 #include "kernels.h"
 
