@@ -58,8 +58,11 @@ __device__ __forceinline__ uint32_t swz(int row, int col) {   // byte offset of 
 // KS: how many warps share 16 query rows.  Each of them takes KT / KS keys of every tile with a softmax of its own (running maximum, sum
 // and O), merged through shared memory when the chunk is done.  With one warp per 16 rows a call with few rows was one warp's
 // dependent chain, 4 us per tile; four warps also run a quarter of the code, which a step always finds cold in the instruction cache.
+// The bounds leave the compiler 128 registers at heads of 64 (two CTAs of 256 threads per SM; at 133 there is one, 128 rows 171 -> 220 us), 168 where
+// two warps share rows of 128 (two CTAs at 48 rows; 254, where only a CTA of 256 threads has to fit, keeps more loads in flight and pays for one
+// and four warps: 128 rows, 4096 CTAs 1113 us against 1234 at 182).
 template <int DH, int KS>
-__global__ void __launch_bounds__(KS > 1 ? 352 : 256)
+__global__ void __launch_bounds__(DH == 128 && KS == 2 ? 384 : 256, DH == 64 ? 2 : 1)
 attn_partial_kernel(AttnArgs a) {
   if (!a.early) { pdl_wait(); pdl_trigger(); }
   extern __shared__ __align__(128) uint8_t smem[];
@@ -86,11 +89,7 @@ attn_partial_kernel(AttnArgs a) {
   constexpr int CPR = DH / 8;                        // 16-byte chunks per row
   constexpr int KW = KT / KS;                        // keys of a tile per warp
 
-  // KS warps per 16 query rows compute.  The block's further warps, where it has any, do all the K/V loading, so that those that
-  // compute never wait for a page id.
-  const int n_compute = a.RT * 2 * KS, slab16 = warp / KS, part = warp % KS;     // (threads; the warp's rows; its part of the keys)
-  const bool compute = tid < n_compute;
-  const int n_loaders = nthr > n_compute ? nthr - n_compute : nthr, loader = nthr > n_compute ? tid - n_compute : tid;   // (loader < 0: none)
+  const int slab16 = warp / KS, part = warp % KS;    // the warp's rows; its part of the keys
 
   const int32_t* ptab = a.page_table + size_t(b) * a.page_table_stride;
   auto load_tile = [&](int t) {
@@ -98,36 +97,25 @@ attn_partial_kernel(AttnArgs a) {
     const uint32_t dK = smem_u32(sK) + st * KT * DH * 2, dV = smem_u32(sV) + st * KT * DH * 2;
     if (t < n_pre) {
       const int base = p_begin + t * KT;
-      constexpr int U = 4;                             // rows in flight per thread: their page ids are fetched together
-      for (int idx0 = loader; idx0 < KT * CPR; idx0 += U * n_loaders) {
-        int page[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int idx = idx0 + u * n_loaders, p = base + idx / CPR;
-          page[u] = (idx < KT * CPR && p < p_end) ? ptab[p / a.page_size] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int idx = idx0 + u * n_loaders;
-          if (idx >= KT * CPR) break;
-          const int r = idx / CPR, ch = idx % CPR;
-          const int p = base + r;
-          bool ok = p < p_end;
-          size_t off = 0;
-          if (ok) {
-            if (unsigned(page[u]) >= unsigned(a.num_pages)) {     // never form an address from a bad id: zero row, counted once
-              ok = false;
-              if (ch == 0 && p % a.page_size == 0) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
-            } else {
-              off = ((size_t(page[u]) * a.page_size + (p % a.page_size)) * a.Hkv + kvh) * DH + ch * 8;
-            }
+      for (int idx = tid; idx < KT * CPR; idx += nthr) {
+        const int r = idx / CPR, ch = idx % CPR;
+        const int p = base + r;
+        bool ok = p < p_end;
+        size_t off = 0;
+        if (ok) {
+          const int page = ptab[p / a.page_size];
+          if (unsigned(page) >= unsigned(a.num_pages)) {     // never form an address from a bad id: zero row, counted once
+            ok = false;
+            if (ch == 0 && p % a.page_size == 0) atomicAdd(a.status + STATUS_WORD_BAD_INPUT, 1u);
+          } else {
+            off = ((size_t(page) * a.page_size + (p % a.page_size)) * a.Hkv + kvh) * DH + ch * 8;
           }
-          cp_async16(dK + swz<DH>(r, ch * 8), a.k_pool + off, ok);
-          cp_async16(dV + swz<DH>(r, ch * 8), a.v_pool + off, ok);
         }
+        cp_async16(dK + swz<DH>(r, ch * 8), a.k_pool + off, ok);
+        cp_async16(dV + swz<DH>(r, ch * 8), a.v_pool + off, ok);
       }
     } else {                                          // the block's own keys / values
-      for (int idx = loader; idx < KT * CPR; idx += n_loaders) {
+      for (int idx = tid; idx < KT * CPR; idx += nthr) {
         const int r = idx / CPR, ch = idx % CPR;
         const bool ok = r < a.k;
         const size_t off = ok ? ((size_t(b) * a.k + r) * a.Hkv + kvh) * DH + ch * 8 : 0;
@@ -139,7 +127,7 @@ attn_partial_kernel(AttnArgs a) {
 
   // the first group holds tile 0 and the Q rows
   const bool tile0_early = a.early && n_pre > 0;
-  if (tile0_early && loader >= 0) load_tile(0);
+  if (tile0_early) load_tile(0);
   if (a.early) { pdl_wait(); pdl_trigger(); }
   // ---- Q rows of this tile -> shared (zero for padding rows)
   const int row0 = rt * a.RT;
@@ -151,11 +139,11 @@ attn_partial_kernel(AttnArgs a) {
     const __nv_bfloat16* src = a.q + ((size_t(b) * a.k + i) * a.Hq + kvh * a.rep + gq) * DH + ch * 8;
     cp_async16(smem_u32(sQ) + swz<DH>(r, ch * 8), src, ok);
   }
-  if (!tile0_early && n_tiles > 0 && loader >= 0) load_tile(0);
+  if (!tile0_early && n_tiles > 0) load_tile(0);
   cp_async_commit();
 #pragma unroll
   for (int t = 1; t < NSTAGE - 1; ++t) {
-    if (t < n_tiles && loader >= 0) load_tile(t);
+    if (t < n_tiles) load_tile(t);
     cp_async_commit();
   }
 
@@ -173,9 +161,8 @@ attn_partial_kernel(AttnArgs a) {
   for (int t = 0; t < n_tiles; ++t) {
     cp_async_wait<NSTAGE - 2>();
     __syncthreads();
-    if (t + NSTAGE - 1 < n_tiles && loader >= 0) load_tile(t + NSTAGE - 1);
+    if (t + NSTAGE - 1 < n_tiles) load_tile(t + NSTAGE - 1);
     cp_async_commit();
-    if (!compute) continue;
     if (!q_loaded) {                                   // Q landed with the first group
       q_loaded = true;
 #pragma unroll
@@ -259,7 +246,6 @@ attn_partial_kernel(AttnArgs a) {
     }
   }
   cp_async_wait<0>();
-  if (KS == 1 && !compute) return;
 
   // ---- partial (m, l, O) of this chunk, or the finished rows of a request with a single one
   l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
@@ -272,7 +258,7 @@ attn_partial_kernel(AttnArgs a) {
     float* so = reinterpret_cast<float*>(sK);          // [KS][RT][LD]
     float* sml = so + KS * a.RT * LD;                  // [KS][RT][2]
     __syncthreads();                                   // every warp is done with the ring
-    if (compute) {
+    {
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         const int rl = part * a.RT + slab16 * 16 + g + half * 8;
@@ -503,15 +489,20 @@ cudaError_t attention_launch(const AttnCall& c, cudaStream_t stream, Tracker* tr
   a.ws_ml = a.ws_o + slabs * a.R * c.dh;
   static bool attr_done[2][3][MAX_DEVICES] = {};
   dim3 grid(a.max_chunks * a.n_row_tiles, c.Hkv, c.B);
-  // Sharing rows shortens a CTA's chain but costs work (each part rescales its own O and keeps its own sums), so it stops where the
-  // CTAs fill the chip anyway.  Test-sized drafter, us per step, one warp per 16 rows / shared: 16 or 32 rows with four warps, up to
-  // four CTAs per SM: 8 CTAs 73.1 / 66.3, 256 88.8 / 81.3, 544 115.2 / 110.5, 540 121.4 / 119.6; 640 148 / 169.  64 rows with two warps,
-  // up to one CTA per SM: 144 CTAs 116.6 / 112.4; 384 113.7 / 119.0, 512 121.4 / 127.2.
+  // Sharing rows shortens a CTA's chain but costs work (each part rescales its own O and keeps its own sums) and registers (fewer CTAs per
+  // SM), so it stops where the CTAs fill the chip anyway.  8 KV heads, us, one warp per 16 rows / two / four.  Heads of 64: 16 rows 64 CTAs
+  // 54 / 32 / 23, 4096 345 / 208 / 155; 32 rows 288 CTAs 46 / 32 / 28, 512 48 / 36 / 42, 4096 280 / 210 / 249; 48 rows 288 CTAs 44 / 32, 512 46 / 50;
+  // 64 rows 288 42 / 34, 320 52 / 56.  Heads of 128: 16 rows 64 CTAs 79 / 48 / 30, 4096 1019 / 564 / 347; 32 rows 64 CTAs 54 / 36 / 26, 512
+  // 200 / 130 / 144, 4096 708 / 474 / 542; 64 rows 64 CTAs 44 / 34, 512 171 / 194, 4096 632 / 748.  Three further warps that do all the loading lost
+  // wherever there was more than a CTA per SM (48 rows, heads of 128, 4096 CTAs 1242 us against 740 with none).
   const long long ctas = (long long)grid.x * grid.y * grid.z;
-  const int ks = a.RT <= 32 && ctas <= 4 * 148 ? 4 : (a.RT <= 64 && ctas <= 148 ? 2 : 1);
+  int ks = 1;
+  if (a.RT <= 16) ks = 4;
+  else if (a.RT <= 32) ks = ctas <= (c.dh == 64 ? 2 * 148 : 148) ? 4 : 2;
+  else if (a.RT <= 64) ks = (c.dh == 64 ? ctas <= 2 * 148 : a.RT <= 48 || ctas <= 148) ? 2 : 1;
   const size_t ring = size_t(2) * NSTAGE * KT * c.dh * 2, parts = ks > 1 ? size_t(ks) * a.RT * (c.dh + 10) * 4 : 0;
   const size_t smem = size_t(a.RT) * c.dh * 2 + std::max(ring, parts);
-  const int threads = a.RT * 2 * ks + (ks > 1 || a.RT < 64 ? 96 : 0);      // three more warps that only load where few compute
+  const int threads = a.RT * 2 * ks;
   auto kernel = c.dh == 128 ? (ks == 4 ? attn_partial_kernel<128, 4> : ks == 2 ? attn_partial_kernel<128, 2> : attn_partial_kernel<128, 1>)
                             : (ks == 4 ? attn_partial_kernel<64, 4> : ks == 2 ? attn_partial_kernel<64, 2> : attn_partial_kernel<64, 1>);
   cudaError_t e = once_per_device(attr_done[c.dh == 128][ks / 2], [kernel](int) {

@@ -197,10 +197,12 @@ def test_attention_row_copies(hs, k, rep, window, chunk, dh, Hkv):
     _attention_against_fp64(hs, [0, 1, 31, 97, 128, 500, 1111], k, rep, window, chunk, dh, Hkv)
 
 
-# the mma.sync kernel's forms: four, two and one warps per 16 query rows, with and without warps that only load, on either side of the CTA counts
-# that choose between them (592 with up to 32 rows, 148 with up to 64); heads of 128 come here with pages that are not 16 tokens
-@pytest.mark.parametrize("dh,page,B,Hkv,k,rep", [(64, 16, 74, 8, 8, 4), (64, 16, 75, 8, 8, 4), (64, 16, 75, 8, 1, 1), (64, 16, 18, 8, 16, 4), (64, 16, 19, 8, 16, 4),
-                                                 (128, 32, 3, 2, 4, 4), (128, 8, 3, 2, 16, 4), (128, 8, 75, 8, 8, 4), (128, 5, 2, 2, 16, 8), (128, 1, 1, 1, 32, 16)])
+# the mma.sync kernel's forms: four, two and one warps per 16 query rows, on either side of the CTA counts that choose between them (8 KV heads,
+# one chunk: 37 | 38 requests with heads of 64, 18 | 19 with heads of 128); heads of 128 come here with pages that are not 16 tokens
+@pytest.mark.parametrize("dh,page,B,Hkv,k,rep", [(64, 16, 75, 8, 1, 1), (64, 16, 37, 8, 8, 4), (64, 16, 38, 8, 8, 4), (64, 16, 37, 8, 12, 4), (64, 16, 38, 8, 12, 4),
+                                                 (64, 16, 18, 8, 16, 4), (64, 16, 38, 8, 16, 4), (128, 32, 3, 2, 4, 4), (128, 8, 18, 8, 8, 4),
+                                                 (128, 128, 19, 8, 8, 4), (128, 8, 75, 8, 12, 4), (128, 8, 18, 8, 16, 4), (128, 64, 19, 8, 16, 4),
+                                                 (128, 5, 2, 2, 16, 8), (128, 1, 1, 1, 32, 16)])
 @pytest.mark.parametrize("window", [0, 40])
 def test_attention_warps_per_row(hs, dh, page, B, Hkv, k, rep, window):
     _attention_against_fp64(hs, [(37 * b + 61) % 129 for b in range(B)], k, rep, window, 256, dh, Hkv, page)
