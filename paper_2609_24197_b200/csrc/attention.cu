@@ -411,11 +411,12 @@ int visible_tokens(int max_ctx, int window) {
 
 }  // namespace
 
-int attn_pick_chunk(int B, int Hkv, int dh, int rows, int max_ctx, int window, int num_sms) {
+int attn_pick_chunk(int B, int Hkv, int dh, int page_size, int rows, int max_ctx, int window, int num_sms) {
   const int lmax = visible_tokens(max_ctx, window);
   const ChunkRule rule = chunk_rule(B, Hkv, dh, num_sms);
-  if (dh == 128 && window > 0 && lmax == window + 15) {
-    // Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
+  if (dh == 128 && page_size == 16 && window > 0 && lmax == window + 15) {
+    // (The tcgen05 kernel only, whose tiles are the unit of the costs below; by this rule the mma.sync kernel, heads of 128 on other pages,
+    // took 209 us where the general one takes 122: 11 requests, window 2048.)  Under a window the long requests all have the same few tiles, so what counts is how the rounds of equal items fill the SMs.
     // Cost of a round in tiles: the chunk's own, three for an item's set-up and read-out, one more for a partial and its merge.
     // 32 requests x 8 KV heads, window 2048 (256 items of 17 tiles on 148 SMs): one chunk 65.7 us, two 73.1, four 80.  Over windows of 512,
     // 2048 and 4096 tokens, 1 to 128 requests and 32 to 256 rows per KV head, the chunk this picks was the best of nine or within 13 %
@@ -453,9 +454,10 @@ size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, 
 }
 
 // A call with a smaller bound on its contexts can be cut into more chunks than one with the largest: below the window the rule is
-// another one, and a range of pieces x least tokens makes more chunks than a longer one whose chunks have grown.
+// another one, and a range of pieces x least tokens makes more chunks than a longer one whose chunks have grown.  (Pages of 16 tokens may
+// be cut by the rule for a window as well, others by the general rule alone: the size covers both.)
 size_t attn_workspace_bytes_any_ctx(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int num_sms) {
-  const int chunk = attn_pick_chunk(B, Hkv, dh, k * (Hq / Hkv), max_ctx, window, num_sms);
+  const int chunk = attn_pick_chunk(B, Hkv, dh, 16, k * (Hq / Hkv), max_ctx, window, num_sms);
   const int n = std::max(attn_max_chunks(max_ctx, window, chunk), chunk_rule(B, Hkv, dh, num_sms).max_chunks(visible_tokens(max_ctx, window)));
   return attn_bytes(B, k, Hq, Hkv, dh, n);
 }

@@ -85,7 +85,7 @@ Plan make_plan(const hspec_config& c, int B, int k, int max_ctx, bool any_ctx = 
   p.KB = take(M * size_t(c.Hkv) * c.dh * 2);
   p.VB = take(M * size_t(c.Hkv) * c.dh * 2);
   p.max_ctx = max_ctx;
-  p.attn_chunk = attn_pick_chunk(B, c.Hkv, c.dh, k * (c.Hq / c.Hkv), max_ctx, c.window, kNumSMs);
+  p.attn_chunk = attn_pick_chunk(B, c.Hkv, c.dh, c.page_size, k * (c.Hq / c.Hkv), max_ctx, c.window, kNumSMs);
   p.att_bytes = any_ctx ? attn_workspace_bytes_any_ctx(B, k, c.Hq, c.Hkv, c.dh, max_ctx, c.window, kNumSMs)
                         : attn_workspace_bytes(B, k, c.Hq, c.Hkv, c.dh, max_ctx, c.window, p.attn_chunk);
   p.ATT = take(p.att_bytes);
@@ -937,15 +937,15 @@ int hspec_op_qk_norm_rope(const float* qkv, const float* qw, const float* kw, co
   return HSPEC_OK;
 }
 
-static int resolve_chunk(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens) {
+static int resolve_chunk(int B, int k, int Hq, int Hkv, int dh, int page_size, int max_ctx, int window, int chunk_tokens) {
   if (chunk_tokens > 0) return ((chunk_tokens + 127) / 128) * 128;
-  return attn_pick_chunk(B, Hkv, dh, k * (Hq / Hkv), max_ctx, window, kNumSMs);
+  return attn_pick_chunk(B, Hkv, dh, page_size, k * (Hq / Hkv), max_ctx, window, kNumSMs);
 }
 
 size_t hspec_attention_workspace_bytes(int32_t B, int32_t k, int32_t Hq, int32_t Hkv, int32_t dh, int32_t max_ctx,
                                        int32_t window, int32_t chunk_tokens) {
   if (chunk_tokens <= 0) return attn_workspace_bytes_any_ctx(B, k, Hq, Hkv, dh, max_ctx, window, kNumSMs);
-  return attn_workspace_bytes(B, k, Hq, Hkv, dh, max_ctx, window, resolve_chunk(B, k, Hq, Hkv, dh, max_ctx, window, chunk_tokens));
+  return attn_workspace_bytes(B, k, Hq, Hkv, dh, max_ctx, window, resolve_chunk(B, k, Hq, Hkv, dh, 16, max_ctx, window, chunk_tokens));
 }
 
 int hspec_op_attention(const void* q, const void* kb, const void* vb, const void* k_pool, const void* v_pool,
@@ -963,7 +963,7 @@ int hspec_op_attention(const void* q, const void* kb, const void* vb, const void
   a.page_table_stride = page_table_stride; a.ctx_lens = ctx_lens;
   a.max_ctx = max_ctx > 0 ? max_ctx : page_table_stride * page_size;
   a.o = o; a.B = B; a.k = k; a.Hq = Hq; a.Hkv = Hkv; a.dh = dh; a.page_size = page_size; a.window = window;
-  a.chunk_tokens = resolve_chunk(B, k, Hq, Hkv, dh, a.max_ctx, window, chunk_tokens);
+  a.chunk_tokens = resolve_chunk(B, k, Hq, Hkv, dh, page_size, a.max_ctx, window, chunk_tokens);
   a.ws = workspace; a.ws_bytes = workspace_bytes;
   OP_TRY(attention_launch(a, reinterpret_cast<cudaStream_t>(stream), nullptr, &errtxt));
   return HSPEC_OK;

@@ -265,7 +265,7 @@ struct AttnPlan {
   int* count;
   int4* items;
 };
-int attn_pick_chunk(int B, int Hkv, int dh, int rows, int max_ctx, int window, int num_sms);   // rows: query rows per KV head
+int attn_pick_chunk(int B, int Hkv, int dh, int page_size, int rows, int max_ctx, int window, int num_sms);   // rows: query rows per KV head
 size_t attn_workspace_bytes(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int chunk_tokens);
 // The most any call with a bound of at most max_ctx and a chunk picked by the library needs.
 size_t attn_workspace_bytes_any_ctx(int B, int k, int Hq, int Hkv, int dh, int max_ctx, int window, int num_sms);

@@ -72,9 +72,18 @@ def test_workspace_covers_every_smaller_context_bound(lib, name, window, B, k):
 @pytest.mark.parametrize("window", [512, 2048, 4096])
 @pytest.mark.parametrize("B", [1, 2, 4, 8, 12, 24, 37])
 def test_chunks_under_a_window_count_row_tiles(lib, B, window):
-    chunk = lambda b, rows: lib._ZN5hspec15attn_pick_chunkEiiiiiii(b, 8, 128, rows, 20000, window, 148)
+    chunk = lambda b, rows: lib._ZN5hspec15attn_pick_chunkEiiiiiiii(b, 8, 128, 16, rows, 20000, window, 148)
     assert chunk(B, 256) == chunk(2 * B, 128) == chunk(2 * B, 7)
     assert chunk(B, 129) == chunk(B, 256)
+
+
+# that rule is for the kernel with 128-key tiles (heads of 128 on 16-token pages); on other pages a window is cut like a context of its length
+@pytest.mark.parametrize("B", [1, 4, 11, 30, 64])
+@pytest.mark.parametrize("page", [1, 8, 32, 128])
+def test_chunks_under_a_window_on_other_pages(lib, B, page):
+    chunk = lambda max_ctx, window: lib._ZN5hspec15attn_pick_chunkEiiiiiiii(B, 8, 128, page, 336, max_ctx, window, 148)
+    for window in (100, 300, 2048, 4096):
+        assert chunk(20000, window) == chunk(window + 15, 0)
 
 
 def test_no_cpu_path(lib):
