@@ -5,8 +5,9 @@
 // 152 064 and rank 256; it stays in the L2 for the next position) and the batch's logits rows (read, and written back when the
 // caller wants them).  As one GEMM and one reduction launch per position it took 47.6 + 8.9 us at 32 requests and that
 // vocabulary and 44 + 9.8 us at 96 requests and 32 000 rows: CTAs too short to fill their pipelines, a reduction network per
-// 16 columns, and a launch boundary on each side.  As one launch for all positions: 21 and 14 us per position (and 52 against 72 at
-// 128 requests and 152 064 rows, logits not written).
+// 16 columns, and a launch boundary on each side.  As one launch for all positions: 20 and 14 us per position (and 46 against 64 at
+// 128 requests and 152 064 rows, logits not written; with few rows to go over and 97 requests or more it is 12 us of gathers, barriers and
+// reductions a position, where two launches took 10).
 //
 // Here one cooperative kernel (one CTA per SM) walks the positions with a grid barrier between them:
 //   warp 16       producer: 64-column boxes of W_out (128 vocabulary rows each) through a ring of 16 KB stages; it does not
@@ -52,7 +53,7 @@ struct __align__(8) ChainTail {
   uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   uint64_t acc_full[2], acc_empty[2];
   uint64_t x_ready;
-  unsigned long long key[MAX_B];
+  unsigned long long key[4][MAX_B];   // per TMEM lane quarter
   int token[MAX_B];
   uint32_t tmem_base;
   uint32_t epi_abort;
@@ -113,7 +114,6 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
     tail->epi_abort = 0;
     fence_mbar_init();
   }
-  if (tid < MAX_B) tail->key[tid] = 0ull;
   if (warp == 17) {
     tmem_alloc(smem_u32(&tail->tmem_base), a.tmem_cols);
     tmem_relinquish();
@@ -210,6 +210,13 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
         step_row(src);
       }
     };
+    // With a single chunk in flight the others' lines are at least in the L2: a warp's 32 columns of a tile are 32 lines, one per lane.  (128
+    // requests, rank 256, us per position, logits not written / written, without -> with: V = 32 000 19.6 / 20.9 -> 17.2 / 18.3, 152 064 52 / 63 -> 46 / 52.)
+    auto prefetch_add = [&](int pos, int t) {
+      const int n = (cta + t * grid) * TILE_W + q * 32, c = (lane >> 3) * 32 + cg * 8 + (lane & 7);
+      if (n < a.Vd && c < a.B) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.logits + size_t(pos) * a.ld + n + size_t(c) * req_stride));
+    };
+    if (AQ < NCH) prefetch_add(0, 0);
 #pragma unroll
     for (int u = 0; u < AQ; ++u) load_add(u, 0, 0);
     gather([&](int b) { return a.last_token[b]; });
@@ -227,6 +234,7 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
         const bool n_ok = n < a.Vd;
         const bool more = t + 1 < n_my || pos + 1 < a.k;
         const int pos2 = t + 1 < n_my ? pos : pos + 1, t2 = t + 1 < n_my ? t + 1 : 0;
+        if (AQ < NCH && more) prefetch_add(pos2, t2);
         if (ok && !mbar_wait(smem_u32(&tail->acc_full[acc]), (gt >> 1) & 1, 6000000000ull)) {
           atomicExch(a.status, STATUS_TIMEOUT_EPILOGUE);
           ok = false;
@@ -282,14 +290,15 @@ markov_chain_kernel(const __grid_constant__ CUtensorMap tmW, ChainArgs a) {
         }
         int col;
         const unsigned long long m = max_over_lanes8(v, lane, col);
-        if ((lane & 3) == 0 && c0 + col < a.B) atomicMax(&tail->key[c0 + col], m);
+        if ((lane & 3) == 0) tail->key[q][c0 + col] = m;         // (one warp per quarter and chunk: written once a position)
       }
       if (!ok && lane == 0) *reinterpret_cast<volatile uint32_t*>(&tail->epi_abort) = 1;
       epi_sync();
       unsigned long long* gkeys = a.keys + size_t(pos % 3) * a.B;
       if (tid < a.B) {
-        const unsigned long long m = tail->key[tid];
-        tail->key[tid] = 0ull;
+        unsigned long long m = tail->key[0][tid];
+#pragma unroll
+        for (int i = 1; i < 4; ++i) m = m > tail->key[i][tid] ? m : tail->key[i][tid];
         if (m) atomicMax(gkeys + tid, m);
         __threadfence();
       }
