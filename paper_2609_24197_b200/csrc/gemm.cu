@@ -411,8 +411,9 @@ int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode) {
   // 4 17.6, 5 24.1; 96 tiles 2 23.8, 3 29.9.  Clusters of two still fit at 274 CTAs (137 tiles: 1 slice 26.9 us, 2 25.7, 3 31.7).
   int want = 256 * num_sms / 148 / tiles;
   if (want < 2 && 2 * tiles <= 276 * num_sms / 148) want = 2;
-  int max_by_k = k_tiles / 4;               // at least 4 K-tiles per slice
-  int s = want < max_by_k ? want : max_by_k;
+  // (down to one K-tile per slice: the cluster's read-out, a slice's share of the columns in turn, is longer than a short K loop, and it is more
+  // slices that shorten it.  K = 512, n_out = 256, 2 / 4 / 8 slices: 128 rows 18.4 / 11.8 / 9.2 us, 64 11.8 / 8.2 / 6.6, 16 6.6 / 5.6 / 5.1)
+  int s = want < k_tiles ? want : k_tiles;
   if (s > GEMM_MAX_SPLITS) s = GEMM_MAX_SPLITS;
   return s < 1 ? 1 : s;
 }
