@@ -58,14 +58,7 @@ struct ScanNorm {
 
 __device__ __forceinline__ float softplus_f(float v) { return v > 20.f ? v : log1pf(expf(v)); }
 
-// BLOCKS: blocks of an SM that the compiler has to leave registers for.  With one (128 registers, four blocks fit) more loads of a block
-// are in flight; with five it has 96.  Where the shared memory lets five or more blocks in and the grid fills the SMs more than four
-// times, the blocks make up for it and the second is faster, elsewhere the first (heads x requests, block 12 or 32; first / second):
-// P = 64, N = 20, 736 blocks 38.8 / 28.2 us, 640 of 32 positions 75.8 / 51.9; P = 128, N = 17, 736 blocks 45.1 / 37.1;
-// eight blocks of P = 64, N = 20 17.2 / 21.3; four to an SM (P = 64, N = 64) 736 blocks 74.5 / 93.2, 640 of 32 positions 197 / 212.
-template <int BLOCKS>
-__global__ void __launch_bounds__(SCAN_THREADS, BLOCKS)
-mamba_scan_kernel(ScanArgs a) {
+__device__ __forceinline__ void scan_general(const ScanArgs& a) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) float sm[];
@@ -179,6 +172,16 @@ mamba_scan_kernel(ScanArgs a) {
     }
   }
 }
+
+// The compiler's own choice: 128 registers, many loads of a block in flight, four blocks to an SM.
+__global__ void __launch_bounds__(SCAN_THREADS)
+mamba_scan_kernel(ScanArgs a) { scan_general(a); }
+
+// 96 registers, five blocks to an SM: 1.1 to 1.5 times slower over the same number of waves, but 593 to 740 blocks are one wave
+// instead of two.  Us, the kernel above / this one, 608 blocks of 8 positions: P = 64, N = 20 30.7 / 24.6, P = 24, N = 64 55.3 / 42.6,
+// P = 128, N = 24 36.9 / 32.8; 736 of 12, P = 64, N = 20 38.8 / 28.2; 1184 blocks of 8, P = 64, N = 20 38.9 / 47.1; 4480 of 4 90.1 / 103.
+__global__ void __launch_bounds__(SCAN_THREADS, 5)
+mamba_scan_five_kernel(ScanArgs a) { scan_general(a); }
 
 // ---------------------------------------------------------------------------------------------------
 // Small states (N <= 16: the paper's own drafter has N = 4).  The state of a channel fits in registers, so a thread owns one
@@ -923,23 +926,24 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   }
   const size_t smem = sizeof(float) * (size_t(KMAX) * c.P + 2 * size_t(KMAX) * c.N + KMAX * KMAX + 3 * KMAX +
                                        size_t(c.P) * a.NP);
-  // five blocks of an SM: each takes its shared memory and 1 KB of the 228 KB
-  const bool many = 5 * (smem + 1024) <= 228 * 1024 && size_t(a.H) * c.B > 4 * 148;
-  if (smem > 48 * 1024) {            // (never with `many`)
+  // one wave of five blocks to an SM, each with its shared memory and 1 KB of the 228 KB, where four would need two
+  const size_t blocks = size_t(a.H) * c.B;
+  const bool five = 5 * (smem + 1024) <= 228 * 1024 && blocks > 4 * 148 && blocks <= 5 * 148;
+  if (smem > 48 * 1024) {            // (never with `five`)
     // the largest size asked for so far, per device (the attribute is a per-device property of the function)
     static size_t smem_set[MAX_DEVICES] = {};
     const int dev = current_device();
     if (dev < 0) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(device_setup_mutex());
     if (smem > smem_set[dev]) {
-      cudaError_t e = cudaFuncSetAttribute(mamba_scan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+      cudaError_t e = cudaFuncSetAttribute(mamba_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
       if (e != cudaSuccess) { if (err) *err = "scan: state tile does not fit in shared memory"; return e; }
       smem_set[dev] = smem;
     }
   }
   dim3 grid(a.H, c.B);
   trk_begin(trk, "mamba_scan", 0, double(c.B) * a.H * c.P * c.N * 2);
-  const cudaError_t e = launch_pdl(many ? mamba_scan_kernel<5> : mamba_scan_kernel<1>, grid, dim3(SCAN_THREADS), smem, stream, a);
+  const cudaError_t e = launch_pdl(five ? mamba_scan_five_kernel : mamba_scan_kernel, grid, dim3(SCAN_THREADS), smem, stream, a);
   trk_end(trk);
   return e;
 }
