@@ -375,3 +375,38 @@ def test_low_rank_dt_in_the_scan(hs, Di, N, G, dt_rank, B, k, bf16):
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[20] * B)
     check_step(cfg, drafter, w, batch, k, requests=[0, B - 1], what=f"low rank {Di} {N} {dt_rank} {B}", **(dict(tol=5e-2) if bf16 else {}))
     drafter.close()
+
+
+# the tcgen05 scan (P = 64, N = 128): one tile of 16 positions and two, on both sides; one tile per CTA and enough of them that every ring goes round
+# several times; groups of two tiles, so that C changes with every other tile, and one group of all; x by TMA and, from rows that are no
+# multiples of 16 bytes, by plain loads; no state
+@pytest.mark.parametrize("B,k,H,G,ld_extra,state", [(1, 1, 4, 1, 0, True), (3, 15, 8, 2, 0, True), (41, 16, 64, 16, 0, True), (41, 17, 64, 16, 0, True),
+                                                    (75, 32, 32, 1, 0, True), (40, 9, 36, 3, 1, True), (40, 31, 36, 3, 2, True), (64, 5, 32, 2, 0, False)])
+def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
+    import numpy as np
+    from oracle import hspec_oracle as O
+    P, N = 64, 128
+    Di, d_xBC, f32 = H * P, H * P + 2 * G * N, torch.float32
+    ld = Di + d_xBC + H + ld_extra
+    zx = _rand((B * k, ld), 1, f32)
+    s0 = _rand((B, H, P, N), 3, torch.float16, 1.5) if state else None
+    conv_w, conv_b = _rand((d_xBC, 4), 4, f32, 0.3), _rand((d_xBC,), 5, f32, 0.02)
+    A_log, dt_bias, D = _rand((H,), 6, f32).abs(), _rand((H,), 7, f32) - 4.0, 1 + _rand((H,), 8, f32, 0.1)
+    y = torch.full((B * k, Di), float("nan"), device="cuda")
+    ws = torch.full((hs.hspec_scan_workspace_bytes(B, k, Di, N, G),), 255, dtype=torch.uint8, device="cuda")      # NaN wherever nothing is written
+    hs.hspec_op_mamba_scan(zx, None, s0, conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, 4, ws)
+    assert bool(torch.isfinite(y).all())
+    f64 = lambda t: t.double().cpu().numpy()
+    for b in sorted({0, 1 % B, B // 2, B - 1}):
+        rows = f64(zx[b * k:(b + 1) * k])
+        xBC = O.conv_silu(rows[:, Di:Di + d_xBC], f64(conv_w), f64(conv_b))
+        dt, a = O.discretise(rows[:, Di + d_xBC:Di + d_xBC + H], f64(dt_bias), f64(A_log))
+        S = f64(s0[b]) if state else np.zeros((H, P, N))
+        yy, _ = O.scan_sequential(S, xBC[:, :Di].reshape(k, H, P), xBC[:, Di:Di + G * N].reshape(k, G, N),
+                                  xBC[:, Di + G * N:].reshape(k, G, N), dt, a, f64(D))
+        ref = yy.reshape(k, Di) * O.silu(rows[:, :Di])
+        got = f64(y[b * k:(b + 1) * k])
+        # sums of 128 products with C in 22 bits and of 32 in fp32, SiLU and decay by the special-function unit (2^-22 relative each): together some
+        # 10 x 2^-22 of the terms' absolute sum, which is below 20 RMS; 1e-4 leaves a factor of two
+        assert np.abs(got - ref).max() <= 1e-4 * max(1.0, np.sqrt((ref ** 2).mean())), np.abs(got - ref).max()
+    assert hs.hspec_op_device_status()["rc"] == 0
