@@ -62,90 +62,122 @@ __device__ __forceinline__ const float4* tail_src(const GemmTail& t, const TailR
 }
 __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 
-// y = x / sqrt(mean(x^2) + eps) * w, one CTA per row, fp16 (or bf16) out.  VPT = 16-byte vectors a thread keeps in
-// registers between the two passes.  TAIL: the residual GEMM in front left the K-slices of its last wave's tiles unsummed; they are
-// added to x here, on the way (a launch of its own cost 6 us and a pass over x).
-template <int VPT, bool TAIL>
+// y = x / sqrt(mean(x^2) + eps) * w, fp16 (or bf16) out.  A CTA takes every gridDim.x-th row; VPT = 16-byte vectors of a row that a thread keeps
+// in registers between the two passes.
+// TAIL: the residual GEMM in front left the K-slices of its last wave's tiles unsummed; they are added to x here, on the way (a launch
+// of its own cost 6 us and a pass over x).  A warp's vector lies in one weight tile, so whether it has slices is uniform; where it has none
+// x is not written back, and where it has, all slices are under way together.  (With x written back everywhere and a slice fetched only after
+// the one before had come: 2048 rows of 5120, 12 of 160 tiles with six slices each, 41 us; now 26.)
+// AHEAD: the next row's loads go out before this one's sum is there.  It pays where a row takes 512 threads and an SM holds two CTAs (2048 rows of
+// 10240 35 -> 31 us, 1536 25 -> 21); shorter rows have five CTAs of other rows to hide behind (8192 rows of 4096 44 -> 52).
+template <int VPT, bool TAIL, bool AHEAD>
 __global__ void __launch_bounds__(512, 2) rmsnorm_kernel(float* __restrict__ x, const float* __restrict__ w, void* __restrict__ y,
-                               int n, float eps, GemmTail tail, uint32_t* status, int bf16_out) {
+                               int M, int n, float eps, GemmTail tail, uint32_t* status, int bf16_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
-  const TailRow tail_row = TAIL ? TailRow(tail, blockIdx.x) : TailRow();
-  float* xr = x + size_t(blockIdx.x) * n;
-  uint16_t* yr = reinterpret_cast<uint16_t*>(y) + size_t(blockIdx.x) * n;      // a row of 16-bit values, either type
-  if ((n & 3) == 0 && n <= 4 * VPT * int(blockDim.x)) {
-    // 16-byte loads, the row stays in registers between the two passes
-    float4 v[VPT];
-    const int nv = n >> 2;
+  const bool vec = (n & 3) == 0 && n <= 4 * VPT * int(blockDim.x);
+  const int nv = n >> 2;
+  float4 next[AHEAD ? VPT : 1];
+  auto load_row = [&](float4 (&v)[VPT], int m) {
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int d4 = threadIdx.x + i * blockDim.x;
+      v[i] = d4 < nv ? reinterpret_cast<const float4*>(x + size_t(m) * n)[d4] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if constexpr (AHEAD)
+    if (vec) load_row(next, blockIdx.x);
+  for (int m = blockIdx.x; m < M; m += gridDim.x) {
+    float* xr = x + size_t(m) * n;
+    uint16_t* yr = reinterpret_cast<uint16_t*>(y) + size_t(m) * n;             // a row of 16-bit values, either type
+    if (vec) {
+      // 16-byte loads, the row stays in registers between the two passes
+      float4 v[VPT];
+      float ss = 0.f;
+      if constexpr (TAIL) {
+        load_row(v, m);
+        const TailRow tail_row(tail, m);
+        // each element is (0 + slice 0 + slice 1 ..) added to x
+        const size_t step = size_t(tail.BNT) * 64;
+        if (tail.splits <= 2) {
+          constexpr int U = 3;                                 // three vectors' two slices in flight
+          static_assert(VPT % U == 0, "vectors are taken in threes");
+#pragma unroll
+          for (int i0 = 0; i0 < VPT; i0 += U) {
+            const float4* src[U];
+            float4 p0[U], p1[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+              const int d4 = threadIdx.x + (i0 + i) * blockDim.x;
+              src[i] = d4 < nv ? tail_src(tail, tail_row, d4 * 4) : nullptr;
+              p0[i] = src[i] ? __ldcs(src[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
+              p1[i] = src[i] && tail.splits > 1 ? __ldcs(src[i] + step) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+              if (src[i] == nullptr) continue;
+              add4(p0[i], p1[i]);
+              add4(v[i0 + i], p0[i]);
+              reinterpret_cast<float4*>(xr)[threadIdx.x + (i0 + i) * blockDim.x] = v[i0 + i];
+            }
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < VPT; ++i) {
+            const int d4 = threadIdx.x + i * blockDim.x;
+            const float4* src = d4 < nv ? tail_src(tail, tail_row, d4 * 4) : nullptr;
+            if (src == nullptr) continue;
+            float4 p[8];
+#pragma unroll
+            for (int sp = 0; sp < 8; ++sp) p[sp] = sp < tail.splits ? __ldcs(src + sp * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int sp = 1; sp < 8; ++sp)
+              if (sp < tail.splits) add4(p[0], p[sp]);
+            add4(v[i], p[0]);
+            reinterpret_cast<float4*>(xr)[d4] = v[i];
+          }
+        }
+      } else if constexpr (AHEAD) {
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) v[i] = next[i];
+        if (m + int(gridDim.x) < M) load_row(next, m + gridDim.x);
+      } else {
+        load_row(v, m);
+      }
+#pragma unroll
+      for (int i = 0; i < VPT; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+      const float inv = rsqrtf(block_sum(ss, red) / float(n) + eps);
+#pragma unroll
+      for (int i = 0; i < VPT; ++i) {
+        const int d4 = threadIdx.x + i * blockDim.x;
+        if (d4 < nv) {
+          // (fetching the gains together with the row, before the block-wide sum, measured slower: 27 against 23 us)
+          const float4 g = reinterpret_cast<const float4*>(w)[d4];
+          store_norm4(yr, d4, v[i], inv, g, bf16_out, status);
+        }
+      }
+      continue;
+    }
+    if constexpr (TAIL) {                             // (n is a multiple of four: the host sees to it)
+      const TailRow tail_row(tail, m);
+      for (int d4 = threadIdx.x; d4 < nv; d4 += blockDim.x) {
+        float4 v = reinterpret_cast<const float4*>(xr)[d4];
+        if (const float4* src = tail_src(tail, tail_row, d4 * 4)) {
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int sp = 0; sp < tail.splits; ++sp) add4(acc, __ldcs(src + size_t(sp) * tail.BNT * 64));
+          add4(v, acc);
+        }
+        reinterpret_cast<float4*>(xr)[d4] = v;
+      }
+      __syncthreads();
+    }
     float ss = 0.f;
-#pragma unroll
-    for (int i = 0; i < VPT; ++i) {
-      const int d4 = threadIdx.x + i * blockDim.x;
-      v[i] = d4 < nv ? reinterpret_cast<const float4*>(xr)[d4] : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (TAIL) continue;
-      ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
-    }
-    if (TAIL) {
-      // three vectors at a time (64 registers: four blocks per SM), slice after slice with the three loads of a slice in flight
-      // together; each element is (0 + slice 0 + slice 1 ..) added to x
-      static_assert(VPT % 3 == 0, "vectors are taken in threes");
-#pragma unroll
-      for (int i0 = 0; i0 < VPT; i0 += 3) {
-        const float4* src[3];
-        float4 acc[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const int d4 = threadIdx.x + (i0 + i) * blockDim.x;
-          src[i] = d4 < nv ? tail_src(tail, tail_row, d4 * 4) : nullptr;
-          acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (int sp = 0; sp < tail.splits; ++sp) {
-          float4 part[3];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) part[i] = src[i] ? __ldcs(src[i] + size_t(sp) * tail.BNT * 64) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int i = 0; i < 3; ++i) add4(acc[i], part[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const int d4 = threadIdx.x + (i0 + i) * blockDim.x;
-          float4& x4 = v[i0 + i];
-          add4(x4, acc[i]);
-          if (d4 < nv) reinterpret_cast<float4*>(xr)[d4] = x4;
-          ss += x4.x * x4.x + x4.y * x4.y + x4.z * x4.z + x4.w * x4.w;
-        }
-      }
-    }
-    const float inv = rsqrtf(block_sum(ss, red) / float(n) + eps);
-#pragma unroll
-    for (int i = 0; i < VPT; ++i) {
-      const int d4 = threadIdx.x + i * blockDim.x;
-      if (d4 < nv) {
-        // (fetching the gains together with the row, before the block-wide sum, measured slower: 27 against 23 us)
-        const float4 g = reinterpret_cast<const float4*>(w)[d4];
-        store_norm4(yr, d4, v[i], inv, g, bf16_out, status);
-      }
-    }
-    return;
+    for (int d = threadIdx.x; d < n; d += blockDim.x) { const float v = xr[d]; ss += v * v; }
+    const float tot = block_sum(ss, red);
+    const float inv = rsqrtf(tot / float(n) + eps);
+    for (int d = threadIdx.x; d < n; d += blockDim.x) store_act16(yr, d, xr[d] * inv * w[d], bf16_out != 0, status);
   }
-  if (TAIL) {                                       // (n is a multiple of four: the host sees to it)
-    for (int d4 = threadIdx.x; d4 < (n >> 2); d4 += blockDim.x) {
-      float4 v = reinterpret_cast<const float4*>(xr)[d4];
-      if (const float4* src = tail_src(tail, tail_row, d4 * 4)) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int sp = 0; sp < tail.splits; ++sp) add4(acc, __ldcs(src + size_t(sp) * tail.BNT * 64));
-        add4(v, acc);
-      }
-      reinterpret_cast<float4*>(xr)[d4] = v;
-    }
-    __syncthreads();
-  }
-  float ss = 0.f;
-  for (int d = threadIdx.x; d < n; d += blockDim.x) { const float v = xr[d]; ss += v * v; }
-  const float tot = block_sum(ss, red);
-  const float inv = rsqrtf(tot / float(n) + eps);
-  for (int d = threadIdx.x; d < n; d += blockDim.x) store_act16(yr, d, xr[d] * inv * w[d], bf16_out != 0, status);
 }
 
 // Block rows: row 0 of each request is the embedding of its last token, rows 1..k-1 the mask-token embedding; no positional
@@ -456,8 +488,10 @@ cudaError_t rmsnorm_launch(float* x, const float* w, void* y_16, int M, int n, f
   const int threads = n <= 4 * 6 * 256 ? 256 : 512;
   const bool pending = tail != nullptr && tail->part != nullptr;
   if (pending && (n & 3)) return cudaErrorInvalidValue;
-  cudaError_t e = launch_pdl(pending ? rmsnorm_kernel<6, true> : rmsnorm_kernel<6, false>, dim3(M), dim3(threads), 0, stream, x, w, y_16, n, eps,
-                             pending ? *tail : GemmTail{}, status, bf16_out ? 1 : 0);
+  const bool ahead = !pending && threads == 512 && M > 2 * 148;
+  auto kernel = pending ? rmsnorm_kernel<6, true, false> : ahead ? rmsnorm_kernel<6, false, true> : rmsnorm_kernel<6, false, false>;
+  cudaError_t e = launch_pdl(kernel, dim3(ahead ? 2 * 148 : M), dim3(threads), 0, stream, x, w, y_16, M, n, eps, pending ? *tail : GemmTail{}, status,
+                             bf16_out ? 1 : 0);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

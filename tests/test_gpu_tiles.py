@@ -410,3 +410,18 @@ def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
         # 10 x 2^-22 of the terms' absolute sum, which is below 20 RMS; 1e-4 leaves a factor of two
         assert np.abs(got - ref).max() <= 1e-4 * max(1.0, np.sqrt((ref ** 2).mean())), np.abs(got - ref).max()
     assert hs.hspec_op_device_status()["rc"] == 0
+
+
+# the norm of wide rows, where a CTA fetches its next row ahead: one row per CTA and several, row lengths around 6144 (256 or 512 threads) and
+# 12 288 (the row no longer fits the registers), one that is no multiple of four
+@pytest.mark.parametrize("M", [1, 296, 297, 593])
+@pytest.mark.parametrize("n", [6144, 6148, 8192, 12288, 12292, 7001])
+def test_rmsnorm_rows_ahead(hs, M, n):
+    x, w = _rand((M, n), 1, torch.float32, 3.0), 1 + _rand((n,), 2, torch.float32, 0.1)
+    y = torch.full((M, n), float("nan"), dtype=torch.float16, device="cuda")
+    before = x.clone()
+    hs.hspec_op_rmsnorm(x, w, y, 1e-6)
+    ref = x.double() / torch.sqrt((x.double() ** 2).mean(1, keepdim=True) + 1e-6) * w.double()
+    # one fp16 rounding (2^-11 of the value) and a few fp32 ones
+    assert bool(((y.double() - ref).abs() <= ref.abs() * 2.0 ** -10.9 + 1e-6).all())
+    assert torch.equal(x, before)
