@@ -408,4 +408,9 @@ __device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
   u = (u & 0x80000000u) ? ~u : u | 0x80000000u;
   return (static_cast<unsigned long long>(u) << 32) | (0xffffffffu - uint32_t(idx));
 }
+// The value of a key; -infinity for the zero key.
+__device__ __forceinline__ float argmax_key_value(unsigned long long key) {
+  const uint32_t u = uint32_t(key >> 32);
+  return key == 0ull ? -INFINITY : __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
+}
 }  // namespace hspec

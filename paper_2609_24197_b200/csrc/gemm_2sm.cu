@@ -61,15 +61,14 @@ struct Gemm2Args {
   uint32_t* status;
 };
 
-struct __align__(8) Tail2 {
+struct __align__(16) Tail2 {
   uint64_t full[GEMM_MAX_STAGES];
   uint64_t empty[GEMM_MAX_STAGES];
   uint64_t tmem_full[2];
   uint64_t tmem_empty[2];
   uint32_t tmem_base;
   uint32_t abort_flag;
-  float red_val[4][256];
-  int red_idx[4][256];
+  float4 best[EPI_WARPS][32];   // LM head: what each column of a warp's share has to reach to matter
 };
 
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
@@ -264,6 +263,17 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       int tn, tm;
       g.raster.tile_at(tile, tn, tm);
       const int mode = sp >= 0 ? EPI_PARTIAL_F32 : g.mode;
+      if (mode == EPI_ARGMAX) {
+        // The rows' maxima over the tiles that are done by now, asked for while this one is still computed.  They only grow, so an older value costs
+        // a reduction too many at worst.
+        float* best = reinterpret_cast<float*>(tail->best[warp - 2]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int c = ((warp - 2) >> 2) * 16 + (2 * i + (lane >> 4)) * 32 + (lane & 15), m = tm * g.BNT + c;
+          best[i * 32 + lane] = c < g.BNT && m < g.M ? argmax_key_value(__ldcg(g.keys + m)) : INFINITY;
+        }
+        __syncwarp();
+      }
       const uint32_t acc = tile_count & 1, use = tile_count >> 1;
       if (!mbar_wait(smem_u32(&tail->tmem_full[acc]), use & 1)) {
         atomicExch(g.status, STATUS_TIMEOUT_EPILOGUE);
@@ -277,7 +287,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const int m0 = tm * g.BNT;
       const uint32_t tmem_acc = tmem_base + acc * g.acc_cols + (uint32_t(q * 32) << 16);
       for (int c0 = ((warp - 2) >> 2) * 16; c0 < g.BNT; c0 += EPI_WARPS * 4) {
-        if (m0 + c0 >= g.M && mode != EPI_ARGMAX) break;    // rows past M: nothing to store (warp-uniform)
+        if (m0 + c0 >= g.M) break;                          // rows past M: nothing to store (warp-uniform)
         uint32_t r[16];
         tmem_ld16(tmem_acc + uint32_t(c0), r);
         tmem_ld_wait();
@@ -323,45 +333,40 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __float2bfloat16_rn(__uint_as_float(r[j]));
           }
         } else {  // EPI_ARGMAX
-          float v[16];
-          int vi[16];
+          // A lane that does not reach its row's maximum so far has nothing to say about the arg-max, and after the first few of a
+          // row's tiles hardly one does: the reduction network (64 shuffles for 16 rows) runs for the few groups with one that reaches it.  (For
+          // every group it cost the LM head 4 %, mostly as clock under the power cap; one redux.sync maximum + ballot per column more still.)
+          const float4* best = tail->best[warp - 2] + (c0 >> 5) * 4;
+          bool reached = false;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            const float x = __uint_as_float(r[j]);
-            if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
-            v[j] = argmax_value(x, n_ok);
-            vi[j] = n;
+          for (int j = 0; j < 16; j += 4) {
+            const float4 t = best[j >> 2];
+            const float tj[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int m = m0 + c0 + j + e;
+              const float x = __uint_as_float(r[j + e]);
+              if (g.logits != nullptr && n_ok && m < g.M) g.logits[size_t(m) * g.ldo + n] = x;
+              reached |= !(x < tj[e]);
+            }
           }
-          // (The network costs the LM head 4 % - 2.34 -> 2.24 ms per step without it - mostly as clock under the power cap.
-          // One redux.sync maximum + ballot per column instead of the shuffle rounds: 2.56 ms.)
-          int row = 0;
-          warp_argmax16(v, vi, lane, row);
-          if ((lane & 1) == 0) { tail->red_val[q][c0 + row] = v[0]; tail->red_idx[q][c0 + row] = vi[0]; }
+          if (__any_sync(0xffffffffu, reached && n_ok)) {
+            float v[16];
+            int vi[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) { v[j] = argmax_value(__uint_as_float(r[j]), n_ok); vi[j] = n; }
+            int row = 0;
+            warp_argmax16(v, vi, lane, row);
+            const int m = m0 + c0 + row;
+            if ((lane & 1) == 0 && m < g.M && vi[0] < g.N_out && !(v[0] < reinterpret_cast<const float*>(best)[row]))
+              atomicMax(g.keys + m, argmax_key(v[0], vi[0]));
+          }
         }
       }
       // accumulator drained: hand it back to the MMA issuer in the leader CTA
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc ? empty_leader1 : empty_leader0);
-      if (mode == EPI_ARGMAX) {
-        asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
-        const int t = threadIdx.x - 64;
-        for (int c = t; c < g.BNT; c += EPI_THREADS) {
-          const int m = m0 + c;
-          if (m >= g.M || tile_n128 * 128 >= g.N_out) continue;   // the pair's second half may lie wholly past V
-          float v = tail->red_val[0][c];
-          int idx = tail->red_idx[0][c];
-#pragma unroll
-          for (int qq = 1; qq < 4; ++qq) {
-            const float ov = tail->red_val[qq][c];
-            const int oi = tail->red_idx[qq][c];
-            if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-          }
-          if (idx != 0x7fffffff) atomicMax(g.keys + m, argmax_key(v, idx));
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");        // red_* is reused by the next tile
-      }
     }
   }
   tc_fence_before();
