@@ -425,3 +425,37 @@ def test_rmsnorm_rows_ahead(hs, M, n):
     # one fp16 rounding (2^-11 of the value) and a few fp32 ones
     assert bool(((y.double() - ref).abs() <= ref.abs() * 2.0 ** -10.9 + 1e-6).all())
     assert torch.equal(x, before)
+
+
+# the pair GEMM's wide tiles (257 to 512 activation rows, two instructions): every width in steps of 32 with as many rows as it holds and with one
+# more than the width before, a last weight tile that is part full, K that ends in a part k-step, one slice and three to six, two wide tiles
+@pytest.mark.parametrize("M,n_out,K", [(257, 17000, 520), (288, 17000, 512), (289, 17000, 72), (352, 17000, 128), (353, 17000, 192), (416, 17000, 64), (417, 17000, 512),
+                                       (480, 17000, 512), (481, 17000, 8), (512, 17408, 256), (257, 5000, 4096), (270, 4096, 4096), (257, 2560, 4096),
+                                       (549, 4096, 8192)])
+@pytest.mark.parametrize("kind,out", [(torch.float16, torch.float32), (torch.float16, torch.float16), (torch.bfloat16, torch.bfloat16), (torch.float16, "add")])
+def test_wide_gemm_tiles(hs, M, n_out, K, kind, out):
+    x, W = _rand((M, K), 1, kind), _rand((n_out, K), 2, kind, 0.05)
+    add = out == "add"
+    y = _rand((M, n_out), 3, torch.float32) if add else torch.full((M, n_out), float("nan"), dtype=out, device="cuda")
+    ref = x.double() @ W.double().t() + (y.double() if add else 0.)
+    # every partial sum of K products is rounded to fp32 (2^-24): K / 64 roundings per element in a chain at most, here taken as 64; and the store's
+    # rounding
+    terms = x.double().abs() @ W.double().abs().t() + (y.double().abs() if add else 0.)
+    store = {torch.float16: 2.0 ** -11, torch.bfloat16: 2.0 ** -8}.get(out, 2.0 ** -23)
+    ws = torch.full((hs.hspec_gemm_workspace_bytes(M, n_out, K),), 255, dtype=torch.uint8, device="cuda")
+    hs.hspec_op_gemm(x, W, y, accumulate=add, workspace=ws)
+    assert bool(((y.double() - ref).abs() <= terms * 2.0 ** -18 + ref.abs() * store + 1e-7).all())
+    assert hs.hspec_op_device_status()["rc"] == 0
+
+
+# the SwiGLU epilogue of a wide tile, with 300 and 512 rows
+@pytest.mark.parametrize("B,k", [(30, 10), (16, 32)])
+def test_wide_gemm_tiles_with_swiglu(hs, B, k):
+    import synth
+    from harness import check_step, cuda_setup
+    cfg = synth.derived(dict(D=256, n_fuse=1, r=64, L=1, has_attn=[0], kv_slot=[-1], n_slots=0, Di=512, P=64, N=4, G=1, d_conv=4, dt_rank=0,
+                             Hq=2, Hkv=1, dh=64, rope_theta=1.0e4, window=0, qk_norm=1, F=8512, V=300, rms_eps=1e-6, page_size=16, name="wide",
+                             B=B, k=k, ctx=("const", 16, 16)))
+    drafter, w, batch = cuda_setup(cfg, ctx_lens=[16] * B)
+    check_step(cfg, drafter, w, batch, k, requests=[0, B // 2, B - 1], what=f"wide {B}")
+    drafter.close()
