@@ -667,7 +667,7 @@ def case_scan(reps, B=32, Di=8192):
     torch.cuda.synchronize()
     us = [round(ev[i].elapsed_time(ev[i + 1]) * 1e3, 1) for i in range(reps)]
     print(f"scan: B={B} H={H} S_init bytes per launch={B * H * P * N * 2} activation bytes (z, xBC, dt in; y out)="
-          f"{B * k * (ld + Di) * 4} us per call (conv + stream)={us}")
+          f"{B * k * (ld + Di) * 4} us per call (both kernels)={us}")
 
 
 def case_rowwise(reps, M=2048, D=5120, Hq=64, Hkv=8, dh=128, k=16):
