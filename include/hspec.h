@@ -310,7 +310,7 @@ int hspec_op_rmsnorm(const float* x, const float* w, void* y_f16, int32_t M, int
  *   dt_raw fp32 [B*k, H] or NULL;  s_init fp16 [B, H, P, N] or NULL (zero state)
  *   y_gated fp32 [B*k, Di] = (scan output) * SiLU(z).
  *   workspace: optional device scratch of hspec_scan_workspace_bytes(...) bytes (256-byte aligned); with it the serving
- *   shapes (P = 64, N = 128) run as two kernels (B, C, their products and dt; the rest on tcgen05), without it as one. */
+ *   shapes (P = 64, N = 128) run as two kernels (conv with the C.B table, state stream), without it as one fused kernel. */
 int hspec_op_mamba_scan(const float* zxbcdt, int64_t ld_in, const float* dt_raw, const void* s_init,
                         const float* conv_w, const float* conv_b, const float* dt_bias, const float* A_log,
                         const float* Dskip, float* y_gated, int32_t B, int32_t k, int32_t Di, int32_t P,

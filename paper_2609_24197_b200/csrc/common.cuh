@@ -50,15 +50,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// x / (1 + 2^(-x log2 e)) on the special-function unit: exponential and reciprocal, about an ulp each, far inside every tolerance that follows an fp16
-// or bf16 rounding.  The flush-to-zero forms have no range fix-up around them (__expf and __fdividef do, twice the instructions); below 2^-126
-// there is nothing to keep, and past +-88 the exponential is 0 or infinite either way.
-__device__ __forceinline__ float silu_f(float v) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(v * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-  return v * r;
-}
+// (fast exponential and fast division: ~2 ulp each, far inside every tolerance that follows an fp16 or bf16 rounding)
+__device__ __forceinline__ float silu_f(float v) { return __fdividef(v, 1.0f + __expf(-v)); }
 
 // Stores v into a 16-bit activation buffer: fp16 with saturation (counted), or bf16 (fp32's range: nothing to clamp).
 __device__ __forceinline__ void store_act16(void* base, size_t idx, float v, bool bf16, uint32_t* status) {
@@ -355,22 +348,6 @@ __device__ __forceinline__ void mma_f16_16816(float (&c)[4], const uint32_t (&a)
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// Loads that stay where they are written (behind a wait under a condition); the first for what is read once and needs no place in the L1.
-__device__ __forceinline__ float ld_stream(const float* p) {
-  float v;
-  asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ float ld_f1(const float* p) {
-  float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ float4 ld_f4(const float* p) {
-  float4 v;
-  asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
-  return v;
 }
 // one 32-byte read-only load (sm_100: 256-bit global loads); p must be 32-byte aligned
 __device__ __forceinline__ void ldg_nc_32B(const void* p, uint4& lo, uint4& hi) {

@@ -391,23 +391,6 @@ bool make_tmap_16bit_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t
   return true;
 }
 
-// 2-D fp32 row-major [rows, cols] tensor without gaps between its rows, box [box_rows x box_cols], no swizzle.
-bool make_tmap_f32_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int box_cols, int box_rows, std::string* err) {
-  EncodeTiledFn enc = get_encode();
-  if (!enc) { if (err) *err = "cuTensorMapEncodeTiled is not available from the CUDA driver"; return false; }
-  cuuint64_t dims[2] = {cuuint64_t(cols), cuuint64_t(rows)};
-  cuuint64_t strides[1] = {cuuint64_t(cols) * 4};
-  cuuint32_t box[2] = {cuuint32_t(box_cols), cuuint32_t(box_rows)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    if (err) *err = "cuTensorMapEncodeTiled failed with CUresult " + std::to_string(int(r));
-    return false;
-  }
-  return true;
-}
-
 int gemm_pick_bn(int M) {
   if (M >= 256) return 256;
   return ((M + 15) / 16) * 16;

@@ -918,8 +918,6 @@ int hspec_op_mamba_scan(const float* zxbcdt, int64_t ld_in, const float* dt_raw,
   sc.dt_bias = dt_bias; sc.A_log = A_log; sc.Dskip = Dskip; sc.y_gated = y_gated;
   sc.B = B; sc.k = k; sc.Di = Di; sc.P = P; sc.N = N; sc.G = G; sc.d_conv = d_conv;
   sc.ws = workspace; sc.ws_bytes = workspace_bytes;
-  sc.status = global_status();
-  if (!sc.status) return fail(nullptr, HSPEC_ERR_CUDA, "hspec_op_mamba_scan: cannot allocate the status word");
   OP_TRY(scan_launch(sc, reinterpret_cast<cudaStream_t>(stream), nullptr, &errtxt));
   return HSPEC_OK;
 }

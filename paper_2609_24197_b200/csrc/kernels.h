@@ -201,7 +201,6 @@ struct GemmCall {       // host-side description of one y = x W^T
 
 bool make_tmap_16bit_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int64_t ld_elems,
                        int box_rows, bool f16, std::string* err);
-bool make_tmap_f32_2d(CUtensorMap* tm, const void* base, int64_t rows, int64_t cols, int box_cols, int box_rows, std::string* err);
 int gemm_pick_bn(int M);
 int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode = EPI_STORE_F32);
 cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);

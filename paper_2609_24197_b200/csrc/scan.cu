@@ -501,10 +501,14 @@ mamba_scan_mma_kernel(ScanArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------------
-// The serving shapes with scratch, as two kernels:
-//   scan_prep_kernel   per request and group: conv + SiLU of the B and C channels, C as fp16 head + fp16 remainder in the form of a tensor-core
-//                      operand tile, C_t . B_s in fp32; dt and the prefix sums of dt A of the group's heads
-//   scan_tc_kernel     state term of two heads at a time on tcgen05; conv of x, intra-block term, skip and gate with one thread per channel
+// Two-kernel form of the fast path (used when the caller provides scratch): the small per-position
+// operands are prepared once per request and group, so the kernel that streams S_init has no
+// block-wide phases in front of its loads.
+//   scan_conv_kernel   causal depthwise conv + SiLU of every xBC channel (thread = 4 channels x 4 positions); for the B and C channels
+//                      of a group one block does all positions, writes C as fp16 head + fp16 remainder for the tensor-core
+//                      contraction and CB[b, g, t, s] = C_t . B_s for s <= t
+//   mamba_scan_stream_kernel  one warp per head: everything it needs is fetched up front (cp.async for the
+//                      shared operands, 32-byte loads of S_init straight into the MMA fragments)
 constexpr int CONV_ROWS = 4;                                 // block positions per thread
 // thread = (VEC adjacent channels, group of four block positions): the filter reads raw inputs only, so the groups are
 // independent; a thread's seven (vector) loads are in flight together and it needs few registers.  VEC = 4 (16-byte
@@ -551,85 +555,52 @@ __device__ __forceinline__ void conv_rows(const ScanArgs& a, int b, int i0, int 
       out[r][v] = silu_f(bias[v] + w[v][0] * in[r][v] + w[v][1] * in[r + 1][v] + w[v][2] * in[r + 2][v] + w[v][3] * in[r + 3][v]);
 }
 
-// Where the prepared operands lie in the scratch (rows = block positions padded to 16 or 32).
-struct ScanPrep {
-  uint8_t* c;     // [B][G][head, remainder][2 halves of 64 n] tiles of [rows x 64] fp16, K-major, 128-byte swizzle
-  float* cb;      // [B][G] C_t . B_s, quads of neighbouring s up to the diagonal, row after row (tri_quad); zero for s > t and for t >= k
-  float* dt;      // [B][H][rows], zero past k
-  float* cum;     // [B][H][rows]
-};
-
-// Quads (t; 4 s4 .. 4 s4 + 3) of a lower triangle, row after row: row t has t / 4 + 1 of them.
-__host__ __device__ constexpr int tri_quad(int t, int s4) { return 2 * (t / 4) * (t / 4 + 1) + (t & 3) * (t / 4 + 1) + s4; }
-__host__ __device__ constexpr int tri_quads(int rows) { return tri_quad(rows, 0); }
-
-// Blocks x < G: B, C and their products of a group; x >= G: dt of eight warps' heads, one to four each.  (As part
-// of a kernel that also activated x and wrote it back for the scan to read: 184 us at 256 requests of 32 positions, 128 heads.)  The
-// rows are padded by four floats so that the 16-byte reads of a warp's threads spread over the banks.
-template <int VEC, int MT>
+// Blocks x < G: the B and C channels of one group and, from shared memory, their products CB (a launch of its own before that read
+// both back from memory: conv 8 us + CB 4 us at 32 requests of the 8B-class shapes, k = 16).  The rows are padded by four floats
+// so that the 16-byte reads of a warp's threads spread over the banks.  Blocks x >= G: 256 VEC channels of x at CONV_ROWS positions.
+template <int VEC>
 __global__ void __launch_bounds__(256)
-scan_prep_kernel(ScanArgs a, ScanPrep sp, int heads_per_warp) {
-  constexpr int N = 128, LDR = N + 4, ROWS = MT * 16, HW = 4;
-  extern __shared__ __align__(16) float cb_sm[];
-  const int k = a.k, n_grp = (k + CONV_ROWS - 1) / CONV_ROWS, g = blockIdx.x, b = blockIdx.y, GN = a.G * N;
-  if (!a.w_stable) { pdl_wait(); pdl_trigger(); }
-  if (g >= a.G) {
-    // a lane per position; what the weights give before the wait for the kernel in front
-    const int lane = threadIdx.x & 31, h0 = ((g - a.G) * 8 + (threadIdx.x >> 5)) * heads_per_warp;
-    float bias[HW], A[HW], raw[HW];
+scan_conv_kernel(ScanArgs a, float* __restrict__ xact, __half* __restrict__ c16, float* __restrict__ cb) {
+  pdl_wait();
+  pdl_trigger();
+  const int k = a.k, N = a.N, n_grp = (k + CONV_ROWS - 1) / CONV_ROWS;
+  const int b = blockIdx.y / n_grp, grp = blockIdx.y % n_grp;
+  const size_t row0 = size_t(b) * k;
+  float o[CONV_ROWS][VEC];
+  if (int(blockIdx.x) >= a.G) {
+    const int ch = ((blockIdx.x - a.G) * 256 + threadIdx.x) * VEC, i0 = grp * CONV_ROWS;
+    if (ch >= a.Di) return;
+    conv_rows<VEC>(a, b, i0, ch, o);
 #pragma unroll
-    for (int i = 0; i < HW; ++i) {
-      const bool on = i < heads_per_warp && h0 + i < a.H;
-      bias[i] = on ? a.dt_bias[h0 + i] : 0.f;
-      A[i] = on ? -expf(a.A_log[h0 + i]) : 0.f;
-    }
-    if (a.w_stable) { pdl_wait(); pdl_trigger(); }
-#pragma unroll
-    for (int i = 0; i < HW; ++i) raw[i] = i < heads_per_warp && h0 + i < a.H && lane < k ? a.dt_pre(b, lane, h0 + i) : 0.f;
-#pragma unroll
-    for (int i = 0; i < HW; ++i) {
-      if (i >= heads_per_warp || h0 + i >= a.H) break;         // (the same for the warp)
-      const float dt = lane < k ? softplus_f(raw[i] + bias[i]) : 0.f;
-      float cum = dt * A[i];
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float up = __shfl_up_sync(0xffffffffu, cum, off);
-        if (lane >= off) cum += up;
-      }
-      if (lane < ROWS) {
-        sp.dt[(size_t(b) * a.H + h0 + i) * ROWS + lane] = dt;
-        sp.cum[(size_t(b) * a.H + h0 + i) * ROWS + lane] = cum;
-      }
+    for (int r = 0; r < CONV_ROWS; ++r) {
+      if (i0 + r >= k) break;
+      float* dst = xact + (row0 + i0 + r) * a.Di + ch;
+      if (VEC == 4) *reinterpret_cast<float4*>(dst) = make_float4(o[r][0], o[r][VEC > 1 ? 1 : 0], o[r][VEC > 1 ? 2 : 0], o[r][VEC > 1 ? 3 : 0]);
+      else dst[0] = o[r][0];
     }
     return;
   }
-  if (a.w_stable) {
-    const int c = threadIdx.x & (2 * N - 1), ch = a.Di + (c >= N ? GN : 0) + g * N + (c & (N - 1));
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.conv_w + size_t(ch) * a.d_conv));
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.conv_b + ch));
-    pdl_wait();
-    pdl_trigger();
-  }
-  float* Bs = cb_sm;                 // [k][LDR]
-  float* Cs = cb_sm + k * LDR;       // [k][LDR]
-  uint8_t* ct = sp.c + (size_t(b) * a.G + g) * (4 * ROWS * 128);
+  if (grp != 0) return;
+  extern __shared__ __align__(16) float cb_sm[];
+  const int g = blockIdx.x, ldr = N + 4, GN = a.G * N;
+  float* Bs = cb_sm;                 // [k][N + 4]
+  float* Cs = cb_sm + k * ldr;       // [k][N + 4]
   for (int idx = threadIdx.x; idx < n_grp * (2 * N / VEC); idx += 256) {
     const int i0 = idx / (2 * N / VEC) * CONV_ROWS, c = idx % (2 * N / VEC) * VEC, is_c = c >= N, n = is_c ? c - N : c;
-    float o[CONV_ROWS][VEC];
     conv_rows<VEC>(a, b, i0, a.Di + is_c * GN + g * N + n, o);
 #pragma unroll
     for (int r = 0; r < CONV_ROWS; ++r) {
       const int i = i0 + r;
       if (i >= k) break;
-      float* dst = (is_c ? Cs : Bs) + i * LDR + n;
+      float* dst = (is_c ? Cs : Bs) + i * ldr + n;
 #pragma unroll
       for (int v = 0; v < VEC; ++v) dst[v] = o[r][v];
       if (is_c) {
         __half hi[VEC], lo[VEC];
 #pragma unroll
         for (int v = 0; v < VEC; ++v) { hi[v] = __float2half_rn(o[r][v]); lo[v] = __float2half_rn(o[r][v] - __half2float(hi[v])); }
-        uint8_t* tile = ct + (n >> 6) * ROWS * 128 + (i >> 3) * 1024 + (i & 7) * 128 + ((((n >> 3) & 7) ^ (i & 7)) << 4);
-        __half *d_hi = reinterpret_cast<__half*>(tile) + (n & 7), *d_lo = reinterpret_cast<__half*>(tile + 2 * ROWS * 128) + (n & 7);
+        __half* d_hi = c16 + ((row0 + i) * 2 + 0) * GN + g * N + n;
+        __half* d_lo = c16 + ((row0 + i) * 2 + 1) * GN + g * N + n;
         if (VEC == 4) {
           *reinterpret_cast<uint2*>(d_hi) = *reinterpret_cast<const uint2*>(hi);
           *reinterpret_cast<uint2*>(d_lo) = *reinterpret_cast<const uint2*>(lo);
@@ -641,372 +612,196 @@ scan_prep_kernel(ScanArgs a, ScanPrep sp, int heads_per_warp) {
     }
   }
   __syncthreads();
-  // C_t . B_s: a thread makes MT x MT neighbouring products, so that 136 of them have work either way (two by two from four rows of shared
-  // memory: with one product per thread and 32 positions the reads of the rows set the kernel's pace)
-  float* cbt = sp.cb + (size_t(b) * a.G + g) * tri_quads(ROWS) * 4;
-  for (int idx = threadIdx.x; idx < 16 * 17 / 2; idx += 256) {
-    int tb = int((sqrtf(8.f * float(idx) + 1.f) - 1.f) * 0.5f);
-    if ((tb + 1) * (tb + 2) / 2 <= idx) ++tb;
-    if (tb * (tb + 1) / 2 > idx) --tb;
-    const int t = MT * tb, s0 = MT * (idx - tb * (tb + 1) / 2);
-    float d[MT][MT];
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-      for (int j = 0; j < MT; ++j) d[i][j] = 0.f;
-    if (t < k) {
-      const float4 *cr[MT], *br[MT];
-#pragma unroll
-      for (int i = 0; i < MT; ++i) {
-        cr[i] = reinterpret_cast<const float4*>(Cs + min(t + i, k - 1) * LDR);
-        br[i] = reinterpret_cast<const float4*>(Bs + min(s0 + i, k - 1) * LDR);
-      }
-#pragma unroll 4
+  for (int idx = threadIdx.x; idx < k * k; idx += 256) {
+    const int t = idx / k, s2 = idx % k;
+    float dot = 0.f;
+    if (s2 <= t) {
+      const float4* cr = reinterpret_cast<const float4*>(Cs + t * ldr);
+      const float4* br = reinterpret_cast<const float4*>(Bs + s2 * ldr);
       for (int n4 = 0; n4 < N / 4; ++n4) {
-        float4 cv[MT], bv[MT];
-#pragma unroll
-        for (int i = 0; i < MT; ++i) { cv[i] = cr[i][n4]; bv[i] = br[i][n4]; }
-#pragma unroll
-        for (int i = 0; i < MT; ++i)
-#pragma unroll
-          for (int j = 0; j < MT; ++j) {
-            d[i][j] += cv[i].x * bv[j].x; d[i][j] += cv[i].y * bv[j].y; d[i][j] += cv[i].z * bv[j].z; d[i][j] += cv[i].w * bv[j].w;
-          }
+        const float4 c = cr[n4], bb = br[n4];
+        dot += c.x * bb.x; dot += c.y * bb.y; dot += c.z * bb.z; dot += c.w * bb.w;
       }
     }
+    cb[((size_t(b) * a.G + g) * KMAX + t) * KMAX + s2] = dot;
+  }
+}
+
+template <int P, int N, int MT>
+__global__ void __launch_bounds__(128, MT == 1 ? 4 : 3)
+mamba_scan_stream_kernel(ScanArgs a, const float* __restrict__ xact, const __half* __restrict__ c16,
+                         const float* __restrict__ cb) {
+  constexpr int HPC = 4, NT = P / 8, ROWS = MT * 16;
+  constexpr int XS = P + 8;                                    // floats per x row in shared memory (padded: the fragment reads
+                                                               // of rows tq and columns gq then fall on 32 different banks)
+  constexpr int CS = 2 * N + 8;                                // halves per C row (hi | lo | 16 bytes of padding: the 16-byte
+                                                               // fragment reads, 32 bytes apart along a row, of rows gq and gq + 1
+                                                               // then fall on different banks)
+  extern __shared__ __align__(16) float sm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int h0 = blockIdx.x * HPC, b = blockIdx.y;
+  const int hpg = a.H / a.G, g = h0 / hpg, k = a.k, GN = a.G * N;
+  const int h = h0 + warp;
+  const size_t row0 = size_t(b) * k;
+  __half* C16 = reinterpret_cast<__half*>(sm);                 // [ROWS][CS]  (hi, lo), rows >= k zero
+  float* CB = sm + ROWS * CS / 2;                                   // [ROWS][ROWS]
+  float* xs = CB + ROWS * ROWS + warp * (ROWS * XS);           // per warp [ROWS][XS]
+  float* Wh = CB + ROWS * ROWS + HPC * ROWS * XS + warp * ROWS * (ROWS + 1);   // per warp [ROWS][ROWS+1]
+
+  // ---- state fragments of the first two k-step pairs: issued before anything else, and before the wait for the kernel in front: that
+  // kernel (the conv) started its dependents only once everything ahead of it, the state's producer included, had finished
+  const int gq = lane >> 2, tq = lane & 3;
+  const __half* S = a.s_init ? a.s_init + (size_t(b) * a.H + h) * P * N : nullptr;
+  // (32-byte loads: the four lanes of a row then cover a whole 128-byte line per instruction; with 16-byte loads every
+  // line was touched twice, and the state's loads were a quarter of the L1's work)
+  uint4 sv0[NT][2];
+  if (S != nullptr) {
 #pragma unroll
-    for (int i = 0; i < MT; ++i) {
-      float* row = cbt + tri_quad(t + i, s0 >> 2) * 4;
+    for (int j = 0; j < NT; ++j) ldg_nc_32B(S + size_t(j * 8 + gq) * N + tq * 16, sv0[j][0], sv0[j][1]);
+  }
+  pdl_wait();
+  pdl_trigger();
+  // ---- shared operands (C halves, CB) and this head's x rows: cp.async, zero fill for the padding rows
+  for (int idx = tid; idx < ROWS * 2 * N / 8; idx += 128) {
+    const int r = idx / (2 * N / 8), rest = idx % (2 * N / 8), half = rest / (N / 8), c8 = rest % (N / 8);
+    cp_async16(smem_u32(C16 + r * CS + half * N + c8 * 8), c16 + ((row0 + min(r, k - 1)) * 2 + half) * GN + g * N + c8 * 8, r < k);
+  }
+  for (int idx = tid; idx < ROWS * ROWS / 4; idx += 128) {
+    const int r = idx / (ROWS / 4), c4 = idx % (ROWS / 4);
+    cp_async16(smem_u32(CB + r * ROWS + c4 * 4), cb + ((size_t(b) * a.G + g) * KMAX + r) * KMAX + c4 * 4, true);
+  }
+  for (int idx = lane; idx < ROWS * P / 4; idx += 32) {
+    const int r = idx / (P / 4), c4 = idx % (P / 4);
+    cp_async16(smem_u32(xs + r * XS + c4 * 4), xact + (row0 + min(r, k - 1)) * a.Di + h * P + c4 * 4, r < k);
+  }
+  cp_async_commit();
+  // ---- dt, inclusive prefix sum of dt * A over the block positions (one warp shuffle scan per head)
+  float dt = 0.f, dA = 0.f;
+  if (lane < k) {
+    const float raw = a.dt_pre(b, lane, h);
+    dt = softplus_f(raw + a.dt_bias[h]);
+    dA = dt * (-expf(a.A_log[h]));
+  }
+  float cum = dA;
 #pragma unroll
-      for (int j = 0; j < MT; ++j) row[(s0 & 3) + j] = t + i < k && s0 + j <= t + i ? d[i][j] : 0.f;
-      if (s0 + MT > t)                                         // the places behind the diagonal's block in its quad
-        for (int e = (s0 & 3) + MT; e < 4; ++e) row[e] = 0.f;
+  for (int off = 1; off < 32; off <<= 1) {
+    const float up = __shfl_up_sync(0xffffffffu, cum, off);
+    if (lane >= off) cum += up;
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  // ---- W[t][s] = exp(c_t - c_s) dt_s CB[t][s] for s <= t, plus the skip weight D on the diagonal: lane s owns
+  // column s; the rows past k are zero
+  const float Dh = a.Dskip[h];
+  for (int t = 0; t < ROWS; ++t) {
+    const float ct = __shfl_sync(0xffffffffu, cum, t & 31);
+    float w = 0.f;
+    if (t < k && lane <= t) w = __expf(ct - cum) * dt * CB[t * ROWS + lane];
+    if (t < k && lane == t) w += Dh;
+    if (lane < ROWS) Wh[t * (ROWS + 1) + lane] = w;
+  }
+  __syncwarp();
+  // ---- state term on the tensor cores
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) { acc[mt][j][0] = acc[mt][j][1] = acc[mt][j][2] = acc[mt][j][3] = 0.f; }
+  if (S != nullptr) {
+#pragma unroll
+    // the contraction index is permuted (the same way for C and for the state): within a chunk of 64, lane tq's 16
+    // consecutive elements serve four k-steps, four elements each
+    for (int kq = 0; kq < N / 64; ++kq) {
+      uint4 sv[NT][2];
+      if (kq >= 1) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j) ldg_nc_32B(S + size_t(j * 8 + gq) * N + kq * 64 + tq * 16, sv[j][0], sv[j][1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < NT; ++j) { sv[j][0] = sv0[j][0]; sv[j][1] = sv0[j][1]; }
+      }
+#pragma unroll
+      for (int piece = 0; piece < 2; ++piece) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          const __half* c0 = C16 + (mt * 16 + gq) * CS + kq * 64 + tq * 16 + piece * 8;
+          const __half* c1 = C16 + (mt * 16 + gq + 8) * CS + kq * 64 + tq * 16 + piece * 8;
+          const uint4 c_lo = *reinterpret_cast<const uint4*>(c0), c_hi = *reinterpret_cast<const uint4*>(c1);
+          const uint4 r_lo = *reinterpret_cast<const uint4*>(c0 + N), r_hi = *reinterpret_cast<const uint4*>(c1 + N);
+          const uint32_t a0[4] = {c_lo.x, c_hi.x, c_lo.y, c_hi.y}, a1[4] = {c_lo.z, c_hi.z, c_lo.w, c_hi.w};
+          const uint32_t e0[4] = {r_lo.x, r_hi.x, r_lo.y, r_hi.y}, e1[4] = {r_lo.z, r_hi.z, r_lo.w, r_hi.w};
+#pragma unroll
+          for (int j = 0; j < NT; ++j) {
+            mma_f16_16816(acc[mt][j], a0, sv[j][piece].x, sv[j][piece].y);
+            mma_f16_16816(acc[mt][j], a1, sv[j][piece].z, sv[j][piece].w);
+            mma_f16_16816(acc[mt][j], e0, sv[j][piece].x, sv[j][piece].y);
+            mma_f16_16816(acc[mt][j], e1, sv[j][piece].z, sv[j][piece].w);
+          }
+        }
+      }
+    }
+  }
+  // ---- decay of the state term: row t of the accumulator times exp(c_t)
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt) {
+    const float d_lo = __expf(__shfl_sync(0xffffffffu, cum, (mt * 16 + gq) & 31));
+    const float d_hi = __expf(__shfl_sync(0xffffffffu, cum, (mt * 16 + gq + 8) & 31));
+#pragma unroll
+    for (int j = 0; j < NT; ++j) { acc[mt][j][0] *= d_lo; acc[mt][j][1] *= d_lo; acc[mt][j][2] *= d_hi; acc[mt][j][3] *= d_hi; }
+  }
+  // ---- intra-block term and D skip, y_t += sum_{s <= t} W[t][s] x_s, as a [ROWS x ROWS] x [ROWS x P] product on the
+  // tensor cores: tf32 operands keep fp32's range (W is a product of exponentials, dt and a 128-term dot product), and
+  // each operand is split in two tf32 parts, three products per k-step, for ~21 bits.  (The scalar form read x from
+  // shared memory once per (t, s) pair and thread, and the kernel ran at the L1's limit.)
+#pragma unroll
+  for (int ks = 0; ks < ROWS / 8; ++ks) {
+    uint32_t ah[MT][4], al[MT][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      const float* wr = Wh + (mt * 16 + gq) * (ROWS + 1) + ks * 8 + tq;
+      split_tf32(wr[0], ah[mt][0], al[mt][0]);
+      split_tf32(wr[8 * (ROWS + 1)], ah[mt][1], al[mt][1]);
+      split_tf32(wr[4], ah[mt][2], al[mt][2]);
+      split_tf32(wr[8 * (ROWS + 1) + 4], ah[mt][3], al[mt][3]);
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      uint32_t bh[2], bl[2];
+      split_tf32(xs[(ks * 8 + tq) * XS + j * 8 + gq], bh[0], bl[0]);
+      split_tf32(xs[(ks * 8 + tq + 4) * XS + j * 8 + gq], bh[1], bl[1]);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        if (ks * 8 > mt * 16 + 15) continue;                   // W is lower triangular: nothing in this k-step for these rows
+        mma_tf32_1688(acc[mt][j], al[mt], bh[0], bh[1]);
+        mma_tf32_1688(acc[mt][j], ah[mt], bl[0], bl[1]);
+        mma_tf32_1688(acc[mt][j], ah[mt], bh[0], bh[1]);
+      }
+    }
+  }
+  // ---- gate and store
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int t = mt * 16 + gq + half * 8;
+      if (t >= k) continue;
+      const size_t row = row0 + t;
+      float2 z[NT];
+#pragma unroll
+      for (int j = 0; j < NT; ++j) z[j] = *reinterpret_cast<const float2*>(a.zxbcdt + a.in_row(b, t) * a.ld_in + h * P + j * 8 + tq * 2);
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+        *reinterpret_cast<float2*>(a.y + row * a.Di + h * P + j * 8 + tq * 2) =
+            make_float2(acc[mt][j][half * 2] * silu_f(z[j].x), acc[mt][j][half * 2 + 1] * silu_f(z[j].y));
     }
   }
 }
 
-// A tile is two heads of one group of one request (128 channels); a CTA per SM walks a contiguous stretch of the tiles.
-//   warp 0        producer: the tile's state rows (32 KB, two boxes [128 channels x 64 n], 128-byte swizzle) through a ring of four stages; the
-//                 group's C (head and remainder, both operand tiles as the preparation left them) when the group changes
-//   warp 1        state term  D[p, t] = sum_n S[p, n] C[t, n]: A = state (M = 128 channels), B = C (N = 16 or 32 positions), head and remainder into
-//                 the same accumulator (~22 bits of C), one of four in tensor memory
-//   warps 2..13   three groups of four warps take the tiles in turn; a thread owns a channel (= TMEM lane) with all its positions in registers:
-//                 conv + SiLU of x, then  y_t = e^{c_t} D_t + sum_{s <= t} W[t][s] x_s,  W[t][s] = exp(c_t - c_s) dt_s (C_t . B_s) (+ skip on the
-//                 diagonal) in fp32 from a table in shared memory that the head's two warps make together, gate, store.
-// What has to move is the state, x, z and y, once each (1.34 GB at 256 requests of 32 positions and 128 heads, 205 us at the copy peak); the issue of
-// the channel threads' instructions comes next (about 1 900 per warp and tile).  Before, the products were mma.sync fragments (1 600 clocks of a
-// scheduler per 32 channels, and as many instructions again for the lanes' pieces of C and x), and a kernel of its own activated x and wrote it
-// back.  Us of both kernels, before -> now, requests x positions, 128 heads: 1 x 16 9.6 -> 6.8, 5 x 7 9.7 -> 8.3, 16 x 1 13.7 -> 11.7, 32 x 16
-// 35.0 -> 24.3, 61 x 9 52.3 -> 33.3, 256 x 32 514 -> 317; 160 heads: 128 x 16 147 -> 114, 40 x 32 116 -> 71.
-constexpr int TC_BUFS = 4, TC_GROUPS = 3, TC_THREADS = 64 + TC_GROUPS * 128;
-constexpr uint32_t TC_S_BYTES = 128 * 128 * 2;
-constexpr int TC_MAX_STAGES = 5;
-struct __align__(8) ScanTcBars {
-  uint64_t s_full[TC_MAX_STAGES], s_empty[TC_MAX_STAGES], x_full[TC_MAX_STAGES], x_empty[TC_MAX_STAGES], c_full[2], c_empty[2], d_full[TC_BUFS], d_empty[TC_BUFS];
-  uint32_t tmem_base;
-};
-// Shared memory: bars, [6 heads' tables], [2][C], [NS][state], [NX][slot].
 template <int MT>
-struct ScanTcSmem {
-  static constexpr int ROWS = MT * 16, NS = MT == 1 ? 3 : 2, NX = MT == 1 ? 5 : 3;       // most stages of the state, of the rest
-  static constexpr int C_BYTES = 4 * ROWS * 128, X_BYTES = ROWS * 512, CB_BYTES = tri_quads(ROWS) * 16, W_FLOATS = tri_quads(ROWS) * 4 + ROWS;
-  // a slot: x, z, the group's table, prefix sums and dt of the two heads
-  static constexpr int SLOT = 2 * X_BYTES + CB_BYTES + 4 * ROWS * 4;
-  static constexpr int W_AT = 512, C_AT = (W_AT + 2 * TC_GROUPS * W_FLOATS * 4 + 1023) / 1024 * 1024, S_AT = C_AT + 2 * C_BYTES;
-  static_assert(sizeof(ScanTcBars) <= W_AT, "");
-  static constexpr size_t BYTES = S_AT + NS * size_t(TC_S_BYTES) + NX * size_t(SLOT) + 1024;
-};
-static_assert(ScanTcSmem<1>::BYTES <= 227 * 1024 && ScanTcSmem<2>::BYTES <= 227 * 1024, "shared memory of an SM");
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
+size_t scan_stream_smem() {
+  constexpr int P = 64, N = 128, HPC = 4, ROWS = MT * 16;
+  return sizeof(__half) * ROWS * (2 * N + 8) + sizeof(float) * (ROWS * ROWS + HPC * ROWS * (P + 8) + HPC * ROWS * (ROWS + 1));
 }
-__device__ __forceinline__ float exp_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.4426950408889634f));
-  return y;
-}
-
-// TMA_X: x and z come by TMA as well (rows of 16-byte multiples), else by plain loads of their channel's thread.
-template <int MT, bool TMA_X>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-scan_tc_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUtensorMap tmX, ScanArgs a, ScanPrep sp, int n_tiles, uint32_t* status) {
-  using L = ScanTcSmem<MT>;
-  constexpr int P = 64, ROWS = L::ROWS, NS = L::NS, NX = L::NX;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  ScanTcBars* bars = reinterpret_cast<ScanTcBars*>(smem);
-  uint8_t *sC = smem + L::C_AT, *sS = smem + L::S_AT, *sX = sS + NS * TC_S_BYTES;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = a.k;
-  const int t_begin = int((long long)n_tiles * blockIdx.x / gridDim.x), n_my = int((long long)n_tiles * (blockIdx.x + 1) / gridDim.x) - t_begin;
-  const int per_group = a.H / a.G / 2, per_req = a.H / 2;      // tiles of a group and of a request
-  const bool has_state = a.s_init != nullptr;
-  constexpr uint32_t TMEM_COLS = TC_BUFS * ROWS;               // 64 or 128
-
-  if (threadIdx.x == 0) {
-    if (has_state) tma_prefetch_desc(&tmS);
-    if (TMA_X) tma_prefetch_desc(&tmX);
-    for (int i = 0; i < NS; ++i) { mbar_init(smem_u32(&bars->s_full[i]), 1); mbar_init(smem_u32(&bars->s_empty[i]), 1); }
-    for (int i = 0; i < NX; ++i) { mbar_init(smem_u32(&bars->x_full[i]), 1); mbar_init(smem_u32(&bars->x_empty[i]), 4); }
-    for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bars->c_full[i]), 1); mbar_init(smem_u32(&bars->c_empty[i]), 1); }
-    for (int i = 0; i < TC_BUFS; ++i) { mbar_init(smem_u32(&bars->d_full[i]), 1); mbar_init(smem_u32(&bars->d_empty[i]), 4); }
-    fence_mbar_init();
-  }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(&bars->tmem_base), TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = bars->tmem_base;
-
-  if (warp == 0) {
-    if (elect_one()) {
-      const uint64_t pol = policy_evict_first();
-      bool ok = true;
-      int n_c = 0;                                             // groups so far
-      auto load_state = [&](int i) {
-        const uint32_t dst = smem_u32(sS + (i % NS) * TC_S_BYTES), full = smem_u32(&bars->s_full[i % NS]);
-        mbar_expect_tx(full, TC_S_BYTES);
-        tma_load_2d(dst, &tmS, 0, (t_begin + i) * 128, full, pol);
-        tma_load_2d(dst + TC_S_BYTES / 2, &tmS, 64, (t_begin + i) * 128, full, pol);
-      };
-      auto load_x = [&](int i) {
-        const int b = (t_begin + i) / per_req, c = (t_begin + i - b * per_req) * 128;
-        const uint32_t dst = smem_u32(sX + (i % NX) * L::SLOT), full = smem_u32(&bars->x_full[i % NX]);
-        const int n = !TMA_X ? 0 : !a.shared_rows ? k : k > 1 ? 2 : 1;
-        mbar_expect_tx(full, n * 1024 + L::CB_BYTES + 4 * ROWS * 4);
-        if (!TMA_X) return;
-        if (a.shared_rows) {                                   // boxes of one row: position 0, every later position
-          for (int r = 0; r < n; ++r) {
-            tma_load_2d(dst + r * 512, &tmX, a.Di + c, r == 0 ? b : a.B, full, pol);
-            tma_load_2d(dst + L::X_BYTES + r * 512, &tmX, c, r == 0 ? b : a.B, full, pol);
-          }
-        } else {
-          tma_load_2d(dst, &tmX, a.Di + c, b * k, full, pol);
-          tma_load_2d(dst + L::X_BYTES, &tmX, c, b * k, full, pol);
-        }
-      };
-      auto load_prep = [&](int i) {                            // what the kernel in front makes
-        const int tile = t_begin + i;
-        const uint32_t dst = smem_u32(sX + (i % NX) * L::SLOT) + 2 * L::X_BYTES, full = smem_u32(&bars->x_full[i % NX]);
-        bulk_load(dst, sp.cb + size_t(tile / per_group) * (L::CB_BYTES / 4), L::CB_BYTES, full);
-        bulk_load(dst + L::CB_BYTES, sp.cum + size_t(tile) * 2 * ROWS, 2 * ROWS * 4, full);
-        bulk_load(dst + L::CB_BYTES + 2 * ROWS * 4, sp.dt + size_t(tile) * 2 * ROWS, 2 * ROWS * 4, full);
-      };
-      // The kernel in front (the preparation) started this one only after everything ahead of it had finished: state and in-projection are there.
-      const int early_s = has_state ? min(NS, n_my) : 0, early_x = min(NX, n_my);
-      for (int i = 0; i < early_s; ++i) load_state(i);
-      for (int i = 0; i < early_x; ++i) load_x(i);
-      pdl_wait();
-      pdl_trigger();
-      for (int i = 0; i < n_my && ok; ++i) {
-        if (has_state) {
-          const int tile = t_begin + i;
-          if (i == 0 || tile % per_group == 0) {               // a group's first tile here
-            const int cb = n_c & 1;
-            if (n_c >= 2 && !mbar_wait(smem_u32(&bars->c_empty[cb]), ((n_c >> 1) - 1) & 1)) { ok = false; break; }
-            mbar_expect_tx(smem_u32(&bars->c_full[cb]), L::C_BYTES);
-            bulk_load(smem_u32(sC + cb * L::C_BYTES), sp.c + size_t(tile / per_group) * L::C_BYTES, L::C_BYTES, smem_u32(&bars->c_full[cb]));
-            ++n_c;
-          }
-          if (i >= early_s) {
-            if (!mbar_wait(smem_u32(&bars->s_empty[i % NS]), (i / NS - 1) & 1)) { ok = false; break; }
-            load_state(i);
-          }
-        }
-        if (i >= early_x) {
-          if (!mbar_wait(smem_u32(&bars->x_empty[i % NX]), (i / NX - 1) & 1)) { ok = false; break; }
-          load_x(i);
-        }
-        load_prep(i);
-      }
-      if (!ok) atomicExch(status, STATUS_TIMEOUT_PRODUCER);
-    }
-  } else if (warp == 1) {
-    if (has_state && elect_one()) {
-      const uint32_t idesc = umma_idesc_m128(ROWS, true);
-      bool ok = true;
-      int n_c = 0;
-      for (int i = 0; i < n_my && ok; ++i) {
-        const int tile = t_begin + i, s = i % NS, d = i % TC_BUFS;
-        if (i == 0 || tile % per_group == 0) {
-          ok = mbar_wait(smem_u32(&bars->c_full[n_c & 1]), (n_c >> 1) & 1);
-          ++n_c;
-        }
-        ok = ok && mbar_wait(smem_u32(&bars->s_full[s]), (i / NS) & 1);
-        if (ok && i >= TC_BUFS) ok = mbar_wait(smem_u32(&bars->d_empty[d]), (i / TC_BUFS - 1) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t st = smem_u32(sS + s * TC_S_BYTES), sc = smem_u32(sC + ((n_c - 1) & 1) * L::C_BYTES);
-#pragma unroll
-        for (int hl = 0; hl < 2; ++hl)
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t da = umma_desc_kmajor_sw128(st + (kk >> 2) * (TC_S_BYTES / 2)) + uint64_t((kk & 3) * 2);
-            const uint64_t db = umma_desc_kmajor_sw128(sc + (hl * 2 + (kk >> 2)) * ROWS * 128) + uint64_t((kk & 3) * 2);
-            umma_bf16(tmem + d * ROWS, da, db, idesc, (hl > 0 || kk > 0) ? 1u : 0u);
-          }
-        umma_commit(smem_u32(&bars->s_empty[s]));
-        umma_commit(smem_u32(&bars->d_full[d]));
-        if ((tile + 1) % per_group == 0) umma_commit(smem_u32(&bars->c_empty[(n_c - 1) & 1]));
-      }
-      if (!ok) atomicExch(status, STATUS_TIMEOUT_MMA);
-    }
-  } else {
-    const int wg = (warp - 2) >> 2, q = warp & 3, pair = q >> 1;          // TMEM lane quarter; head of the tile
-    float* Wt = reinterpret_cast<float*>(smem + L::W_AT) + (wg * 2 + pair) * L::W_FLOATS;     // triangle, then exp(c_t)
-    float* dec = Wt + tri_quads(ROWS) * 4;
-    const int bar_id = 1 + wg * 2 + pair, j64 = (q & 1) * 32 + lane;
-    bool ok = true;
-    // this thread's quads of the table: t and s4
-    constexpr int QUADS = tri_quads(ROWS), ITS = (QUADS + 63) / 64;
-    int q_t[ITS], q_s[ITS];
-#pragma unroll
-    for (int it = 0; it < ITS; ++it) {
-      const int i = min(it * 64 + j64, QUADS - 1);
-      int r = 0;
-      while (2 * (r + 1) * (r + 2) <= i) ++r;                  // group of four rows with r + 1 quads each
-      const int rem = i - 2 * r * (r + 1);
-      q_t[it] = 4 * r + rem / (r + 1);
-      q_s[it] = rem % (r + 1);
-    }
-    // taps, bias and skip weight of the thread's channel, a tile ahead
-    float w[4], bias, Dh;
-    auto load_taps = [&](int i) {
-      const int tile = t_begin + i, h = (tile % per_req) * 2 + pair, ch = h * P + j64;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = j >= 4 - a.d_conv ? a.conv_w[ch * a.d_conv + j - (4 - a.d_conv)] : 0.f;   // right-aligned
-      bias = a.conv_b[ch];
-      Dh = a.Dskip[h];
-    };
-    if (a.w_stable && wg < n_my) load_taps(wg);
-    pdl_wait();
-    if (!a.w_stable && wg < n_my) load_taps(wg);
-    for (int i = wg; i < n_my; i += TC_GROUPS) {
-      const int tile = t_begin + i, b = tile / per_req, ch = ((tile - b * per_req) * 2 + pair) * P + j64;
-      // ---- raw x and gate of the channel at every position
-      float x[ROWS], z[ROWS];
-      const int sx = i % NX;
-      const uint8_t* slot = sX + sx * L::SLOT;
-      if (ok && !mbar_wait(smem_u32(&bars->x_full[sx]), (i / NX) & 1)) {
-        atomicExch(status, STATUS_TIMEOUT_EPILOGUE);
-        ok = false;
-      }
-      if constexpr (TMA_X) {
-        const float* px = reinterpret_cast<const float*>(slot) + q * 32 + lane;
-        if (a.shared_rows) {
-          x[0] = px[0]; z[0] = px[ROWS * 128];
-          const float x1 = px[128], z1 = px[ROWS * 128 + 128];
-#pragma unroll
-          for (int t = 1; t < ROWS; ++t) { x[t] = x1; z[t] = z1; }
-        } else {
-#pragma unroll
-          for (int t = 0; t < ROWS; ++t) { x[t] = px[t * 128]; z[t] = px[ROWS * 128 + t * 128]; }
-        }
-      } else {
-        const float* row = a.zxbcdt + a.in_row(b, 0) * a.ld_in + ch;
-        const size_t first_step = a.shared_rows ? size_t(a.B - b) * a.ld_in : size_t(a.ld_in), step = a.shared_rows ? 0 : size_t(a.ld_in);
-#pragma unroll
-        for (int t = 0; t < ROWS; ++t) {
-          x[t] = t < k ? ld_stream(row + a.Di) : 0.f;
-          z[t] = t < k ? ld_stream(row) : 0.f;
-          row += t == 0 ? first_step : step;
-        }
-      }
-      // ---- the head's table, by its 64 threads.  (The products are zero for s > t and for t >= k; the decay only must not overflow there.)
-      {
-        const float* cbt = reinterpret_cast<const float*>(slot + 2 * L::X_BYTES);
-        const float *cum = reinterpret_cast<const float*>(slot + 2 * L::X_BYTES + L::CB_BYTES) + pair * ROWS, *dts = cum + 2 * ROWS;
-#pragma unroll
-        for (int it = 0; it < ITS; ++it) {
-          if (QUADS % 64 != 0 && it == ITS - 1 && it * 64 + j64 >= QUADS) break;
-          const int t = q_t[it], s4 = q_s[it], d = t - s4 * 4;
-          const float4 cb = *reinterpret_cast<const float4*>(cbt + (it * 64 + j64) * 4);
-          const float4 cs = *reinterpret_cast<const float4*>(cum + s4 * 4), ds = *reinterpret_cast<const float4*>(dts + s4 * 4);
-          const float c = cum[t];
-          float4 v;
-          v.x = exp_ftz(fminf(c - cs.x, 0.f)) * ds.x * cb.x + (d == 0 ? Dh : 0.f);
-          v.y = exp_ftz(fminf(c - cs.y, 0.f)) * ds.y * cb.y + (d == 1 ? Dh : 0.f);
-          v.z = exp_ftz(fminf(c - cs.z, 0.f)) * ds.z * cb.z + (d == 2 ? Dh : 0.f);
-          v.w = exp_ftz(fminf(c - cs.w, 0.f)) * ds.w * cb.w + (d == 3 ? Dh : 0.f);
-          *reinterpret_cast<float4*>(Wt + (it * 64 + j64) * 4) = v;
-        }
-        if (j64 < ROWS) dec[j64] = exp_ftz(cum[j64]);
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->x_empty[sx]));
-      asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-      // ---- conv + SiLU of x, zero left context
-      {
-        float c1 = 0.f, c2 = 0.f, c3 = 0.f;
-#pragma unroll
-        for (int t = 0; t < ROWS; ++t) {
-          const float in = x[t];
-          x[t] = silu_f(bias + w[0] * c3 + w[1] * c2 + w[2] * c1 + w[3] * in);
-          c3 = c2; c2 = c1; c1 = in;
-        }
-      }
-      if (i + TC_GROUPS < n_my) load_taps(i + TC_GROUPS);
-      // ---- state term
-      float acc[ROWS];
-      if (has_state) {
-        const int d = i % TC_BUFS;
-        if (ok && !mbar_wait(smem_u32(&bars->d_full[d]), (i / TC_BUFS) & 1)) {
-          atomicExch(status, STATUS_TIMEOUT_EPILOGUE);
-          ok = false;
-        }
-        tc_fence_after();
-#pragma unroll
-        for (int c0 = 0; c0 < ROWS; c0 += 16)
-          tmem_ld16(tmem + (uint32_t(q * 32) << 16) + d * ROWS + c0, *reinterpret_cast<uint32_t(*)[16]>(acc + c0));
-        tmem_ld_wait();
-#pragma unroll
-        for (int t = 0; t < ROWS; ++t) asm volatile("" : "+f"(acc[t]));     // (no use of the registers ahead of the wait)
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars->d_empty[d]));
-      } else {
-#pragma unroll
-        for (int t = 0; t < ROWS; ++t) acc[t] = 0.f;
-      }
-      // ---- four positions at a time
-      float* yr = a.y + size_t(b) * k * a.Di + ch;
-#pragma unroll
-      for (int t0 = 0; t0 < ROWS; t0 += 4) {
-        if (t0 >= k) break;
-        const float4 dc = *reinterpret_cast<const float4*>(dec + t0);
-        float y[4] = {dc.x * acc[t0], dc.y * acc[t0 + 1], dc.z * acc[t0 + 2], dc.w * acc[t0 + 3]};
-#pragma unroll
-        for (int s4 = 0; s4 <= t0 / 4; ++s4)
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const float4 v = *reinterpret_cast<const float4*>(Wt + tri_quad(t0 + r, s4) * 4);
-            const int s = s4 * 4, t = t0 + r;
-            y[r] += v.x * x[s];
-            if (s + 1 <= t) y[r] += v.y * x[s + 1];
-            if (s + 2 <= t) y[r] += v.z * x[s + 2];
-            if (s + 3 <= t) y[r] += v.w * x[s + 3];
-          }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          if (t0 + r < k && ok) { *yr = y[r] * silu_f(z[t0 + r]); yr += a.Di; }
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");           // the table may be written again
-    }
-    tc_fence_before();
-  }
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem, TMEM_COLS);
-  }
-}
-
-// rows of a request's prepared operands: block positions padded to a tile of the tensor-core products
-int unit_rows(int k) { return k > 16 ? 32 : 16; }
 
 template <int MT>
 size_t scan_mma_smem() {
@@ -1018,8 +813,8 @@ size_t scan_mma_smem() {
 }  // namespace
 
 size_t scan_workspace_bytes(int B, int k, int Di, int N, int G) {
-  const size_t rows = size_t(unit_rows(k));
-  return size_t(B) * (G * (rows * 2 * N * 2 + size_t(tri_quads(int(rows))) * 16) + size_t(Di / 64) * 2 * rows * 4) + 256;
+  const size_t M = size_t(B) * k, d_xBC = size_t(Di) + 2 * size_t(G) * N;
+  return M * d_xBC * 4 + size_t(B) * G * KMAX * KMAX * 4 + M * 2 * size_t(G) * N * 2 + 256;
 }
 
 namespace {
@@ -1058,43 +853,37 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   a.w_stable = c.w_stable ? 1 : 0;
   a.NP = c.N + 1;                                    // odd pitch: threads of a warp own consecutive p
   if (a.H % c.G) { if (err) *err = "scan: heads must divide into groups"; return cudaErrorInvalidValue; }
-  // serving shapes: tcgen05 path (16-byte copies of the state and of the scratch)
-  if (c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ws != nullptr && c.status != nullptr &&
-      ((reinterpret_cast<uintptr_t>(c.s_init) | reinterpret_cast<uintptr_t>(c.ws)) & 15) == 0 &&
+  // serving shapes: tensor-core path (needs 8-byte aligned rows for the float2 accesses)
+  if (c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ld_in % 2 == 0 && c.Di % 4 == 0 && c.ws != nullptr &&
+      (reinterpret_cast<uintptr_t>(c.s_init) & 31) == 0 &&     // its 32-byte loads of the state
       c.ws_bytes >= scan_workspace_bytes(c.B, c.k, c.Di, c.N, c.G)) {
-    // (a grid of the conv that this path once had: calls past its limit stay refused)
-    if ((long long)c.B * ((c.k + CONV_ROWS - 1) / CONV_ROWS) > 65535) return cudaErrorInvalidConfiguration;
     const bool two = c.k > 16;
-    const int rows = unit_rows(c.k);
-    ScanPrep sp{};
-    sp.c = reinterpret_cast<uint8_t*>(c.ws);
-    sp.cb = reinterpret_cast<float*>(sp.c + size_t(c.B) * c.G * rows * 2 * c.N * 2);
-    sp.dt = sp.cb + size_t(c.B) * c.G * tri_quads(rows) * 4;
-    sp.cum = sp.dt + size_t(c.B) * a.H * rows;
-    const bool vec4 = a.ld_in % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.zxbcdt) | reinterpret_cast<uintptr_t>(a.conv_w) |
-                                            reinterpret_cast<uintptr_t>(a.conv_b)) & 15) == 0;
-    CUtensorMap tmS{}, tmX{};
-    if (c.s_init != nullptr && !make_tmap_16bit_2d(&tmS, c.s_init, int64_t(c.B) * a.H * c.P, c.N, c.N, 128, true, err)) return cudaErrorInvalidValue;
-    const bool tma_x = a.ld_in % 4 == 0 && (reinterpret_cast<uintptr_t>(a.zxbcdt) & 15) == 0;
-    if (tma_x && !make_tmap_f32_2d(&tmX, a.zxbcdt, a.shared_rows ? c.B + 1 : int64_t(c.B) * c.k, a.ld_in, 128, a.shared_rows ? 1 : c.k, err))
-      return cudaErrorInvalidValue;
-    trk_begin(trk, "scan_prep", 0, double(c.B) * c.k * (2 * c.G * c.N + a.H) * 4);
-    auto prep = two ? (vec4 ? scan_prep_kernel<4, 2> : scan_prep_kernel<1, 2>) : (vec4 ? scan_prep_kernel<4, 1> : scan_prep_kernel<1, 1>);
-    const int hw = (long long)c.B * a.H > 148 * 32 ? 4 : 1;    // one head per warp while the blocks for them fit the chip at once
-    const cudaError_t e_prep = launch_pdl(prep, dim3(c.G + (a.H + 8 * hw - 1) / (8 * hw), c.B), dim3(256), size_t(2) * c.k * (c.N + 4) * sizeof(float), stream,
-                                          a, sp, hw);
+    const size_t M = size_t(c.B) * c.k;
+    float* xact = reinterpret_cast<float*>(c.ws);
+    float* cbw = xact + M * a.d_xBC;
+    __half* c16 = reinterpret_cast<__half*>(cbw + size_t(c.B) * c.G * KMAX * KMAX);
+    trk_begin(trk, "scan_conv", 0, double(M) * (a.d_xBC + a.Di) * 4);
+    const bool vec4 = a.Di % 4 == 0 && (c.G * c.N) % 4 == 0 && a.ld_in % 4 == 0 &&
+                      ((reinterpret_cast<uintptr_t>(a.zxbcdt) | reinterpret_cast<uintptr_t>(c.ws) | reinterpret_cast<uintptr_t>(a.conv_w) |
+                        reinterpret_cast<uintptr_t>(a.conv_b)) & 15) == 0;
+    const dim3 grid_c(c.G + (a.Di / (vec4 ? 4 : 1) + 255) / 256, c.B * ((c.k + CONV_ROWS - 1) / CONV_ROWS));
+    const size_t smem_c = size_t(2) * c.k * (c.N + 4) * sizeof(float);
+    const cudaError_t e_conv = launch_pdl(vec4 ? scan_conv_kernel<4> : scan_conv_kernel<1>, grid_c, dim3(256), smem_c, stream, a, xact, c16, cbw);
     trk_end(trk);
-    if (e_prep != cudaSuccess) return e_prep;        // (the next kernel reads the state early on the strength of this launch in front of it)
-    const int n_tiles = c.B * (a.H / 2), ctas = n_tiles < 148 ? n_tiles : 148;
-    const size_t smem_t = two ? ScanTcSmem<2>::BYTES : ScanTcSmem<1>::BYTES;
-    auto kernel = two ? (tma_x ? scan_tc_kernel<2, true> : scan_tc_kernel<2, false>) : (tma_x ? scan_tc_kernel<1, true> : scan_tc_kernel<1, false>);
-    static bool tset[4][MAX_DEVICES] = {};
-    const cudaError_t e0 = once_per_device(tset[two * 2 + tma_x], [kernel](int) {
-      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    });
-    if (e0 != cudaSuccess) return e0;
+    if (e_conv != cudaSuccess) return e_conv;        // (the stream kernel reads the state early on the strength of this launch in front of it)
+    const size_t smem_s = two ? scan_stream_smem<2>() : scan_stream_smem<1>();
+    static bool sset[2][MAX_DEVICES] = {};
+    {
+      const cudaError_t e = once_per_device(sset[two ? 1 : 0], [two, smem_s](int) {
+        return two ? cudaFuncSetAttribute(mamba_scan_stream_kernel<64, 128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_s))
+                   : cudaFuncSetAttribute(mamba_scan_stream_kernel<64, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_s));
+      });
+      if (e != cudaSuccess) return e;
+    }
+    dim3 grid_s(a.H / 4, c.B);
     trk_begin(trk, "mamba_scan", 2.0 * c.B * c.k * a.H * c.P * c.N, double(c.B) * a.H * c.P * c.N * 2);
-    const cudaError_t e = launch_pdl(kernel, dim3(ctas), dim3(TC_THREADS), smem_t, stream, tmS, tmX, a, sp, n_tiles, c.status);
+    const cudaError_t e = launch_pdl(two ? mamba_scan_stream_kernel<64, 128, 2> : mamba_scan_stream_kernel<64, 128, 1>, grid_s, dim3(128), smem_s, stream, a,
+                                     (const float*)xact, (const __half*)c16, (const float*)cbw);
     trk_end(trk);
     return e;
   }

@@ -377,9 +377,9 @@ def test_low_rank_dt_in_the_scan(hs, Di, N, G, dt_rank, B, k, bf16):
     drafter.close()
 
 
-# the tcgen05 scan (P = 64, N = 128): one tile of 16 positions and two, on both sides; one tile per CTA and enough of them that every ring goes round
-# several times; groups of two tiles, so that C changes with every other tile, and one group of all; x by TMA and, from rows that are no
-# multiples of 16 bytes, by plain loads; no state
+# the scan of the serving shapes (P = 64, N = 128), with scratch: one tile of 16 positions and two, on both sides; few blocks and several waves of
+# them; groups of four heads and one group of all; rows of 16-byte multiples (vector loads of the conv), of 8-byte ones (scalar) and, off the 8 bytes,
+# the general kernel; no state
 @pytest.mark.parametrize("B,k,H,G,ld_extra,state", [(1, 1, 4, 1, 0, True), (3, 15, 8, 2, 0, True), (41, 16, 64, 16, 0, True), (41, 17, 64, 16, 0, True),
                                                     (75, 32, 32, 1, 0, True), (40, 9, 36, 3, 1, True), (40, 31, 36, 3, 2, True), (64, 5, 32, 2, 0, False)])
 def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
@@ -410,6 +410,68 @@ def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
         # 10 x 2^-22 of the terms' absolute sum, which is below 20 RMS; 1e-4 leaves a factor of two
         assert np.abs(got - ref).max() <= 1e-4 * max(1.0, np.sqrt((ref ** 2).mean())), np.abs(got - ref).max()
     assert hs.hspec_op_device_status()["rc"] == 0
+
+
+# Draws on a grid, from integers alone: the same bits on every platform.
+def _grid(shape, seed, low, high, dtype=torch.float32):
+    import numpy as np
+    v = np.random.default_rng(seed).integers(0, 1 << 16, size=shape)
+    return torch.from_numpy((low + (high - low) * v / 65536.0).astype(np.float32)).to("cuda", dtype)
+
+
+def _scan_of_few_rows(hs, B, k, H, G, state, a_log=(0.0, 2.0), scratch=True):
+    P, N = 64, 128
+    Di, d_xBC = H * P, H * P + 2 * G * N
+    zx = _grid((B * k, Di + d_xBC + H), 1, -2.0, 2.0)
+    s0 = _grid((B, H, P, N), 2, -2.0, 2.0, torch.float16) if state else None
+    conv_w, conv_b = _grid((d_xBC, 4), 3, -0.5, 0.5), _grid((d_xBC,), 4, -0.05, 0.05)
+    dt_bias, A_log, D = _grid((H,), 5, -6.0, -2.0), _grid((H,), 6, *a_log), _grid((H,), 7, 0.5, 1.5)
+    y = torch.full((B * k, Di), float("nan"), device="cuda")
+    ws = torch.full((hs.hspec_scan_workspace_bytes(B, k, Di, N, G),), 255, dtype=torch.uint8, device="cuda") if scratch else None
+    hs.hspec_op_mamba_scan(zx, None, s0, conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, 4, ws)
+    return y
+
+
+# A step's logits carry the scan's last bits through the 16-bit roundings behind it, up to 5e-4 (fp16 operands) and 4e-3 (bf16) of their size, and
+# there the arg-max of near-tied tokens turns: of a few tokens, one is several per cent.  So the sums of this path keep their order, and its
+# outputs are compared to the bit with those on record (CRC-32 of the fp32 outputs).
+@pytest.mark.parametrize("B,k,H,G,state", [(1, 1, 4, 1, True), (1, 16, 128, 4, True), (1, 17, 128, 4, True), (2, 32, 8, 2, True), (3, 29, 64, 4, True),
+                                           (5, 7, 128, 4, True), (3, 16, 64, 4, False), (8, 20, 16, 1, False)])
+def test_scan_outputs_keep_their_bits(hs, B, k, H, G, state):
+    import json
+    import os
+    import zlib
+    y = _scan_of_few_rows(hs, B, k, H, G, state)
+    with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "scan_crc32.json")) as f:
+        want = json.load(f)
+    assert zlib.crc32(y.cpu().numpy().tobytes()) == want["%d,%d,%d,%d,%d" % (B, k, H, G, state)]
+
+
+# Prefix sums of dt A at -infinity: exp of their differences is NaN, with scratch as without, and is not turned into a factor.
+def test_scan_lets_a_nan_decay_through(hs):
+    with_scratch = _scan_of_few_rows(hs, 2, 9, 8, 2, True, a_log=(100.0, 101.0))
+    without = _scan_of_few_rows(hs, 2, 9, 8, 2, True, a_log=(100.0, 101.0), scratch=False)
+    assert bool(torch.isnan(without).all()) and bool(torch.isnan(with_scratch).all())
+
+
+# The scan allocates nothing, also as the first call of a process: it can be captured.
+def test_scan_as_a_process_first_call_under_capture():
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import torch, paper_2609_24197_b200 as hs; hs.load_library()\n"
+            "B, k, H, P, N, G = 2, 5, 8, 64, 128, 2; Di = H * P; W = Di + 2 * G * N\n"
+            "r = lambda *s: torch.rand(s, device='cuda') - 0.5\n"
+            "a = [r(B * k, Di + W + H), None, r(B, H, P, N).half(), r(W, 4), r(W), r(H), r(H), r(H)]; y = torch.zeros(B * k, Di, device='cuda')\n"
+            "ws = torch.zeros(hs.hspec_scan_workspace_bytes(B, k, Di, N, G), dtype=torch.uint8, device='cuda')\n"
+            "run = lambda: hs.hspec_op_mamba_scan(*a, y, B, k, Di, P, N, G, 4, ws)\n"
+            "g = torch.cuda.CUDAGraph(); torch.cuda.synchronize()\n"
+            "with torch.cuda.graph(g): run()\n"
+            "g.replay(); torch.cuda.synchronize(); got = y.clone(); y.zero_(); run(); torch.cuda.synchronize()\n"
+            "assert bool(got.any()) and torch.equal(got, y); print('same')\n")
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and "same" in res.stdout, res.stdout[-2000:] + res.stderr[-2000:]
 
 
 # the norm of wide rows, where a CTA fetches its next row ahead: one row per CTA and several, row lengths around 6144 (256 or 512 threads) and
