@@ -307,11 +307,11 @@ __device__ __forceinline__ uint32_t umma_idesc_m128(uint32_t n, bool f16) {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// SwiGLU epilogue for 16 accumulator columns (column j is activation row m_lo + j, from the eighth on m_hi + j).  Weight rows are interleaved in blocks
+// SwiGLU epilogue for 16 accumulator columns (activation rows m0 + c0 .. +15).  Weight rows are interleaved in blocks
 // of 16: lanes 0..15 of a warp hold the gate pre-activation of 16 features, lanes 16..31 the up projection of the same
 // features.  Columns are handled in pairs: the lower half-warp finishes the even column, the upper half the odd one,
 // so all 32 lanes compute and store.  `f` is the feature index of this lane (same for lane and lane ^ 16).
-__device__ __forceinline__ void swiglu_store16(const uint32_t (&r)[16], void* out, bool bf16, long long ldo, int m_lo, int m_hi, int M, int f,
+__device__ __forceinline__ void swiglu_store16(const uint32_t (&r)[16], void* out, bool bf16, long long ldo, int m_first, int M, int f,
                                                bool f_ok, int lane, uint32_t* status) {
   const bool upper = lane >= 16;
 #pragma unroll
@@ -321,7 +321,7 @@ __device__ __forceinline__ void swiglu_store16(const uint32_t (&r)[16], void* ou
     const float recv = __shfl_xor_sync(0xffffffffu, send, 16);
     const float gate = upper ? recv : mine_even;               // upper half: partner's gate of the odd column
     const float up = upper ? mine_odd : recv;                  // lower half: partner's up of the even column
-    const int m = (j < 8 ? m_lo : m_hi) + j + (upper ? 1 : 0);
+    const int m = m_first + j + (upper ? 1 : 0);
     if (f_ok && m < M) store_act16(out, size_t(m) * ldo + f, silu_f(gate) * up, bf16, status);
   }
 }

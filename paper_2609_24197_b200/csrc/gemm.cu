@@ -216,7 +216,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       } else if (g.mode == EPI_SWIGLU_F16 || g.mode == EPI_SWIGLU_BF16) {
         const int f = tile_n * 64 + q * 16 + (lane & 15);
-        swiglu_store16(r, g.out, g.mode == EPI_SWIGLU_BF16, g.ldo, m0 + c0, m0 + c0, g.M, f, 2 * f < g.N_out, lane, g.status);
+        swiglu_store16(r, g.out, g.mode == EPI_SWIGLU_BF16, g.ldo, m0 + c0, g.M, f, 2 * f < g.N_out, lane, g.status);
       } else if (g.mode == EPI_STORE_F16) {
         __half* out = reinterpret_cast<__half*>(g.out);
 #pragma unroll
@@ -399,7 +399,7 @@ int gemm_pick_bn(int M) {
 int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode) {
   if (gemm2_preferred(M, n_out)) {
     int bnt = 256, s = 1;
-    gemm2_pick(M, n_out, K, mode, &bnt, &s, true);
+    gemm2_pick(M, n_out, K, mode, &bnt, &s);
     return s;
   }
   // Weight streaming (few rows): keep every SM fed.  Many rows: one slice (tensor-bound, no reduction pass).

@@ -42,8 +42,7 @@ constexpr uint32_t A_BYTES = 128 * TILE_K * 2;     // 16 KiB: this CTA's 128 wei
 
 struct Gemm2Args {
   int M, N_out, K;
-  int BNT;                 // activation rows per cluster tile; each CTA stages BNT/2.  A multiple of 16 up to 256 (two accumulators take
-                           // turns), or of 32 up to 512 (one accumulator, two instructions wide: a cluster then has a single unit)
+  int BNT;                 // activation rows per cluster tile (a multiple of 16, at most 256); each CTA stages BNT/2
   uint32_t acc_cols;       // TMEM columns per accumulator: BNT rounded up to a power of two
   int k_tiles, stages;
   int ksub;                // 64-column k-steps per pipeline stage (1 or 2): one barrier round per stage
@@ -115,9 +114,8 @@ __device__ __forceinline__ uint32_t idesc_m256(uint32_t n, bool f16) {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((n >> 3) << 17) | ((256u >> 4) << 24);
 }
 
-// WIDE: tiles of more than 256 activation rows.  (As a branch in one kernel the others' instruction issue suffered: 512 rows, n_out = 4096, K = 14336
-// 70 -> 85 us.)  ARGMAX: the LM head's epilogue, apart so that the other launches do not carry its registers (96 for all of them instead of 66 and 77).
-template <bool WIDE, bool ARGMAX>
+// ARGMAX: the LM head's epilogue, apart so that the other launches do not carry its registers (96 for all of them instead of 64).
+template <bool ARGMAX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
 gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Gemm2Args g) {
   extern __shared__ uint8_t smem_raw[];
@@ -141,15 +139,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     kt_begin = (v % g.tail_splits) * g.k_tiles_per_split;
     kt_end = min(g.k_tiles, kt_begin + g.k_tiles_per_split);
   };
-  const uint32_t tmem_cols = WIDE ? g.acc_cols : 2u * g.acc_cols;
-  // A wide tile is two instructions of BNT / 2 columns each: instruction h takes rows h * BNT/4 .. of what either CTA has staged.  Column
-  // c of the accumulator is activation row row_of(c) of the tile.
-  const int half_cols = WIDE ? g.BNT / 2 : g.BNT;
-  auto row_of = [&](int c) {
-    if (!WIDE) return c;
-    const int q = g.BNT / 4, h = c >= half_cols ? 1 : 0, cc = c - h * half_cols;
-    return h * q + (cc < q ? cc : cc + q);
-  };
+  const uint32_t tmem_cols = 2u * g.acc_cols;                // two accumulators
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
@@ -230,8 +220,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
   } else if (warp == 1) {
     if (rank == 0 && elect_one()) {
-      const uint32_t idesc = idesc_m256(uint32_t(half_cols), g.f16 != 0);
-      const uint64_t db_half = uint64_t(g.BNT / 4 * 128 >> 4);
+      const uint32_t idesc = idesc_m256(uint32_t(g.BNT), g.f16 != 0);
       uint32_t it = 0, tile_count = 0;
       bool ok = true;
       for (int unit = cluster_id; unit < total_units && ok; unit += n_clusters, ++tile_count) {
@@ -253,11 +242,8 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const uint32_t sa = smem_u32(smem + size_t(s) * stage_bytes + size_t(sub) * sub_bytes);
             const uint64_t da = umma_desc_kmajor_sw128(sa), db = umma_desc_kmajor_sw128(sa + A_BYTES);
 #pragma unroll
-            for (int kk = 0; kk < TILE_K / 16; ++kk) {
-              const uint32_t add = (kt > kt_begin || sub > 0 || kk > 0) ? 1u : 0u;
-              umma_2sm(tmem_acc, da + uint64_t(kk * 2), db + uint64_t(kk * 2), idesc, add);
-              if (WIDE) umma_2sm(tmem_acc + uint32_t(half_cols), da + uint64_t(kk * 2), db + db_half + uint64_t(kk * 2), idesc, add);
-            }
+            for (int kk = 0; kk < TILE_K / 16; ++kk)
+              umma_2sm(tmem_acc, da + uint64_t(kk * 2), db + uint64_t(kk * 2), idesc, (kt > kt_begin || sub > 0 || kk > 0) ? 1u : 0u);
           }
           umma_commit_pair(smem_u32(&tail->empty[s]));
         }
@@ -303,11 +289,7 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const int m0 = tm * g.BNT;
       const uint32_t tmem_acc = tmem_base + acc * g.acc_cols + (uint32_t(q * 32) << 16);
       for (int c0 = ((warp - 2) >> 2) * 16; c0 < g.BNT; c0 += EPI_WARPS * 4) {
-        // activation rows of the first and of the last eight columns (a wide tile's rows make a jump every BNT / 4 columns)
-        const int ma = m0 + row_of(c0), mb = WIDE ? m0 + row_of(c0 + 8) - 8 : ma;
-        auto row = [&](int j) { return (j < 8 ? ma : mb) + j; };
-        if (!WIDE && ma >= g.M) break;                      // rows past M: nothing to store (warp-uniform)
-        if (WIDE && ma >= g.M && mb + 8 >= g.M) continue;
+        if (m0 + c0 >= g.M) break;                          // rows past M: nothing to store (warp-uniform)
         uint32_t r[16];
         tmem_ld16(tmem_acc + uint32_t(c0), r);
         tmem_ld_wait();
@@ -345,12 +327,12 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           float* out = g.part + (size_t(tile - g.n_full_tiles) * g.tail_splits + sp) * size_t(g.BNT) * 256 +
                        int(rank) * 128 + q * 32 + lane;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) out[size_t(row(j) - m0) * 256] = __uint_as_float(r[j]);
+          for (int j = 0; j < 16; ++j) out[size_t(c0 + j) * 256] = __uint_as_float(r[j]);
         } else if (mode == EPI_STORE_F32) {
           float* out = reinterpret_cast<float*>(g.out);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int m = row(j);
+            const int m = m0 + c0 + j;
             if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __uint_as_float(r[j]);
           }
         } else if (mode == EPI_ACCUM_F32) {
@@ -361,24 +343,24 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           float* out = reinterpret_cast<float*>(g.out);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int m = row(j);
+            const int m = m0 + c0 + j;
             if (n_ok && m < g.M) red_add_f32(out + size_t(m) * g.ldo + n, __uint_as_float(r[j]));
           }
         } else if (mode == EPI_SWIGLU_F16 || mode == EPI_SWIGLU_BF16) {
           const int f = tile_n128 * 64 + q * 16 + (lane & 15);
-          swiglu_store16(r, g.out, mode == EPI_SWIGLU_BF16, g.ldo, ma, mb, g.M, f, 2 * f < g.N_out, lane, g.status);
+          swiglu_store16(r, g.out, mode == EPI_SWIGLU_BF16, g.ldo, m0 + c0, g.M, f, 2 * f < g.N_out, lane, g.status);
         } else if (mode == EPI_STORE_F16) {
           __half* out = reinterpret_cast<__half*>(g.out);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int m = row(j);
+            const int m = m0 + c0 + j;
             if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = f16_sat(__uint_as_float(r[j]), g.status);
           }
         } else if (mode == EPI_STORE_BF16) {
           __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(g.out);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int m = row(j);
+            const int m = m0 + c0 + j;
             if (n_ok && m < g.M) out[size_t(m) * g.ldo + n] = __float2bfloat16_rn(__uint_as_float(r[j]));
           }
         }
@@ -469,38 +451,29 @@ bool gemm2_preferred(int M, int n_out) {
 // One cost unit ~ 2.2 ns (a k-step of a 256-wide pair tile = 256 units ~ 0.56 us).
 // The rows are spread evenly over the tiles, in steps of 16, so that the last one is not mostly padding: 549 rows are three tiles of 192
 // and not of 256 (n_out = 28672, K = 4096: 134 -> 122 us; n_out = 4096, K = 14336: 70 -> 66 us).
-// Tiles of more than 256 rows (one accumulator of up to all 512 columns) where every cluster then has a single unit, so that nothing waits for
-// the accumulator: 549 rows as two tiles of 288 instead of four of 144, 512 rows of n_out = 17536 as 69 units instead of 138 in two waves.  Us, without
-// -> with: 549 rows, n_out = 4096, K = 14336 67 -> 61 in the step; 257 rows, 5120, 25600 100 -> 76; 17536, 4096: 300 rows 48 -> 44.5, 400 65 -> 62,
-// 512 65 -> 62.5.  (Slices of wide tiles are charged 14 us: with the 2 of the others 549 x 4096 x 8192 was sliced and went from 41 to 51.)
-void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out, bool may_be_wide) {
+void gemm2_pick(int M, int n_out, int K, int mode, int* bnt_out, int* splits_out) {
   const int tw = (n_out + 255) / 256;
   const int k_tiles = (K + TILE_K - 1) / TILE_K;
   const bool may_split = mode != EPI_ARGMAX;            // every other epilogue can be applied after the slices are summed
   double best_cost = 1e30;
   int best_bnt = 256, best_s = 1;
-  for (int i = 0; i < 13; ++i) {
-    const int widest = i < 5 ? 256 - 32 * i : 288 + 32 * (i - 5);
-    const bool wide = widest > 256;
-    if (wide && (!may_be_wide || mode == EPI_ARGMAX)) break;
-    const int nm = (M + widest - 1) / widest, grain = wide ? 32 : 16;
-    const int bnt = ((M + nm - 1) / nm + grain - 1) / grain * grain;
-    if (wide && bnt <= 256) continue;
+  for (int widest = 256; widest >= 128; widest -= 32) {
+    const int nm = (M + widest - 1) / widest;
+    const int bnt = ((M + nm - 1) / nm + 15) / 16 * 16;
     const int tiles = tw * nm;
     const int full_waves = tiles / 74, tail = tiles % 74;
     // a k-step fills 16 KB of weights and BNT x 64 bytes of activations per SM: below 256 rows it is this fill that sets the
-    // pace (measured, a 128-wide tile runs 1.5x slower per flop than a 256-wide one), above them the instructions
-    const double kstep = wide ? bnt : 128.0 + 0.5 * bnt;
+    // pace (measured, a 128-wide tile runs 1.5x slower per flop than a 256-wide one)
+    const double kstep = 128.0 + 0.5 * bnt;
     for (int s = 1; s <= 8; ++s) {
       if (s > 1 && (!may_split || tail == 0 || tail * s > 74 || k_tiles / s < 8)) continue;
-      if (wide && (tiles * s > 74 || (s > 1 && tail * s * bnt > 74 * 256))) continue;       // one unit per cluster; the scratch for slices
       const int kps = (k_tiles + s - 1) / s;
       if (s > 1 && kps * (s - 1) >= k_tiles) continue;         // an empty last slice
       double cost = double(full_waves) * (k_tiles * kstep + 1500.0);
       if (tail > 0) cost += kps * kstep + 1500.0;
       // (the pass that sums the slices: its bytes at 4 TB/s plus 2 us; with 4, 8, 12 or 20 us fewer launches are sliced and
       // the 256-row steps get slower, 1.93 -> 1.95 / 2.02 / 2.07 / 2.10 ms at paper_8b; no difference at 2048 rows)
-      if (s > 1) cost += (double(s + 2) * tail * bnt * 256 * 4.0 / 4.0e6 + (wide ? 14.0 : 2.0)) * 455.0;
+      if (s > 1) cost += (double(s + 2) * tail * bnt * 256 * 4.0 / 4.0e6 + 2.0) * 455.0;
       if (cost < best_cost) { best_cost = cost; best_bnt = bnt; best_s = s; }
     }
   }
@@ -515,10 +488,9 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   {
     const cudaError_t e = once_per_device(g_attr_done2, [](int dev) {
       cudaError_t e2 = cudaDeviceGetAttribute(&g_smem_optin2[dev], cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      if (e2 == cudaSuccess) e2 = cudaFuncSetAttribute(gemm_2sm_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_smem_optin2[dev]);
-      if (e2 == cudaSuccess) e2 = cudaFuncSetAttribute(gemm_2sm_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_smem_optin2[dev]);
-      if (e2 == cudaSuccess) e2 = cudaFuncSetAttribute(gemm_2sm_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_smem_optin2[dev]);
-      return e2;
+      if (e2 != cudaSuccess) return e2;
+      e2 = cudaFuncSetAttribute(gemm_2sm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_smem_optin2[dev]);
+      return e2 != cudaSuccess ? e2 : cudaFuncSetAttribute(gemm_2sm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_smem_optin2[dev]);
     });
     if (e != cudaSuccess) return e;
   }
@@ -526,10 +498,8 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   Gemm2Args g{};
   g.M = c.M; g.N_out = c.n_out; g.K = c.K;
   int splits = 1;
-  gemm2_pick(c.M, c.n_out, c.K, c.mode, &g.BNT, &splits, true);
-  if (g.BNT > 256 && c.splits > 0 && c.splits != splits)      // another number of slices could give a cluster a second unit
-    gemm2_pick(c.M, c.n_out, c.K, c.mode, &g.BNT, &splits, false);
-  g.acc_cols = g.BNT > 256 ? 512 : g.BNT > 128 ? 256 : (g.BNT > 64 ? 128 : 64);
+  gemm2_pick(c.M, c.n_out, c.K, c.mode, &g.BNT, &splits);
+  g.acc_cols = g.BNT > 128 ? 256 : (g.BNT > 64 ? 128 : 64);
   g.k_tiles = (c.K + TILE_K - 1) / TILE_K;
   g.raster.n_tiles_w = (c.n_out + 255) / 256;
   g.raster.n_tiles_m = (c.M + g.BNT - 1) / g.BNT;
@@ -558,7 +528,7 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   if (c.addend != nullptr) { if (err) *err = "the 2-SM kernel has no addend epilogue"; return cudaErrorInvalidValue; }
   g.logits = c.logits; g.keys = c.keys; g.status = c.status;
   static const int ksub_env = [] { const char* e = getenv("HSPEC_GEMM2_KSUB"); return e ? atoi(e) : 0; }();   // measurements only
-  g.ksub = (ksub_env == 1 || ksub_env == 2) ? ksub_env : g.BNT > 256 ? 1 : 2;   // (eight instructions per barrier round either way)
+  g.ksub = (ksub_env == 1 || ksub_env == 2) ? ksub_env : 2;
   const size_t stage_bytes = size_t(g.ksub) * (A_BYTES + size_t(g.BNT / 2) * TILE_K * 2);
   const size_t fixed = sizeof(Tail2) + 1024;
   int stages = int((size_t(smem_optin2) - fixed) / stage_bytes);
@@ -578,7 +548,8 @@ cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, s
   }
   trk_begin(trk, label, 2.0 * c.M * c.n_out * c.K, 2.0 * c.n_out * c.K,
             gemm_io_bytes(c.M, c.n_out, c.K, c.mode, c.logits != nullptr));
-  cudaError_t e = launch_pdl(g.BNT > 256 ? gemm_2sm_kernel<true, false> : c.mode == EPI_ARGMAX ? gemm_2sm_kernel<false, true> : gemm_2sm_kernel<false, false>, dim3(2 * clusters), dim3(GEMM2_THREADS), smem, stream, *c.tmW, tmB, g);
+  cudaError_t e = launch_pdl(c.mode == EPI_ARGMAX ? gemm_2sm_kernel<true> : gemm_2sm_kernel<false>, dim3(2 * clusters), dim3(GEMM2_THREADS), smem, stream,
+                             *c.tmW, tmB, g);
   trk_end(trk);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (c.defer_tail) *c.defer_tail = GemmTail{};

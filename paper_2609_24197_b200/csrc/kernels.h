@@ -206,7 +206,7 @@ int gemm_pick_splits(int M, int n_out, int K, int num_sms, int mode = EPI_STORE_
 cudaError_t gemm_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 bool gemm2_preferred(int M, int n_out);        // many rows and at least one full round of cluster tiles
 size_t gemm2_tail_bytes();                     // scratch the 2-SM kernel's K-sliced tail wave may use
-void gemm2_pick(int M, int n_out, int K, int mode, int* bnt, int* splits, bool may_be_wide);   // tile width and K-slices of the 2-SM kernel
+void gemm2_pick(int M, int n_out, int K, int mode, int* bnt, int* splits);   // tile width and K-slices of the 2-SM kernel
 cudaError_t gemm2_launch(const GemmCall& c, cudaStream_t stream, Tracker* trk, std::string* err);
 // Zeroes the keys, for callers that have no kernel of their own in front to do it; ids from the keys (id_map: vocabulary row -> token id).
 cudaError_t argmax_init_launch(unsigned long long* keys, int M, cudaStream_t stream);

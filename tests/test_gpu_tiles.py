@@ -489,8 +489,22 @@ def test_rmsnorm_rows_ahead(hs, M, n):
     assert torch.equal(x, before)
 
 
-# the pair GEMM's wide tiles (257 to 512 activation rows, two instructions): every width in steps of 32 with as many rows as it holds and with one
-# more than the width before, a last weight tile that is part full, K that ends in a part k-step, one slice and three to six, two wide tiles
+# Launches of the pair GEMM that take no K-slices add a row's products in the order of K, whatever the tile's width: a call's rows are the bits that the
+# same rows have among others.  (Tiles of more than 256 rows, sliced where the others are not, moved the sums of 257 rows of 5120 and of 549 of 4096.)
+@pytest.mark.parametrize("M,others,n_out,K", [(257, 300, 5120, 8192), (549, 640, 4096, 14336), (320, 301, 5120, 25600), (400, 512, 17536, 256)])
+@pytest.mark.parametrize("kind", [torch.float16, torch.bfloat16])
+def test_gemm_rows_keep_their_bits_among_others(hs, M, others, n_out, K, kind):
+    x, W = _rand((max(M, others), K), 1, kind), _rand((n_out, K), 2, kind, 0.05)
+
+    def rows(m):
+        y = torch.full((m, n_out), float("nan"), device="cuda")
+        hs.hspec_op_gemm(x[:m].contiguous(), W, y, workspace=torch.empty(hs.hspec_gemm_workspace_bytes(m, n_out, K), dtype=torch.uint8, device="cuda"))
+        return y[:min(M, others)]
+    assert torch.equal(rows(M), rows(others))
+
+
+# the pair GEMM at 257 to 549 rows, where the rows are spread over two to four tiles: a whole wave and a tail of almost one, a last weight tile that is part full,
+# K that ends in a part k-step or is shorter than one, one slice (most), two (270 rows) and three (257 of 2560)
 @pytest.mark.parametrize("M,n_out,K", [(257, 17000, 520), (288, 17000, 512), (289, 17000, 72), (352, 17000, 128), (353, 17000, 192), (416, 17000, 64), (417, 17000, 512),
                                        (480, 17000, 512), (481, 17000, 8), (512, 17408, 256), (257, 5000, 4096), (270, 4096, 4096), (257, 2560, 4096),
                                        (549, 4096, 8192)])
@@ -510,7 +524,7 @@ def test_wide_gemm_tiles(hs, M, n_out, K, kind, out):
     assert hs.hspec_op_device_status()["rc"] == 0
 
 
-# the SwiGLU epilogue of a wide tile, with 300 and 512 rows
+# the SwiGLU epilogue with several tiles of rows: 300 and 512 rows
 @pytest.mark.parametrize("B,k", [(30, 10), (16, 32)])
 def test_wide_gemm_tiles_with_swiglu(hs, B, k):
     import synth
