@@ -113,7 +113,7 @@ __device__ __forceinline__ void scan_general(const ScanArgs& a) {
   // ---- stage S_init[b, h] (fp16 -> fp32), 16-byte loads
   if (a.s_init != nullptr) {
     const __half* src = a.s_init + (size_t(b) * a.H + h) * P * N;
-    if ((N & 7) == 0) {
+    if ((N & 7) == 0 && (reinterpret_cast<uintptr_t>(a.s_init) & 15) == 0) {
       const int vec = P * N / 8;
       for (int idx = tid; idx < vec; idx += SCAN_THREADS) {
         const uint4 raw = reinterpret_cast<const uint4*>(src)[idx];
@@ -853,9 +853,12 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
   a.w_stable = c.w_stable ? 1 : 0;
   a.NP = c.N + 1;                                    // odd pitch: threads of a warp own consecutive p
   if (a.H % c.G) { if (err) *err = "scan: heads must divide into groups"; return cudaErrorInvalidValue; }
-  // serving shapes: tensor-core path (needs 8-byte aligned rows for the float2 accesses)
-  if (c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ld_in % 2 == 0 && c.Di % 4 == 0 && c.ws != nullptr &&
-      (reinterpret_cast<uintptr_t>(c.s_init) & 31) == 0 &&     // its 32-byte loads of the state
+  // serving shapes: tensor-core paths.  z and y are read and written in pairs; the state comes by 32-byte loads with scratch (which is read in
+  // 16-byte copies) and by 16-byte ones without.  What is off these boundaries takes the general kernel.
+  const bool mma = c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ld_in % 2 == 0 &&
+                   ((reinterpret_cast<uintptr_t>(c.zxbcdt) | reinterpret_cast<uintptr_t>(c.y_gated)) & 7) == 0 &&
+                   (reinterpret_cast<uintptr_t>(c.s_init) & 15) == 0;
+  if (mma && c.ws != nullptr && (reinterpret_cast<uintptr_t>(c.s_init) & 31) == 0 && (reinterpret_cast<uintptr_t>(c.ws) & 15) == 0 &&
       c.ws_bytes >= scan_workspace_bytes(c.B, c.k, c.Di, c.N, c.G)) {
     const bool two = c.k > 16;
     const size_t M = size_t(c.B) * c.k;
@@ -887,7 +890,7 @@ cudaError_t scan_launch(const ScanCall& c, cudaStream_t stream, Tracker* trk, st
     trk_end(trk);
     return e;
   }
-  if (c.P == 64 && c.N == 128 && (a.H / c.G) % 4 == 0 && c.ld_in % 2 == 0 && c.Di % 2 == 0) {
+  if (mma) {
     const bool two = c.k > 16;
     const size_t smem_f = two ? scan_mma_smem<2>() : scan_mma_smem<1>();
     static bool fset[2][MAX_DEVICES] = {};

@@ -474,6 +474,34 @@ def test_scan_as_a_process_first_call_under_capture():
     assert res.returncode == 0 and "same" in res.stdout, res.stdout[-2000:] + res.stderr[-2000:]
 
 
+# Operands off the boundaries that the vector loads of a path want: state (16-bit values) 2, 8 and 16 bytes behind a 32-byte boundary, rows in and out
+# 4 and 8 bytes behind a 16-byte one, scratch 8; the serving shapes and the general kernel, with scratch and without.  Each call has to give what the
+# aligned one gives: two kernels' fp32 sums of 128 products (2^-22 of some 20 RMS, as above).
+@pytest.mark.parametrize("P,N", [(64, 128), (24, 40)])
+@pytest.mark.parametrize("off_state,off_in,off_out,off_ws", [(1, 0, 0, 0), (4, 0, 0, 0), (8, 0, 0, 0), (0, 1, 0, 0), (0, 2, 0, 0), (0, 0, 1, 0), (0, 0, 2, 0), (0, 0, 0, 8),
+                                                             (4, 1, 1, 8)])
+@pytest.mark.parametrize("scratch", [True, False])
+def test_scan_of_misaligned_operands(hs, P, N, off_state, off_in, off_out, off_ws, scratch):
+    B, k, H, G, f32 = 2, 18, 8, 2, torch.float32
+    Di, d_xBC = H * P, H * P + 2 * G * N
+    conv_w, conv_b = _rand((d_xBC, 4), 4, f32, 0.3), _rand((d_xBC,), 5, f32, 0.02)
+    A_log, dt_bias, D = _rand((H,), 6, f32).abs(), _rand((H,), 7, f32) - 4.0, 1 + _rand((H,), 8, f32, 0.1)
+    zx, s0 = _rand((B * k, Di + d_xBC + H), 1, f32), _rand((B, H, P, N), 3, torch.float16, 1.5)
+
+    def at(t, off):                                            # a copy of t, `off` elements into its storage
+        flat = torch.empty(t.numel() + off, dtype=t.dtype, device="cuda")
+        flat[off:] = t.flatten()
+        return flat[off:].view(t.shape)
+
+    def run(o_state, o_in, o_out, o_ws):
+        y = at(torch.full((B * k, Di), float("nan"), device="cuda"), o_out)
+        ws = at(torch.zeros(hs.hspec_scan_workspace_bytes(B, k, Di, N, G), dtype=torch.uint8, device="cuda"), o_ws) if scratch else None
+        hs.hspec_op_mamba_scan(at(zx, o_in), None, at(s0, o_state), conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, 4, ws)
+        return y
+    want, got = run(0, 0, 0, 0), run(off_state, off_in, off_out, off_ws)
+    assert float((got - want).abs().max()) <= 1e-4 * max(1.0, float(want.square().mean().sqrt()))
+
+
 # the norm of wide rows, where a CTA fetches its next row ahead: one row per CTA and several, row lengths around 6144 (256 or 512 threads) and
 # 12 288 (the row no longer fits the registers), one that is no multiple of four
 @pytest.mark.parametrize("M", [1, 296, 297, 593])
