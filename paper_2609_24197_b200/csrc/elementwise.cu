@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(512, 2) rmsnorm_kernel(float* __restrict__ x, 
   pdl_wait();
   pdl_trigger();
   __shared__ float red[32];
-  const bool vec = (n & 3) == 0 && n <= 4 * VPT * int(blockDim.x);
+  const bool vec = (n & 3) == 0 && n <= 4 * VPT * int(blockDim.x) &&
+                   ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w) | (reinterpret_cast<uintptr_t>(y) << 1)) & 15) == 0;
   const int nv = n >> 2;
   float4 next[AHEAD ? VPT : 1];
   auto load_row = [&](float4 (&v)[VPT], int m) {

@@ -517,6 +517,18 @@ def test_rmsnorm_rows_ahead(hs, M, n):
     assert torch.equal(x, before)
 
 
+# the norm of operands off the boundaries of its vector loads and stores (x and w 16 bytes, y 8), in one CTA per row and with rows ahead
+@pytest.mark.parametrize("M,n", [(3, 256), (300, 8192)])
+@pytest.mark.parametrize("off_x,off_w,off_y", [(1, 0, 0), (2, 0, 0), (0, 1, 0), (0, 0, 1), (0, 0, 4), (3, 2, 6)])
+def test_rmsnorm_of_misaligned_operands(hs, M, n, off_x, off_w, off_y):
+    x = _rand((M * n + off_x,), 1, torch.float32, 3.0)[off_x:].view(M, n)
+    w = (1 + _rand((n + off_w,), 2, torch.float32, 0.1))[off_w:]
+    y = torch.full((M * n + off_y,), float("nan"), dtype=torch.float16, device="cuda")[off_y:].view(M, n)
+    hs.hspec_op_rmsnorm(x, w, y, 1e-6)
+    ref = x.double() / torch.sqrt((x.double() ** 2).mean(1, keepdim=True) + 1e-6) * w.double()
+    assert bool(((y.double() - ref).abs() <= ref.abs() * 2.0 ** -10.9 + 1e-6).all())
+
+
 # Launches of the pair GEMM that take no K-slices add a row's products in the order of K, whatever the tile's width: a call's rows are the bits that the
 # same rows have among others.  (Tiles of more than 256 rows, sliced where the others are not, moved the sums of 257 rows of 5120 and of 549 of 4096.)
 @pytest.mark.parametrize("M,others,n_out,K", [(257, 300, 5120, 8192), (549, 640, 4096, 14336), (320, 301, 5120, 25600), (400, 512, 17536, 256)])
