@@ -338,6 +338,9 @@ size_t hspec_attention_workspace_bytes(int32_t B, int32_t k, int32_t Hq, int32_t
  * bit-exact; used to check the page-table addressing of the attention kernel, Sec. 3.3.2). */
 int hspec_debug_gather_kv(const void* pool, const int32_t* page_table_row, int32_t ctx_len, int32_t page_size,
                           int32_t Hkv, int32_t dh, void* dst, void* stream);
+/* How y [M, n_out] = x [M, K] W^T is cut up where the kernel on pairs of SMs takes it (host only, for tests): tiles4 = activation rows
+ * per tile, K-slices of the tiles of the last wave, tiles, tiles of the last wave.  All zero where the one-SM kernel takes it. */
+int hspec_debug_gemm_tiles(int32_t M, int32_t n_out, int32_t K, int32_t* tiles4);
 /* h fp16 [M, F] = SiLU(gu[:, :F]) * gu[:, F:], gu fp32 [M, 2F] (App. B.1 "MLP"). */
 int hspec_op_swiglu(const float* gu, void* h_f16, int32_t M, int32_t F, void* stream);
 

@@ -23,7 +23,7 @@ EXPORTS = [
     "hspec_op_lm_head_argmax", "hspec_op_lm_head_argmax_noalloc", "hspec_op_rmsnorm", "hspec_op_mamba_scan", "hspec_scan_workspace_bytes", "hspec_op_qk_norm_rope",
     "hspec_op_attention", "hspec_attention_workspace_bytes", "hspec_debug_gather_kv", "hspec_op_swiglu",
     "hspec_op_accept", "hspec_op_token_probs", "hspec_op_markov_head", "hspec_markov_workspace_bytes",
-    "hspec_op_kv_inject_write", "hspec_op_device_status",
+    "hspec_op_kv_inject_write", "hspec_op_device_status", "hspec_debug_gemm_tiles",
 ]
 
 
@@ -119,6 +119,7 @@ def load_library(path=None):
                                        i32, vp, sz, vp]
     lib.hspec_attention_workspace_bytes.argtypes = [i32, i32, i32, i32, i32, i32, i32, i32]
     lib.hspec_attention_workspace_bytes.restype = sz
+    lib.hspec_debug_gemm_tiles.argtypes = [i32, i32, i32, C.POINTER(C.c_int32)]
     lib.hspec_debug_gather_kv.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp]
     lib.hspec_op_swiglu.argtypes = [vp, vp, i32, i32, vp]
     lib.hspec_op_device_status.argtypes = [C.POINTER(C.c_uint32), i32]
@@ -366,6 +367,13 @@ def hspec_debug_gather_kv(pool, page_table_row, ctx_len, dst):
     _check(load_library().hspec_debug_gather_kv(_ptr(pool, torch.bfloat16), _ptr(page_table_row, torch.int32),
                                                 int(ctx_len), page_size, Hkv, dh, _ptr(dst, torch.bfloat16),
                                                 _stream()), None, "hspec_debug_gather_kv")
+
+
+def hspec_debug_gemm_tiles(M, n_out, K):
+    """(activation rows per tile, K-slices of the last wave's tiles, tiles, tiles of the last wave); zeros: the one-SM kernel's call."""
+    t = (C.c_int32 * 4)()
+    _check(load_library().hspec_debug_gemm_tiles(int(M), int(n_out), int(K), t), None, "hspec_debug_gemm_tiles")
+    return tuple(t)
 
 
 def hspec_op_swiglu(gu, h):

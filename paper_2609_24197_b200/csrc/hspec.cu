@@ -978,6 +978,17 @@ int hspec_debug_gather_kv(const void* pool, const int32_t* page_table_row, int32
   return HSPEC_OK;
 }
 
+int hspec_debug_gemm_tiles(int32_t M, int32_t n_out, int32_t K, int32_t* tiles4) {
+  if (!tiles4 || M < 1 || n_out < 1 || K < 1) return fail(nullptr, HSPEC_ERR_INVALID_ARG, "hspec_debug_gemm_tiles: bad argument");
+  for (int i = 0; i < 4; ++i) tiles4[i] = 0;
+  if (!gemm2_preferred(M, n_out)) return HSPEC_OK;
+  int bnt = 0, splits = 0;
+  gemm2_pick(M, n_out, K, EPI_STORE_F32, &bnt, &splits);
+  const int tiles = (n_out + 255) / 256 * ((M + bnt - 1) / bnt);
+  tiles4[0] = bnt; tiles4[1] = splits; tiles4[2] = tiles; tiles4[3] = tiles % 74;
+  return HSPEC_OK;
+}
+
 int hspec_op_swiglu(const float* gu, void* h_f16, int32_t M, int32_t F, void* stream) {
   if (!gu || !h_f16 || M < 1 || F < 1) return fail(nullptr, HSPEC_ERR_INVALID_ARG, "hspec_op_swiglu: bad argument");
   std::string errtxt;

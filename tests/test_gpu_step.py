@@ -116,6 +116,29 @@ def test_request_independence_across_batch_sizes():
     d3.close()
 
 
+# One and a few requests at the serving width (state of 128, 128 heads), block lengths on both sides of the scan's tiles of 16 and no multiples of four: a
+# single id is several per cent of such a step, so every id whose margin in 64 bits is above the step's own error has to be the oracle's.
+@pytest.mark.parametrize("bf16", [False, True])
+def test_ids_of_few_requests_at_serving_width(bf16):
+    cfg = synth.derived(dict(D=4096, n_fuse=1, r=64, L=1, has_attn=[1], kv_slot=[0], n_slots=1, Di=8192, P=64, N=128, G=4, d_conv=4, dt_rank=0, Hq=32, Hkv=8,
+                             dh=128, rope_theta=1.0e6, window=0, qk_norm=1, F=2048, V=8000, rms_eps=1e-6, page_size=16, name="few", act_bf16=int(bf16),
+                             B=4, k=32, ctx=("uniform", 100, 700)))
+    w = synth.make_weights(cfg, device="cuda")
+    for ctx, k in [([300], 17), ([41], 20), ([129], 32), ([700, 3], 31), ([64, 500, 222], 27), ([1, 90, 333, 128], 24)]:
+        drafter, _, batch = cuda_setup(cfg, ctx_lens=ctx, max_k=32, weights=w)
+        ids, logits, _ = drafter.draft(batch, k, want_logits=True, max_ctx=max(ctx))
+        torch.cuda.synchronize()
+        ids, logits, ref = ids.cpu().numpy(), logits.cpu().numpy(), oracle_step(cfg, w, batch, k)
+        assert np.array_equal(ids, logits.argmax(-1))
+        e = assert_close(logits, ref["logits"], f"{len(ctx)} x {k}", TOL_BF16 if bf16 else 2e-2)
+        # two logits' errors (Gaussian, as sums of many roundings are) against each other, four of their deviations
+        margin = 4 * 2 ** 0.5 * float(np.sqrt(((logits - ref["logits"]) ** 2).mean()))
+        sure = ref["margin"] > margin
+        print(f"{len(ctx)} x {k}: max error {e:.1e}, margin {margin:.1e}, {int(sure.sum())} of {sure.size} ids above it, {int((ids != ref['draft_ids']).sum())} differ")
+        assert sure.mean() > 0.5 and np.array_equal(ids[sure], ref["draft_ids"][sure])
+        drafter.close()
+
+
 def _full_size(name, n_check, **over):
     """The workload at its full size, in the launch configuration bench.py times, compared with the oracle on `n_check`
     sampled requests (requests are independent, so each is a complete comparison): the longest, the shortest and the

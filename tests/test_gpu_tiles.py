@@ -20,13 +20,17 @@ def _rand(shape, seed, dtype=torch.float16, std=1.0):
     return (torch.randn(shape, generator=g, device="cuda") * std).to(dtype)
 
 
-# rows that make the 2-SM kernel take tiles of 256, 224, 192, 160 and 128 rows, full and with a remainder, whole waves and tail
-# waves; weight rows that end inside a tile of the pair; more activation tiles than one group of the walk holds
-@pytest.mark.parametrize("M,n_out,K", [(256, 256, 64), (257, 300, 520), (289, 1000, 512), (430, 2048, 1024), (448, 2048, 1024),
-                                       (449, 512, 2048), (549, 4096, 1024), (640, 19200, 256), (1153, 1111, 264),
-                                       (4500, 1200, 2048)])
+# rows that make the 2-SM kernel take tiles of many widths, full and with a remainder, whole waves and tail waves with one to eight slices (as
+# asserted: rows per tile, slices, tiles, tiles of the last wave); weight rows that end inside a tile of the pair; more activation tiles (29) than
+# one group of the walk holds
+@pytest.mark.parametrize("M,n_out,K,tiles", [(256, 256, 64, (128, 1, 2, 2)), (257, 300, 520, (96, 1, 6, 6)), (289, 1000, 512, (112, 1, 12, 12)),
+                                             (430, 2048, 1024, (112, 1, 32, 32)), (448, 2048, 1024, (112, 1, 32, 32)), (449, 512, 2048, (128, 4, 8, 8)),
+                                             (549, 4096, 1024, (144, 1, 64, 64)), (640, 19200, 256, (224, 1, 225, 3)), (1153, 1111, 264, (128, 1, 50, 50)),
+                                             (4500, 1200, 2048, (160, 1, 145, 71)), (270, 4096, 4096, (144, 2, 32, 32)), (257, 2560, 4096, (144, 3, 20, 20)),
+                                             (130, 1024, 8192, (80, 8, 8, 8)), (1130, 4096, 4096, (240, 8, 80, 6))])
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
-def test_many_row_gemm_tile_widths(hs, M, n_out, K, kind):
+def test_many_row_gemm_tile_widths(hs, M, n_out, K, tiles, kind):
+    assert hs.hspec_debug_gemm_tiles(M, n_out, K) == tiles
     x, w = _rand((M, K), 1), _rand((n_out, K), 2, std=0.05)
     ref = x.double() @ w.double().t()
     y = torch.zeros((M, n_out), dtype=torch.float16 if kind == "f16" else torch.float32, device="cuda")
@@ -218,10 +222,14 @@ def test_attention_warps_per_row(hs, dh, page, B, Hkv, k, rep, window):
     _attention_against_fp64(hs, [(37 * b + 61) % 129 for b in range(B)], k, rep, window, 256, dh, Hkv, page)
 
 
-# the norm behind a residual GEMM adds the GEMM's K-sliced tail tiles: row counts with a whole-wave part and a tail, all tail, and no tail,
-# widths above and below what the norm keeps in registers (6 x 4 x 256 and 6 x 4 x 512 floats), hidden state asked for
-@pytest.mark.parametrize("D,F,B,k", [(512, 4096, 9, 32), (4096, 2048, 20, 13), (7168, 1024, 9, 30), (12544, 512, 10, 26), (1280, 1024, 141, 32)])
-def test_residual_tail_is_added_by_the_norm(hs, D, F, B, k):
+# the norm behind a residual GEMM adds the GEMM's K-sliced tail tiles: two slices and three to eight (behind the out and the down projection, as asserted),
+# one (nothing to add), all tail and a whole wave in front of it; widths that take 256 and 512 threads and those that no longer fit the norm's
+# registers (6 x 4 x 256 and 6 x 4 x 512 floats); hidden state asked for
+@pytest.mark.parametrize("D,F,B,k,out_slices,down_slices", [(512, 4096, 9, 32, 2, 8), (4096, 2048, 20, 13, 1, 1), (4096, 4096, 5, 29, 1, 4), (2048, 4096, 9, 31, 1, 4),
+                                                          (7168, 1024, 9, 30, 1, 1), (12544, 512, 10, 26, 1, 1), (12544, 4096, 10, 26, 1, 3), (12800, 4096, 9, 31, 1, 2),
+                                                          (1280, 1024, 141, 32, 1, 1)])
+def test_residual_tail_is_added_by_the_norm(hs, D, F, B, k, out_slices, down_slices):
+    assert (hs.hspec_debug_gemm_tiles(B * k, D, 1024)[1], hs.hspec_debug_gemm_tiles(B * k, D, F)[1]) == (out_slices, down_slices)
     import synth
     from harness import check_step, cuda_setup
     cfg = synth.derived(dict(D=D, n_fuse=1, r=64, L=1, has_attn=[0], kv_slot=[-1], n_slots=0, Di=1024, P=64, N=4, G=1, d_conv=4, dt_rank=0,
@@ -246,13 +254,17 @@ def test_small_state_scan_with_norm(hs, Di, P, N, G, dt_rank, B, k):
     drafter.close()
 
 
-# the QK norm behind the QKV projection adds that GEMM's K-sliced tail tiles up to 512 rows (here 260 to 512; 513 and a whole wave with a tail behind
-# it take the pass of their own): heads of a quarter and of half a weight tile, a last weight tile that is only part full
-@pytest.mark.parametrize("dh,Hq,Hkv,B,k", [(64, 16, 4, 9, 32), (128, 8, 2, 9, 32), (128, 6, 1, 20, 13), (128, 8, 2, 16, 32), (64, 14, 2, 27, 19), (64, 14, 2, 141, 32)])
-def test_qkv_tail_is_added_by_the_qk_norm(hs, dh, Hq, Hkv, B, k):
+# the QK norm behind the QKV projection adds that GEMM's K-sliced tail tiles up to 512 rows (513 and a whole wave with a tail behind it take the pass
+# of their own, where there are slices): one slice to eight, as asserted; heads of a quarter and of half a weight tile, a last weight tile that is only part full
+@pytest.mark.parametrize("D,dh,Hq,Hkv,B,k,slices", [(1024, 64, 16, 4, 9, 32, 1), (1024, 128, 8, 2, 9, 32, 1), (1024, 128, 6, 1, 20, 13, 1), (1024, 128, 8, 2, 16, 32, 1),
+                                                     (1024, 64, 14, 2, 27, 19, 1), (1024, 64, 14, 2, 141, 32, 1), (1024, 64, 14, 2, 5, 29, 2), (2048, 64, 16, 4, 9, 32, 4),
+                                                     (2048, 128, 6, 1, 20, 13, 4), (2048, 128, 8, 2, 16, 32, 3), (2048, 64, 14, 2, 27, 19, 4), (4096, 128, 8, 2, 9, 32, 6),
+                                                     (4096, 64, 14, 2, 5, 29, 7)])
+def test_qkv_tail_is_added_by_the_qk_norm(hs, D, dh, Hq, Hkv, B, k, slices):
     import synth
     from harness import check_step, cuda_setup
-    cfg = synth.derived(dict(D=1024, n_fuse=1, r=64, L=1, has_attn=[1], kv_slot=[0], n_slots=1, Di=1024, P=64, N=4, G=1, d_conv=4, dt_rank=0,
+    assert hs.hspec_debug_gemm_tiles(B * k, (Hq + 2 * Hkv) * dh, D)[1] == slices
+    cfg = synth.derived(dict(D=D, n_fuse=1, r=64, L=1, has_attn=[1], kv_slot=[0], n_slots=1, Di=1024, P=64, N=4, G=1, d_conv=4, dt_rank=0,
                              Hq=Hq, Hkv=Hkv, dh=dh, rope_theta=1.0e4, window=0, qk_norm=1, F=512, V=600, rms_eps=1e-6, page_size=16, name="qkvtail",
                              B=B, k=k, ctx=("const", 20, 20)))
     drafter, w, batch = cuda_setup(cfg, ctx_lens=[b % 40 for b in range(B)])
@@ -287,6 +299,28 @@ def test_lm_head_argmax_ties(hs, M, V, alloc):
         best = z.max(1, keepdim=True).values
         first = torch.where(z == best, torch.arange(V, device="cuda"), V).min(1).values.int()     # exact: the kernel's own logits
         assert torch.equal(ids, first)
+
+
+# logits that rise along the vocabulary (every column group reaches its rows' maxima so far and runs the reduction), that fall (only the first ones do) and
+# that are all the same; whole and part tiles, with logits written and without
+@pytest.mark.parametrize("M", [33, 77, 128, 300])
+@pytest.mark.parametrize("V", [16384, 16500, 40001])
+@pytest.mark.parametrize("write", [True, False])
+def test_lm_head_argmax_in_its_worst_orders(hs, M, V, write):
+    K, v = 64, torch.arange(V, device="cuda")
+    x, W = torch.zeros((M, K), dtype=torch.float16, device="cuda"), _rand((V, K), 2, torch.float16)
+    W[:, 0], W[:, 1] = (v // 128 * 128).half(), (v % 128).half()                  # v, exactly, over two columns
+    x[0::3, :2], x[1::3, :2] = 1.0, -1.0
+    want = torch.zeros(M, dtype=torch.int32, device="cuda")
+    want[0::3] = V - 1
+    ids, logits = torch.full((M,), -1, dtype=torch.int32, device="cuda"), torch.full((M, V), float("nan"), device="cuda") if write else None
+    hs.hspec_op_lm_head_argmax_noalloc(x, W, ids, logits=logits)
+    assert torch.equal(ids, want)
+    ws = torch.full((((V + 127) // 128) * M * 8 + 1024,), 255, dtype=torch.uint8, device="cuda")
+    hs.hspec_op_lm_head_argmax(x, W, ids.fill_(-1), logits, ws)
+    assert torch.equal(ids, want)
+    if write:
+        assert torch.equal(logits[0], v.float()) and torch.equal(logits[1], -v.float()) and not bool(logits[2].any())
 
 
 # a NaN logit counts as -inf: one at the first and the last row of a tile and of the matrix, next to and away from the maximum, a row that is
@@ -380,9 +414,10 @@ def test_low_rank_dt_in_the_scan(hs, Di, N, G, dt_rank, B, k, bf16):
 # the scan of the serving shapes (P = 64, N = 128), with scratch: one tile of 16 positions and two, on both sides; few blocks and several waves of
 # them; groups of four heads and one group of all; rows of 16-byte multiples (vector loads of the conv), of 8-byte ones (scalar) and, off the 8 bytes,
 # the general kernel; no state
-@pytest.mark.parametrize("B,k,H,G,ld_extra,state", [(1, 1, 4, 1, 0, True), (3, 15, 8, 2, 0, True), (41, 16, 64, 16, 0, True), (41, 17, 64, 16, 0, True),
-                                                    (75, 32, 32, 1, 0, True), (40, 9, 36, 3, 1, True), (40, 31, 36, 3, 2, True), (64, 5, 32, 2, 0, False)])
-def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
+@pytest.mark.parametrize("B,k,H,G,ld_extra,state,d_conv", [(1, 1, 4, 1, 0, True, 4), (3, 15, 8, 2, 0, True, 4), (41, 16, 64, 16, 0, True, 4), (41, 17, 64, 16, 0, True, 4),
+                                                           (75, 32, 32, 1, 0, True, 4), (40, 9, 36, 3, 1, True, 4), (40, 31, 36, 3, 2, True, 4), (64, 5, 32, 2, 0, False, 4),
+                                                           (2, 9, 8, 2, 0, True, 3), (2, 17, 8, 2, 0, True, 2), (2, 32, 8, 2, 2, True, 1)])
+def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state, d_conv):
     import numpy as np
     from oracle import hspec_oracle as O
     P, N = 64, 128
@@ -390,11 +425,11 @@ def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
     ld = Di + d_xBC + H + ld_extra
     zx = _rand((B * k, ld), 1, f32)
     s0 = _rand((B, H, P, N), 3, torch.float16, 1.5) if state else None
-    conv_w, conv_b = _rand((d_xBC, 4), 4, f32, 0.3), _rand((d_xBC,), 5, f32, 0.02)
+    conv_w, conv_b = _rand((d_xBC, d_conv), 4, f32, 0.3), _rand((d_xBC,), 5, f32, 0.02)
     A_log, dt_bias, D = _rand((H,), 6, f32).abs(), _rand((H,), 7, f32) - 4.0, 1 + _rand((H,), 8, f32, 0.1)
     y = torch.full((B * k, Di), float("nan"), device="cuda")
     ws = torch.full((hs.hspec_scan_workspace_bytes(B, k, Di, N, G),), 255, dtype=torch.uint8, device="cuda")      # NaN wherever nothing is written
-    hs.hspec_op_mamba_scan(zx, None, s0, conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, 4, ws)
+    hs.hspec_op_mamba_scan(zx, None, s0, conv_w, conv_b, dt_bias, A_log, D, y, B, k, Di, P, N, G, d_conv, ws)
     assert bool(torch.isfinite(y).all())
     f64 = lambda t: t.double().cpu().numpy()
     for b in sorted({0, 1 % B, B // 2, B - 1}):
@@ -406,8 +441,10 @@ def test_scan_tiles_on_tensor_cores(hs, B, k, H, G, ld_extra, state):
                                   xBC[:, Di + G * N:].reshape(k, G, N), dt, a, f64(D))
         ref = yy.reshape(k, Di) * O.silu(rows[:, :Di])
         got = f64(y[b * k:(b + 1) * k])
-        # sums of 128 products with C in 22 bits and of 32 in fp32, SiLU and decay by the special-function unit (2^-22 relative each): together some
-        # 10 x 2^-22 of the terms' absolute sum, which is below 20 RMS; 1e-4 leaves a factor of two
+        # sums of 128 products with C in 22 bits and of up to 32 with both factors in 21 or 22; exp(x), in SiLU and decay, to about (2 + |x|) x 2^-23 of itself
+        # (x log2 e is rounded before the power), so of no weight where |x| is large and the value e^-|x|: in all some 3 x 2^-22 of the
+        # result, RMS over RMS (4.9e-7 to 6e-7 measured; twice that allowed), and at a single place 10 x 2^-22 of the terms' absolute sum, which is below 20 RMS
+        assert np.sqrt(((got - ref) ** 2).mean()) <= 6 * 2.0 ** -22 * np.sqrt((ref ** 2).mean())
         assert np.abs(got - ref).max() <= 1e-4 * max(1.0, np.sqrt((ref ** 2).mean())), np.abs(got - ref).max()
     assert hs.hspec_op_device_status()["rc"] == 0
 
