@@ -31,6 +31,10 @@ def _rand(shape, seed, dtype=torch.float16, std=1.0):
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
 def test_many_row_gemm_tile_widths(hs, M, n_out, K, tiles, kind):
     assert hs.hspec_debug_gemm_tiles(M, n_out, K) == tiles
+    _gemm_against_fp64(hs, M, n_out, K, kind)
+
+
+def _gemm_against_fp64(hs, M, n_out, K, kind):
     x, w = _rand((M, K), 1), _rand((n_out, K), 2, std=0.05)
     ref = x.double() @ w.double().t()
     y = torch.zeros((M, n_out), dtype=torch.float16 if kind == "f16" else torch.float32, device="cuda")
@@ -161,7 +165,7 @@ def test_step_with_shared_first_layer_rows(hs, B, k, over):
 @pytest.mark.parametrize("n_out,K", [(256, 4096), (130, 1000), (4096, 2048), (9000, 520), (17000, 640)])
 @pytest.mark.parametrize("kind", ["f32", "accumulate", "f16"])
 def test_few_row_gemm_slices(hs, M, n_out, K, kind):
-    test_many_row_gemm_tile_widths(hs, M, n_out, K, kind)
+    _gemm_against_fp64(hs, M, n_out, K, kind)
 
 
 def _attention_against_fp64(hs, ctx, k, rep, window, chunk, dh, Hkv, page=16):
