@@ -1,12 +1,16 @@
 // Mamba-2 mixer core over the k block rows, started from the injected state (paper Sec. 3.3.1).
 //
-// One CTA per (request, head).  Because the recurrence S_i = a_i S_{i-1} + dt_i x_i B_i^T is linear,
-// all k positions are evaluated in one pass without carrying the state:
+// Because the recurrence S_i = a_i S_{i-1} + dt_i x_i B_i^T is linear, all k positions are evaluated in one
+// pass without carrying the state:
 //   y_t = exp(c_t) * (S_init C_t)  +  sum_{s<=t} exp(c_t - c_s) dt_s (C_t . B_s) x_s  +  D x_t,
 //   c_t = sum_{r<=t} dt_r A   (inclusive prefix sum over the block positions, one warp shuffle scan).
-// S_init (fp16 [P, N] per head) is read from HBM exactly once with 16-byte loads; it is the only
-// large operand, so the kernel is bound by that read.  The causal depthwise conv + SiLU of x, B, C
-// (zero left context), softplus(dt), the D skip and the SiLU(z) gate are fused around it.
+// S_init (fp16 [P, N] per head) is read from HBM exactly once; it is the largest operand where N is large.  The causal
+// depthwise conv + SiLU of x, B, C (zero left context), softplus(dt), the D skip and the SiLU(z) gate are part of it.
+// Forms, as scan_launch() chooses them:
+//   P = 64, N = 128 with scratch     scan_conv_kernel, then mamba_scan_stream_kernel (one warp per head, tensor-core fragments)
+//   the same without scratch         mamba_scan_mma_kernel, everything in one
+//   N <= 16                          scan_small_state_kernel, the state in registers; with the gated norm where a cluster holds a request
+//   everything else                  mamba_scan_kernel / mamba_scan_five_kernel, one CTA per (request, head), the state staged in fp32
 #include "common.cuh"
 #include "kernels.h"
 
