@@ -296,7 +296,8 @@ gemm_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if constexpr (ARGMAX) {
           // A lane that does not reach its row's maximum so far has nothing to say about the arg-max, and after the first few of a
           // row's tiles hardly one does: the reduction network (64 shuffles for 16 rows) runs for the few groups with one that reaches it.  (For
-          // every group it cost the LM head 4 %, mostly as clock under the power cap; one redux.sync maximum + ballot per column more still.)
+          // every group it cost the LM head 4 %, mostly as clock under the power cap; one redux.sync maximum + ballot per column more still.  Logits that rise along the
+          // vocabulary still run it for every group, equal ones too: within 1 % of the form without the test, 77 rows of 152 064 256 -> 255.5 and 255 -> 254.7 us.)
           const float4* best = tail->best[warp - 2] + (c0 >> 5) * 4;
           bool reached = false;
 #pragma unroll

@@ -590,7 +590,7 @@ def test_gemm_rows_keep_their_bits_among_others(hs, M, others, n_out, K, kind):
                                        (480, 17000, 512), (481, 17000, 8), (512, 17408, 256), (257, 5000, 4096), (270, 4096, 4096), (257, 2560, 4096),
                                        (549, 4096, 8192)])
 @pytest.mark.parametrize("kind,out", [(torch.float16, torch.float32), (torch.float16, torch.float16), (torch.bfloat16, torch.bfloat16), (torch.float16, "add")])
-def test_wide_gemm_tiles(hs, M, n_out, K, kind, out):
+def test_gemm_rows_over_several_tiles(hs, M, n_out, K, kind, out):
     x, W = _rand((M, K), 1, kind), _rand((n_out, K), 2, kind, 0.05)
     add = out == "add"
     y = _rand((M, n_out), 3, torch.float32) if add else torch.full((M, n_out), float("nan"), dtype=out, device="cuda")
@@ -607,7 +607,7 @@ def test_wide_gemm_tiles(hs, M, n_out, K, kind, out):
 
 # the SwiGLU epilogue with several tiles of rows: 300 and 512 rows
 @pytest.mark.parametrize("B,k", [(30, 10), (16, 32)])
-def test_wide_gemm_tiles_with_swiglu(hs, B, k):
+def test_gemm_rows_over_several_tiles_with_swiglu(hs, B, k):
     import synth
     from harness import check_step, cuda_setup
     cfg = synth.derived(dict(D=256, n_fuse=1, r=64, L=1, has_attn=[0], kv_slot=[-1], n_slots=0, Di=512, P=64, N=4, G=1, d_conv=4, dt_rank=0,
